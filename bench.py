@@ -569,8 +569,10 @@ def main():
     n_spmv = (cycles * rms0, int(lvl[1]) * 3)
     np_, S = pr.np_, 2 * pr.d + 1
     N0, N1 = pr.ndof, pr.ndof // (2 ** pr.d)
-    sweep_flop = (2 * ((S - 1) * np_ + np_) * N0, 2 * ((S - 1) * np_ + np_) * N1)
-    spmv_flop = (2 * S * np_ * N0, 2 * S * np_ * N1)
+    # one multiply-add per stored matrix entry (8 bytes): the reported bytes less the vectors'
+    # (the finest level stores and multiplies its blocks' nonzero entries only)
+    sweep_flop = tuple(2 * (rep[k] - 24.0 * n) / 8 for k, n in (("sweep_bytes", N0), ("sweep1_bytes", N1)))
+    spmv_flop = tuple(2 * (rep[k] - 16.0 * n) / 8 for k, n in (("spmv_bytes", N0), ("spmv1_bytes", N1)))
 
     def alu_kernel(name, what, t, n, flop):
         tot_ms = n[0] * t[0] + n[1] * t[1]

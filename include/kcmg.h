@@ -80,7 +80,13 @@ typedef struct {
     const double *blocks;    /* fine operator, [2*dim+1][ncells][np][np] row-major blocks;
                                 slot 0 = diagonal block of the cell, slot 1+2k / 2+2k = the
                                 coupling to the -e_k / +e_k face neighbour (zero where the
-                                neighbour is outside the grid).  Copied at setup. */
+                                neighbour is outside the grid).  Copied at setup.  Blocks with
+                                the zero pattern of a total-degree tensor basis (modes by total
+                                degree, then decreasing power of x, then of y; face blocks couple
+                                modes that differ in the face's direction only, diagonal blocks
+                                modes that differ in at most one) are found at setup, and the
+                                finest level's kernels then skip the zeros; results do not
+                                depend on it. */
     const double *prolong;   /* [2^dim][np][np]: P_k maps coarse modes to the modes of child
                                 k = cx + 2 cy + 4 cz of an agglomerated cell; the same P_k on
                                 every level.  R = P^T; coarse operators are P^T A P. */

@@ -38,6 +38,12 @@ struct Level {
   void *as_inv0 = nullptr, *as_inv1 = nullptr, *as_z = nullptr, *as_r = nullptr;
   // matrix-free level-0 coupling (FP32 sweeps): coefficient per cell, face matrices
   float *mf_nu = nullptr, *mf_F = nullptr;
+  // finest level with a tensor basis's zero pattern: the nonzero entries and the inverses in the
+  // pattern kernels' layout (pattern_ops.cuh); A64, D64, A32, D32, D16 are then not stored
+  bool pat = false;
+  double *V64 = nullptr, *PD64 = nullptr;
+  float *V32 = nullptr, *PD32 = nullptr;
+  __nv_bfloat16* PD16 = nullptr;
   int lcap = 0;
   int nblk = 1;                     // blocks of the multi-column dot kernels
   int nblk2 = 1;                    // blocks of the update / finish / norm kernels
@@ -149,12 +155,36 @@ int level_cells(const int* n, int dim) { return n[0] * n[1] * (dim == 3 ? n[2] :
 
 // operator of a level's residual minimisation and the prolongation matrices, in the
 // level's vector type (FP64; FP32 in the inner solve of the iterative-refinement forms)
-template <typename V> const V* level_op(const Level& L);
-template <> const double* level_op<double>(const Level& L) { return L.A64; }
-template <> const float* level_op<float>(const Level& L) { return L.A32; }
+template <typename V> const V* dense_op(const Level& L);
+template <> const double* dense_op<double>(const Level& L) { return L.A64; }
+template <> const float* dense_op<float>(const Level& L) { return L.A32; }
+template <typename V> const V* pattern_op(const Level& L);
+template <> const double* pattern_op<double>(const Level& L) { return L.V64; }
+template <> const float* pattern_op<float>(const Level& L) { return L.V32; }
 template <typename V> const V* prolong_mats(const kcmg_ctx* c);
 template <> const double* prolong_mats<double>(const kcmg_ctx* c) { return c->P64; }
 template <> const float* prolong_mats<float>(const kcmg_ctx* c) { return c->P32; }
+
+// y = A x (b null) or y = b - A x on a level, with the epilogue's ||y||^2
+template <typename V>
+void apply_op(const kcmg_ctx* c, const Level& L, const V* x, V* y, const V* b, double* partial, const EpiArgs& e,
+              int conditional, cudaStream_t s) {
+  if (L.pat)
+    launch_pattern_spmv<V>(c->np, c->dim, L.n, pattern_op<V>(L), x, y, b, partial, e, conditional, s);
+  else
+    launch_spmv<V>(c->np, c->dim, dense_op<V>(L), L.nbr, L.N, L.G, L.rows_pad, L.block_rows, x, y, b, partial, e,
+                   conditional, s);
+}
+
+// r = b - A x on a level with compensated sums
+void apply_residual_dd(const kcmg_ctx* c, const Level& L, const double* x, double* r, const double* b, double* partial,
+                       const EpiArgs& e, int conditional, cudaStream_t s) {
+  if (L.pat)
+    launch_pattern_residual_dd(c->np, c->dim, L.n, L.V64, x, r, b, partial, e, conditional, s);
+  else
+    launch_residual_dd(c->np, c->dim, L.A64, L.nbr, L.N, L.G, L.rows_pad, L.block_rows, x, r, b, partial, e,
+                       conditional, s);
+}
 
 // ------------------------------------------------------------------ setup
 void setup_level_geometry(kcmg_ctx* ctx, Level& L, int l) {
@@ -192,10 +222,42 @@ void alloc_cycle_vectors(kcmg_ctx* ctx, Level& L, int lcap) {
   const size_t spmv_blocks = L.rows_pad / L.block_rows;
   size_t plen = (size_t)kDotBlocksMax * (lcap + 1);
   if (spmv_blocks > plen) plen = spmv_blocks;
+  if (L.pat) plen = std::max(plen, (size_t)pattern_blocks(ctx->np, ctx->dim, L.ncell));
   if ((size_t)4 * 65536 > plen) plen = 4 * 65536;
   L.partial = dalloc<double>(ctx, plen);
   L.st = dalloc<LevelState>(ctx, 1);
   CK(cudaMemsetAsync(L.st, 0, sizeof(LevelState), ctx->s));
+}
+
+// The finest level's blocks and inverses (natural layout) in the pattern kernels' storage, if
+// every block has the pattern.
+void store_pattern(kcmg_ctx* ctx, Level& L, const double* inv_nat, bool bf16) {
+  const int np = ctx->np, dim = ctx->dim;
+  CK(cudaMemsetAsync(ctx->dflag, 0, sizeof(int), ctx->s));
+  launch_pattern_check(np, dim, L.nat, L.nbr, L.ncell, ctx->dflag, ctx->s);
+  CK(cudaGetLastError());
+  int outside = 0;
+  CK(cudaMemcpyAsync(&outside, ctx->dflag, sizeof(int), cudaMemcpyDeviceToHost, ctx->s));
+  CK(cudaStreamSynchronize(ctx->s));
+  if (outside) return;
+  L.pat = true;
+  const size_t nv = pattern_values(np, dim, L.ncell), ni = pattern_inverse_values(np, dim, L.ncell);
+  L.V64 = dalloc<double>(ctx, nv);
+  launch_pattern_pack<double>(np, dim, L.nat, L.nbr, L.ncell, L.V64, ctx->s);
+  if (!ctx->mixed) {
+    L.PD64 = dalloc<double>(ctx, ni);
+    launch_pattern_pack_inverse<double>(np, dim, inv_nat, L.ncell, L.PD64, ctx->s);
+    return;
+  }
+  L.V32 = dalloc<float>(ctx, nv);
+  launch_pattern_pack<float>(np, dim, L.nat, L.nbr, L.ncell, L.V32, ctx->s);
+  if (bf16) {
+    L.PD16 = dalloc<__nv_bfloat16>(ctx, ni);
+    launch_pattern_pack_inverse<__nv_bfloat16>(np, dim, inv_nat, L.ncell, L.PD16, ctx->s);
+  } else {
+    L.PD32 = dalloc<float>(ctx, ni);
+    launch_pattern_pack_inverse<float>(np, dim, inv_nat, L.ncell, L.PD32, ctx->s);
+  }
 }
 
 void build_hierarchy(kcmg_ctx* ctx, const double* blocks_src) {
@@ -229,14 +291,20 @@ void build_hierarchy(kcmg_ctx* ctx, const double* blocks_src) {
     }
     const size_t opsz = (size_t)S * L.G * ((np + 1) / 2) * 64;
     const size_t invsz = (size_t)L.G * ((np + 1) / 2) * 64;
-    L.A64 = dalloc<double>(ctx, opsz);
-    L.D64 = dalloc<double>(ctx, invsz);
-    launch_interleave<double>(np, S, L.nat, L.ncell, L.G, L.A64, ctx->s);
-    launch_interleave<double>(np, 1, inv_nat, L.ncell, L.G, L.D64, ctx->s);
-    if (ctx->mixed) {
+    const bool bf16 = ctx->p.precision == KCMG_MIXED_BF16INV || ctx->p.precision == KCMG_IR32_BF16INV;
+    if (l == 0) store_pattern(ctx, L, inv_nat, bf16);
+    if (!L.pat) {
+      L.A64 = dalloc<double>(ctx, opsz);
+      L.D64 = dalloc<double>(ctx, invsz);
+      launch_interleave<double>(np, S, L.nat, L.ncell, L.G, L.A64, ctx->s);
+      launch_interleave<double>(np, 1, inv_nat, L.ncell, L.G, L.D64, ctx->s);
+    }
+    if (ctx->mixed && !L.pat) {
       L.A32 = dalloc<float>(ctx, opsz);
       launch_interleave<float>(np, S, L.nat, L.ncell, L.G, L.A32, ctx->s);
-      if (ctx->p.precision == KCMG_MIXED_BF16INV || ctx->p.precision == KCMG_IR32_BF16INV) {
+    }
+    if (ctx->mixed && (!L.pat || ctx->p.mf_nu)) {   // the matrix-free sweeps read this layout
+      if (bf16) {
         L.D16 = dalloc<__nv_bfloat16>(ctx, invsz);
         launch_interleave<__nv_bfloat16>(np, 1, inv_nat, L.ncell, L.G, L.D16, ctx->s);
       } else {
@@ -348,9 +416,6 @@ struct Cycle {
 
   static constexpr bool kMixed = !std::is_same<T0, T>::value;
 
-  const T* Ainner(const Level& L) const;   // operator in T
-  const T* Pm() const;
-
   EpiArgs epi(int lev, int kind) const {
     Level& L = ctx->lv[lev];
     EpiArgs e;
@@ -371,7 +436,7 @@ struct Cycle {
 
   // Alg. AS in T on buffers z/t: per sweep the residual r - A z_old (skipped on the first
   // sweep from z = 0), both partitions' patch solves, and z_new = z_old + omega (z_0 + z_1)
-  T* as_sweeps(const Level& L, const T* r, T* z, T* t, cudaStream_t s) {
+  T* as_sweeps(const Level& L, const T* r, T* z, T* t, T* dst, cudaStream_t s) {
     T* buf[2] = {z, t};
     T* res = static_cast<T*>(L.as_r);
     T* zp = static_cast<T*>(L.as_z);
@@ -379,12 +444,12 @@ struct Cycle {
     const int sw = ctx->p.sweeps;
     const bool bf16 = ctx->p.precision == KCMG_MIXED_BF16INV || ctx->p.precision == KCMG_IR32_BF16INV;
     for (int k = 0; k < sw; ++k) {
-      T* out = buf[k & 1];
+      T* out = k == sw - 1 && dst ? dst : buf[k & 1];
       const T* old = buf[(k + 1) & 1];
       const T* rk = r;
       if (k > 0) {
         launches += 1;
-        launch_spmv<T>(ctx->np, ctx->dim, Ainner(L), L.nbr, L.N, L.G, L.rows_pad, L.block_rows, old, res, r,
+        apply_op<T>(ctx, L, old, res, r,
                        nullptr, EpiArgs{}, 0, s);
         rk = res;
       }
@@ -400,61 +465,89 @@ struct Cycle {
                                       (const float*)rk, (float*)zp, s);
       launch_as_combine<T>(ctx->np, ctx->dim, L.n, L.N, zp, old, out, om, k == 0, s);
     }
-    return buf[(sw - 1) & 1];
+    return dst ? dst : buf[(sw - 1) & 1];
   }
 
-  // the smoother sweeps in T on buffers z/t; returns the buffer holding the result
-  T* sweeps(const Level& L, const T* r, T* z, T* t, cudaStream_t s) {
-    if (ctx->p.smoother == 1) return as_sweeps(L, r, z, t, s);
+  // the smoother sweeps in T on buffers z/t; the result goes to dst if given, else to the
+  // buffer returned
+  T* sweeps(const Level& L, const T* r, T* z, T* t, T* dst, cudaStream_t s) {
+    if (ctx->p.smoother == 1) return as_sweeps(L, r, z, t, dst, s);
     T* buf[2] = {z, t};
     const double om = ctx->p.omega;
     const int sw = ctx->p.sweeps;
     launches += sw;
     for (int k = 0; k < sw; ++k) {
-      T* out = buf[k & 1];
+      T* out = k == sw - 1 && dst ? dst : buf[k & 1];
       const T* old = buf[(k + 1) & 1];
-      if (!std::is_same<T, double>::value && L.mf_nu) {   // level 0, coupling matrix-free
+      if constexpr (std::is_same<T, double>::value) {
+        if (L.pat)
+          launch_pattern_sweep<double, double, double, double>(ctx->np, ctx->dim, L.n, L.V64, L.PD64, r, nullptr, old,
+                                                               out, om, k == 0, s);
+        else
+          launch_bj_sweep<double, double>(ctx->np, ctx->dim, L.A64, L.D64, L.nbr, L.N, L.G, L.rows_pad, L.block_rows,
+                                          r, old, out, om, k == 0, s);
+      } else if (L.mf_nu) {   // level 0, coupling matrix-free
         if (L.D16)
           launch_bj_sweep_mf<__nv_bfloat16>(ctx->np, ctx->dim, L.n, L.mf_nu, L.mf_F, L.D16, L.N, L.rows_pad,
-                                            L.block_rows, (const float*)r, (const float*)old, (float*)out, om,
-                                            k == 0, s);
+                                            L.block_rows, r, old, out, om, k == 0, s);
         else
           launch_bj_sweep_mf<float>(ctx->np, ctx->dim, L.n, L.mf_nu, L.mf_F, L.D32, L.N, L.rows_pad,
-                                    L.block_rows, (const float*)r, (const float*)old, (float*)out, om, k == 0, s);
-      } else if (std::is_same<T, double>::value) {
-        launch_bj_sweep<double, double>(ctx->np, ctx->dim, (const double*)Ainner(L), L.D64, L.nbr, L.N,
-                                        L.G, L.rows_pad, L.block_rows, (const double*)r,
-                                        (const double*)old, (double*)out, om, k == 0, s);
+                                    L.block_rows, r, old, out, om, k == 0, s);
+      } else if (L.pat) {
+        pattern_sweep32<float, float>(L, r, nullptr, old, out, k == 0, s);
       } else if (L.D16) {
-        launch_bj_sweep<float, __nv_bfloat16>(ctx->np, ctx->dim, (const float*)Ainner(L), L.D16, L.nbr,
-                                              L.N, L.G, L.rows_pad, L.block_rows, (const float*)r,
-                                              (const float*)old, (float*)out, om, k == 0, s);
+        launch_bj_sweep<float, __nv_bfloat16>(ctx->np, ctx->dim, L.A32, L.D16, L.nbr, L.N, L.G, L.rows_pad,
+                                              L.block_rows, r, old, out, om, k == 0, s);
       } else {
-        launch_bj_sweep<float, float>(ctx->np, ctx->dim, (const float*)Ainner(L), L.D32, L.nbr, L.N,
-                                      L.G, L.rows_pad, L.block_rows, (const float*)r,
-                                      (const float*)old, (float*)out, om, k == 0, s);
+        launch_bj_sweep<float, float>(ctx->np, ctx->dim, L.A32, L.D32, L.nbr, L.N, L.G, L.rows_pad, L.block_rows, r,
+                                      old, out, om, k == 0, s);
       }
     }
-    return buf[(sw - 1) & 1];
+    return dst ? dst : buf[(sw - 1) & 1];
   }
 
-  // z = BJ(r) from z = 0 on level lev (Alg. BJ); V is the level's vector type
+  // one FP32 pattern sweep with either kind of stored inverse
+  template <typename TR, typename TZ>
+  void pattern_sweep32(const Level& L, const TR* r, float* r_lo, const float* old, TZ* out, bool first,
+                       cudaStream_t s) {
+    if (L.PD16)
+      launch_pattern_sweep<float, __nv_bfloat16, TR, TZ>(ctx->np, ctx->dim, L.n, L.V32, L.PD16, r, r_lo, old, out,
+                                                         ctx->p.omega, first, s);
+    else
+      launch_pattern_sweep<float, float, TR, TZ>(ctx->np, ctx->dim, L.n, L.V32, L.PD32, r, r_lo, old, out,
+                                                 ctx->p.omega, first, s);
+  }
+
+  // z = BJ(r) from z = 0 on level lev (Alg. BJ); V is the level's vector type.  The result goes
+  // to dst if given (dst must not overlap r), else to the level buffer returned.
   template <typename V>
-  V* smooth(int lev, const V* r, cudaStream_t s) {
+  V* smooth(int lev, const V* r, cudaStream_t s, V* dst = nullptr) {
     Level& L = ctx->lv[lev];
-    if (kMixed) {
+    if constexpr (kMixed) {
+      double* z = dst ? (double*)dst : (double*)L.z;
+      const int sw = ctx->p.sweeps;
+      if (L.pat && !L.mf_nu && ctx->p.smoother == 0 && sw > 1) {   // conversions ride in the sweeps
+        float* buf[2] = {L.z_lo, L.t_lo};
+        launches += sw;
+        pattern_sweep32<double, float>(L, (const double*)r, L.r_lo, nullptr, buf[0], true, s);
+        for (int k = 1; k < sw - 1; ++k)
+          pattern_sweep32<float, float>(L, L.r_lo, nullptr, buf[(k + 1) & 1], buf[k & 1], false, s);
+        pattern_sweep32<float, double>(L, L.r_lo, nullptr, buf[sw & 1], z, false, s);
+        return (V*)z;
+      }
       launches += 2;
       launch_convert<double, float>((const double*)r, L.r_lo, L.N, s);
-      const float* out = (const float*)sweeps(L, (const T*)L.r_lo, (T*)L.z_lo, (T*)L.t_lo, s);
-      launch_convert<float, double>(out, (double*)L.z, L.N, s);
-      return static_cast<V*>(L.z);
+      const float* out = (const float*)sweeps(L, (const T*)L.r_lo, (T*)L.z_lo, (T*)L.t_lo, nullptr, s);
+      launch_convert<float, double>(out, z, L.N, s);
+      return (V*)z;
+    } else {
+      return (V*)sweeps(L, (const T*)r, static_cast<T*>(L.z), static_cast<T*>(L.t), (T*)dst, s);
     }
-    return (V*)sweeps(L, (const T*)r, static_cast<T*>(L.z), static_cast<T*>(L.t), s);
   }
 
-  // Alg. 1 on level lev with correction z (vectors in V, operator Aop)
+  // Alg. 1 on level lev with correction z (vectors in V)
   template <typename V>
-  void rm(int lev, const V* Aop, const V* z, int end_iter, int htype, cudaStream_t s) {
+  void rm(int lev, const V* z, int end_iter, int htype, cudaStream_t s) {
     Level& L = ctx->lv[lev];
     V* W = static_cast<V*>(L.W);
     V* Z = static_cast<V*>(L.Z);
@@ -462,7 +555,7 @@ struct Cycle {
     V* wre = static_cast<V*>(L.wre);
     EpiArgs none = epi(lev, EPI_NONE);
     launches += 6;
-    launch_spmv<V>(ctx->np, ctx->dim, Aop, L.nbr, L.N, L.G, L.rows_pad, L.block_rows, z, w,
+    apply_op<V>(ctx, L, z, w,
                    nullptr, L.partial, none, 0, s);
     launch_gram_dots<V>(W, L.N, w, L.lcap, L.nblk, L.partial, epi(lev, EPI_GRAM1), 0, s);
     launch_gram_apply<V>(W, L.N, w, wre, L.lcap, L.nblk2, L.st, L.h, s);
@@ -478,11 +571,11 @@ struct Cycle {
 
   // one pass of the while body of Alg. 2 on level lev; V is the level's vector type
   template <typename V>
-  void body(int lev, const V* Aop, cudaStream_t s) {
+  void body(int lev, cudaStream_t s) {
     Level& L = ctx->lv[lev];
     Level& C = ctx->lv[lev + 1];
     V* z = smooth<V>(lev, static_cast<V*>(L.r), s);                       // pre-smoother
-    rm<V>(lev, Aop, z, 0, 1, s);
+    rm<V>(lev, z, 0, 1, s);
     launches += 3;                                                         // transfers, restart check
     if (lev + 1 == ctx->nlev - 1) {                                        // direct solve
       launches += 1;
@@ -509,22 +602,20 @@ struct Cycle {
       launch_restrict<V, V>(ctx->np, ctx->dim, L.n, C.n, prolong_mats<V>(ctx), static_cast<V*>(L.r),
                             static_cast<V*>(C.b), static_cast<V*>(C.r), static_cast<V*>(C.x),
                             C.partial, epi(lev + 1, EPI_MG_BEGIN), s);
-      loop<V>(lev + 1, level_op<V>(C), s);
+      loop<V>(lev + 1, s);
     }
     launch_prolong<V, V>(ctx->np, ctx->dim, L.n, C.n, prolong_mats<V>(ctx), static_cast<V*>(C.x),
                          static_cast<V*>(L.z), s);                         // z = P z_c
-    rm<V>(lev, Aop, static_cast<V*>(L.z), 0, 2, s);
+    rm<V>(lev, static_cast<V*>(L.z), 0, 2, s);
     z = smooth<V>(lev, static_cast<V*>(L.r), s);                           // post-smoother
-    rm<V>(lev, Aop, z, 1, 3, s);
+    rm<V>(lev, z, 1, 3, s);
     // restart check: r = b - A x on request, then the loop condition of this level
     // (compensated on level 0, where the tolerance can sit near the attainable accuracy)
     if (lev == 0 && std::is_same<V, double>::value)
-      launch_residual_dd(ctx->np, ctx->dim, (const double*)Aop, L.nbr, L.N, L.G, L.rows_pad, L.block_rows,
-                         (const double*)L.x, (double*)L.r, (const double*)L.b, L.partial,
+      apply_residual_dd(ctx, L, (const double*)L.x, (double*)L.r, (const double*)L.b, L.partial,
                          epi(lev, EPI_RESTART), 1, s);
     else
-      launch_spmv<V>(ctx->np, ctx->dim, Aop, L.nbr, L.N, L.G, L.rows_pad, L.block_rows,
-                     static_cast<V*>(L.x), static_cast<V*>(L.r), static_cast<V*>(L.b), L.partial,
+      apply_op<V>(ctx, L, static_cast<V*>(L.x), static_cast<V*>(L.r), static_cast<V*>(L.b), L.partial,
                      epi(lev, EPI_RESTART), 1, s);
   }
 
@@ -535,7 +626,7 @@ struct Cycle {
   // with zc closes the cycle.  The two paths share no buffer: the smoother path writes the
   // level-0 z, t, w, W, Z, x, r and state, the coarse path level >= 1 buffers and zc.
   template <typename V>
-  void body_async(const V* Aop, cudaStream_t s) {
+  void body_async(cudaStream_t s) {
     Level& L = ctx->lv[0];
     Level& C = ctx->lv[1];
     cudaStream_t cs = ctx->cap[KCMG_MAX_LEVELS + 1];
@@ -568,7 +659,7 @@ struct Cycle {
     // smoother path first, so that host-driven coarse control overlaps it
     for (int k = 0; k < ctx->p.async_smooth; ++k) {
       V* z = smooth<V>(0, static_cast<V*>(L.r), s);
-      rm<V>(0, Aop, z, 0, 1, s);
+      rm<V>(0, z, 0, 1, s);
     }
     // coarse path
     if (direct) {
@@ -578,22 +669,20 @@ struct Cycle {
       launches += 1;
       launch_coarse(ctx, cs);
     } else {
-      loop<V>(1, level_op<V>(C), cs);
+      loop<V>(1, cs);
     }
     launches += 1;
     launch_prolong<V, V>(ctx->np, ctx->dim, L.n, C.n, prolong_mats<V>(ctx), static_cast<V*>(C.x),
                          reinterpret_cast<V*>(ctx->zc), cs);                // z_cor = P z_c
     CK(cudaEventRecord(ctx->join_ev, cs));                               // join
     CK(cudaStreamWaitEvent(s, ctx->join_ev, 0));
-    rm<V>(0, Aop, reinterpret_cast<const V*>(ctx->zc), 1, 2, s);
+    rm<V>(0, reinterpret_cast<const V*>(ctx->zc), 1, 2, s);
     launches += 1;                                                       // restart check
     if (std::is_same<V, double>::value)
-      launch_residual_dd(ctx->np, ctx->dim, (const double*)Aop, L.nbr, L.N, L.G, L.rows_pad, L.block_rows,
-                         (const double*)L.x, (double*)L.r, (const double*)L.b, L.partial,
+      apply_residual_dd(ctx, L, (const double*)L.x, (double*)L.r, (const double*)L.b, L.partial,
                          epi(0, EPI_RESTART), 1, s);
     else
-      launch_spmv<V>(ctx->np, ctx->dim, Aop, L.nbr, L.N, L.G, L.rows_pad, L.block_rows,
-                     static_cast<V*>(L.x), static_cast<V*>(L.r), static_cast<V*>(L.b), L.partial,
+      apply_op<V>(ctx, L, static_cast<V*>(L.x), static_cast<V*>(L.r), static_cast<V*>(L.b), L.partial,
                      epi(0, EPI_RESTART), 1, s);
   }
 
@@ -611,12 +700,12 @@ struct Cycle {
 
   // while (cond_lev) body(lev): host-driven, or a conditional while node when capturing
   template <typename V>
-  void loop(int lev, const V* Aop, cudaStream_t s) {
+  void loop(int lev, cudaStream_t s) {
     const bool task_parallel = lev == 0 && ctx->p.async_smooth > 0;
     if (!capture) {
       while (read_cond(lev, s)) {
-        if (task_parallel) body_async<V>(Aop, s);
-        else body<V>(lev, Aop, s);
+        if (task_parallel) body_async<V>(s);
+        else body<V>(lev, s);
       }
       return;
     }
@@ -640,8 +729,8 @@ struct Cycle {
                                      cudaStreamCaptureModeRelaxed));
     const long long before = launches;
     loop_total[lev + 1] = 0;
-    if (task_parallel) body_async<V>(Aop, bs);
-    else body<V>(lev, Aop, bs);
+    if (task_parallel) body_async<V>(bs);
+    else body<V>(lev, bs);
     loop_total[lev] = launches - before;
     body_kernels[lev] = loop_total[lev] - loop_total[lev + 1];
     if (lev == 0) body_launches = launches - before;
@@ -663,23 +752,14 @@ struct Cycle {
       CK(cudaGraphConditionalHandleCreate(&handle[0], g, 0, 0));
     }
     if (std::is_same<T0, double>::value)
-      launch_residual_dd(ctx->np, ctx->dim, L.A64, L.nbr, L.N, L.G, L.rows_pad, L.block_rows,
-                         static_cast<double*>(L.x), static_cast<double*>(L.r), static_cast<double*>(L.b),
+      apply_residual_dd(ctx, L, static_cast<double*>(L.x), static_cast<double*>(L.r), static_cast<double*>(L.b),
                          L.partial, epi(0, EPI_MG_BEGIN), 0, s);
     else
-      launch_spmv<T0>(ctx->np, ctx->dim, level_op<T0>(L), L.nbr, L.N, L.G, L.rows_pad, L.block_rows,
-                      static_cast<T0*>(L.x), static_cast<T0*>(L.r), static_cast<T0*>(L.b), L.partial,
+      apply_op<T0>(ctx, L, static_cast<T0*>(L.x), static_cast<T0*>(L.r), static_cast<T0*>(L.b), L.partial,
                       epi(0, EPI_MG_BEGIN), 0, s);
-    loop<T0>(0, level_op<T0>(L), s);
+    loop<T0>(0, s);
   }
 };
-
-template <> const double* Cycle<double, double>::Ainner(const Level& L) const { return L.A64; }
-template <> const float* Cycle<double, float>::Ainner(const Level& L) const { return L.A32; }
-template <> const double* Cycle<double, double>::Pm() const { return ctx->P64; }
-template <> const float* Cycle<double, float>::Pm() const { return ctx->P32; }
-template <> const float* Cycle<float, float>::Ainner(const Level& L) const { return L.A32; }
-template <> const float* Cycle<float, float>::Pm() const { return ctx->P32; }
 
 // host copy of the level states before a cycle
 void init_states(kcmg_ctx* ctx, double rtol0, double atol0, int maxit0) {
@@ -754,7 +834,7 @@ double fp64_residual(kcmg_ctx* ctx, const double* x, const double* b, double* r)
   e.st = L.st;  // only its reduction ticket is used
   e.kind = EPI_NORM;
   e.out = ctx->scal;
-  launch_residual_dd(ctx->np, ctx->dim, L.A64, L.nbr, L.N, L.G, L.rows_pad, L.block_rows, x, r, b,
+  apply_residual_dd(ctx, L, x, r, b,
                      L.partial, e, 0, ctx->s);
   CK(cudaGetLastError());
   double v = 0;
@@ -1267,6 +1347,7 @@ kcmg_ctx* build_ctx(const kcmg_params* p, cudaStream_t user, const double* block
     ctx->stage_out = dalloc<double>(ctx, maxN);
     // the no-allocation residual's static scratch on this device (address and kernels)
     CK(noalloc_prepare(dev, &ctx->na_scratch));
+    if (ctx->lv[0].pat) CK(pattern_residual_load(ctx->np, ctx->dim));
     CK(cudaStreamSynchronize(ctx->s));
     *out_status = KCMG_OK;
     return ctx;
@@ -1293,6 +1374,24 @@ void store_vec(kcmg_ctx* ctx, int lev, double* dst, const void* src, size_t n) {
   else CK(cudaMemcpyAsync(ctx->stage_out, src, n * sizeof(double), cudaMemcpyDeviceToDevice, ctx->s));
   copy_out(ctx, dst, ctx->stage_out, n);
   CK(cudaStreamSynchronize(ctx->s));
+}
+
+// Whether a component call can read in and write out (n doubles each) where they are, without
+// staging: both in the context's device memory, on the 16-byte boundary the kernels' vector loads
+// need, and not overlapping (the kernels read a cell's neighbours after other cells are written).
+bool in_place_ok(const kcmg_ctx* ctx, const void* in, const void* out, size_t n) {
+  const uintptr_t a = (uintptr_t)in, b = (uintptr_t)out, len = n * sizeof(double);
+  if ((a | b) & 15 || (a < b + len && b < a + len)) return false;
+  for (const void* p : {in, out}) {
+    cudaPointerAttributes at;
+    const bool ok = cudaPointerGetAttributes(&at, p) == cudaSuccess && at.type == cudaMemoryTypeDevice &&
+                    at.device == ctx->dev;
+    if (!ok) {
+      cudaGetLastError();
+      return false;
+    }
+  }
+  return true;
 }
 
 template <typename F>
@@ -1389,21 +1488,26 @@ kcmg_status kcmg_apply(kcmg_ctx* ctx, int level, int op, const double* x, double
     REQUIRE(level >= 0 && level < ctx->nlev && x && y, "bad level or null vector");
     REQUIRE(op == 0 || (op == 1 && ctx->mixed), "op 1 needs a mixed-precision context");
     Level& L = ctx->lv[level];
-    copy_in(ctx, ctx->stage_in, x, L.N);
+    const bool direct = in_place_ok(ctx, x, y, L.N);
+    const double* xi = x;
+    double* yo = y;
+    if (!direct) {
+      copy_in(ctx, ctx->stage_in, x, L.N);
+      xi = ctx->stage_in;
+      yo = ctx->stage_out;
+    }
     EpiArgs none;
     if (op == 0) {
-      launch_spmv<double>(ctx->np, ctx->dim, L.A64, L.nbr, L.N, L.G, L.rows_pad, L.block_rows,
-                          ctx->stage_in, ctx->stage_out, nullptr, nullptr, none, 0, ctx->s);
+      apply_op<double>(ctx, L, xi, yo, nullptr, nullptr, none, 0, ctx->s);
     } else {
-      float* xi = ctx->lv[0].r_lo;    // FP32 scratch of the finest size
-      float* yi = ctx->lv[0].z_lo;     // (the inner-precision operator of the mixed forms)
-      launch_convert<double, float>(ctx->stage_in, xi, L.N, ctx->s);
-      launch_spmv<float>(ctx->np, ctx->dim, L.A32, L.nbr, L.N, L.G, L.rows_pad, L.block_rows, xi,
-                         yi, nullptr, nullptr, none, 0, ctx->s);
-      launch_convert<float, double>(yi, ctx->stage_out, L.N, ctx->s);
+      float* xf = ctx->lv[0].r_lo;    // FP32 scratch of the finest size
+      float* yf = ctx->lv[0].z_lo;     // (the inner-precision operator of the mixed forms)
+      launch_convert<double, float>(xi, xf, L.N, ctx->s);
+      apply_op<float>(ctx, L, xf, yf, nullptr, nullptr, none, 0, ctx->s);
+      launch_convert<float, double>(yf, yo, L.N, ctx->s);
     }
     CK(cudaGetLastError());
-    copy_out(ctx, y, ctx->stage_out, L.N);
+    if (!direct) copy_out(ctx, y, ctx->stage_out, L.N);
     CK(cudaStreamSynchronize(ctx->s));
     return KCMG_OK;
   });
@@ -1413,6 +1517,13 @@ kcmg_status kcmg_smooth(kcmg_ctx* ctx, int level, const double* r, double* z) {
   return guarded(ctx, [&]() -> kcmg_status {
     REQUIRE(level >= 0 && level < ctx->nlev - 1 && r && z, "bad level or null vector");
     Level& L = ctx->lv[level];
+    if (!ctx->ir && in_place_ok(ctx, r, z, L.N)) {   // on the caller's vectors
+      if (ctx->mixed) Cycle<double, float>{ctx}.smooth<double>(level, r, ctx->s, z);
+      else Cycle<double, double>{ctx}.smooth<double>(level, r, ctx->s, z);
+      CK(cudaGetLastError());
+      CK(cudaStreamSynchronize(ctx->s));
+      return KCMG_OK;
+    }
     load_vec(ctx, level, L.b, r, L.N);
     const void* out;
     if (ctx->ir) {
@@ -1494,13 +1605,11 @@ template <typename T0, typename T, typename V>
 void rm_sequence_impl(kcmg_ctx* ctx, int level, const double* z, int ncorr) {
   Level& L = ctx->lv[level];
   Cycle<T0, T> cy{ctx};
-  const V* Aop = level_op<V>(L);
-  launch_spmv<V>(ctx->np, ctx->dim, Aop, L.nbr, L.N, L.G, L.rows_pad, L.block_rows,
-                 static_cast<V*>(L.x), static_cast<V*>(L.r), static_cast<V*>(L.b), L.partial,
+  apply_op<V>(ctx, L, static_cast<V*>(L.x), static_cast<V*>(L.r), static_cast<V*>(L.b), L.partial,
                  cy.epi(level, EPI_MG_BEGIN), 0, ctx->s);
   for (int k = 0; k < ncorr; ++k) {
     load_vec(ctx, level, L.z, z + (size_t)k * L.N, L.N);
-    cy.template rm<V>(level, Aop, static_cast<V*>(L.z), 0, 1, ctx->s);
+    cy.template rm<V>(level, static_cast<V*>(L.z), 0, 1, ctx->s);
   }
 }
 }  // namespace
@@ -1609,20 +1718,20 @@ kcmg_status kcmg_kernel_report(kcmg_ctx* ctx, int reps, double* out, int nout) {
         CK(cudaEventRecord(e0, ctx->s));
         for (int k = 0; k < reps; ++k) {
           if (ctx->ir)
-            launch_spmv<float>(np, ctx->dim, L.A32, L.nbr, L.N, L.G, L.rows_pad, L.block_rows,
-                               static_cast<float*>(L.t), static_cast<float*>(L.w), nullptr, nullptr, none, 0, ctx->s);
+            apply_op<float>(ctx, L, static_cast<float*>(L.t), static_cast<float*>(L.w), nullptr, nullptr, none, 0, ctx->s);
           else
-            launch_spmv<double>(np, ctx->dim, L.A64, L.nbr, L.N, L.G, L.rows_pad, L.block_rows,
-                                static_cast<double*>(L.t), static_cast<double*>(L.w), nullptr, nullptr, none, 0, ctx->s);
+            apply_op<double>(ctx, L, static_cast<double*>(L.t), static_cast<double*>(L.w), nullptr, nullptr, none, 0, ctx->s);
         }
         CK(cudaEventRecord(e1, ctx->s));
         CK(cudaEventSynchronize(e1));
         float ms = 0;
         CK(cudaEventElapsedTime(&ms, e0, e1));
         out[o] = ms / reps;
-        out[o + 1] = (double)S * L.N * np * vb + 2.0 * L.N * vb;
+        // stored entries of the operator (the zero pattern's only, or every entry)
+        const double ents = L.pat ? (double)pattern_values(np, ctx->dim, L.ncell) : (double)S * L.N * np;
+        out[o + 1] = ents * vb + 2.0 * L.N * vb;
         const double sb = ctx->mixed ? 4 : 8;
-        const double ib = !ctx->mixed ? 8 : ((L.D16 || ctx->p.precision == KCMG_IR32_BF16INV) ? 2 : 4);
+        const double ib = !ctx->mixed ? 8 : ((L.D16 || L.PD16) ? 2 : 4);
         if (ctx->mixed) {
           CK(cudaMemsetAsync(L.r_lo, 0, L.N * sizeof(float), ctx->s));
           CK(cudaMemsetAsync(L.t_lo, 0, L.N * sizeof(float), ctx->s));
@@ -1636,14 +1745,14 @@ kcmg_status kcmg_kernel_report(kcmg_ctx* ctx, int reps, double* out, int nout) {
           for (int k = 0; k < reps; ++k) {
             if (!ctx->mixed) {
               const double *r = static_cast<double*>(L.b), *zo = static_cast<double*>(L.t);
-              launch_spmv<double>(np, ctx->dim, L.A64, L.nbr, L.N, L.G, L.rows_pad, L.block_rows, zo,
+              apply_op<double>(ctx, L, zo,
                                   static_cast<double*>(L.as_r), r, nullptr, EpiArgs{}, 0, ctx->s);
               launch_as_patch<double, double>(np, ctx->dim, L.n, (const double*)L.as_inv0, (const double*)L.as_inv1,
                                               static_cast<double*>(L.as_r), static_cast<double*>(L.as_z), ctx->s);
               launch_as_combine<double>(np, ctx->dim, L.n, L.N, static_cast<double*>(L.as_z), zo,
                                         static_cast<double*>(L.z), ctx->p.omega, 0, ctx->s);
             } else {
-              launch_spmv<float>(np, ctx->dim, L.A32, L.nbr, L.N, L.G, L.rows_pad, L.block_rows, L.t_lo,
+              apply_op<float>(ctx, L, L.t_lo,
                                  static_cast<float*>(L.as_r), L.r_lo, nullptr, EpiArgs{}, 0, ctx->s);
               if (b16)
                 launch_as_patch<float, __nv_bfloat16>(np, ctx->dim, L.n, (const __nv_bfloat16*)L.as_inv0,
@@ -1668,7 +1777,11 @@ kcmg_status kcmg_kernel_report(kcmg_ctx* ctx, int reps, double* out, int nout) {
         }
         CK(cudaEventRecord(e0, ctx->s));
         for (int k = 0; k < reps; ++k) {
-          if (!ctx->mixed)
+          if (!ctx->mixed && L.pat)
+            launch_pattern_sweep<double, double, double, double>(
+                np, ctx->dim, L.n, L.V64, L.PD64, static_cast<double*>(L.b), nullptr, static_cast<double*>(L.t),
+                static_cast<double*>(L.z), ctx->p.omega, 0, ctx->s);
+          else if (!ctx->mixed)
             launch_bj_sweep<double, double>(np, ctx->dim, L.A64, L.D64, L.nbr, L.N, L.G, L.rows_pad, L.block_rows,
                                             static_cast<double*>(L.b), static_cast<double*>(L.t),
                                             static_cast<double*>(L.z), ctx->p.omega, 0, ctx->s);
@@ -1678,6 +1791,8 @@ kcmg_status kcmg_kernel_report(kcmg_ctx* ctx, int reps, double* out, int nout) {
           else if (L.mf_nu)
             launch_bj_sweep_mf<float>(np, ctx->dim, L.n, L.mf_nu, L.mf_F, L.D32, L.N, L.rows_pad, L.block_rows,
                                       L.r_lo, L.t_lo, L.z_lo, ctx->p.omega, 0, ctx->s);
+          else if (L.pat)
+            Cycle<double, float>{ctx}.pattern_sweep32<float, float>(L, L.r_lo, nullptr, L.t_lo, L.z_lo, false, ctx->s);
           else if (L.D16)
             launch_bj_sweep<float, __nv_bfloat16>(np, ctx->dim, L.A32, L.D16, L.nbr, L.N, L.G, L.rows_pad,
                                                   L.block_rows, L.r_lo, L.t_lo, L.z_lo, ctx->p.omega, 0, ctx->s);
@@ -1689,8 +1804,10 @@ kcmg_status kcmg_kernel_report(kcmg_ctx* ctx, int reps, double* out, int nout) {
         CK(cudaEventSynchronize(e1));
         CK(cudaEventElapsedTime(&ms, e0, e1));
         out[o + 2] = ms / reps;
+        // entries of the coupling blocks
+        const double pattern_coupling = L.pat ? (double)pattern_coupling_values(np, ctx->dim, L.ncell) : 0.0;
         out[o + 3] = L.mf_nu ? (double)L.ncell * 4 + (double)L.N * np * ib + 3.0 * L.N * sb   // coefficient,
-                             : (double)(S - 1) * L.N * np * sb + (double)L.N * np * ib + 3.0 * L.N * sb;  // inverses, vectors
+                             : (L.pat ? pattern_coupling : (double)(S - 1) * L.N * np) * sb + (double)L.N * np * ib + 3.0 * L.N * sb;  // inverses, vectors
       };
       time_level(0, 3);
       const int o1 = 7 + KCMG_MAX_LEVELS + kCoarsePhases;
@@ -1780,8 +1897,8 @@ kcmg_status kcmg_residual_noalloc(kcmg_ctx* ctx, const double* b, const double* 
       REQUIRE(dev, "kcmg_residual_noalloc: b, x and r must be device memory");
     }
     const Level& L = ctx->lv[0];
-    Level0View v{L.A64, L.nbr, L.N, L.G, L.rows_pad, L.block_rows, ctx->np, ctx->dim, ctx->s,
-                 ctx->na_scratch};
+    Level0View v{L.pat ? L.V64 : L.A64, L.nbr, L.N, L.G, L.rows_pad, L.block_rows, ctx->np, ctx->dim, ctx->s,
+                 ctx->na_scratch, L.pat, {L.n[0], L.n[1], L.n[2]}};
     // run on the context's device (its scratch address, operator and stream live there)
     int cur = 0;
     CK(cudaGetDevice(&cur));

@@ -126,6 +126,31 @@ void launch_axpy_to_double(const T* e, double* x, size_t n, cudaStream_t s); // 
 void launch_scale_to_float(const double* src, float* dst, double a, size_t n, cudaStream_t s);
 void launch_axpy_scaled_to_double(const float* e, double* x, double a, size_t n, cudaStream_t s);
 
+// the finest level's operator and sweeps over the nonzero entries only, for operators whose
+// blocks have a tensor basis's zero pattern (pattern_ops.cuh); n: cells per direction
+int pattern_blocks(int np, int dim, int C);               // blocks of a launch (partial sums)
+size_t pattern_values(int np, int dim, int C);            // stored operator entries
+size_t pattern_coupling_values(int np, int dim, int C);   // nonzero entries of the coupling blocks
+size_t pattern_inverse_values(int np, int dim, int C);    // stored inverse entries
+void launch_pattern_check(int np, int dim, const double* nat, const int* nbr, int C, int* outside, cudaStream_t s);
+template <typename T>
+void launch_pattern_pack(int np, int dim, const double* nat, const int* nbr, int C, T* V, cudaStream_t s);
+template <typename TI>
+void launch_pattern_pack_inverse(int np, int dim, const double* inv, int C, TI* D, cudaStream_t s);
+template <typename T>
+void launch_pattern_spmv(int np, int dim, const int* n, const T* V, const T* x, T* y, const T* b, double* partial,
+                         const EpiArgs& e, int conditional, cudaStream_t s);
+void launch_pattern_residual_dd(int np, int dim, const int* n, const double* V, const double* x, double* r,
+                                const double* b, double* partial, const EpiArgs& e, int conditional, cudaStream_t s);
+// TR, TZ: the residual's and the correction's type; FP32 sweeps take an FP64 residual in the
+// first sweep (which leaves the FP32 copy in r_lo) and can write an FP64 correction in the others
+template <typename T, typename TI, typename TR, typename TZ>
+void launch_pattern_sweep(int np, int dim, const int* n, const T* V, const TI* D, const TR* r, T* r_lo, const T* zold,
+                          TZ* znew, double omega, int first, cudaStream_t s);
+void launch_pattern_residual_scratch(int np, int dim, const int* n, const double* V, const double* x, const double* b,
+                                     double* r, double* scratch, int norm_at, cudaStream_t s);
+cudaError_t pattern_residual_load(int np, int dim);       // load that kernel's code now
+
 // additive Schwarz smoother on cell patches (schwarz.cu, schwarz.cuh)
 cudaError_t launch_patch_inverse(int np, int dim, const double* nat, const int* nbr, const int* n, int part,
                                  double* invT, int* fail, cudaStream_t s);
@@ -238,6 +263,8 @@ struct Level0View {
   int N, G, rows_pad, block_rows, np, dim;
   cudaStream_t stream;
   double* scratch;   // device address of the static scratch (from noalloc_prepare)
+  bool pat;          // A holds the pattern kernels' storage
+  int n[3];
 };
 // With device dev current: look up the static scratch's device address (once per device)
 // and load the no-allocation kernels.  Called by kcmg_setup.

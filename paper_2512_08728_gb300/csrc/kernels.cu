@@ -3,8 +3,7 @@
 // Operator application, block-Jacobi sweeps, transfers, the coarsest solve, the Gram /
 // residual-minimisation kernels of Alg. 1, the device-side loop control of Alg. 2 and
 // the setup kernels (Galerkin product, block inverses, dense coarsest inverse).
-#include "kcmg_internal.h"
-#include "reduce.cuh"
+#include "epilogue.cuh"
 
 #include <cmath>
 
@@ -38,158 +37,6 @@ template <> struct InvPair<__nv_bfloat16> {
     return __bfloat1622float2(v);
   }
 };
-
-// Sum over the block with a fixed shuffle/shared-memory tree (deterministic).
-// Result valid in thread 0.  sh: >= 32 doubles of shared memory.
-__device__ __forceinline__ double block_sum(double v, double* sh) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x >> 5, ln = threadIdx.x & 31;
-  __syncthreads();
-  if (ln == 0) sh[w] = v;
-  __syncthreads();
-  double r = 0.0;
-  if (w == 0) {
-    const int nw = (blockDim.x + 31) >> 5;
-    r = (ln < nw) ? sh[ln] : 0.0;
-#pragma unroll
-    for (int o = 16; o; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
-  }
-  return r;
-}
-
-// True in every thread of the block that finished last (all partials visible).
-__device__ __forceinline__ bool last_block(unsigned int* ticket) {
-  __shared__ int s_last;
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = (atomicAdd(ticket, 1u) == gridDim.x - 1);
-  __syncthreads();
-  if (s_last) __threadfence();
-  return s_last != 0;
-}
-
-// Final reduction of few columns: out[c] = sum_b partial[b*ncol + c] (fixed order).
-__device__ void reduce_few(const double* partial, int nblk, int ncol, double* out, double* sh) {
-  for (int c = 0; c < ncol; ++c) {
-    double s = 0.0;
-    for (int b = threadIdx.x; b < nblk; b += blockDim.x) s += __ldcg(partial + (size_t)b * ncol + c);
-    s = block_sum(s, sh);
-    if (threadIdx.x == 0) out[c] = s;
-  }
-  __syncthreads();
-}
-
-__device__ __forceinline__ void set_cond(const EpiArgs& e, int c) {
-  e.st->cond = c;
-  if (e.use_handle) cudaGraphSetConditional(e.handle, c ? 1u : 0u);
-}
-
-// Loop condition of Alg. 2 on a level.  The guard (loop bodies executed in this solve,
-// counted outside the reductions) bounds every while loop independently of the rest.
-__device__ __forceinline__ int more_cycles(const LevelState* st) {
-  return (st->rnorm > st->eps) && (st->it < st->maxit) && (st->status == KCMG_OK) &&
-         (st->guard < st->guard_cap);
-}
-
-__device__ __forceinline__ void record(const EpiArgs& e, int type) {
-  LevelState* st = e.st;
-  if (st->level == 0 && e.hist && st->hist_len < st->hist_cap) {
-    e.hist[st->hist_len] = st->rnorm;
-    e.hist_type_buf[st->hist_len] = type;
-    st->hist_len++;
-  }
-}
-
-// Epilogues run by thread 0 of the last block with the reduced sums.
-__device__ void epilogue(const EpiArgs& e, const double* sums) {
-  LevelState* st = e.st;
-  switch (e.kind) {
-    case EPI_MG_BEGIN: {
-      st->rnorm0 = st->rnorm = sqrt(sums[0]);
-      st->eps = fmax(st->rtol * st->rnorm0, st->atol);
-      st->l = 0; st->it = 0; st->flags = 0; st->breakdowns = 0; st->restart_req = 0;
-      if (!isfinite(st->rnorm)) st->status = KCMG_NONFINITE;
-      record(e, 0);
-      set_cond(e, more_cycles(st));
-    } break;
-    case EPI_GRAM1: {
-      const int l = st->l;
-      double hh = 0.0;
-      for (int i = 0; i < l; ++i) { e.h[i] = sums[i]; hh += sums[i] * sums[i]; }
-      const double naz2 = sums[l];
-      st->naz2 = naz2;
-      int f = 0;
-      // Pythagoras estimate of ||w - W h||^2; reorthogonalise when it fell below a
-      // quarter of ||w||^2 (a second Gram-Schmidt pass, "twice is enough")
-      if (l > 0 && naz2 - hh < 0.25 * naz2) f |= F_REORTH;
-      if (!isfinite(naz2) || !(naz2 > 0.0)) f |= F_DISCARD;
-      st->flags = f;
-    } break;
-    case EPI_GRAM2: {
-      for (int i = 0; i < st->l; ++i) e.h2[i] = sums[i];
-    } break;
-    case EPI_UPDATE: {
-      const double nw = sqrt(sums[0]), naz = sqrt(st->naz2);
-      if ((st->flags & F_DISCARD) || !isfinite(nw) || !(nw > st->brk * naz)) {
-        st->flags |= F_DISCARD;
-        if (!isfinite(nw) && st->level == 0) st->status = KCMG_NONFINITE;
-      } else {
-        st->gamma = 1.0 / nw;
-        st->alpha = st->gamma * sums[1];   // alpha = (gamma w_hat) . r
-      }
-    } break;
-    case EPI_FINISH: {
-      if (!(st->flags & F_DISCARD)) {
-        st->l++;
-        st->breakdowns = 0;
-      } else if (st->level == 0) {
-        if (++st->breakdowns >= 2 && st->status == KCMG_OK) st->status = KCMG_BREAKDOWN;
-      }
-      st->rnorm = sqrt(sums[0]);
-      if (!isfinite(st->rnorm) && st->status == KCMG_OK) st->status = KCMG_NONFINITE;
-      record(e, e.hist_type);
-      if (e.end_iter) {
-        st->it++;
-        st->iters_total++;
-        const int cap = (st->lmax > 0 && st->lmax < st->lcap) ? st->lmax : st->lcap;
-        if (st->level == 0 && !(st->rnorm > st->eps) && st->l > 0) st->restart_req = 1;
-        if (st->l + st->per_cycle > cap) st->restart_req = 1;
-      }
-    } break;
-    case EPI_RESTART: {
-      st->rnorm = sqrt(sums[0]);
-      st->l = 0;
-      st->restart_req = 0;
-      st->nrestart++;
-      if (!isfinite(st->rnorm) && st->status == KCMG_OK) st->status = KCMG_NONFINITE;
-      record(e, 4);
-      set_cond(e, more_cycles(st));
-    } break;
-    case EPI_NORM: {
-      if (e.out) *e.out = sqrt(sums[0]);
-    } break;
-    default: break;
-  }
-}
-
-// Write this block's partial sums, and if last, reduce and run the epilogue.
-template <int NC>
-__device__ __forceinline__ void finish_reduction(double (&v)[NC], double* partial, const EpiArgs& e,
-                                                 double* sh) {
-  bsum_n<NC>(v, sh);
-  if (threadIdx.x == 0)
-#pragma unroll
-    for (int c = 0; c < NC; ++c) partial[(size_t)blockIdx.x * NC + c] = v[c];
-  if (last_block(&e.st->ticket)) {
-    __shared__ double sums[NC];
-    reduce_few(partial, gridDim.x, NC, sums, sh);
-    if (threadIdx.x == 0) {
-      epilogue(e, sums);
-      e.st->ticket = 0u;
-    }
-  }
-}
 
 // ------------------------------------------------------------------ operator kernels
 // y = A x (or y = b - A x), one thread per DOF row, optional ||y||^2 with an epilogue.
@@ -245,16 +92,7 @@ __global__ void __launch_bounds__(320)
 k_residual_dd(const double* __restrict__ A, const int* __restrict__ nbr, int N, int G,
               const double* __restrict__ x, double* __restrict__ r, const double* __restrict__ b,
               double* partial, EpiArgs e, int conditional) {
-  if (conditional) {   // end of a loop body: count it, then restart or set the condition
-    if (!e.st->restart_req) {
-      if (blockIdx.x == 0 && threadIdx.x == 0) {
-        e.st->guard++;
-        set_cond(e, more_cycles(e.st));
-      }
-      return;
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&e.st->guard, 1);
-  }
+  if (conditional && !restart_begin(e)) return;
   __shared__ double sh[32 * 8];   // bsum_n<NC> needs 32 * NC
   const int row = blockIdx.x * blockDim.x + threadIdx.x;
   double out = 0.0;
@@ -274,17 +112,7 @@ k_spmv(const T* __restrict__ A, const int* __restrict__ nbr, int N, int G,
   using V2 = typename Vec2<T>::type;
   constexpr int JP = (NP + 1) / 2;
   constexpr int NF = S - 1;
-  if (conditional) {
-    // end of a loop body: count it, then either restart (below) or set the condition
-    if (!e.st->restart_req) {
-      if (blockIdx.x == 0 && threadIdx.x == 0) {
-        e.st->guard++;
-        set_cond(e, more_cycles(e.st));
-      }
-      return;
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&e.st->guard, 1);
-  }
+  if (conditional && !restart_begin(e)) return;
   __shared__ double sh[32 * 8];   // bsum_n<NC> needs 32 * NC
   const int row = blockIdx.x * blockDim.x + threadIdx.x;
   const int g = row >> 5, lane = row & 31;

@@ -140,7 +140,9 @@ cudaError_t residual_noalloc(const Level0View& v, const double* b, const double*
   cudaError_t e;
   // the counter must start at zero (the previous call may have been interrupted)
   if ((e = cudaMemsetAsync(scratch + kNoallocMaxBlocks + 1, 0, sizeof(double), v.stream)) != cudaSuccess) return e;
-  switch (v.np * 10 + v.dim) {
+  if (v.pat)
+    launch_pattern_residual_scratch(v.np, v.dim, v.n, v.A, x, b, r, scratch, kNoallocMaxBlocks, v.stream);
+  else switch (v.np * 10 + v.dim) {
     case 32: k_residual_noalloc<3, 5><<<grid, v.block_rows, 0, v.stream>>>(v.A, v.nbr, v.N, v.G, x, b, r, scratch); break;
     case 62: k_residual_noalloc<6, 5><<<grid, v.block_rows, 0, v.stream>>>(v.A, v.nbr, v.N, v.G, x, b, r, scratch); break;
     case 102: k_residual_noalloc<10, 5><<<grid, v.block_rows, 0, v.stream>>>(v.A, v.nbr, v.N, v.G, x, b, r, scratch); break;
