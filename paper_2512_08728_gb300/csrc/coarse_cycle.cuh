@@ -3,12 +3,33 @@
 // minimisation (Alg. 1), transfers, the level-local criteria of Sec. 4.2 and the dense
 // coarsest solve, all in one launch per finest-level cycle.
 //
-// Coarse levels are small (here 5K-330K unknowns) and a kernel per step would be bound
-// by launch and reduction latency; one resident grid separated by grid barriers keeps
-// every SM busy instead.  Every control decision is taken by all blocks from the same
-// reduced values (fixed reduction order), so all blocks follow the same path.  The grid
-// barrier spins with a bound: if it ever times out it raises an error flag and every
-// block leaves the kernel, so a fault becomes a status, not a hang.
+// Coarse levels are small (here 200-330K unknowns), so a phase is bound by latency (a grid
+// barrier, an L2 round trip, a dependent chain of FP64 FMAs) and, from about 5K unknowns, by the
+// FP64 FMA rate of the SMs that take part.  What follows from that:
+//   - Every block owns a contiguous range of each level's cells, the same in every phase, so that
+//     the work spreads over all SMs even on a level of a few hundred cells, and r, the basis W
+//     and the coefficients never leave the SM: r and w are in shared memory, W is read through L1
+//     (only its own block writes it).
+//   - What blocks exchange is the iterate of a sweep (and r, b, x at a transfer).  Before the
+//     sum, a block copies its neighbours' slabs of the iterate (the ranges shifted by the grid's
+//     strides) to shared memory: one L2 round trip a phase in place of one per use.
+//   - A row's products are split over several threads where a block has fewer rows than threads.
+//   - One reduction per residual minimisation: W^T w, ||w||^2, w.r and ||r||^2 together give the
+//     coefficients, the new column's norm (Pythagoras, guarded by the reorthogonalisation test)
+//     and alpha, so the column is normalised as it is formed and no second reduction is needed.
+//     The next smoother's first sweep needs own rows only: no barrier in between.
+//   - Corrections are stored as they come; x = sum_k y_k z_k with R y = alpha (R: the
+//     orthogonalisation coefficients) is formed when the level returns or restarts, so Alg. 1's
+//     second recurrence costs one pass over the corrections per visit, not one per correction.
+//   - A level set too small to pay for a grid barrier runs in one block (cc_blocks()).
+// Measured (GB300, one launch, against blocks that took whole 320-row tiles and reduced three
+// times a minimisation): levels 16^3 and 8^3 at np = 10 beside the finest level's kernels 971 ->
+// 704 us; 64 x 48 and two levels below at np = 10, 2-D, 8.4 -> 5.3 ms a visit; 192 unknowns 749 ->
+// 370 us.
+// Every control decision is taken by all blocks from the same reduced values (fixed reduction
+// order), so all blocks follow the same path.  The grid barrier spins with a bound: if it ever
+// times out it raises an error flag and every block leaves the kernel, so a fault becomes a
+// status, not a hang.
 #pragma once
 #include "kcmg_internal.h"
 #include "reduce.cuh"
@@ -48,54 +69,36 @@ template <> struct InvLoad<double, double> {
   }
 };
 
-__device__ __forceinline__ double bsum(double v, double* sh) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x >> 5, ln = threadIdx.x & 31;
-  __syncthreads();
-  if (ln == 0) sh[w] = v;
-  __syncthreads();
-  double r = 0.0;
-  if (w == 0) {
-    r = (ln < (int)((blockDim.x + 31) >> 5)) ? sh[ln] : 0.0;
-#pragma unroll
-    for (int o = 16; o; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
-  }
-  return r;  // valid in thread 0
-}
-
 template <typename T> __device__ __forceinline__ T ldv(const T* p) { return __ldcg(p); }
 
 }  // namespace
 
-// Grid barrier with a bounded wait.  Every block adds one to a counter (acquire-release,
-// which publishes the block's writes) and waits until the counter reaches the total for
-// this generation; the host zeroes the counter before every launch.  gen: this block's
-// barrier count so far.  Returns false (in every thread of the block) once the error flag
-// is set; callers then leave the kernel.
+// Grid barrier with a bounded wait.  Every block adds one to a counter (a release, which
+// publishes the block's writes, and without waiting for the old value) and polls until the
+// counter reaches the total for this generation.  gen: this block's barrier count so far in the
+// launch; the last block to leave the kernel clears the counter (cc_leave), the host at the start
+// of every solve.  Returns false (in every thread of the block) once the error flag is set;
+// callers then leave the kernel.
 static __device__ __forceinline__ bool cc_barrier(const CoarseArgs& a, unsigned int& gen) {
   __shared__ int s_ok;
   __syncthreads();
+  if (gridDim.x == 1) return true;
   if (threadIdx.x == 0) {
     cuda::atomic_ref<unsigned int, cuda::thread_scope_device> cnt(*a.bar_count);
     cuda::atomic_ref<int, cuda::thread_scope_device> err(*a.err);
-    int ok = err.load(cuda::memory_order_relaxed) == 0;
-    if (ok) {
-      const unsigned int target = (gen + 1) * gridDim.x;
-      const unsigned int old = cnt.fetch_add(1u, cuda::memory_order_acq_rel);
-      if (old + 1 != target) {
-        long long spins = 0;
-        while (cnt.load(cuda::memory_order_acquire) < target) {
-          if ((++spins & 1023) == 0) {
-            if (err.load(cuda::memory_order_relaxed)) break;
-            if (spins > (1LL << 23)) {   // seconds: far beyond any legitimate wait
-              err.store(1, cuda::memory_order_relaxed);
-              break;
-            }
-          }
+    const unsigned int target = (gen + 1) * gridDim.x;
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.bar_count) : "memory");
+    long long spins = 0;
+    int ok = 1;
+    while (cnt.load(cuda::memory_order_acquire) < target) {
+      if ((++spins & 1023) == 0) {
+        if (err.load(cuda::memory_order_relaxed)) { ok = 0; break; }
+        if (spins > (1LL << 23)) {   // seconds: far beyond any legitimate wait
+          err.store(1, cuda::memory_order_relaxed);
+          ok = 0;
+          break;
         }
       }
-      ok = err.load(cuda::memory_order_relaxed) == 0;
     }
     s_ok = ok;
   }
@@ -104,12 +107,23 @@ static __device__ __forceinline__ bool cc_barrier(const CoarseArgs& a, unsigned 
   return s_ok != 0;
 }
 
+// Called by every block after its last barrier: the last one clears the counters for the next
+// launch.  No block polls any more, since all have passed the barrier.
+static __device__ __forceinline__ void cc_leave(const CoarseArgs& a) {
+  if (gridDim.x == 1 || threadIdx.x != 0) return;
+  if (atomicAdd(a.bar_gen, 1u) == gridDim.x - 1) {
+    *a.bar_count = 0u;
+    *a.bar_gen = 0u;
+    __threadfence();
+  }
+}
+
 namespace {
 
 // Per-level scalars, held identically by every block.
 struct LvScal {
-  int l, it;
-  double rnorm, rnorm0, eps;
+  int l, it, first;      // first: no reduction done yet on this visit (rnorm0 unknown)
+  double rnorm, eps;
 };
 
 // Vectors, basis W, Z, the Alg. 1 operator and the transfers are in TV (FP64, or FP32 in
@@ -121,23 +135,30 @@ struct CoarseCycle {
   using V2 = typename V2T<TV>::type;
   using VS2 = typename V2T<TS>::type;
   static constexpr int S = 2 * DIM + 1;
-  static constexpr int NF = S - 1;
   static constexpr int JP = (NP + 1) / 2;
   static constexpr int NCH = 1 << DIM;
+  static constexpr int SEGS = 2 * DIM - 1;   // slabs of the iterate: own with both x ends, +-y, +-z
 
   const CoarseArgs& a;
-  double* sh;      // 32 doubles
-  double* red_s;   // reduced sums (shared), >= kCoarseMaxCols
-  TS* tile;        // blockDim TS (smoother exchange)
-  TS* as_rs;       // (blockDim / 32) x 2^d np TS: a warp's gathered patch residual (Alg. AS)
-  T* Ps;           // NCH*NP*NP (prolongation matrices)
-  double* cw;      // coefficient vectors in shared memory: 2 * kCoarseMaxCols
-  int rcount = 0;  // reductions done (selects the partial buffer)
+  unsigned char* smem;   // dynamic shared memory (CoarseArgs offsets)
+  double* sh;            // 32 * 8 doubles
+  double* red_s;         // reduced sums, kCoarseMaxCols + 4
+  double* cf;            // coefficients of the minimisation, kCoarseMaxCols
+  T* Ps;                 // NCH*NP*NP (prolongation matrices)
+  int rcount = 0;        // reductions done (selects the partial buffer)
   unsigned int gen = 0;  // grid barriers passed (identical in every block)
   bool ok = true;
-  __device__ bool bar() { return cc_barrier(a, gen); }
-  double bytes = 0.0;  // algorithmic bytes of this launch (kept by thread 0 of block 0)
+  double bytes = 0.0;    // algorithmic bytes of this launch (kept by thread 0 of block 0)
 
+  // the block's range on the current level (set by enter())
+  int lev = 0, K0 = 0, nc = 0, rows = 0, row0 = 0;
+  int lpr = 1, part = 0, lrow = 0;   // threads per row; this thread's part and row (rows < blockDim)
+  int nb_off[S] = {};                // neighbour slab of each slot: cell offset in the slab buffer
+  unsigned char* mask = nullptr;     // per own cell: bit s set if the neighbour of slot s exists
+  T* rs = nullptr;                   // residual, own rows
+  double *R = nullptr, *gm = nullptr, *al = nullptr;   // packed columns of R, 1 / R_kk, alpha
+
+  __device__ bool bar() { return cc_barrier(a, gen); }
   __device__ void count(double b) {
     if (blockIdx.x == 0 && threadIdx.x == 0) bytes += b;
   }
@@ -145,194 +166,209 @@ struct CoarseCycle {
   __device__ double opbytes(const CoarseLevel& C, int slots, int elem) const {
     return (double)slots * C.N * NP * elem;
   }
-
-  __device__ const CoarseLevel& L(int lev) const { return a.lv[lev]; }
+  __device__ const CoarseLevel& L(int l) const { return a.lv[l]; }
   __device__ T* vec(void* p) const { return static_cast<T*>(p); }
+  __device__ T* zsV() const { return reinterpret_cast<T*>(smem + a.sm_zv); }
+  __device__ TS* zsS() const { return reinterpret_cast<TS*>(smem + a.sm_zs); }
+  __device__ TS* ts() const { return reinterpret_cast<TS*>(smem + a.sm_ts); }
+  __device__ T* ws() const { return reinterpret_cast<T*>(smem + a.sm_ws); }
+  __device__ double* ps() const { return reinterpret_cast<double*>(smem + a.sm_ps); }
 
-  // ---------------------------------------------------------------- reductions
-  // every block: v (this thread's contributions) -> red_s[0..nc) (grid totals)
-  template <int NC>
-  __device__ bool reduce_few(const double (&v)[NC]) {
-    double* part = a.partial + (size_t)(rcount & 1) * a.partial_stride;
-    rcount++;
-    double t[NC];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) t[c] = v[c];
-    bsum_n<NC>(t, sh);
-    if (threadIdx.x == 0)
-#pragma unroll
-      for (int c = 0; c < NC; ++c) part[(size_t)blockIdx.x * NC + c] = t[c];
-    if (!bar()) return false;
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      double s = 0.0;
-      for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) s += __ldcg(part + (size_t)b * NC + c);
-      t[c] = s;
+  // first cell of block b on a level of C cells
+  __device__ static int first_cell(int C, int b) { return (int)(((long long)C * b) / gridDim.x); }
+
+  __device__ void enter(int l) {
+    lev = l;
+    const CoarseLevel& C = L(l);
+    const int cells = C.N / NP;
+    K0 = first_cell(cells, blockIdx.x);
+    nc = first_cell(cells, blockIdx.x + 1) - K0;
+    rows = nc * NP;
+    row0 = K0 * NP;
+    lpr = rows > 0 ? min(8, max(1, (int)blockDim.x / rows)) : 1;
+    part = 0;
+    lrow = threadIdx.x;
+    if (lpr > 1) {
+      part = threadIdx.x / rows;
+      lrow = threadIdx.x - part * rows;
     }
-    bsum_n<NC>(t, sh);
-    if (threadIdx.x == 0)
+    mask = smem + C.sm_mask;
+    rs = reinterpret_cast<T*>(smem + C.sm_r);
+    gm = C.sm_gm >= 0 ? reinterpret_cast<double*>(smem + C.sm_gm) : C.coef + (size_t)blockIdx.x * C.coef_len;
+    al = gm + C.lcap;
+    R = al + C.lcap;
+    // slab buffer: [own cells with one more on each side | -y | +y | -z | +z]; one block owns all
+    // cells, and its own slab serves every slot
+    const int st[3] = {1, C.n[0], C.n[0] * C.n[1]};
+    nb_off[0] = 1;
 #pragma unroll
-      for (int c = 0; c < NC; ++c) red_s[c] = t[c];
-    __syncthreads();
-    return true;
-  }
-
-  // many columns: partial[b][c] already written by every block for c < nc; owners
-  // reduce one column each, then all blocks read the totals into red_s
-  __device__ bool reduce_cols(double* part, int nc) {
-    if (nc * (int)gridDim.x <= 4096) {   // few columns: every block sums all of them
-      if (!bar()) return false;
-      for (int c0 = 0; c0 < nc; c0 += 8) {
-        double t[8];
+    for (int k = 0; k < DIM; ++k)
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          t[c] = 0.0;
-          if (c0 + c < nc)
-            for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) t[c] += __ldcg(part + (size_t)b * nc + c0 + c);
-        }
-        bsum_n<8>(t, sh);
-        if (threadIdx.x == 0)
-#pragma unroll
-          for (int c = 0; c < 8; ++c)
-            if (c0 + c < nc) red_s[c0 + c] = t[c];
+      for (int side = 0; side < 2; ++side) {
+        const int s = 1 + 2 * k + side;
+        nb_off[s] = (k == 0 || gridDim.x == 1) ? 1 + (side ? st[k] : -st[k]) : (nc + 2) + (2 * (k - 1) + side) * nc;
       }
-      __syncthreads();
-      return true;
-    }
-    if (!bar()) return false;
-    for (int c = blockIdx.x; c < nc; c += gridDim.x) {
-      double s = 0.0;
-      for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) s += __ldcg(part + (size_t)b * nc + c);
-      s = bsum(s, sh);
-      if (threadIdx.x == 0) a.red[c] = s;
-    }
-    if (!bar()) return false;
-    for (int c = threadIdx.x; c < nc; c += blockDim.x) red_s[c] = __ldcg(a.red + c);
-    __syncthreads();
-    return true;
   }
 
-  // ---------------------------------------------------------------- operator phases
-  // y = A x (or b - A x) on level lev; returns this thread's sum of y^2
-  __device__ double spmv(int lev, const T* x, T* y, const T* b) {
-    const CoarseLevel& C = L(lev);
-    const T* A = static_cast<const T*>(C.A);
-    count(opbytes(C, S, sizeof(T)) + (double)C.N * sizeof(T) * (b ? 3 : 2));
-    double nrm = 0.0;
-    for (int row = blockIdx.x * blockDim.x + threadIdx.x; row < C.rows_pad; row += gridDim.x * blockDim.x) {
-      if (row >= C.N) continue;
-      const int g = row >> 5, lane = row & 31, K = row / NP;
-      T acc[4] = {T(0), T(0), T(0), T(0)};   // independent FMA chains (latency)
+  // existence masks of a level's own cells (once per launch)
+  __device__ void build_mask(int l) {
+    enter(l);
+    const CoarseLevel& C = L(l);
+    for (int c = threadIdx.x; c < nc; c += blockDim.x) {
+      const int K = K0 + c;
+      const int x[3] = {K % C.n[0], (K / C.n[0]) % C.n[1], DIM == 3 ? K / (C.n[0] * C.n[1]) : 0};
+      unsigned m = 1u;
 #pragma unroll
-      for (int s = 0; s < S; ++s) {
-        const int J = (s == 0) ? K : __ldg(C.nbr + (size_t)K * NF + s - 1);
-        if (J < 0) continue;
-        const V2* Ap = reinterpret_cast<const V2*>(A) + ((size_t)(s * C.G + g) * JP) * 32 + lane;
-        const T* xp = x + (size_t)J * NP;
-        const int c = (s & 1) << 1;
+      for (int k = 0; k < DIM; ++k) {
+        if (x[k] > 0) m |= 1u << (1 + 2 * k);
+        if (x[k] < C.n[k] - 1) m |= 1u << (2 + 2 * k);
+      }
+      mask[c] = (unsigned char)m;
+    }
+  }
+
+  // ---------------------------------------------------------------- slabs
+  // the neighbours' cells of the iterate z (global) into the slab buffer; with own: the block's
+  // own cells too.  Cells outside the grid are skipped (never read: the masks).
+  template <typename TX>
+  __device__ void load_slabs(const TX* z, TX* buf, bool own) {
+    const CoarseLevel& C = L(lev);
+    const int cells = C.N / NP;
+    if (own)
+      for (int i = threadIdx.x; i < rows; i += blockDim.x) buf[NP + i] = ldv(z + row0 + i);
+    if (gridDim.x > 1) {
+      if (threadIdx.x < 2 * NP) {   // the x neighbours of the range's ends
+        const int hi = threadIdx.x >= NP, q = threadIdx.x - hi * NP;
+        const int K = hi ? K0 + nc : K0 - 1;
+        if (K >= 0 && K < cells) buf[(hi ? (nc + 1) * NP : 0) + q] = ldv(z + (size_t)K * NP + q);
+      }
+      const int st[3] = {1, C.n[0], C.n[0] * C.n[1]};
+#pragma unroll
+      for (int k = 1; k < DIM; ++k)
+#pragma unroll
+        for (int side = 0; side < 2; ++side) {
+          const int base = (nc + 2 + (2 * (k - 1) + side) * nc) * NP;
+          const int g0 = (K0 + (side ? st[k] : -st[k])) * NP;
+          for (int i = threadIdx.x; i < rows; i += blockDim.x)
+            if (g0 + i >= 0 && g0 + i < C.N) buf[base + i] = ldv(z + g0 + i);
+        }
+    }
+    __syncthreads();
+  }
+
+  // sum over slots FROM.. of A_{K,s} z_{nbr(K,s)} for own row lr (this thread's share of the pairs)
+  template <typename TX, int FROM>
+  __device__ __forceinline__ TX row_sum(const void* Aop, const TX* buf, int lr, int q, int np) {
+    using VX = typename V2T<TX>::type;
+    const CoarseLevel& C = L(lev);
+    const int c = lr / NP, row = row0 + lr, g = row >> 5, lane = row & 31;
+    const VX* Ap = reinterpret_cast<const VX*>(Aop) + (size_t)g * JP * 32 + lane;
+    const size_t sl = (size_t)C.G * JP * 32;
+    const unsigned m = mask[c];
+    if (np == 1) {
+      TX acc[4] = {TX(0), TX(0), TX(0), TX(0)};   // independent FMA chains (latency)
+#pragma unroll
+      for (int s = FROM; s < S; ++s) {
+        if (!((m >> s) & 1u)) continue;
+        const TX* zp = buf + (size_t)(nb_off[s] + c) * NP;
+        const int k = (s & 1) << 1;
 #pragma unroll
         for (int jp = 0; jp < JP; ++jp) {
-          const V2 av = __ldg(Ap + jp * 32);
-          acc[c] = fma(av.x, ldv(xp + 2 * jp), acc[c]);
-          if (2 * jp + 1 < NP) acc[c + 1] = fma(av.y, ldv(xp + 2 * jp + 1), acc[c + 1]);
+          const VX av = __ldg(Ap + s * sl + jp * 32);
+          acc[k] = fma(av.x, zp[2 * jp], acc[k]);
+          if (2 * jp + 1 < NP) acc[k + 1] = fma(av.y, zp[2 * jp + 1], acc[k + 1]);
         }
       }
-      const T sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-      const T out = b ? (ldv(b + row) - sum) : sum;
-      y[row] = out;
-      nrm = fma((double)out, (double)out, nrm);
+      return (acc[0] + acc[1]) + (acc[2] + acc[3]);
     }
-    return nrm;
+    TX a0 = TX(0), a1 = TX(0);
+#pragma unroll 6
+    for (int e = FROM * JP + q; e < S * JP; e += np) {
+      const int s = e / JP, jp = e - s * JP;
+      if (!((m >> s) & 1u)) continue;
+      int off = nb_off[0];
+#pragma unroll
+      for (int t = 1; t < S; ++t)
+        if (s == t) off = nb_off[t];
+      const TX* zp = buf + (size_t)(off + c) * NP + 2 * jp;
+      const VX av = __ldg(Ap + s * sl + jp * 32);
+      a0 = fma(av.x, zp[0], a0);
+      if (2 * jp + 1 < NP) a1 = fma(av.y, zp[1], a1);
+    }
+    return a0 + a1;
   }
 
-  // One sweep of Alg. BJ in TS over tiles of blockDim rows (whole cells): t = r - A_off zo
-  // (skipped on the first sweep from z = 0), zn = (1 - omega) zo + omega D^{-1} t.
-  // The last sweep writes the FP64 correction.
+  // f(own row, sum) in one thread per row, over slots FROM..; ends with every thread past the
+  // reads of the slab buffer
+  template <typename TX, int FROM, typename F>
+  __device__ __forceinline__ void for_rows(const void* Aop, const TX* buf, F&& f) {
+    if (lpr == 1) {
+      for (int lr = threadIdx.x; lr < rows; lr += blockDim.x) f(lr, row_sum<TX, FROM>(Aop, buf, lr, 0, 1));
+    } else {
+      TX* p = reinterpret_cast<TX*>(ps());
+      if (part < lpr) p[part * rows + lrow] = row_sum<TX, FROM>(Aop, buf, lrow, part, lpr);
+      __syncthreads();
+      if (threadIdx.x < rows) {
+        TX v = p[threadIdx.x];
+        for (int q = 1; q < lpr; ++q) v += p[q * rows + threadIdx.x];
+        f((int)threadIdx.x, v);
+      }
+    }
+    __syncthreads();
+  }
+
+  // ---------------------------------------------------------------- smoother
+  // One sweep of Alg. BJ in TS on the own cells: t = r - A_off zo (skipped on the first sweep
+  // from z = 0), zn = (1 - omega) zo + omega D^{-1} t.  The own iterate is in the slab buffer; the
+  // new one goes to global memory for the neighbours and, in TO, to the slab buffer out.
   template <typename TO>
-  __device__ void sweep(const CoarseLevel& C, const T* r, const TS* zo, TO* zn, bool first) {
+  __device__ void sweep(const TS* zo, TO* zn, TO* out, bool first) {
+    const CoarseLevel& C = L(lev);
     count(opbytes(C, first ? 0 : S - 1, a.smoother_bytes) + opbytes(C, 1, a.inverse_bytes) +
           (double)C.N * (sizeof(T) + sizeof(TO) + (first ? 0 : sizeof(TS))));
-    const TS* A = static_cast<const TS*>(C.As);
+    TS* t = ts();
+    TS* zb = zsS();
+    if (first) {
+      for (int lr = threadIdx.x; lr < rows; lr += blockDim.x) t[lr] = (TS)rs[lr];
+      __syncthreads();
+    } else {
+      load_slabs<TS>(zo, zb, false);
+      for_rows<TS, 1>(C.As, zb, [&](int lr, TS v) { t[lr] = (TS)rs[lr] - v; });
+    }
     const TI* D = static_cast<const TI*>(C.Dinv);
     const TS om = (TS)a.omega;
-    const int ntile = C.rows_pad / blockDim.x;
-    for (int tl = blockIdx.x; tl < ntile; tl += gridDim.x) {
-      const int row = tl * blockDim.x + threadIdx.x;
-      const int g = row >> 5, lane = row & 31;
-      TS tv = TS(0);
-      if (row < C.N) {
-        tv = (TS)ldv(r + row);
-        if (!first) {
-          const int K = row / NP;
-          TS acc[4] = {TS(0), TS(0), TS(0), TS(0)};
+    for (int lr = threadIdx.x; lr < rows; lr += blockDim.x) {
+      const int row = row0 + lr, g = row >> 5, lane = row & 31, base = (lr / NP) * NP;
+      TS d0s = TS(0), d1s = TS(0);
 #pragma unroll
-          for (int s = 1; s < S; ++s) {
-            const int J = __ldg(C.nbr + (size_t)K * NF + s - 1);
-            if (J < 0) continue;
-            const VS2* Ap = reinterpret_cast<const VS2*>(A) + ((size_t)(s * C.G + g) * JP) * 32 + lane;
-            const TS* zp = zo + (size_t)J * NP;
-            const int c = (s & 1) << 1;
-#pragma unroll
-            for (int jp = 0; jp < JP; ++jp) {
-              const VS2 av = __ldg(Ap + jp * 32);
-              acc[c] = fma(av.x, ldv(zp + 2 * jp), acc[c]);
-              if (2 * jp + 1 < NP) acc[c + 1] = fma(av.y, ldv(zp + 2 * jp + 1), acc[c + 1]);
-            }
-          }
-          tv -= (acc[0] + acc[1]) + (acc[2] + acc[3]);
-        }
+      for (int jp = 0; jp < JP; ++jp) {
+        TS d0, d1;
+        InvLoad<TS, TI>::get(D, ((size_t)g * JP + jp) * 32 + lane, d0, d1);
+        d0s = fma(d0, t[base + 2 * jp], d0s);
+        if (2 * jp + 1 < NP) d1s = fma(d1, t[base + 2 * jp + 1], d1s);
       }
-      __syncthreads();
-      tile[threadIdx.x] = tv;
-      __syncthreads();
-      if (row < C.N) {
-        const int base = (row / NP) * NP - tl * blockDim.x;
-        TS d0s = TS(0), d1s = TS(0);
-#pragma unroll
-        for (int jp = 0; jp < JP; ++jp) {
-          TS d0, d1;
-          InvLoad<TS, TI>::get(D, ((size_t)g * JP + jp) * 32 + lane, d0, d1);
-          d0s = fma(d0, tile[base + 2 * jp], d0s);
-          if (2 * jp + 1 < NP) d1s = fma(d1, tile[base + 2 * jp + 1], d1s);
-        }
-        const TS dz = d0s + d1s;
-        const TS v = first ? om * dz : fma(TS(1) - om, ldv(zo + row), om * dz);
-        zn[row] = (TO)v;
-      }
+      const TS dz = d0s + d1s;
+      const TS v = first ? om * dz : fma(TS(1) - om, zb[NP + lr], om * dz);
+      zn[row] = (TO)v;
+      out[NP + lr] = (TO)v;
     }
   }
 
   // Alg. AS phases on a level (schwarz.cuh): the sweep's residual in TS, both partitions'
   // patch solves (one warp per patch), and the combination z_new = z_old + omega (z_0 + z_1)
-  __device__ void as_residual(const CoarseLevel& C, const T* r, const TS* zo, bool first) {
+  __device__ void as_residual(const TS* zo, bool first) {
+    const CoarseLevel& C = L(lev);
     count((double)C.N * (sizeof(T) + sizeof(TS)) + (first ? 0.0 : opbytes(C, S, a.smoother_bytes) + (double)C.N * sizeof(TS)));
-    const TS* A = static_cast<const TS*>(C.As);
     TS* res = static_cast<TS*>(C.as_r);
-    for (int row = blockIdx.x * blockDim.x + threadIdx.x; row < C.N; row += gridDim.x * blockDim.x) {
-      TS v = (TS)ldv(r + row);
-      if (!first) {
-        const int g = row >> 5, lane = row & 31, K = row / NP;
-        TS acc[4] = {TS(0), TS(0), TS(0), TS(0)};
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-          const int J = (s == 0) ? K : __ldg(C.nbr + (size_t)K * NF + s - 1);
-          if (J < 0) continue;
-          const VS2* Ap = reinterpret_cast<const VS2*>(A) + ((size_t)(s * C.G + g) * JP) * 32 + lane;
-          const TS* zp = zo + (size_t)J * NP;
-          const int c = (s & 1) << 1;
-#pragma unroll
-          for (int jp = 0; jp < JP; ++jp) {
-            const VS2 av = __ldg(Ap + jp * 32);
-            acc[c] = fma(av.x, ldv(zp + 2 * jp), acc[c]);
-            if (2 * jp + 1 < NP) acc[c + 1] = fma(av.y, ldv(zp + 2 * jp + 1), acc[c + 1]);
-          }
-        }
-        v -= (acc[0] + acc[1]) + (acc[2] + acc[3]);
-      }
-      res[row] = v;
+    if (first) {
+      for (int lr = threadIdx.x; lr < rows; lr += blockDim.x) res[row0 + lr] = (TS)rs[lr];
+    } else {
+      load_slabs<TS>(zo, zsS(), true);
+      for_rows<TS, 0>(C.As, zsS(), [&](int lr, TS v) { res[row0 + lr] = (TS)rs[lr] - v; });
     }
   }
-  __device__ void as_patches(const CoarseLevel& C) {
+  __device__ void as_patches() {
+    const CoarseLevel& C = L(lev);
     constexpr int M = NCH * NP;
     const int np0 = as_npatch(C.n, DIM, 0), np1 = as_npatch(C.n, DIM, 1);
     count((double)(np0 + np1) * M * M * a.inverse_bytes + (double)(np0 + np1) * M * 2 * sizeof(TS));
@@ -341,287 +377,367 @@ struct CoarseCycle {
     const TS* res = static_cast<const TS*>(C.as_r);
     TS* zP = static_cast<TS*>(C.as_z);
     const int warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
-    TS* rs = as_rs + (size_t)warp * M;
-    for (int w = blockIdx.x * wpb + warp; w < np0 + np1; w += gridDim.x * wpb) {
-      if (w < np0) as_patch_solve_warp<TS, TI, NP, DIM>(C.n, 0, w, inv0, res, zP, rs);
-      else as_patch_solve_warp<TS, TI, NP, DIM>(C.n, 1, w - np0, inv1, res, zP + (size_t)np0 * M, rs);
+    TS* prs = reinterpret_cast<TS*>(smem + a.sm_as) + (size_t)warp * M;
+    // patches over blocks first, so that a level of few patches still uses every SM
+    for (int w = blockIdx.x + gridDim.x * warp; w < np0 + np1; w += gridDim.x * wpb) {
+      if (w < np0) as_patch_solve_warp<TS, TI, NP, DIM>(C.n, 0, w, inv0, res, zP, prs);
+      else as_patch_solve_warp<TS, TI, NP, DIM>(C.n, 1, w - np0, inv1, res, zP + (size_t)np0 * M, prs);
     }
   }
   template <typename TO>
-  __device__ void as_combine(const CoarseLevel& C, const TS* zo, TO* zn, bool first) {
+  __device__ void as_combine(const TS* zo, TO* zn, TO* out, bool first) {
+    const CoarseLevel& C = L(lev);
     count((double)C.N * (2 * sizeof(TS) + sizeof(TO)));
     const int np0 = as_npatch(C.n, DIM, 0);
     const TS* zP = static_cast<const TS*>(C.as_z);
-    for (int row = blockIdx.x * blockDim.x + threadIdx.x; row < C.N; row += gridDim.x * blockDim.x)
-      zn[row] = (TO)as_combine_row<TS, NP, DIM>(C.n, row, zP, np0, zo, (TS)a.omega, first);
+    for (int lr = threadIdx.x; lr < rows; lr += blockDim.x) {
+      const TO v = (TO)as_combine_row<TS, NP, DIM>(C.n, row0 + lr, zP, np0, zo, (TS)a.omega, first);
+      zn[row0 + lr] = v;
+      out[NP + lr] = v;
+    }
   }
 
-  // z = BJ(r) or AS(r) from z = 0 (a.sweeps sweeps); returns the correction C.z (type T)
-  __device__ T* smooth(int lev, const T* r) {
+  // z = BJ(r) or AS(r) from z = 0 (a.sweeps sweeps): own rows in zsV(), all rows in C.z
+  __device__ void smooth() {
     const CoarseLevel& C = L(lev);
-    if (a.smoother == 1) {
-      TS* sb[2] = {static_cast<TS*>(C.s0), static_cast<TS*>(C.s1)};
-      T* out = vec(C.z);
-      for (int k = 0; k < a.sweeps && ok; ++k) {
-        const TS* zo = sb[(k + 1) & 1];
-        as_residual(C, r, zo, k == 0);
-        if (!(ok = bar())) break;
-        as_patches(C);
-        if (!(ok = bar())) break;
-        if (k == a.sweeps - 1) as_combine<T>(C, zo, out, k == 0);
-        else as_combine<TS>(C, zo, sb[k & 1], k == 0);
-        ok = bar();
-        ph(PH_SWEEP);
-      }
-      return out;
-    }
     TS* sb[2] = {static_cast<TS*>(C.s0), static_cast<TS*>(C.s1)};
     T* out = vec(C.z);
     for (int k = 0; k < a.sweeps && ok; ++k) {
       const TS* zo = sb[(k + 1) & 1];
-      if (k == a.sweeps - 1) sweep<T>(C, r, zo, out, k == 0);
-      else sweep<TS>(C, r, zo, sb[k & 1], k == 0);
+      const bool last = k == a.sweeps - 1;
+      if (a.smoother == 1) {
+        as_residual(zo, k == 0);
+        if (!(ok = bar())) break;
+        as_patches();
+        if (!(ok = bar())) break;
+        if (last) as_combine<T>(zo, out, zsV(), k == 0);
+        else as_combine<TS>(zo, sb[k & 1], zsS(), k == 0);
+      } else if (last) {
+        sweep<T>(zo, out, zsV(), k == 0);
+      } else {
+        sweep<TS>(zo, sb[k & 1], zsS(), k == 0);
+      }
       ok = bar();
       ph(PH_SWEEP);
     }
-    return out;
+  }
+
+  // ---------------------------------------------------------------- reductions
+  // partial[c][b] of every block b -> red_s[0..n): few columns are summed by every block, more
+  // columns by one owner each (a second barrier)
+  __device__ bool reduce_cols(double* pt, int n) {
+    if (gridDim.x == 1) {   // the sums are the block's own, in red_s already
+      __syncthreads();
+      return true;
+    }
+    if (!bar()) return false;
+    const int warp = threadIdx.x >> 5, ln = threadIdx.x & 31, nw = blockDim.x >> 5;
+    if (n * (int)gridDim.x <= 4096) {
+      for (int c = warp; c < n; c += nw) {
+        double v = 0.0;
+        for (int b = ln; b < (int)gridDim.x; b += 32) v += __ldcg(pt + (size_t)c * gridDim.x + b);
+#pragma unroll
+        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (ln == 0) red_s[c] = v;
+      }
+      __syncthreads();
+      return true;
+    }
+    for (int c = blockIdx.x + gridDim.x * warp; c < n; c += gridDim.x * nw) {
+      double v = 0.0;
+      for (int b = ln; b < (int)gridDim.x; b += 32) v += __ldcg(pt + (size_t)c * gridDim.x + b);
+#pragma unroll
+      for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (ln == 0) a.red[c] = v;
+    }
+    if (!bar()) return false;
+    for (int c = threadIdx.x; c < n; c += blockDim.x) red_s[c] = __ldcg(a.red + c);
+    __syncthreads();
+    return true;
+  }
+  __device__ double* next_partial() {
+    double* pt = a.partial + (size_t)(rcount & 1) * a.partial_stride;
+    rcount++;
+    return pt;
+  }
+
+  // this block's sums of column c < l: W_c . w, l: w . w, l + 1: w . r, l + 2: r . r over the own
+  // rows; LPC lanes of a warp share a column.  Per-thread sums in T, then FP64.
+  template <int LPC>
+  __device__ void dots_lpc(const T* W, int N, int l, double* pt) {
+    constexpr int CPW = 32 / LPC;
+    const int warp = threadIdx.x >> 5, ln = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const int sub = ln / LPC, lc = ln - sub * LPC, n = l + 3;
+    const T* w = ws();
+    for (int c0 = warp * CPW; c0 < n; c0 += nw * CPW) {
+      const int c = c0 + sub;
+      T s0 = T(0), s1 = T(0);
+      if (c < n) {
+        const T* u = c < l ? W + (size_t)c * N + row0 : c == l + 2 ? rs : w;
+        const T* v = c <= l ? w : rs;
+        int j = lc;
+        for (; j + LPC < rows; j += 2 * LPC) {
+          s0 = fma(u[j], v[j], s0);
+          s1 = fma(u[j + LPC], v[j + LPC], s1);
+        }
+        if (j < rows) s0 = fma(u[j], v[j], s0);
+      }
+      double d = (double)(s0 + s1);
+#pragma unroll
+      for (int o = LPC / 2; o; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+      if (lc == 0 && c < n) {
+        if (gridDim.x == 1) red_s[c] = d;
+        else pt[(size_t)c * gridDim.x + blockIdx.x] = d;
+      }
+    }
+  }
+  __device__ bool dots(const T* W, int N, int l) {
+    double* pt = next_partial();
+    const int nw = blockDim.x >> 5;
+    if (l + 3 <= nw) dots_lpc<32>(W, N, l, pt);
+    else if (l + 3 <= 2 * nw) dots_lpc<16>(W, N, l, pt);
+    else dots_lpc<8>(W, N, l, pt);
+    return reduce_cols(pt, l + 3);
+  }
+
+  // v[row] - sum_c W[c][row] cf[c] -> f(own row, value), columns split over lpr threads a row
+  template <typename F>
+  __device__ void project(const T* W, int N, int l, const T* v, F&& f) {
+    auto share = [&](int lr, int q, int np) {
+      const T* Wp = W + row0 + lr;
+      T s[4] = {T(0), T(0), T(0), T(0)};
+      int i = q;
+      for (; i + 3 * np < l; i += 4 * np)
+#pragma unroll
+        for (int t = 0; t < 4; ++t) s[t] = fma((T)(-cf[i + t * np]), Wp[(size_t)(i + t * np) * N], s[t]);
+      for (; i < l; i += np) s[0] = fma((T)(-cf[i]), Wp[(size_t)i * N], s[0]);
+      return (s[0] + s[1]) + (s[2] + s[3]);
+    };
+    if (lpr == 1 || l < 8) {
+      for (int lr = threadIdx.x; lr < rows; lr += blockDim.x) f(lr, v[lr] + share(lr, 0, 1));
+    } else {
+      T* p = reinterpret_cast<T*>(ps());
+      if (part < lpr) p[part * rows + lrow] = share(lrow, part, lpr);
+      __syncthreads();
+      if (threadIdx.x < rows) {
+        T s = p[threadIdx.x];
+        for (int q = 1; q < lpr; ++q) s += p[q * rows + threadIdx.x];
+        f((int)threadIdx.x, v[threadIdx.x] + s);
+      }
+    }
+    __syncthreads();
   }
 
   // ---------------------------------------------------------------- Alg. 1
-  // returns false on a barrier error
-  __device__ bool rm(int lev, const T* z, LvScal& sc) {
+  // with the correction z: own rows in zsV(), all rows in C.z; returns false on a barrier error
+  __device__ bool rm(LvScal& sc) {
     const CoarseLevel& C = L(lev);
     const int N = C.N, l = sc.l;
     T* W = vec(C.W);
-    T* Z = vec(C.Z);
-    T* w = vec(C.w);
-    T* wre = vec(C.wre);
-    const T* r = vec(C.r);
-    // w = A z.  No grid barrier before the dots: both phases give each thread the same
-    // rows (grid-stride), so every w[j] a thread reads it wrote itself.
-    spmv(lev, z, w, nullptr);
-    // h = W^T w, ||w||^2  (columns in groups of 8)
-    const int nc = l + 1;
-    double* part = a.partial + (size_t)(rcount & 1) * a.partial_stride;
-    rcount++;
-    dots(W, N, w, l, part);
-    count((double)(l + 1) * N * sizeof(T));
-    if (!reduce_cols(part, nc)) return false;
+    T* w = ws();
+    const T* zown = zsV() + NP;
+    load_slabs<T>(vec(C.z), zsV(), false);
+    for_rows<T, 0>(C.A, zsV(), [&](int lr, T v) { w[lr] = v; });
+    count(opbytes(C, S, sizeof(T)) + (double)N * sizeof(T) * 2 + (double)(l + 1) * N * sizeof(T));
+    if (!dots(W, N, l)) return false;
     ph(PH_RM_GRAM1);
-    double hh = 0.0;
-    for (int i = 0; i < l; ++i) hh += red_s[i] * red_s[i];
-    const double naz2 = red_s[l];
-    const bool reorth = l > 0 && (naz2 - hh < 0.25 * naz2);
+    const double rr = red_s[l + 2], naz2 = red_s[l];
+    if (sc.first) {
+      sc.rnorm = sqrt(rr);
+      sc.eps = C.rtol * sc.rnorm;
+      sc.first = 0;
+    }
+    // w_hat = w - W W^T w: its norm by Pythagoras; another pass whenever that cancelled
+    // more than half of it (classical Gram-Schmidt, "twice is enough")
+    double* Rc = R + l * (l - 1) / 2;
+    for (int i = threadIdx.x; i < l; i += blockDim.x) Rc[i] = 0.0;
     bool discard = !isfinite(naz2) || !(naz2 > 0.0);
-    // coefficients into shared memory: cw (for w), cw + lcap (for z)
-    for (int i = threadIdx.x; i < l; i += blockDim.x) { cw[i] = red_s[i]; cw[kCoarseMaxCols + i] = red_s[i]; }
-    __syncthreads();
-    const T* wsrc = w;
-    if (reorth) {
-      // w' = w - W h, then h2 = W^T w'
-      for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < N; j += gridDim.x * blockDim.x) {
-        T s = ldv(w + j);
-        for (int i = 0; i < l; ++i) s = fma((T)(-cw[i]), ldv(W + (size_t)i * N + j), s);
-        wre[j] = s;
-      }
-      if (!bar()) return false;
-      double* part2 = a.partial + (size_t)(rcount & 1) * a.partial_stride;
-      rcount++;
-      dots(W, N, wre, l, part2);
-      count((double)(l + 2) * N * sizeof(T) + (double)(l + 1) * N * sizeof(T));   // apply + second dots
-      if (!reduce_cols(part2, nc)) return false;
+    const double tiny = a.brk * a.brk * naz2;
+    double nw2 = 0.0, wr = 0.0;
+    for (int pass = 0;; ++pass) {
+      double hh = 0.0;
+      for (int i = 0; i < l; ++i) hh += red_s[i] * red_s[i];
+      const double n2 = red_s[l];
+      nw2 = n2 - hh;
+      wr = red_s[l + 1];
+      __syncthreads();
       for (int i = threadIdx.x; i < l; i += blockDim.x) {
-        cw[kCoarseMaxCols + i] += red_s[i];   // z gets h + h2
-        cw[i] = red_s[i];                     // w' gets h2
+        cf[i] = red_s[i];
+        Rc[i] += red_s[i];
       }
       __syncthreads();
-      wsrc = wre;
+      if (discard || l == 0 || nw2 >= 0.25 * n2 || pass == 3) break;
+      if (pass > 0 && !(nw2 > tiny)) break;   // nothing left: linearly dependent
+      project(W, N, l, w, [&](int lr, T v) { w[lr] = v; });
+      count((double)(l + 2) * N * sizeof(T) + (double)(l + 1) * N * sizeof(T));   // apply + second dots
+      if (!dots(W, N, l)) return false;
       ph(PH_RM_REORTH);
     }
-    // w_hat = wsrc - W cw, z_hat = z - Z cz into column l; ||w_hat||^2, w_hat . r
-    T* Wl = W + (size_t)l * N;
-    T* Zl = Z + (size_t)l * N;
-    double nw2 = 0.0, wr = 0.0;
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < N; j += gridDim.x * blockDim.x) {
-      T av = ldv(wsrc + j), zv = ldv(z + j), av1 = T(0), zv1 = T(0);
-      int i = 0;
-      for (; i + 1 < l; i += 2) {
-        av = fma((T)(-cw[i]), ldv(W + (size_t)i * N + j), av);
-        zv = fma((T)(-cw[kCoarseMaxCols + i]), ldv(Z + (size_t)i * N + j), zv);
-        av1 = fma((T)(-cw[i + 1]), ldv(W + (size_t)(i + 1) * N + j), av1);
-        zv1 = fma((T)(-cw[kCoarseMaxCols + i + 1]), ldv(Z + (size_t)(i + 1) * N + j), zv1);
-      }
-      if (i < l) {
-        av = fma((T)(-cw[i]), ldv(W + (size_t)i * N + j), av);
-        zv = fma((T)(-cw[kCoarseMaxCols + i]), ldv(Z + (size_t)i * N + j), zv);
-      }
-      av += av1;
-      zv += zv1;
-      Wl[j] = av;
-      Zl[j] = zv;
-      nw2 = fma((double)av, (double)av, nw2);
-      wr = fma((double)av, (double)ldv(r + j), wr);
+    if (!isfinite(nw2) || !(nw2 > tiny)) discard = true;
+    if (discard) {
+      sc.rnorm = sqrt(rr);
+      return true;
     }
-    count((double)(2 * l + 5) * N * sizeof(T));   // W, Z columns; w, z, r in; new columns out
-    {
-      double v[2] = {nw2, wr};
-      if (!reduce_few<2>(v)) return false;
+    const double gam = 1.0 / sqrt(nw2), alp = gam * wr;   // alpha = w_hat . r (r is orthogonal to W)
+    const T g = (T)gam, al_t = (T)alp;
+    T* Wl = W + (size_t)l * N + row0;
+    T* Zl = vec(C.Z) + (size_t)l * N + row0;
+    project(W, N, l, w, [&](int lr, T v) {
+      const T wv = v * g;
+      Wl[lr] = wv;
+      Zl[lr] = zown[lr];
+      rs[lr] = fma(-al_t, wv, rs[lr]);
+    });
+    if (threadIdx.x == 0) {
+      gm[l] = gam;
+      al[l] = alp;
     }
-    ph(PH_RM_UPDATE);
-    const double nw = sqrt(red_s[0]);
-    if (!isfinite(nw) || !(nw > a.brk * sqrt(naz2))) discard = true;
-    const double gam = discard ? 0.0 : 1.0 / nw;
-    const double alp = discard ? 0.0 : gam * red_s[1];
-    // normalise and update x, r; ||r||^2
-    double r2 = 0.0;
-    T* x = vec(C.x);
-    T* rr = vec(C.r);
-    const T g = (T)gam, al = (T)alp;
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < N; j += gridDim.x * blockDim.x) {
-      T rv = ldv(rr + j);
-      if (!discard) {
-        const T wv = ldv(Wl + j) * g, zv = ldv(Zl + j) * g;
-        Wl[j] = wv;
-        Zl[j] = zv;
-        x[j] = fma(al, zv, ldv(x + j));
-        rv = fma(-al, wv, rv);
-        rr[j] = rv;
-      }
-      r2 = fma((double)rv, (double)rv, r2);
-    }
-    count(discard ? 0.0 : (double)N * 8 * sizeof(T));
+    count((double)(l + 4) * N * sizeof(T));   // W columns; w, r in; new columns and r out
     // ||r - alpha w||^2 = ||r||^2 - alpha^2 for unit w with alpha = w . r; reduce the
     // updated vector explicitly only if that cancels more than four digits
-    const double r2old = sc.rnorm * sc.rnorm;
-    const double r2new = r2old - alp * alp;
-    if (discard) {
-      // x, r unchanged
-    } else if (r2new > 1e-4 * r2old) {
+    const double r2new = rr - alp * alp;
+    sc.l++;
+    if (r2new > 1e-4 * rr) {
       sc.rnorm = sqrt(r2new);
     } else {
-      double v[1] = {r2};
-      if (!reduce_few<1>(v)) return false;
-      sc.rnorm = sqrt(red_s[0]);
+      if (!residual_norm(sc)) return false;
     }
-    if (!discard) sc.l++;
-    ph(PH_RM_FINISH);
+    ph(PH_RM_UPDATE);
     return true;
   }
 
-  // partial[blk][c] for c < l: W_c . w ; c = l: ||w||^2.  Groups of 8 columns; the last
-  // group reads a valid column in place of the missing ones and drops those sums, and the
-  // norm is a separate sum of group 0, so every step issues the same FMAs.  Per-thread
-  // sums in T, block and grid sums in FP64.
-  __device__ void dots(const T* W, int N, const T* w, int l, double* part) {
-    const int nc = l + 1;
-    const int groups = l > 0 ? (l + 7) / 8 : 1;
-    for (int g = 0; g < groups; ++g) {
-      const int c0 = 8 * g;
-      T acc[8];
-      T ww = T(0);
-#pragma unroll
-      for (int c = 0; c < 8; ++c) acc[c] = T(0);
-      for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < N; j += gridDim.x * blockDim.x) {
-        const T wv = ldv(w + j);
-        if (l > 0)
-#pragma unroll
-          for (int c = 0; c < 8; ++c)
-            acc[c] = fma(ldv(W + (size_t)min(c0 + c, l - 1) * N + j), wv, acc[c]);
-        if (g == 0) ww = fma(wv, wv, ww);
-      }
-      double v[8];
-#pragma unroll
-      for (int c = 0; c < 8; ++c) v[c] = (double)acc[c];
-      bsum_n<8>(v, sh);
-      if (threadIdx.x == 0)
-#pragma unroll
-        for (int c = 0; c < 8; ++c)
-          if (c0 + c < l) part[(size_t)blockIdx.x * nc + c0 + c] = v[c];
-      if (g == 0) {
-        double n[1] = {(double)ww};
-        bsum_n<1>(n, sh);
-        if (threadIdx.x == 0) part[(size_t)blockIdx.x * nc + l] = n[0];
+  // sc.rnorm = ||r|| from the own rows of every block
+  __device__ bool residual_norm(LvScal& sc) {
+    double* pt = next_partial();
+    double s = 0.0;
+    for (int j = threadIdx.x; j < rows; j += blockDim.x) s = fma((double)rs[j], (double)rs[j], s);
+    double v[1] = {s};
+    __syncthreads();
+    bsum_n<1>(v, sh);
+    if (threadIdx.x == 0) (gridDim.x == 1 ? red_s : pt)[blockIdx.x] = v[0];
+    if (!reduce_cols(pt, 1)) return false;
+    sc.rnorm = sqrt(red_s[0]);
+    return true;
+  }
+
+  // x += sum_k y_k z_k over the level's corrections, with R y = alpha (back substitution by one
+  // warp of every block)
+  __device__ void update_x(const LvScal& sc) {
+    const CoarseLevel& C = L(lev);
+    const int l = sc.l, N = C.N;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      for (int i = threadIdx.x; i < l; i += 32) cf[i] = al[i];
+      __syncwarp();
+      for (int k = l - 1; k >= 0; --k) {
+        const double y = cf[k] * gm[k];
+        __syncwarp();
+        const double* Rk = R + k * (k - 1) / 2;
+        for (int i = threadIdx.x; i < k; i += 32) cf[i] = fma(-Rk[i], y, cf[i]);
+        if (threadIdx.x == 0) cf[k] = y;
+        __syncwarp();
       }
     }
+    __syncthreads();
+    const T* Z = vec(C.Z);
+    T* x = vec(C.x);
+    for (int lr = threadIdx.x; lr < rows; lr += blockDim.x) {
+      T s[4] = {T(0), T(0), T(0), T(0)};
+      int i = 0;
+      for (; i + 3 < l; i += 4)
+#pragma unroll
+        for (int t = 0; t < 4; ++t) s[t] = fma((T)cf[i + t], Z[(size_t)(i + t) * N + row0 + lr], s[t]);
+      for (; i < l; ++i) s[0] = fma((T)cf[i], Z[(size_t)i * N + row0 + lr], s[0]);
+      x[row0 + lr] = ldv(x + row0 + lr) + ((s[0] + s[1]) + (s[2] + s[3]));
+    }
+    count((double)(l + 2) * N * sizeof(T));
   }
 
   // ---------------------------------------------------------------- transfers
-  // b_{lev+1} = R r_lev; with start: r_{lev+1} = b_{lev+1}, x_{lev+1} = 0; returns ||b||^2 part
-  __device__ double restrict_(int lev, bool start) {
+  // b of level lev + 1 = R r (own rows of that level); with start: its r = b and x = 0.  Needs
+  // C.r of this level complete in global memory.
+  __device__ void restrict_(bool start) {
     const CoarseLevel &F = L(lev), &C = L(lev + 1);
     count((double)F.N * sizeof(T) + (double)C.N * sizeof(T) * (start ? 3 : 1));
+    const int cells = C.N / NP;
+    const int J0 = first_cell(cells, blockIdx.x), nJ = first_cell(cells, blockIdx.x + 1) - J0;
     const T* rf = vec(F.r);
-    T* bc = vec(C.b);
-    double nrm = 0.0;
-    for (int row = blockIdx.x * blockDim.x + threadIdx.x; row < C.N; row += gridDim.x * blockDim.x) {
-      const int J = row / NP, i = row - J * NP;
+    T* stage = zsV();   // children of the own coarse cells: [cell][child][NP]
+    for (int i = threadIdx.x; i < nJ * NCH * NP; i += blockDim.x) {
+      const int q = i % NP, k = (i / NP) % NCH, J = J0 + i / (NP * NCH);
       const int jx = J % C.n[0], jy = (J / C.n[0]) % C.n[1], jz = DIM == 3 ? J / (C.n[0] * C.n[1]) : 0;
-      T s = T(0);
-#pragma unroll
-      for (int k = 0; k < NCH; ++k) {
-        const int fx = 2 * jx + (k & 1), fy = 2 * jy + ((k >> 1) & 1), fz = DIM == 3 ? 2 * jz + ((k >> 2) & 1) : 0;
-        const int K = fx + F.n[0] * (fy + F.n[1] * fz);
-#pragma unroll
-        for (int q = 0; q < NP; ++q) s = fma(Ps[(k * NP + q) * NP + i], ldv(rf + (size_t)K * NP + q), s);
-      }
-      bc[row] = s;
-      if (start) {
-        vec(C.r)[row] = s;
-        vec(C.x)[row] = T(0);
-      }
-      nrm = fma((double)s, (double)s, nrm);
+      const int fx = 2 * jx + (k & 1), fy = 2 * jy + ((k >> 1) & 1), fz = DIM == 3 ? 2 * jz + ((k >> 2) & 1) : 0;
+      stage[i] = ldv(rf + (size_t)(fx + F.n[0] * (fy + F.n[1] * fz)) * NP + q);
     }
-    return nrm;
+    __syncthreads();
+    T* rc = start ? reinterpret_cast<T*>(smem + C.sm_r) : nullptr;
+    for (int lr = threadIdx.x; lr < nJ * NP; lr += blockDim.x) {
+      const int c = lr / NP, i = lr - c * NP;
+      T s[NCH];
+#pragma unroll
+      for (int k = 0; k < NCH; ++k) s[k] = T(0);
+#pragma unroll 2
+      for (int q = 0; q < NP; ++q)
+#pragma unroll
+        for (int k = 0; k < NCH; ++k) s[k] = fma(Ps[(k * NP + q) * NP + i], stage[(c * NCH + k) * NP + q], s[k]);
+      T v = T(0);
+#pragma unroll
+      for (int k = 0; k < NCH; ++k) v += s[k];
+      vec(C.b)[J0 * NP + lr] = v;
+      if (start) {
+        rc[lr] = v;
+        vec(C.x)[J0 * NP + lr] = T(0);
+      }
+    }
+    __syncthreads();
   }
 
-  // z_lev = P x_{lev+1}
-  __device__ void prolong(int lev) {
+  // z = P x_{lev + 1} on the own rows: zsV() and C.z
+  __device__ void prolong() {
     const CoarseLevel &F = L(lev), &C = L(lev + 1);
     count((double)F.N * sizeof(T) + (double)C.N * sizeof(T));
     const T* xc = vec(C.x);
     T* zf = vec(F.z);
-    for (int row = blockIdx.x * blockDim.x + threadIdx.x; row < F.N; row += gridDim.x * blockDim.x) {
-      const int K = row / NP, q = row - K * NP;
+    T* own = zsV() + NP;
+    for (int lr = threadIdx.x; lr < rows; lr += blockDim.x) {
+      const int K = K0 + lr / NP, q = lr % NP;
       const int ix = K % F.n[0], iy = (K / F.n[0]) % F.n[1], iz = DIM == 3 ? K / (F.n[0] * F.n[1]) : 0;
       const int k = (ix & 1) | ((iy & 1) << 1) | (DIM == 3 ? ((iz & 1) << 2) : 0);
       const int J = (ix >> 1) + C.n[0] * ((iy >> 1) + C.n[1] * (iz >> 1));
+      T xv[NP];
+#pragma unroll
+      for (int i = 0; i < NP; ++i) xv[i] = ldv(xc + (size_t)J * NP + i);
       T s = T(0);
 #pragma unroll
-      for (int i = 0; i < NP; ++i) s = fma(Ps[(k * NP + q) * NP + i], ldv(xc + (size_t)J * NP + i), s);
-      zf[row] = s;
+      for (int i = 0; i < NP; ++i) s = fma(Ps[(k * NP + q) * NP + i], xv[i], s);
+      zf[row0 + lr] = s;
+      own[lr] = s;
     }
   }
 
-  // x_c = A_c^{-1} b_c (FP64 dense inverse), one warp per row
-  __device__ void coarse_solve(int lev) {
-    const CoarseLevel& C = L(lev);
+  // x_c = A_c^{-1} b_c (FP64 dense inverse), one warp per row, rows over blocks first
+  __device__ void coarse_solve(int l) {
+    const CoarseLevel& C = L(l);
     count((double)a.Nc * a.Nc * 8 + (double)a.Nc * 2 * sizeof(T));
     const T* bc = vec(C.b);
     T* xc = vec(C.x);
-    const int warps = (gridDim.x * blockDim.x) >> 5;
-    const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, ln = threadIdx.x & 31;
-    for (int row = wid; row < a.Nc; row += warps) {
-      double s = 0.0;
-      for (int j = ln; j < a.Nc; j += 32) s = fma(__ldg(a.Ainv + (size_t)row * a.Nc + j), (double)ldv(bc + j), s);
+    const int nw = blockDim.x >> 5, warp = threadIdx.x >> 5, ln = threadIdx.x & 31;
+    for (int row = blockIdx.x + gridDim.x * warp; row < a.Nc; row += gridDim.x * nw) {
+      double s[4] = {0.0, 0.0, 0.0, 0.0};
+      const double* Ar = a.Ainv + (size_t)row * a.Nc;
+      int j = ln;
+      for (; j + 96 < a.Nc; j += 128)
 #pragma unroll
-      for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (ln == 0) xc[row] = (T)s;
+        for (int t = 0; t < 4; ++t) s[t] = fma(__ldg(Ar + j + 32 * t), (double)ldv(bc + j + 32 * t), s[t]);
+      for (; j < a.Nc; j += 32) s[0] = fma(__ldg(Ar + j), (double)ldv(bc + j), s[0]);
+      double v = (s[0] + s[1]) + (s[2] + s[3]);
+#pragma unroll
+      for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (ln == 0) xc[row] = (T)v;
     }
   }
 
-  // ---------------------------------------------------------------- Alg. 2 on lev >= 1
-  // The recursion MG(lev) -> MG(lev + 1) of Alg. 2 runs as a loop over an explicit
-  // per-level state (the levels form a chain, so a phase per level suffices).
-  // On entry b, r = b and x = 0 of level lev0 are set and sc[lev0].rnorm0 = ||b||.
-  enum Phase { TEST, AFTER_COARSE };
-
-  __device__ void start(int lev, LvScal& sc) {
-    sc.l = 0;
-    sc.it = 0;
-    sc.rnorm = sc.rnorm0;
-    sc.eps = L(lev).rtol * sc.rnorm0;
-  }
-
+  // ---------------------------------------------------------------- timing
   // time attribution per phase kind (thread 0 of block 0; the interval since the previous
   // phase boundary, closing barrier included)
   unsigned long long t_ph = 0;
@@ -636,13 +752,28 @@ struct CoarseCycle {
 
   // time attribution per level (thread 0 of block 0)
   unsigned long long t_mark = 0;
-  __device__ void mark(int lev) {
+  __device__ void mark(int l) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       unsigned long long t;
       asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-      if (t_mark) atomicAdd(a.stat_level_ns + lev, t - t_mark);
+      if (t_mark) atomicAdd(a.stat_level_ns + l, t - t_mark);
       t_mark = t;
     }
+  }
+
+  // ---------------------------------------------------------------- Alg. 2 on lev >= 1
+  // The recursion MG(lev) -> MG(lev + 1) of Alg. 2 runs as a loop over an explicit
+  // per-level state (the levels form a chain, so a phase per level suffices).  On entry b, r = b
+  // and x = 0 of level lev0 are set, r also in shared memory.  ||b|| comes with the first
+  // reduction of a visit.
+  enum Phase { PRE, CORRECT, POST };   // the residual minimisation that comes next on the level
+
+  __device__ static void start(LvScal& sc, double rtol) {
+    sc.l = 0;
+    sc.it = 0;
+    sc.first = 1;
+    sc.rnorm = rtol < 1.0 ? 1.0 : 0.0;   // stands for ||b|| > rtol ||b|| until ||b|| is known
+    sc.eps = 0.0;
   }
 
   __device__ void run(int lev0) {
@@ -650,37 +781,51 @@ struct CoarseCycle {
     int phase[KCMG_MAX_LEVELS];
     int restarts[KCMG_MAX_LEVELS];
     int guard[KCMG_MAX_LEVELS];
-    for (int i = 0; i < KCMG_MAX_LEVELS; ++i) { phase[i] = TEST; restarts[i] = 0; guard[i] = 0; }
-    int lev = lev0;
+    for (int i = 0; i < KCMG_MAX_LEVELS; ++i) { phase[i] = PRE; restarts[i] = 0; guard[i] = 0; }
+    enter(lev0);
     mark(lev);
     ph(PH_CONTROL);
-    sc[lev].rnorm0 = red_s[0];
-    sc[lev].rnorm0 = sqrt(sc[lev].rnorm0);
-    start(lev, sc[lev]);
+    start(sc[lev], L(lev).rtol);
+    // one smoother call or prolongation and one residual minimisation per pass
     while (ok) {
       const CoarseLevel& C = L(lev);
       LvScal& s = sc[lev];
-      if (phase[lev] == TEST) {
+      if (phase[lev] == CORRECT) {
+        prolong();                                                 // z = P z_c
+        if (!(ok = bar())) break;
+        ph(PH_TRANSFER);
+      } else {
         // while ||r|| > eps (level-local criteria of Sec. 4.2)
-        if (!(s.rnorm > s.eps && s.it < C.maxit && guard[lev] < (1 << 24))) {
+        if (phase[lev] == PRE && !(s.rnorm > s.eps && s.it < C.maxit && guard[lev] < (1 << 24))) {
           if (blockIdx.x == 0 && threadIdx.x == 0 && C.st) {
             C.st->iters_total += s.it;
             C.st->nrestart += restarts[lev];
           }
+          restarts[lev] = 0;
+          update_x(s);
           mark(lev);
           if (lev == lev0) break;
-          --lev;                                                   // return to the caller
-          if (!(ok = bar())) break;
+          if (!(ok = bar())) break;                                // x complete everywhere
           ph(PH_CONTROL);
+          enter(lev - 1);                                          // return to the caller
           continue;
         }
+        smooth();                                                  // pre- or post-smoother
+        if (!ok) break;
+      }
+      if (!(ok = rm(s))) break;
+      if (phase[lev] == PRE) {
         ++guard[lev];
-        T* z = smooth(lev, vec(C.r));                              // pre-smoother
-        if (!ok || !(ok = rm(lev, z, s))) break;
+        if (s.it == 0 && s.l == 0 && !(s.rnorm > 0.0)) {           // b = 0 (or not finite): x = 0
+          s.rnorm = 0.0;
+          continue;
+        }
+        T* rg = vec(C.r);
+        for (int lr = threadIdx.x; lr < rows; lr += blockDim.x) rg[row0 + lr] = rs[lr];
         if (!(ok = bar())) break;                                  // r complete everywhere
         const bool direct = (lev + 1 == a.nlev - 1);
-        const double nb = restrict_(lev, !direct);                 // r_c = R r
-        phase[lev] = AFTER_COARSE;
+        restrict_(!direct);                                        // r_c = R r
+        phase[lev] = CORRECT;
         if (direct) {
           if (!(ok = bar())) break;
           ph(PH_TRANSFER);
@@ -690,76 +835,62 @@ struct CoarseCycle {
           ph(PH_COARSEST);
           mark(lev + 1);
         } else {
-          double v[1] = {nb};
-          if (!(ok = reduce_few<1>(v))) break;
           ph(PH_TRANSFER);
           mark(lev);
-          ++lev;                                                   // z_c = MG(A_c, r_c, 0)
-          sc[lev].rnorm0 = sqrt(red_s[0]);
-          start(lev, sc[lev]);
-          phase[lev] = TEST;
+          enter(lev + 1);                                          // z_c = MG(A_c, r_c, 0)
+          start(sc[lev], L(lev).rtol);
+          phase[lev] = PRE;
         }
-        continue;
+      } else if (phase[lev] == CORRECT) {
+        phase[lev] = POST;
+      } else {
+        s.it++;
+        const int cap = (a.lmax > 0 && a.lmax < C.lcap) ? a.lmax : C.lcap;
+        if (s.l + 3 > cap) {                                       // restart: r = b - A x
+          update_x(s);
+          if (!(ok = bar())) break;
+          load_slabs<T>(vec(C.x), zsV(), true);
+          const T* b = vec(C.b);
+          for_rows<T, 0>(C.A, zsV(), [&](int lr, T v) { rs[lr] = ldv(b + row0 + lr) - v; });
+          count(opbytes(C, S, sizeof(T)) + (double)C.N * sizeof(T) * 3);
+          s.l = 0;
+          if (!(ok = residual_norm(s))) break;
+          ph(PH_RESTART);
+          ++restarts[lev];
+        }
+        phase[lev] = PRE;
       }
-      // AFTER_COARSE: prolongate, minimise, post-smooth, minimise
-      prolong(lev);                                                // z = P z_c
-      if (!(ok = bar())) break;
-      ph(PH_TRANSFER);
-      if (!(ok = rm(lev, vec(C.z), s))) break;
-      T* z = smooth(lev, vec(C.r));                                // post-smoother
-      if (!ok || !(ok = rm(lev, z, s))) break;
-      s.it++;
-      const int cap = (a.lmax > 0 && a.lmax < C.lcap) ? a.lmax : C.lcap;
-      if (s.l + 3 > cap) {                                         // restart: r = b - A x
-        if (!(ok = bar())) break;
-        double v[1] = {spmv(lev, vec(C.x), vec(C.r), vec(C.b))};
-        if (!(ok = reduce_few<1>(v))) break;
-        ph(PH_RESTART);
-        s.rnorm = sqrt(red_s[0]);
-        s.l = 0;
-        ++restarts[lev];
-      }
-      phase[lev] = TEST;
     }
   }
 };
 
-// Resident blocks per SM the register allocation must allow.  With 2 the kernel fits in
-// 94 registers without spills (158 with 1), so level-0 kernels of the task-parallel cycle
-// can run on its SMs beside it: measured 75.8 against 77.5 ms per 64^3 cycle, with the
-// coarse kernel itself slower (1.00 against 0.78 ms per launch) as it shares the SMs.
+// Resident blocks per SM the register allocation must allow.  With 2, level-0 kernels of the
+// task-parallel cycle can run on its SMs beside it.
 #ifndef KCMG_CC_MINBLOCKS
 #define KCMG_CC_MINBLOCKS 2
 #endif
 template <typename TV, typename TS, typename TI, int NP, int DIM>
-__global__ void __launch_bounds__(320, KCMG_CC_MINBLOCKS) k_coarse_cycle(CoarseArgs a) {
+__global__ void __launch_bounds__(320, KCMG_CC_MINBLOCKS) k_coarse_cycle(const __grid_constant__ CoarseArgs a) {
   using T = TV;
-  extern __shared__ unsigned char smem_raw[];
+  extern __shared__ __align__(16) unsigned char smem_cc[];
   __shared__ double sh[32 * 8];
-  __shared__ double red_s[kCoarseMaxCols];
-  __shared__ double cw[2 * kCoarseMaxCols];
+  __shared__ double red_s[kCoarseMaxCols + 4];
+  __shared__ double cf[kCoarseMaxCols];
   constexpr int NCH = 1 << DIM;
-  T* Ps = reinterpret_cast<T*>(smem_raw);   // prolongation matrices first (8-byte aligned)
-  TS* tile = reinterpret_cast<TS*>(Ps + NCH * NP * NP);
+  T* Ps = reinterpret_cast<T*>(smem_cc);   // prolongation matrices first
   const double* P = static_cast<const double*>(a.P);   // FP64 prolongation matrices
   for (int i = threadIdx.x; i < NCH * NP * NP; i += blockDim.x) Ps[i] = (T)P[i];
-  __syncthreads();
-  constexpr int M_AS = NCH * NP;
-  TS* as_rs = tile + blockDim.x;            // (blockDim / 32) warps x M_AS
-  CoarseCycle<TV, TS, TI, NP, DIM> cc{a, sh, red_s, tile, as_rs, Ps, cw};
+  CoarseCycle<TV, TS, TI, NP, DIM> cc{a, smem_cc, sh, red_s, cf, Ps};
   unsigned long long t0 = 0;
   if (blockIdx.x == 0 && threadIdx.x == 0) asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+  for (int l = a.lev0; l < a.nlev - 1; ++l) cc.build_mask(l);
   // start of MG on the first coarse level: b, r, x were set by the restriction kernel
-  const CoarseLevel& C = a.lv[a.lev0];
-  double nb = 0.0;
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < C.N; j += gridDim.x * blockDim.x) {
-    const double v = (double)ldv(static_cast<const T*>(C.b) + j);
-    nb += v * v;
-  }
-  double v[1] = {nb};
-  if (!cc.reduce_few<1>(v)) return;
-  cc.count((double)C.N * sizeof(T));
-  cc.run(a.lev0);   // reads ||b||^2 from red_s[0]
+  cc.enter(a.lev0);
+  for (int lr = threadIdx.x; lr < cc.rows; lr += blockDim.x)
+    cc.rs[lr] = ldv(static_cast<const T*>(a.lv[a.lev0].b) + cc.row0 + lr);
+  __syncthreads();
+  cc.count((double)a.lv[a.lev0].N * sizeof(T));
+  cc.run(a.lev0);
   // device time of this launch: every block has passed the last barrier of the cycle
   if (cc.ok) cc.ok = cc.bar();
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -769,6 +900,7 @@ __global__ void __launch_bounds__(320, KCMG_CC_MINBLOCKS) k_coarse_cycle(CoarseA
     atomicAdd(a.stat_launches, 1ull);
     atomicAdd(a.stat_bytes, cc.bytes);
   }
+  cc_leave(a);
 }
 
 }  // namespace

@@ -5,6 +5,8 @@
 #pragma once
 #include "coarse_cycle.cuh"
 
+#include <algorithm>
+
 namespace kcmg {
 
 #define KCMG_CC_SWITCH(np, dim, ...)                                   \
@@ -24,36 +26,86 @@ static void* coarse_kernel_ptr(int np, int dim) {
   return f;
 }
 
-static size_t coarse_cycle_smem(int np, int dim, int threads) {
-  // prolongation matrices (CC_TV), the smoother tile (threads x CC_T), and one gathered
-  // patch residual per warp for the Schwarz smoother ((threads / 32) x 2^d np x CC_T)
-  return (size_t)(1 << dim) * np * np * sizeof(CC_TV) + (size_t)threads * sizeof(CC_T) +
-         (size_t)(threads / 32) * (1 << dim) * np * sizeof(CC_T);
+// Blocks for a hierarchy whose largest level here has N unknowns in cells of np.  One block needs
+// no grid barrier (about 1 us a phase with every SM taking part) but has one SM's FP64 FMA rate,
+// two per clock: it wins while a sweep's FMAs take it less than that.  Otherwise one block per SM,
+// and no more blocks than cells.
+static int cc_blocks(const CoarseArgs& a, int nsm) {
+  const CoarseLevel& L = a.lv[a.lev0];
+  const long long fmas = (long long)L.N * (2 * a.dim + 1) * a.np;
+  if (fmas <= 6000) return 1;
+  const int cells = L.N / a.np;
+  return cells < nsm ? cells : nsm;
+}
+
+// longest basis whose coefficients are kept in shared memory (16 KB a level): the default 63
+constexpr int kCoarseCoefMax = 63;
+
+// shared-memory layout of a block (a multiple of 16 bytes for every piece)
+static void coarse_cycle_layout(CoarseArgs* a, int grid) {
+  int top = 0;
+  auto take = [&](size_t bytes) {
+    const int at = top;
+    top += (int)((bytes + 15) / 16 * 16);
+    return at;
+  };
+  const int nch = 1 << a->dim, segs = 2 * a->dim - 2;
+  take((size_t)nch * a->np * a->np * sizeof(CC_TV));   // prolongation matrices
+  size_t slab = 0, rows_max = 0;
+  for (int l = a->lev0; l < a->nlev; ++l) {
+    CoarseLevel& L = a->lv[l];
+    const int cells = L.N / a->np, own = (cells + grid - 1) / grid;
+    const size_t rows = (size_t)own * a->np;
+    if (l > a->lev0) slab = std::max(slab, rows * nch);                   // children of the own cells
+    if (l == a->nlev - 1) break;
+    slab = std::max(slab, (size_t)(own + 2 + (grid > 1 ? segs * own : 0)) * a->np);
+    rows_max = std::max(rows_max, rows);
+    L.sm_r = take(rows * sizeof(CC_TV));
+    L.coef_len = 2 * L.lcap + L.lcap * (L.lcap - 1) / 2;
+    L.sm_gm = L.lcap <= kCoarseCoefMax ? take((size_t)L.coef_len * sizeof(double)) : -1;
+    L.sm_mask = take(own);
+  }
+  a->sm_zv = take(slab * sizeof(CC_TV));
+  a->sm_zs = sizeof(CC_TV) == sizeof(CC_T) ? a->sm_zv : take(slab * sizeof(CC_T));
+  a->sm_ts = take(rows_max * sizeof(CC_T));
+  a->sm_ws = take(rows_max * sizeof(CC_TV));
+  a->sm_ps = take((size_t)kCoarseThreads * sizeof(double));
+  a->sm_as = a->smoother == 1 ? take((size_t)(kCoarseThreads / 32) * nch * a->np * sizeof(CC_T)) : 0;
+  a->sm_bytes = top;
 }
 
 template <>
-cudaError_t coarse_cycle_grid<CC_TV, CC_T, CC_TI>(int np, int dim, int threads, int* grid) {
-  void* f = coarse_kernel_ptr(np, dim);
+cudaError_t coarse_cycle_prepare<CC_TV, CC_T, CC_TI>(CoarseArgs* a, int* grid) {
+  void* f = coarse_kernel_ptr(a->np, a->dim);
   if (!f) return cudaErrorInvalidValue;
   int per_sm = 0, dev = 0, nsm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, threads,
-                                                                coarse_cycle_smem(np, dim, threads));
-  if (e != cudaSuccess) return e;
+  cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  int g = cc_blocks(*a, nsm);
+  if (*grid > 0 && *grid < g) g = *grid;   // the caller's cap
+  coarse_cycle_layout(a, g);
+  int optin = 0;
+  if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
+  cudaFuncAttributes fa;
+  if ((e = cudaFuncGetAttributes(&fa, f)) != cudaSuccess) return e;
+  if (a->sm_bytes + (int)fa.sharedSizeBytes > optin) return cudaErrorInvalidConfiguration;
+  if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, a->sm_bytes)) != cudaSuccess) return e;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, kCoarseThreads, a->sm_bytes)) != cudaSuccess)
+    return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  *grid = nsm;  // one resident block per SM: measured faster than two (fewer barrier arrivals)
+  *grid = g;
   return cudaSuccess;
 }
 
 template <>
-cudaError_t launch_coarse_cycle<CC_TV, CC_T, CC_TI>(const CoarseArgs& a, int grid, int threads, cudaStream_t s) {
+cudaError_t launch_coarse_cycle<CC_TV, CC_T, CC_TI>(const CoarseArgs& a, int grid, cudaStream_t s) {
   void* f = coarse_kernel_ptr(a.np, a.dim);
   if (!f) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = coarse_cycle_smem(a.np, a.dim, threads);
+  cfg.blockDim = dim3(kCoarseThreads);
+  cfg.dynamicSmemBytes = a.sm_bytes;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;

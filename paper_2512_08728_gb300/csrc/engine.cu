@@ -395,15 +395,13 @@ void build_hierarchy(kcmg_ctx* ctx, const double* blocks_src) {
 // FP64 residual minimisation over FP32-smoothed corrections acts as the iterative
 // refinement (the attainable residual is FP64's).
 void launch_coarse(kcmg_ctx* ctx, cudaStream_t s) {
-  CK(cudaMemsetAsync(ctx->cc.bar_count, 0, sizeof(unsigned int), s));   // barrier counter
   cudaError_t err;
-  const int thr = ctx->lv[ctx->cc_lev0].block_rows;
   const bool bf16 = ctx->p.precision == KCMG_MIXED_BF16INV || ctx->p.precision == KCMG_IR32_BF16INV;
-  if (!ctx->mixed) err = launch_coarse_cycle<double, double, double>(ctx->cc, ctx->cc_grid, thr, s);
-  else if (ctx->ir && bf16) err = launch_coarse_cycle<float, float, __nv_bfloat16>(ctx->cc, ctx->cc_grid, thr, s);
-  else if (ctx->ir) err = launch_coarse_cycle<float, float, float>(ctx->cc, ctx->cc_grid, thr, s);
-  else if (bf16) err = launch_coarse_cycle<double, float, __nv_bfloat16>(ctx->cc, ctx->cc_grid, thr, s);
-  else err = launch_coarse_cycle<double, float, float>(ctx->cc, ctx->cc_grid, thr, s);
+  if (!ctx->mixed) err = launch_coarse_cycle<double, double, double>(ctx->cc, ctx->cc_grid, s);
+  else if (ctx->ir && bf16) err = launch_coarse_cycle<float, float, __nv_bfloat16>(ctx->cc, ctx->cc_grid, s);
+  else if (ctx->ir) err = launch_coarse_cycle<float, float, float>(ctx->cc, ctx->cc_grid, s);
+  else if (bf16) err = launch_coarse_cycle<double, float, __nv_bfloat16>(ctx->cc, ctx->cc_grid, s);
+  else err = launch_coarse_cycle<double, float, float>(ctx->cc, ctx->cc_grid, s);
   CK(err);
 }
 
@@ -787,6 +785,7 @@ void init_states(kcmg_ctx* ctx, double rtol0, double atol0, int maxit0) {
   }
   if (ctx->coarse_kernel) {   // grid-barrier counter and error flag of the coarse cycle
     CK(cudaMemsetAsync(ctx->cc.bar_count, 0, sizeof(unsigned int), ctx->s));
+    CK(cudaMemsetAsync(ctx->cc.bar_gen, 0, sizeof(unsigned int), ctx->s));
     CK(cudaMemsetAsync(ctx->cc.err, 0, sizeof(int), ctx->s));
   }
   CK(cudaStreamSynchronize(ctx->s));
@@ -1252,21 +1251,6 @@ kcmg_ctx* build_ctx(const kcmg_params* p, cudaStream_t user, const double* block
         REQUIRE(ctx->lv[l].lcap + 1 <= kCoarseMaxCols,
                 "level %d keeps %d basis vectors; the persistent coarse cycle supports %d",
                 l, ctx->lv[l].lcap, kCoarseMaxCols - 1);
-      int grid = 0;
-      const int thr = ctx->lv[ctx->cc_lev0].block_rows;
-      cudaError_t ge;
-      const bool bf16 = p->precision == KCMG_MIXED_BF16INV || p->precision == KCMG_IR32_BF16INV;
-      if (!ctx->mixed) ge = coarse_cycle_grid<double, double, double>(ctx->np, ctx->dim, thr, &grid);
-      else if (ctx->ir && bf16) ge = coarse_cycle_grid<float, float, __nv_bfloat16>(ctx->np, ctx->dim, thr, &grid);
-      else if (ctx->ir) ge = coarse_cycle_grid<float, float, float>(ctx->np, ctx->dim, thr, &grid);
-      else if (bf16) ge = coarse_cycle_grid<double, float, __nv_bfloat16>(ctx->np, ctx->dim, thr, &grid);
-      else ge = coarse_cycle_grid<double, float, float>(ctx->np, ctx->dim, thr, &grid);
-      CK(ge);
-      if (const char* ev = getenv("KCMG_COARSE_GRID")) {   // tuning override, capped at residency
-        const int g = atoi(ev);
-        if (g > 0 && g < grid) grid = g;
-      }
-      ctx->cc_grid = grid;
       CoarseArgs& a = ctx->cc;
       memset(&a, 0, sizeof a);
       a.lev0 = ctx->cc_lev0;
@@ -1278,9 +1262,8 @@ kcmg_ctx* build_ctx(const kcmg_params* p, cudaStream_t user, const double* block
       a.sweeps = p->sweeps;
       a.lmax = p->lmax;
       a.brk = 1e-14;
-      a.partial_stride = (size_t)grid * kCoarseMaxCols;
-      a.partial = dalloc<double>(ctx, 2 * a.partial_stride);
-      a.red = dalloc<double>(ctx, kCoarseMaxCols);
+      a.smoother = p->smoother;
+      a.red = dalloc<double>(ctx, kCoarseMaxCols + 4);
       a.bar_count = dalloc<unsigned int>(ctx, 1);
       a.bar_gen = dalloc<unsigned int>(ctx, 1);
       a.err = dalloc<int>(ctx, 1);
@@ -1310,9 +1293,37 @@ kcmg_ctx* build_ctx(const kcmg_params* p, cudaStream_t user, const double* block
         c.as_z = L.as_z;
         c.as_r = L.as_r;
       }
-      a.smoother = p->smoother;
       a.Ainv = ctx->Ainv;
       a.Nc = ctx->Nc;
+      int grid_cap = 0, grid = 0;
+      if (const char* ev = getenv("KCMG_COARSE_GRID")) grid_cap = std::max(0, atoi(ev));   // tuning: fewer blocks
+      const bool bf16 = p->precision == KCMG_MIXED_BF16INV || p->precision == KCMG_IR32_BF16INV;
+      // a level whose blocks' share does not fit in shared memory stays on a kernel per step
+      for (;;) {
+        grid = grid_cap;
+        cudaError_t pe;
+        if (!ctx->mixed) pe = coarse_cycle_prepare<double, double, double>(&a, &grid);
+        else if (ctx->ir && bf16) pe = coarse_cycle_prepare<float, float, __nv_bfloat16>(&a, &grid);
+        else if (ctx->ir) pe = coarse_cycle_prepare<float, float, float>(&a, &grid);
+        else if (bf16) pe = coarse_cycle_prepare<double, float, __nv_bfloat16>(&a, &grid);
+        else pe = coarse_cycle_prepare<double, float, float>(&a, &grid);
+        if (pe != cudaErrorInvalidConfiguration) {
+          CK(pe);
+          break;
+        }
+        cudaGetLastError();
+        if (ctx->cc_lev0 + 1 >= ctx->nlev - 1) {
+          ctx->coarse_kernel = false;
+          break;
+        }
+        a.lev0 = ++ctx->cc_lev0;
+      }
+      if (!ctx->coarse_kernel) grid = 1;
+      for (int l = ctx->cc_lev0; l < ctx->nlev - 1; ++l)
+        if (a.lv[l].sm_gm < 0) a.lv[l].coef = dalloc<double>(ctx, (size_t)grid * a.lv[l].coef_len);
+      ctx->cc_grid = grid;
+      a.partial_stride = (size_t)grid * (kCoarseMaxCols + 4);
+      a.partial = dalloc<double>(ctx, 2 * a.partial_stride);
       ctx->stat_ns = dalloc<unsigned long long>(ctx, 1);
       ctx->stat_launches = dalloc<unsigned long long>(ctx, 1);
       ctx->stat_bytes = dalloc<double>(ctx, 1);

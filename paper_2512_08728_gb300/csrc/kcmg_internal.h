@@ -197,8 +197,8 @@ enum CoarsePhase : int {
   PH_SWEEP = 0,      // one block-Jacobi sweep
   PH_RM_GRAM1,       // w = A z, W^T w, ||w||^2 and their grid reduction
   PH_RM_REORTH,      // second Gram-Schmidt pass
-  PH_RM_UPDATE,      // new basis column, ||w_hat||^2, w_hat . r
-  PH_RM_FINISH,      // normalisation, x and r update
+  PH_RM_UPDATE,      // new basis column, r update
+  PH_RM_FINISH,      // (no phase of its own any more: part of PH_RM_UPDATE)
   PH_TRANSFER,       // restriction (with ||b_c||) or prolongation
   PH_COARSEST,       // dense solve on the coarsest level
   PH_RESTART,        // r = b - A x on a level restart
@@ -222,6 +222,13 @@ struct CoarseLevel {
   // Dinv), patch solutions and the sweep's residual (smoother precision)
   const void *as_inv0, *as_inv1;
   void *as_z, *as_r;
+  // a block's share in dynamic shared memory (byte offsets): residual of the own rows; gamma,
+  // alpha and the packed coefficients of Alg. 1; neighbour masks of the own cells
+  int sm_r, sm_gm, sm_mask;
+  // gamma, alpha and coefficients in global memory (coef_len doubles a block) where sm_gm < 0:
+  // bases so long that they do not fit
+  double* coef;
+  int coef_len;
 };
 
 struct CoarseArgs {
@@ -233,11 +240,14 @@ struct CoarseArgs {
   double omega;
   int sweeps, lmax;
   double brk;                  // breakdown threshold of Alg. 1
+  // dynamic shared memory (byte offsets): iterate slabs in the vector type and in the smoother's
+  // type, t, w, per-thread partial sums, gathered patch residuals; sm_bytes in all
+  int sm_zv, sm_zs, sm_ts, sm_ws, sm_ps, sm_as, sm_bytes;
   double* partial;             // 2 buffers of partial_stride doubles
-  size_t partial_stride;       // grid * kCoarseMaxCols
-  double* red;                 // kCoarseMaxCols reduced sums
-  unsigned int* bar_count;
-  unsigned int* bar_gen;
+  size_t partial_stride;       // grid * (kCoarseMaxCols + 4)
+  double* red;                 // kCoarseMaxCols + 4 reduced sums
+  unsigned int* bar_count;     // arrivals at the grid barrier in this launch
+  unsigned int* bar_gen;       // blocks that have left the kernel
   int* err;                    // set when a grid barrier timed out
   // measurement: launches, device nanoseconds and algorithmic bytes of every launch
   unsigned long long* stat_ns;
@@ -251,10 +261,15 @@ struct CoarseArgs {
 };
 
 // TV: vectors, bases and the residual minimisation; T: smoother sweeps; TI: stored inverses
+// threads per block of the coarse cycle
+constexpr int kCoarseThreads = 320;
+// blocks of the coarse cycle, chosen from its largest level (one block, or up to one per SM), and
+// the shared-memory layout in a (its levels' sizes, capacities and smoother are set);
+// cudaErrorInvalidConfiguration if a block's share does not fit
 template <typename TV, typename T, typename TI>
-cudaError_t coarse_cycle_grid(int np, int dim, int threads, int* grid);
+cudaError_t coarse_cycle_prepare(CoarseArgs* a, int* grid);
 template <typename TV, typename T, typename TI>
-cudaError_t launch_coarse_cycle(const CoarseArgs& a, int grid, int threads, cudaStream_t s);
+cudaError_t launch_coarse_cycle(const CoarseArgs& a, int grid, cudaStream_t s);
 
 // finest-level FP64 operator of a context, for the no-allocation residual (noalloc.cu)
 struct Level0View {
