@@ -276,8 +276,9 @@ MRHS_PRECISION = "mixed_bf16"
 # the batched FP32 sweep kernels the autotuner chooses from (kcmg_mrhs_tuning out[8])
 SWEEP_KERNELS = {0: "tensor-core TF32x3 smoother sweeps (FP32 accumulation)",
                  1: "tensor-core TF32x3 smoother sweeps, bulk-copy staged (FP32 accumulation)",
-                 2: "FP32 CUDA-core smoother sweeps"}
-SWEEP_KERNEL_NAMES = {0: "k_msweep_tc", 1: "k_msweep_tcb", 2: "k_msweep_simt"}
+                 2: "FP32 CUDA-core smoother sweeps",
+                 3: "FP32 CUDA-core smoother sweeps over the blocks' nonzero entries"}
+SWEEP_KERNEL_NAMES = {0: "k_msweep_tc", 1: "k_msweep_tcb", 2: "k_msweep_simt", 3: "k_mpat_sweep"}
 
 
 def run_adjoint(pkg, dev):
@@ -369,13 +370,18 @@ def run_mrhs(pkg, rank, dev, stream, hbm_peak, args, wl_name=None, maxiter=None)
     R = int(pm.b.shape[1])
     C = pm.ndof // pm.np_
     np2, S = pm.np_ * pm.np_, 2 * pm.d + 1
+    # entries a cell's blocks store: all, or those nonzero in some cell where the finest level's
+    # kernels skip the zeros (sweep kernel 3; the SpMM does whenever the blocks have the pattern)
+    nz = int((pm.blocks != 0).any(axis=1).sum())
+    nz0 = int((pm.blocks[0] != 0).any(axis=0).sum())
+    off = nz - nz0 if int(tune["sweep_kernel"]) == 3 else (S - 1) * np2
     inv_b = 2 if prec_m == "mixed_bf16" else 4
     # algorithmic bytes of one FP32 sweep (sweeps 2..5): FP32 off-diagonal blocks, stored
     # inverses, r (FP32) and the old and new iterates (FP32), each once
-    sweep_bytes = C * ((S - 1) * np2 * 4 + np2 * inv_b) + 3 * pm.ndof * R * 4
+    sweep_bytes = C * (off * 4 + np2 * inv_b) + 3 * pm.ndof * R * 4
     sweep_gbs = sweep_bytes / (tune["sweep_ms"] * 1e-3) / 1e9 if tune["sweep_ms"] > 0 else 0.0
-    # FP64 block SpMM: one FMA per block element and column
-    spmm_tflops = 2.0 * S * np2 * C * R / (tune["spmm_ms"] * 1e-3) / 1e12 if tune["spmm_ms"] > 0 else 0.0
+    # FP64 block SpMM: one FMA per nonzero block element and column
+    spmm_tflops = 2.0 * nz * C * R / (tune["spmm_ms"] * 1e-3) / 1e12 if tune["spmm_ms"] > 0 else 0.0
     return {
         "value": pm.ndof * R / (mms * 1e-3), "unit": UNIT, "workload": wname, "nrhs": R,
         # DOF-cycles per second (columns x DOFs x level-0 cycles / s): comparable with the

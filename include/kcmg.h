@@ -292,7 +292,8 @@ kcmg_status kcmg_smooth_multi(kcmg_ctx *ctx, int level, int nrhs, const double *
    out[8] the level-0 sweep kernel, the fastest of three: 0 = tensor cores (one warp per
    cell), 1 = tensor cores with each cell's blocks, inverse, r and neighbour slabs staged
    by double-buffered 1-D bulk copies, 2 = FP32 CUDA cores (register-blocked; exact FP32
-   products).  The environment variable KCMG_SWEEP = tc | tcb | simt, read at the first
+   products); 3 = not tuned: FP32 CUDA cores over the nonzero entries of a finest level with a
+   tensor basis's zero pattern.  The environment variable KCMG_SWEEP = tc | tcb | simt, read at the first
    batched solve, forces one kernel on every level.  Zero-filled up to nout. */
 kcmg_status kcmg_mrhs_tuning(kcmg_ctx *ctx, double *out, int nout);
 

@@ -1014,6 +1014,7 @@ MrhsView mrhs_view(kcmg_ctx* ctx) {
     v.nat[l] = L.nat;
     v.nbr[l] = L.nbr;
   }
+  v.pattern0 = ctx->lv[0].pat;
   v.P = ctx->P64;
   v.Ainv = ctx->Ainv;
   v.Nc = ctx->Nc;
@@ -1658,7 +1659,7 @@ kcmg_status kcmg_apply_multi(kcmg_ctx* ctx, int level, int nrhs, const double* x
     REQUIRE(!ctx->ir, "batched calls support the FP64 and mixed forms");
     kcmg_status st = mrhs_ensure(&ctx->mrhs, mrhs_view(ctx), nrhs, &ctx->err);
     if (st != KCMG_OK) return st;
-    return mrhs_apply(ctx->mrhs, level, x, y);
+    return mrhs_apply(ctx->mrhs, level, x, y, in_place_ok(ctx, x, y, (size_t)ctx->lv[level].N * nrhs));
   });
 }
 
@@ -1669,7 +1670,7 @@ kcmg_status kcmg_smooth_multi(kcmg_ctx* ctx, int level, int nrhs, const double* 
     REQUIRE(!ctx->ir, "batched calls support the FP64 and mixed forms");
     kcmg_status st = mrhs_ensure(&ctx->mrhs, mrhs_view(ctx), nrhs, &ctx->err);
     if (st != KCMG_OK) return st;
-    return mrhs_smooth(ctx->mrhs, level, r, z);
+    return mrhs_smooth(ctx->mrhs, level, r, z, in_place_ok(ctx, r, z, (size_t)ctx->lv[level].N * nrhs));
   });
 }
 

@@ -298,6 +298,7 @@ struct MrhsView {               // the context's hierarchy, as the batched solve
   int n[KCMG_MAX_LEVELS][3];
   int ncell[KCMG_MAX_LEVELS], N[KCMG_MAX_LEVELS];
   const double* nat[KCMG_MAX_LEVELS];   // FP64 blocks [S][C][np][np]
+  bool pattern0;                         // the finest level's blocks have a tensor basis's zeros
   const int* nbr[KCMG_MAX_LEVELS];
   const double* P;                       // [2^dim][np][np]
   const double* Ainv;                    // dense inverse of the coarsest operator
@@ -320,11 +321,25 @@ kcmg_status mrhs_solve(MrhsEngine** eng, const MrhsView& v, const double* b, dou
                        double rtol, double atol, int maxiter, kcmg_info* info, std::string* err);
 // Build (or rebuild for another nrhs / precision) the engine without solving.
 kcmg_status mrhs_ensure(MrhsEngine** eng, const MrhsView& v, int nrhs, std::string* err);
-// Batched component calls on an ensured engine (host or device pointers, [N_level][R]).
-kcmg_status mrhs_apply(MrhsEngine* eng, int level, const double* x, double* y);
-kcmg_status mrhs_smooth(MrhsEngine* eng, int level, const double* r, double* z);
+// Batched component calls on an ensured engine ([N_level][R]; direct: both in device memory and
+// not overlapping, used where they are; else host or device memory, staged).
+kcmg_status mrhs_apply(MrhsEngine* eng, int level, const double* x, double* y, bool direct);
+kcmg_status mrhs_smooth(MrhsEngine* eng, int level, const double* r, double* z, bool direct);
 // Launch shapes the autotuner chose (out[0..nout)), see kcmg_mrhs_tuning.
 int mrhs_tuning(const MrhsEngine* eng, double* out, int nout);
+
+// The finest level's batched operator and sweeps over the nonzero entries only (mrhs_pattern.cuh):
+// V from launch_mpattern_pack, D natural inverses; mode 0: y = A x, 2: y = b - A x compensated.
+// FP32 sweeps: TR = double reads the FP64 residual in the first sweep and leaves the FP32 copy in
+// r_lo, TZ = double writes an FP64 iterate in a later one.
+size_t mpattern_values(int np, int dim, int C);
+template <typename T>
+void launch_mpattern_pack(int np, int dim, const double* nat, const int* nbr, int C, T* V, cudaStream_t s);
+void launch_mpattern_spmm(int np, int dim, const int* n, int R, const double* V, const double* x, double* y,
+                          const double* b, int mode, cudaStream_t s);
+template <typename T, typename TI, typename TR, typename TZ>
+void launch_mpattern_sweep(int np, int dim, const int* n, int R, const T* V, const TI* D, const TR* r, T* r_lo,
+                           const T* zo, TZ* zn, double omega, int first, cudaStream_t s);
 
 // The batched FP32 block-Jacobi sweep on the CUDA cores (mrhs_simt.cu): Ac [C][S][np][np]
 // FP32 cell-major blocks, D [C][np][np] inverses, r32 / zo [C np][R] FP32, zn [C np][R];

@@ -1144,6 +1144,9 @@ struct MLev {
   // tuned launch shapes; sweep_kind: the FP32 sweep kernel (0: tensor cores, k_msweep_tc;
   // 1: tensor cores with bulk-copy staging, k_msweep_tcb; 2: CUDA cores, k_msweep_simt)
   int tc_wpb = 8, tc_grid = 0, sp_wpb = 8, sp_grid = 0, sweep_kind = 0;
+  // finest level with a tensor basis's zero pattern: its nonzero entries (FP64; FP32 sweeps)
+  double* V64 = nullptr;
+  float* V32 = nullptr;
   int tc_grid64 = 0;   // CUDA-core sweep: resident grid of its FP64-output form (last sweep)
 };
 
@@ -1215,6 +1218,11 @@ int grid_for(size_t items, int per_block, int cap) {
 
 // ---------------------------------------------------------------- launch wrappers
 void spmm64(MrhsEngine* E, const MLev& L, const double* x, double* y, const double* b, int mode) {
+  if (L.V64 && mode != 1) {
+    launch_mpattern_spmm(E->v.np, E->v.dim, L.n, E->R, L.V64, x, y, b, mode, E->s);
+    E->launches++;
+    return;
+  }
   const int thr = L.sp_wpb * 32;
   const int grid = L.sp_grid > 0 ? L.sp_grid : grid_for(L.C, L.sp_wpb, 1 << 30);
   MRHS_ND_SWITCH(E->v.np, E->v.dim, {
@@ -1341,21 +1349,48 @@ void read_flags(MrhsEngine* E, int lev) {
 }
 
 // ---------------------------------------------------------------- cycle pieces
-// z = BJ(r) on level lev (sweeps from z = 0); the result is L.z (FP64)
-void smooth(MrhsEngine* E, int lev) {
+// one FP32 pattern sweep with either kind of stored inverse
+template <typename TR, typename TZ>
+void sweep_pattern32(MrhsEngine* E, const MLev& L, const TR* r, float* r_lo, const float* zo, TZ* zn, bool first) {
+  if (L.D16)
+    launch_mpattern_sweep<float, __nv_bfloat16, TR, TZ>(E->v.np, E->v.dim, L.n, E->R, L.V32, L.D16, r, r_lo, zo, zn,
+                                                        E->v.omega, first, E->s);
+  else
+    launch_mpattern_sweep<float, float, TR, TZ>(E->v.np, E->v.dim, L.n, E->R, L.V32, L.D32, r, r_lo, zo, zn,
+                                                E->v.omega, first, E->s);
+  E->launches++;
+}
+
+// z = BJ(r) on level lev (sweeps from z = 0), FP64 in and out (rr, zz: default L.r, L.z)
+void smooth(MrhsEngine* E, int lev, const double* rr = nullptr, double* zz = nullptr) {
   MLev& L = E->lv[lev];
   const int sw = E->v.sweeps;
+  if (!rr) rr = L.r;
+  if (!zz) zz = L.z;
   if (!E->mixed) {
     double* buf[2] = {L.t, L.wre};
     for (int k = 0; k < sw; ++k) {
       const double* zo = buf[(k + 1) & 1];
-      double* zn = (k == sw - 1) ? L.z : buf[k & 1];
-      sweep64(E, L, L.r, zo, zn, k == 0);
+      double* zn = (k == sw - 1) ? zz : buf[k & 1];
+      if (L.V64) {
+        launch_mpattern_sweep<double, double, double, double>(E->v.np, E->v.dim, L.n, E->R, L.V64, L.D64, rr, nullptr,
+                                                              zo, zn, E->v.omega, k == 0, E->s);
+        E->launches++;
+      } else {
+        sweep64(E, L, rr, zo, zn, k == 0);
+      }
     }
     return;
   }
+  if (L.V32 && sw > 1) {   // conversions ride in the first and the last sweep
+    float* buf[2] = {L.s0, L.s1};
+    sweep_pattern32<double, float>(E, L, rr, L.r32, nullptr, buf[0], true);
+    for (int k = 1; k < sw - 1; ++k) sweep_pattern32<float, float>(E, L, L.r32, nullptr, buf[(k + 1) & 1], buf[k & 1], false);
+    sweep_pattern32<float, double>(E, L, L.r32, nullptr, buf[sw & 1], zz, false);
+    return;
+  }
   const size_t n = (size_t)L.N * E->R;
-  k_mto_f32<<<grid_for(n, 256, 4 * E->nsm * 8), 256, 0, E->s>>>(L.r, L.r32, n);
+  k_mto_f32<<<grid_for(n, 256, 4 * E->nsm * 8), 256, 0, E->s>>>(rr, L.r32, n);
   E->launches++;
   float* buf[2] = {L.s0, L.s1};
   for (int k = 0; k < sw; ++k) {
@@ -1364,8 +1399,8 @@ void smooth(MrhsEngine* E, int lev) {
     if (L.sweep_kind == 2) {
       if (k == sw - 1) {
         const int g64 = L.tc_grid64 > 0 ? L.tc_grid64 : grid;
-        if (L.D16) sweep_simt<__nv_bfloat16, double>(E, L, L.D16, L.r32, zo, L.z, k == 0, L.tc_wpb, g64);
-        else sweep_simt<float, double>(E, L, L.D32, L.r32, zo, L.z, k == 0, L.tc_wpb, g64);
+        if (L.D16) sweep_simt<__nv_bfloat16, double>(E, L, L.D16, L.r32, zo, zz, k == 0, L.tc_wpb, g64);
+        else sweep_simt<float, double>(E, L, L.D32, L.r32, zo, zz, k == 0, L.tc_wpb, g64);
       } else {
         if (L.D16) sweep_simt<__nv_bfloat16, float>(E, L, L.D16, L.r32, zo, buf[k & 1], k == 0, L.tc_wpb, grid);
         else sweep_simt<float, float>(E, L, L.D32, L.r32, zo, buf[k & 1], k == 0, L.tc_wpb, grid);
@@ -1374,8 +1409,8 @@ void smooth(MrhsEngine* E, int lev) {
     }
     if (L.sweep_kind == 1) {
       if (k == sw - 1) {
-        if (L.D16) sweep_tcb<__nv_bfloat16, double>(E, L, L.D16, L.r32, zo, L.z, k == 0, L.tc_wpb, grid);
-        else sweep_tcb<float, double>(E, L, L.D32, L.r32, zo, L.z, k == 0, L.tc_wpb, grid);
+        if (L.D16) sweep_tcb<__nv_bfloat16, double>(E, L, L.D16, L.r32, zo, zz, k == 0, L.tc_wpb, grid);
+        else sweep_tcb<float, double>(E, L, L.D32, L.r32, zo, zz, k == 0, L.tc_wpb, grid);
       } else {
         if (L.D16) sweep_tcb<__nv_bfloat16, float>(E, L, L.D16, L.r32, zo, buf[k & 1], k == 0, L.tc_wpb, grid);
         else sweep_tcb<float, float>(E, L, L.D32, L.r32, zo, buf[k & 1], k == 0, L.tc_wpb, grid);
@@ -1383,8 +1418,8 @@ void smooth(MrhsEngine* E, int lev) {
       continue;
     }
     if (k == sw - 1) {
-      if (L.D16) sweep_tc<__nv_bfloat16, double>(E, L, L.D16, L.r32, zo, L.z, k == 0, L.tc_wpb, grid);
-      else sweep_tc<float, double>(E, L, L.D32, L.r32, zo, L.z, k == 0, L.tc_wpb, grid);
+      if (L.D16) sweep_tc<__nv_bfloat16, double>(E, L, L.D16, L.r32, zo, zz, k == 0, L.tc_wpb, grid);
+      else sweep_tc<float, double>(E, L, L.D32, L.r32, zo, zz, k == 0, L.tc_wpb, grid);
     } else {
       if (L.D16) sweep_tc<__nv_bfloat16, float>(E, L, L.D16, L.r32, zo, buf[k & 1], k == 0, L.tc_wpb, grid);
       else sweep_tc<float, float>(E, L, L.D32, L.r32, zo, buf[k & 1], k == 0, L.tc_wpb, grid);
@@ -1580,12 +1615,18 @@ void autotune(MrhsEngine* E) {
   else if (fk && !strcmp(fk, "simt")) force_kind = 2;
   for (int lev = 0; lev < E->v.nlev - 1; ++lev) {
     MLev& L = E->lv[lev];
+    if (L.V64) L.sp_wpb = 4;
+    if (lev == 0) {
+      E->tune[0] = L.sp_wpb;
+      if (L.V32 && E->v.sweeps > 1) E->tune[2] = 4, E->tune[8] = 3;
+    }
     if (L.C < 256) continue;                        // small levels: defaults
     const int reps = lev == 0 ? 3 : 5;
-    // FP64 operator: warps per block
+    // FP64 operator: warps per block (the pattern kernels have one shape)
     float best = 1e30f;
     int best_w = L.sp_wpb;
     for (int wpb : {4, 8}) {
+      if (L.V64 && wpb != 4) continue;
       L.sp_wpb = wpb;
       L.sp_grid = 0;
       const float ms = time_it(E, [&] { spmm64(E, L, L.z, L.w, nullptr, 0); }, reps);
@@ -1594,6 +1635,14 @@ void autotune(MrhsEngine* E) {
     L.sp_wpb = best_w;
     if (lev == 0) { E->tune[0] = best_w; E->tune[1] = best; }
     if (!E->mixed) continue;
+    if (L.V32 && E->v.sweeps > 1) {
+      const float ms = time_it(E, [&] { sweep_pattern32<float, float>(E, L, L.r32, nullptr, L.s0, L.s1, false); }, reps);
+      E->tune[2] = 4;
+      E->tune[3] = 0;
+      E->tune[4] = ms;
+      E->tune[8] = 3;
+      continue;
+    }
     // tensor-core sweep: warps per block and grid (one warp per cell, or a resident grid)
     float bt = 1e30f;
     int bw = L.tc_wpb, bg = 0, bk = 0;
@@ -1701,6 +1750,15 @@ void build(MrhsEngine* E, const MrhsView& v, int R) {
     MCK(cudaMemsetAsync(fail, 0, sizeof(int), E->s));
     launch_block_inverse(np, L.A64, L.C, inv, fail, E->s);
     MCK(cudaGetLastError());
+    if (l == 0 && v.pattern0) {
+      const size_t nv = mpattern_values(np, v.dim, L.C);
+      L.V64 = malloc_dev<double>(E, nv);
+      launch_mpattern_pack<double>(np, v.dim, L.A64, L.nbr, L.C, L.V64, E->s);
+      if (E->mixed && !getenv("KCMG_SWEEP")) {   // a forced sweep kernel runs on every level
+        L.V32 = malloc_dev<float>(E, nv);
+        launch_mpattern_pack<float>(np, v.dim, L.A64, L.nbr, L.C, L.V32, E->s);
+      }
+    }
     if (!E->mixed) {
       L.D64 = malloc_dev<double>(E, L.C * bs);
       MCK(cudaMemcpyAsync(L.D64, inv, L.C * bs * sizeof(double), cudaMemcpyDeviceToDevice, E->s));
@@ -1804,14 +1862,14 @@ kcmg_status mrhs_ensure(MrhsEngine** peng, const MrhsView& v, int R, std::string
   }
 }
 
-kcmg_status mrhs_apply(MrhsEngine* E, int level, const double* x, double* y) {
+kcmg_status mrhs_apply(MrhsEngine* E, int level, const double* x, double* y, bool direct) {
   try {
     MLev& L = E->lv[level];
     const size_t NR = (size_t)L.N * E->R;
-    MCK(cudaMemcpyAsync(L.z, x, NR * sizeof(double), cudaMemcpyDefault, E->s));
-    spmm64(E, L, L.z, L.w, nullptr, 0);
+    if (!direct) MCK(cudaMemcpyAsync(L.z, x, NR * sizeof(double), cudaMemcpyDefault, E->s));
+    spmm64(E, L, direct ? x : L.z, direct ? y : L.w, nullptr, 0);
     MCK(cudaGetLastError());
-    MCK(cudaMemcpyAsync(y, L.w, NR * sizeof(double), cudaMemcpyDefault, E->s));
+    if (!direct) MCK(cudaMemcpyAsync(y, L.w, NR * sizeof(double), cudaMemcpyDefault, E->s));
     MCK(cudaStreamSynchronize(E->s));
     return KCMG_OK;
   } catch (Fail2& f) {
@@ -1819,14 +1877,14 @@ kcmg_status mrhs_apply(MrhsEngine* E, int level, const double* x, double* y) {
   }
 }
 
-kcmg_status mrhs_smooth(MrhsEngine* E, int level, const double* r, double* z) {
+kcmg_status mrhs_smooth(MrhsEngine* E, int level, const double* r, double* z, bool direct) {
   try {
     MLev& L = E->lv[level];
     const size_t NR = (size_t)L.N * E->R;
-    MCK(cudaMemcpyAsync(L.r, r, NR * sizeof(double), cudaMemcpyDefault, E->s));
-    smooth(E, level);
+    if (!direct) MCK(cudaMemcpyAsync(L.r, r, NR * sizeof(double), cudaMemcpyDefault, E->s));
+    smooth(E, level, direct ? r : L.r, direct ? z : L.z);
     MCK(cudaGetLastError());
-    MCK(cudaMemcpyAsync(z, L.z, NR * sizeof(double), cudaMemcpyDefault, E->s));
+    if (!direct) MCK(cudaMemcpyAsync(z, L.z, NR * sizeof(double), cudaMemcpyDefault, E->s));
     MCK(cudaStreamSynchronize(E->s));
     return KCMG_OK;
   } catch (Fail2& f) {

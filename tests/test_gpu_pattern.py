@@ -118,3 +118,42 @@ def test_calls_on_overlapping_and_misaligned_vectors_are_staged():
         assert torch.equal(out[1:], want)
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("d,p,n", GRIDS)
+@pytest.mark.parametrize("nrhs", [2, 8, 9, 32])
+def test_batched_pattern_kernels_equal_the_dense_kernels(d, p, n, nrhs, monkeypatch):
+    """FP64 against the batched dense kernels; FP32 against the CUDA-core sweep (the forced sweep
+    kernel runs on every level).  Columns that fill a lane group, one more, and a full warp."""
+    pr, a, b, rng = _pair(d, p, n, "fp64")
+    X = rng.standard_normal((pr.ndof, nrhs))
+    X[[3, pr.ndof // 2], 1] = np.inf, np.nan            # in one column only
+    assert np.array_equal(a.apply_multi(0, X), b.apply_multi(0, X), equal_nan=True)
+    assert np.array_equal(a.smooth_multi(0, X), b.smooth_multi(0, X), equal_nan=True)
+    Xd = torch.from_numpy(X).cuda()                     # on the caller's vectors
+    assert np.array_equal(a.apply_multi(0, Xd).cpu().numpy(), a.apply_multi(0, X), equal_nan=True)
+    a.close()
+    b.close()
+    for precision in ("mixed", "mixed_bf16"):
+        pr, a, b, rng = _pair(d, p, n, precision)
+        za = a.smooth_multi(0, X)
+        monkeypatch.setenv("KCMG_SWEEP", "simt")
+        zb = b.smooth_multi(0, X)
+        monkeypatch.delenv("KCMG_SWEEP")
+        assert np.array_equal(za, zb, equal_nan=True)
+        assert np.array_equal(a.smooth_multi(0, Xd).cpu().numpy(), za, equal_nan=True)
+        a.close()
+        b.close()
+
+
+@pytest.mark.parametrize("sweeps", [1, 2])
+def test_batched_pattern_sweeps_with_fp32_conversions(sweeps, monkeypatch):
+    pr, a, b, rng = _pair(3, 2, (6, 6, 2), "mixed", sweeps=sweeps)
+    R = rng.standard_normal((pr.ndof, 8))
+    if sweeps == 1:
+        monkeypatch.setenv("KCMG_SWEEP", "simt")        # both on the kernel that a single sweep takes
+    za = a.smooth_multi(0, R)
+    monkeypatch.setenv("KCMG_SWEEP", "simt")
+    assert np.array_equal(za, b.smooth_multi(0, R))
+    a.close()
+    b.close()
