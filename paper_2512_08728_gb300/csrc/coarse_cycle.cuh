@@ -22,10 +22,14 @@
 //     orthogonalisation coefficients) is formed when the level returns or restarts, so Alg. 1's
 //     second recurrence costs one pass over the corrections per visit, not one per correction.
 //   - A level set too small to pay for a grid barrier runs in one block (cc_blocks()).
-// Measured (GB300, one launch, against blocks that took whole 320-row tiles and reduced three
-// times a minimisation): levels 16^3 and 8^3 at np = 10 beside the finest level's kernels 971 ->
-// 704 us; 64 x 48 and two levels below at np = 10, 2-D, 8.4 -> 5.3 ms a visit; 192 unknowns 749 ->
-// 370 us.
+//   - FP64 instructions are scarce (one of a warp takes its SM 16 clocks), so scalars are computed
+//     by one warp, sums over lanes are transposed (several columns at a time) and bytes are
+//     counted in integers.
+// Measured (GB300, one launch; first the kernel whose blocks took whole 320-row tiles, read every
+// neighbour value through L2 and reduced three times a minimisation): levels 16^3 and 8^3 at
+// np = 10 beside the finest level's kernels 971 -> 553 us; 64 x 48 and two levels below at
+// np = 10, 2-D, 16.7 -> 8.4 ms; 16^3 and 8^3 alone, 16 visits, 5.0 -> 2.7 ms; 192 unknowns
+// 749 -> 257 us.
 // Every control decision is taken by all blocks from the same reduced values (fixed reduction
 // order), so all blocks follow the same path.  The grid barrier spins with a bound: if it ever
 // times out it raises an error flag and every block leaves the kernel, so a fault becomes a
@@ -40,6 +44,8 @@
 #include <cmath>
 
 namespace kcmg {
+
+extern __shared__ __align__(16) unsigned char smem_cc[];   // layout: CoarseArgs / CoarseLevel offsets
 
 namespace {
 
@@ -122,8 +128,15 @@ namespace {
 
 // Per-level scalars, held identically by every block.
 struct LvScal {
-  int l, it, first;      // first: no reduction done yet on this visit (rnorm0 unknown)
-  double rnorm, eps;
+  int l, it, first;      // first: no reduction done yet on this visit (||b|| unknown)
+  double r2, eps2;       // ||r||^2 and the squared tolerance
+};
+
+// Scalars of a residual minimisation, computed by warp 0 and read by the block: FP64 instructions
+// are scarce (16 clocks an SM for one of a warp), so what is the same for all threads is done once.
+struct RmScal {
+  double rr, naz2, gam, alp, r2new;
+  int verdict;           // 0 take the correction, 1 another Gram-Schmidt pass, 2 discard it
 };
 
 // Vectors, basis W, Z, the Alg. 1 operator and the transfers are in TV (FP64, or FP32 in
@@ -137,42 +150,43 @@ struct CoarseCycle {
   static constexpr int S = 2 * DIM + 1;
   static constexpr int JP = (NP + 1) / 2;
   static constexpr int NCH = 1 << DIM;
-  static constexpr int SEGS = 2 * DIM - 1;   // slabs of the iterate: own with both x ends, +-y, +-z
 
   const CoarseArgs& a;
-  unsigned char* smem;   // dynamic shared memory (CoarseArgs offsets)
   double* sh;            // 32 * 8 doubles
   double* red_s;         // reduced sums, kCoarseMaxCols + 4
   double* cf;            // coefficients of the minimisation, kCoarseMaxCols
+  RmScal* rms;
+  int* nbs;              // neighbour slab of each slot: cell offset in the slab buffer
+  long long* tph;        // clocks per phase kind, then per level (thread 0 of block 0)
   T* Ps;                 // NCH*NP*NP (prolongation matrices)
   int rcount = 0;        // reductions done (selects the partial buffer)
   unsigned int gen = 0;  // grid barriers passed (identical in every block)
   bool ok = true;
-  double bytes = 0.0;    // algorithmic bytes of this launch (kept by thread 0 of block 0)
+  long long bytes = 0;   // algorithmic bytes of this launch (kept by thread 0 of block 0)
 
   // the block's range on the current level (set by enter())
   int lev = 0, K0 = 0, nc = 0, rows = 0, row0 = 0;
   int lpr = 1, part = 0, lrow = 0;   // threads per row; this thread's part and row (rows < blockDim)
-  int nb_off[S] = {};                // neighbour slab of each slot: cell offset in the slab buffer
-  unsigned char* mask = nullptr;     // per own cell: bit s set if the neighbour of slot s exists
-  T* rs = nullptr;                   // residual, own rows
+  int rs_off = 0;                    // residual, own rows (byte offset)
+  int own0 = 0;                      // the own rows' place in the slab buffer
   double *R = nullptr, *gm = nullptr, *al = nullptr;   // packed columns of R, 1 / R_kk, alpha
 
   __device__ bool bar() { return cc_barrier(a, gen); }
-  __device__ void count(double b) {
+  __device__ void count(long long b) {
     if (blockIdx.x == 0 && threadIdx.x == 0) bytes += b;
   }
   // unique operator bytes of n slots on a level with this element size
-  __device__ double opbytes(const CoarseLevel& C, int slots, int elem) const {
-    return (double)slots * C.N * NP * elem;
+  __device__ long long opbytes(const CoarseLevel& C, int slots, int elem) const {
+    return (long long)slots * C.N * NP * elem;
   }
   __device__ const CoarseLevel& L(int l) const { return a.lv[l]; }
   __device__ T* vec(void* p) const { return static_cast<T*>(p); }
-  __device__ T* zsV() const { return reinterpret_cast<T*>(smem + a.sm_zv); }
-  __device__ TS* zsS() const { return reinterpret_cast<TS*>(smem + a.sm_zs); }
-  __device__ TS* ts() const { return reinterpret_cast<TS*>(smem + a.sm_ts); }
-  __device__ T* ws() const { return reinterpret_cast<T*>(smem + a.sm_ws); }
-  __device__ double* ps() const { return reinterpret_cast<double*>(smem + a.sm_ps); }
+  __device__ T* zsV() const { return reinterpret_cast<T*>(smem_cc + a.sm_zv); }
+  __device__ TS* zsS() const { return reinterpret_cast<TS*>(smem_cc + a.sm_zs); }
+  __device__ TS* ts() const { return reinterpret_cast<TS*>(smem_cc + a.sm_ts); }
+  __device__ T* ws() const { return reinterpret_cast<T*>(smem_cc + a.sm_ws); }
+  __device__ T* rs_() const { return reinterpret_cast<T*>(smem_cc + rs_off); }
+  __device__ double* ps() const { return reinterpret_cast<double*>(smem_cc + a.sm_ps); }
 
   // first cell of block b on a level of C cells
   __device__ static int first_cell(int C, int b) { return (int)(((long long)C * b) / gridDim.x); }
@@ -185,134 +199,157 @@ struct CoarseCycle {
     nc = first_cell(cells, blockIdx.x + 1) - K0;
     rows = nc * NP;
     row0 = K0 * NP;
-    lpr = rows > 0 ? min(8, max(1, (int)blockDim.x / rows)) : 1;
+    // threads per row: 8, 4, 2 or 1, as many as the block has
+    lpr = 1;
+    while (rows > 0 && lpr < 8 && 2 * lpr * rows <= (int)blockDim.x) lpr *= 2;
     part = 0;
     lrow = threadIdx.x;
     if (lpr > 1) {
       part = threadIdx.x / rows;
       lrow = threadIdx.x - part * rows;
     }
-    mask = smem + C.sm_mask;
-    rs = reinterpret_cast<T*>(smem + C.sm_r);
-    gm = C.sm_gm >= 0 ? reinterpret_cast<double*>(smem + C.sm_gm) : C.coef + (size_t)blockIdx.x * C.coef_len;
+    rs_off = C.sm_r;
+    gm = C.sm_gm >= 0 ? reinterpret_cast<double*>(smem_cc + C.sm_gm) : C.coef + (size_t)blockIdx.x * C.coef_len;
     al = gm + C.lcap;
     R = al + C.lcap;
     // slab buffer: [own cells with one more on each side | -y | +y | -z | +z]; one block owns all
-    // cells, and its own slab serves every slot
-    const int st[3] = {1, C.n[0], C.n[0] * C.n[1]};
-    nb_off[0] = 1;
-#pragma unroll
-    for (int k = 0; k < DIM; ++k)
-#pragma unroll
-      for (int side = 0; side < 2; ++side) {
-        const int s = 1 + 2 * k + side;
-        nb_off[s] = (k == 0 || gridDim.x == 1) ? 1 + (side ? st[k] : -st[k]) : (nc + 2) + (2 * (k - 1) + side) * nc;
-      }
-  }
-
-  // existence masks of a level's own cells (once per launch)
-  __device__ void build_mask(int l) {
-    enter(l);
-    const CoarseLevel& C = L(l);
-    for (int c = threadIdx.x; c < nc; c += blockDim.x) {
-      const int K = K0 + c;
-      const int x[3] = {K % C.n[0], (K / C.n[0]) % C.n[1], DIM == 3 ? K / (C.n[0] * C.n[1]) : 0};
-      unsigned m = 1u;
-#pragma unroll
-      for (int k = 0; k < DIM; ++k) {
-        if (x[k] > 0) m |= 1u << (1 + 2 * k);
-        if (x[k] < C.n[k] - 1) m |= 1u << (2 + 2 * k);
-      }
-      mask[c] = (unsigned char)m;
-    }
-  }
-
-  // ---------------------------------------------------------------- slabs
-  // the neighbours' cells of the iterate z (global) into the slab buffer; with own: the block's
-  // own cells too.  Cells outside the grid are skipped (never read: the masks).
-  template <typename TX>
-  __device__ void load_slabs(const TX* z, TX* buf, bool own) {
-    const CoarseLevel& C = L(lev);
-    const int cells = C.N / NP;
-    if (own)
-      for (int i = threadIdx.x; i < rows; i += blockDim.x) buf[NP + i] = ldv(z + row0 + i);
-    if (gridDim.x > 1) {
-      if (threadIdx.x < 2 * NP) {   // the x neighbours of the range's ends
-        const int hi = threadIdx.x >= NP, q = threadIdx.x - hi * NP;
-        const int K = hi ? K0 + nc : K0 - 1;
-        if (K >= 0 && K < cells) buf[(hi ? (nc + 1) * NP : 0) + q] = ldv(z + (size_t)K * NP + q);
-      }
-      const int st[3] = {1, C.n[0], C.n[0] * C.n[1]};
-#pragma unroll
-      for (int k = 1; k < DIM; ++k)
-#pragma unroll
-        for (int side = 0; side < 2; ++side) {
-          const int base = (nc + 2 + (2 * (k - 1) + side) * nc) * NP;
-          const int g0 = (K0 + (side ? st[k] : -st[k])) * NP;
-          for (int i = threadIdx.x; i < rows; i += blockDim.x)
-            if (g0 + i >= 0 && g0 + i < C.N) buf[base + i] = ldv(z + g0 + i);
-        }
+    // cells, and its own slab, with the largest stride of zeros on each side, serves every slot
+    const int pad = gridDim.x == 1 ? (DIM == 2 ? C.n[0] : C.n[0] * C.n[1]) : 1;
+    own0 = pad * NP;
+    __syncthreads();
+    if (threadIdx.x < S) {
+      const int s = threadIdx.x, k = (s - 1) / 2, side = (s - 1) & 1;
+      const int st = k == 0 ? 1 : k == 1 ? C.n[0] : C.n[0] * C.n[1];
+      nbs[s] = s == 0 ? pad
+               : (k == 0 || gridDim.x == 1) ? pad + (side ? st : -st)
+                                            : (nc + 2) + (2 * (k - 1) + side) * nc;
     }
     __syncthreads();
   }
 
-  // sum over slots FROM.. of A_{K,s} z_{nbr(K,s)} for own row lr (this thread's share of the pairs)
-  template <typename TX, int FROM>
-  __device__ __forceinline__ TX row_sum(const void* Aop, const TX* buf, int lr, int q, int np) {
+  // ---------------------------------------------------------------- slabs
+  // The neighbours' cells of the iterate z (global) into the slab buffer; with own: the block's
+  // own cells too.  All loads of a thread are in flight together: one L2 round trip.  Cells past
+  // the grid's ends read as zero.  Cells that are in range but not neighbours (across a face of
+  // the grid) need no mask: a Galerkin block towards a missing neighbour is exactly zero.
+  template <typename TX>
+  __device__ void load_slabs(const TX* z, TX* buf, bool own) {
+    const CoarseLevel& C = L(lev);
+    constexpr int NS = 2 * DIM - 2;
+    if (own)
+      for (int i = threadIdx.x; i < rows; i += blockDim.x) buf[own0 + i] = ldv(z + row0 + i);
+    if (gridDim.x > 1) {
+      const int st[2] = {C.n[0] * NP, C.n[0] * C.n[1] * NP};
+      for (int i = threadIdx.x; i < rows; i += blockDim.x) {
+        TX v[NS];
+#pragma unroll
+        for (int k = 0; k < NS; ++k) {
+          const int g = row0 + i + (k & 1 ? st[k / 2] : -st[k / 2]);
+          v[k] = (g >= 0 && g < C.N) ? ldv(z + g) : TX(0);
+        }
+#pragma unroll
+        for (int k = 0; k < NS; ++k) buf[(nc + 2 + k * nc) * NP + i] = v[k];
+      }
+      const int q = (int)blockDim.x - 1 - (int)threadIdx.x;   // the x neighbours of the range's ends
+      if (q < 2 * NP) {
+        const int g = q < NP ? row0 - NP + q : row0 + rows + q - NP;
+        buf[q < NP ? q : (nc + 1) * NP + q - NP] = (g >= 0 && g < C.N) ? ldv(z + g) : TX(0);
+      }
+    } else {   // one block: zeros on both sides (the transfers use the buffer too)
+      for (int i = threadIdx.x; i < own0; i += blockDim.x) buf[i] = buf[own0 + rows + i] = TX(0);
+    }
+    __syncthreads();
+  }
+
+  // pairs of operator entries of a row over slots FROM.. and how many a thread takes with LPR
+  // threads a row; with eight they are kept in registers over the sweeps of a smoother call
+  template <int FROM, int LPR> struct Trips { static constexpr int N = ((S - FROM) * JP + LPR - 1) / LPR; };
+  static constexpr int kKeep = Trips<1, 8>::N;
+
+  template <typename TX, int FROM, int LPR, int B, int U>
+  __device__ __forceinline__ void load_pairs(const void* Aop, int lr, int q, typename V2T<TX>::type (&av)[U]) const {
     using VX = typename V2T<TX>::type;
     const CoarseLevel& C = L(lev);
-    const int c = lr / NP, row = row0 + lr, g = row >> 5, lane = row & 31;
+    const int row = row0 + lr, g = row >> 5, lane = row & 31;
     const VX* Ap = reinterpret_cast<const VX*>(Aop) + (size_t)g * JP * 32 + lane;
     const size_t sl = (size_t)C.G * JP * 32;
-    const unsigned m = mask[c];
-    if (np == 1) {
-      TX acc[4] = {TX(0), TX(0), TX(0), TX(0)};   // independent FMA chains (latency)
 #pragma unroll
-      for (int s = FROM; s < S; ++s) {
-        if (!((m >> s) & 1u)) continue;
-        const TX* zp = buf + (size_t)(nb_off[s] + c) * NP;
-        const int k = (s & 1) << 1;
-#pragma unroll
-        for (int jp = 0; jp < JP; ++jp) {
-          const VX av = __ldg(Ap + s * sl + jp * 32);
-          acc[k] = fma(av.x, zp[2 * jp], acc[k]);
-          if (2 * jp + 1 < NP) acc[k + 1] = fma(av.y, zp[2 * jp + 1], acc[k + 1]);
-        }
+    for (int u = 0; u < U; ++u) {
+      const int e = FROM * JP + q + (B + u) * LPR;
+      if (LPR == 1 ? B + u < Trips<FROM, LPR>::N : e < S * JP) {
+        const int s = e / JP, jp = e - s * JP;
+        av[u] = __ldg(Ap + s * sl + jp * 32);
+      } else {
+        av[u].x = TX(0);
+        av[u].y = TX(0);
       }
-      return (acc[0] + acc[1]) + (acc[2] + acc[3]);
     }
-    TX a0 = TX(0), a1 = TX(0);
-#pragma unroll 6
-    for (int e = FROM * JP + q; e < S * JP; e += np) {
-      const int s = e / JP, jp = e - s * JP;
-      if (!((m >> s) & 1u)) continue;
-      int off = nb_off[0];
+  }
+  template <typename TX, int FROM, int LPR, int B, int U>
+  __device__ __forceinline__ void apply_pairs(const TX* buf, int c, int q, const typename V2T<TX>::type (&av)[U],
+                                              TX (&acc)[4]) const {
 #pragma unroll
-      for (int t = 1; t < S; ++t)
-        if (s == t) off = nb_off[t];
-      const TX* zp = buf + (size_t)(off + c) * NP + 2 * jp;
-      const VX av = __ldg(Ap + s * sl + jp * 32);
-      a0 = fma(av.x, zp[0], a0);
-      if (2 * jp + 1 < NP) a1 = fma(av.y, zp[1], a1);
+    for (int u = 0; u < U; ++u) {
+      const int e = FROM * JP + q + (B + u) * LPR;
+      if (LPR == 1 ? B + u < Trips<FROM, LPR>::N : e < S * JP) {
+        const int s = e / JP, jp = e - s * JP, k = LPR >= 4 ? 0 : (u & 1) << 1;   // chains
+        const TX* zp = buf + (nbs[s] + c) * NP + 2 * jp;
+        acc[k] = fma(av[u].x, zp[0], acc[k]);
+        if (NP % 2 == 0 || jp + 1 < JP) acc[k + 1] = fma(av[u].y, zp[1], acc[k + 1]);
+      }
     }
-    return a0 + a1;
+  }
+  // sum over slots FROM.. of A_{K,s} z_{nbr(K,s)} for own row lr: this thread's share
+  template <typename TX, int FROM, int LPR, int B = 0>
+  __device__ __forceinline__ void row_share(const void* Aop, const TX* buf, int lr, int q, TX (&acc)[4]) const {
+    constexpr int T0 = Trips<FROM, LPR>::N, U = T0 - B < 8 ? T0 - B : 8;
+    typename V2T<TX>::type av[U];
+    load_pairs<TX, FROM, LPR, B, U>(Aop, lr, q, av);
+    apply_pairs<TX, FROM, LPR, B, U>(buf, lr / NP, q, av, acc);
+    if constexpr (B + U < T0) row_share<TX, FROM, LPR, B + U>(Aop, buf, lr, q, acc);
   }
 
   // f(own row, sum) in one thread per row, over slots FROM..; ends with every thread past the
   // reads of the slab buffer
+  template <typename TX, int FROM, int LPR, typename F>
+  __device__ __forceinline__ void for_rows_l(const void* Aop, const TX* buf, F&& f) {
+    TX* p = reinterpret_cast<TX*>(ps());
+    if (part < LPR) {
+      TX acc[4] = {TX(0), TX(0), TX(0), TX(0)};
+      row_share<TX, FROM, LPR>(Aop, buf, lrow, part, acc);
+      p[part * rows + lrow] = LPR >= 4 ? acc[0] + acc[1] : (acc[0] + acc[1]) + (acc[2] + acc[3]);
+    }
+    sum_shares<TX, LPR>(f);
+  }
+  template <typename TX, int LPR, typename F>
+  __device__ __forceinline__ void sum_shares(F&& f) {
+    const TX* p = reinterpret_cast<const TX*>(ps());
+    __syncthreads();
+    if (threadIdx.x < rows) {
+      TX v[LPR];
+#pragma unroll
+      for (int q = 0; q < LPR; ++q) v[q] = p[q * rows + threadIdx.x];
+#pragma unroll
+      for (int o = LPR / 2; o; o >>= 1)
+#pragma unroll
+        for (int q = 0; q < o; ++q) v[q] += v[q + o];
+      f((int)threadIdx.x, v[0]);
+    }
+  }
   template <typename TX, int FROM, typename F>
   __device__ __forceinline__ void for_rows(const void* Aop, const TX* buf, F&& f) {
     if (lpr == 1) {
-      for (int lr = threadIdx.x; lr < rows; lr += blockDim.x) f(lr, row_sum<TX, FROM>(Aop, buf, lr, 0, 1));
-    } else {
-      TX* p = reinterpret_cast<TX*>(ps());
-      if (part < lpr) p[part * rows + lrow] = row_sum<TX, FROM>(Aop, buf, lrow, part, lpr);
-      __syncthreads();
-      if (threadIdx.x < rows) {
-        TX v = p[threadIdx.x];
-        for (int q = 1; q < lpr; ++q) v += p[q * rows + threadIdx.x];
-        f((int)threadIdx.x, v);
+      for (int lr = threadIdx.x; lr < rows; lr += blockDim.x) {
+        TX acc[4] = {TX(0), TX(0), TX(0), TX(0)};   // independent FMA chains (latency)
+        row_share<TX, FROM, 1>(Aop, buf, lr, 0, acc);
+        f(lr, (acc[0] + acc[1]) + (acc[2] + acc[3]));
       }
+    } else if (lpr == 2) {
+      for_rows_l<TX, FROM, 2>(Aop, buf, f);
+    } else if (lpr == 4) {
+      for_rows_l<TX, FROM, 4>(Aop, buf, f);
+    } else {
+      for_rows_l<TX, FROM, 8>(Aop, buf, f);
     }
     __syncthreads();
   }
@@ -320,23 +357,36 @@ struct CoarseCycle {
   // ---------------------------------------------------------------- smoother
   // One sweep of Alg. BJ in TS on the own cells: t = r - A_off zo (skipped on the first sweep
   // from z = 0), zn = (1 - omega) zo + omega D^{-1} t.  The own iterate is in the slab buffer; the
-  // new one goes to global memory for the neighbours and, in TO, to the slab buffer out.
-  template <typename TO>
-  __device__ void sweep(const TS* zo, TO* zn, TO* out, bool first) {
+  // new one goes to global memory for the neighbours and, in TO, to the slab buffer out.  With
+  // KEEP > 1 the thread's operator entries are in av (KEEP threads a row).
+  template <int KEEP, typename TO>
+  __device__ __forceinline__ void sweep(const TS* zo, TO* zn, TO* out, bool first, const VS2 (&av)[kKeep]) {
     const CoarseLevel& C = L(lev);
     count(opbytes(C, first ? 0 : S - 1, a.smoother_bytes) + opbytes(C, 1, a.inverse_bytes) +
-          (double)C.N * (sizeof(T) + sizeof(TO) + (first ? 0 : sizeof(TS))));
+          (long long)C.N * (sizeof(T) + sizeof(TO) + (first ? 0 : sizeof(TS))));
     TS* t = ts();
     TS* zb = zsS();
+    const T* rs = rs_();
     if (first) {
       for (int lr = threadIdx.x; lr < rows; lr += blockDim.x) t[lr] = (TS)rs[lr];
       __syncthreads();
     } else {
       load_slabs<TS>(zo, zb, false);
-      for_rows<TS, 1>(C.As, zb, [&](int lr, TS v) { t[lr] = (TS)rs[lr] - v; });
+      auto residual = [&](int lr, TS v) { t[lr] = (TS)rs[lr] - v; };
+      if constexpr (KEEP > 1) {
+        if (part < KEEP) {
+          TS acc[4] = {TS(0), TS(0), TS(0), TS(0)};
+          apply_pairs<TS, 1, KEEP, 0, kKeep>(zb, lrow / NP, part, av, acc);
+          reinterpret_cast<TS*>(ps())[part * rows + lrow] = acc[0] + acc[1];
+        }
+        sum_shares<TS, KEEP>(residual);
+        __syncthreads();
+      } else {
+        for_rows<TS, 1>(C.As, zb, residual);
+      }
     }
     const TI* D = static_cast<const TI*>(C.Dinv);
-    const TS om = (TS)a.omega;
+    const TS om = (TS)a.omega, om1 = (TS)a.omega1;
     for (int lr = threadIdx.x; lr < rows; lr += blockDim.x) {
       const int row = row0 + lr, g = row >> 5, lane = row & 31, base = (lr / NP) * NP;
       TS d0s = TS(0), d1s = TS(0);
@@ -348,9 +398,9 @@ struct CoarseCycle {
         if (2 * jp + 1 < NP) d1s = fma(d1, t[base + 2 * jp + 1], d1s);
       }
       const TS dz = d0s + d1s;
-      const TS v = first ? om * dz : fma(TS(1) - om, zb[NP + lr], om * dz);
+      const TS v = first ? om * dz : fma(om1, zb[own0 + lr], om * dz);
       zn[row] = (TO)v;
-      out[NP + lr] = (TO)v;
+      out[own0 + lr] = (TO)v;
     }
   }
 
@@ -358,65 +408,81 @@ struct CoarseCycle {
   // patch solves (one warp per patch), and the combination z_new = z_old + omega (z_0 + z_1)
   __device__ void as_residual(const TS* zo, bool first) {
     const CoarseLevel& C = L(lev);
-    count((double)C.N * (sizeof(T) + sizeof(TS)) + (first ? 0.0 : opbytes(C, S, a.smoother_bytes) + (double)C.N * sizeof(TS)));
+    count((long long)C.N * (sizeof(T) + sizeof(TS)) + (first ? 0ll : opbytes(C, S, a.smoother_bytes) + (long long)C.N * sizeof(TS)));
     TS* res = static_cast<TS*>(C.as_r);
     if (first) {
-      for (int lr = threadIdx.x; lr < rows; lr += blockDim.x) res[row0 + lr] = (TS)rs[lr];
+      for (int lr = threadIdx.x; lr < rows; lr += blockDim.x) res[row0 + lr] = (TS)rs_()[lr];
     } else {
       load_slabs<TS>(zo, zsS(), true);
-      for_rows<TS, 0>(C.As, zsS(), [&](int lr, TS v) { res[row0 + lr] = (TS)rs[lr] - v; });
+      for_rows<TS, 0>(C.As, zsS(), [&](int lr, TS v) { res[row0 + lr] = (TS)rs_()[lr] - v; });
     }
   }
   __device__ void as_patches() {
     const CoarseLevel& C = L(lev);
     constexpr int M = NCH * NP;
     const int np0 = as_npatch(C.n, DIM, 0), np1 = as_npatch(C.n, DIM, 1);
-    count((double)(np0 + np1) * M * M * a.inverse_bytes + (double)(np0 + np1) * M * 2 * sizeof(TS));
+    count((long long)(np0 + np1) * M * M * a.inverse_bytes + (long long)(np0 + np1) * M * 2 * sizeof(TS));
     const TI* inv0 = static_cast<const TI*>(C.as_inv0);
     const TI* inv1 = static_cast<const TI*>(C.as_inv1);
     const TS* res = static_cast<const TS*>(C.as_r);
     TS* zP = static_cast<TS*>(C.as_z);
     const int warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
-    TS* prs = reinterpret_cast<TS*>(smem + a.sm_as) + (size_t)warp * M;
-    // patches over blocks first, so that a level of few patches still uses every SM
-    for (int w = blockIdx.x + gridDim.x * warp; w < np0 + np1; w += gridDim.x * wpb) {
-      if (w < np0) as_patch_solve_warp<TS, TI, NP, DIM>(C.n, 0, w, inv0, res, zP, prs);
-      else as_patch_solve_warp<TS, TI, NP, DIM>(C.n, 1, w - np0, inv1, res, zP + (size_t)np0 * M, prs);
+    TS* prs = reinterpret_cast<TS*>(smem_cc + a.sm_as) + (size_t)warp * M;
+    // a warp takes 32 rows of a patch; units over blocks first, so that few patches use every SM
+    constexpr int JT = (M + 31) / 32;
+    const int units = (np0 + np1) * JT;
+    for (int u = blockIdx.x + gridDim.x * warp; u < units; u += gridDim.x * wpb) {
+      const int w = u / JT, t = u - w * JT;
+      if (w < np0) as_patch_rows_warp<TS, TI, NP, DIM>(C.n, 0, w, t, inv0, res, zP, prs);
+      else as_patch_rows_warp<TS, TI, NP, DIM>(C.n, 1, w - np0, t, inv1, res, zP + (size_t)np0 * M, prs);
     }
   }
   template <typename TO>
   __device__ void as_combine(const TS* zo, TO* zn, TO* out, bool first) {
     const CoarseLevel& C = L(lev);
-    count((double)C.N * (2 * sizeof(TS) + sizeof(TO)));
+    count((long long)C.N * (2 * sizeof(TS) + sizeof(TO)));
     const int np0 = as_npatch(C.n, DIM, 0);
     const TS* zP = static_cast<const TS*>(C.as_z);
     for (int lr = threadIdx.x; lr < rows; lr += blockDim.x) {
       const TO v = (TO)as_combine_row<TS, NP, DIM>(C.n, row0 + lr, zP, np0, zo, (TS)a.omega, first);
       zn[row0 + lr] = v;
-      out[NP + lr] = v;
+      out[own0 + lr] = v;
     }
   }
 
   // z = BJ(r) or AS(r) from z = 0 (a.sweeps sweeps): own rows in zsV(), all rows in C.z
-  __device__ void smooth() {
-    const CoarseLevel& C = L(lev);
-    TS* sb[2] = {static_cast<TS*>(C.s0), static_cast<TS*>(C.s1)};
-    T* out = vec(C.z);
-    for (int k = 0; k < a.sweeps && ok; ++k) {
-      const TS* zo = sb[(k + 1) & 1];
-      const bool last = k == a.sweeps - 1;
-      if (a.smoother == 1) {
+  __device__ __forceinline__ void smooth() {
+    if (a.smoother == 1) {
+      TS* sb[2] = {static_cast<TS*>(L(lev).s0), static_cast<TS*>(L(lev).s1)};
+      for (int k = 0; k < a.sweeps && ok; ++k) {
+        const TS* zo = sb[(k + 1) & 1];
         as_residual(zo, k == 0);
         if (!(ok = bar())) break;
         as_patches();
         if (!(ok = bar())) break;
-        if (last) as_combine<T>(zo, out, zsV(), k == 0);
+        if (k == a.sweeps - 1) as_combine<T>(zo, vec(L(lev).z), zsV(), k == 0);
         else as_combine<TS>(zo, sb[k & 1], zsS(), k == 0);
-      } else if (last) {
-        sweep<T>(zo, out, zsV(), k == 0);
-      } else {
-        sweep<TS>(zo, sb[k & 1], zsS(), k == 0);
+        ok = bar();
+        ph(PH_SWEEP);
       }
+    } else if (lpr == 8) {
+      bj_sweeps<8>();
+    } else {
+      bj_sweeps<1>();
+    }
+  }
+  template <int KEEP>
+  __device__ __forceinline__ void bj_sweeps() {
+    const CoarseLevel& C = L(lev);
+    TS* sb[2] = {static_cast<TS*>(C.s0), static_cast<TS*>(C.s1)};
+    VS2 av[kKeep];
+    if constexpr (KEEP > 1) {
+      if (part < KEEP && a.sweeps > 1) load_pairs<TS, 1, KEEP, 0, kKeep>(C.As, lrow, part, av);
+    }
+    for (int k = 0; k < a.sweeps && ok; ++k) {
+      const TS* zo = sb[(k + 1) & 1];
+      if (k == a.sweeps - 1) sweep<KEEP, T>(zo, vec(C.z), zsV(), k == 0, av);
+      else sweep<KEEP, TS>(zo, sb[k & 1], zsS(), k == 0, av);
       ok = bar();
       ph(PH_SWEEP);
     }
@@ -433,12 +499,17 @@ struct CoarseCycle {
     if (!bar()) return false;
     const int warp = threadIdx.x >> 5, ln = threadIdx.x & 31, nw = blockDim.x >> 5;
     if (n * (int)gridDim.x <= 4096) {
-      for (int c = warp; c < n; c += nw) {
-        double v = 0.0;
-        for (int b = ln; b < (int)gridDim.x; b += 32) v += __ldcg(pt + (size_t)c * gridDim.x + b);
+      // four columns a warp: their loads are in flight together, and the transposed sum takes
+      // fewer FP64 additions than one column at a time
+      for (int c0 = 4 * warp; c0 < n; c0 += 4 * nw) {
+        double v[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int b = ln; b < (int)gridDim.x; b += 32)
 #pragma unroll
-        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (ln == 0) red_s[c] = v;
+          for (int k = 0; k < 4; ++k)
+            v[k] += c0 + k < n ? __ldcg(pt + (size_t)(c0 + k) * gridDim.x + b) : 0.0;
+        int k;
+        const double t = warp_sum_t<4>(v, ln, k);
+        if ((ln & 7) == 0 && c0 + k < n) red_s[c0 + k] = t;
       }
       __syncthreads();
       return true;
@@ -469,6 +540,7 @@ struct CoarseCycle {
     const int warp = threadIdx.x >> 5, ln = threadIdx.x & 31, nw = blockDim.x >> 5;
     const int sub = ln / LPC, lc = ln - sub * LPC, n = l + 3;
     const T* w = ws();
+    const T* rs = rs_();
     for (int c0 = warp * CPW; c0 < n; c0 += nw * CPW) {
       const int c = c0 + sub;
       T s0 = T(0), s1 = T(0);
@@ -493,10 +565,7 @@ struct CoarseCycle {
   }
   __device__ bool dots(const T* W, int N, int l) {
     double* pt = next_partial();
-    const int nw = blockDim.x >> 5;
-    if (l + 3 <= nw) dots_lpc<32>(W, N, l, pt);
-    else if (l + 3 <= 2 * nw) dots_lpc<16>(W, N, l, pt);
-    else dots_lpc<8>(W, N, l, pt);
+    dots_lpc<8>(W, N, l, pt);   // few lanes a column: fewer FP64 instructions in the lanes' sum
     return reduce_cols(pt, l + 3);
   }
 
@@ -535,51 +604,39 @@ struct CoarseCycle {
     const int N = C.N, l = sc.l;
     T* W = vec(C.W);
     T* w = ws();
-    const T* zown = zsV() + NP;
+    const T* zown = zsV() + own0;
+    T* rs = rs_();
     load_slabs<T>(vec(C.z), zsV(), false);
     for_rows<T, 0>(C.A, zsV(), [&](int lr, T v) { w[lr] = v; });
-    count(opbytes(C, S, sizeof(T)) + (double)N * sizeof(T) * 2 + (double)(l + 1) * N * sizeof(T));
+    count(opbytes(C, S, sizeof(T)) + (long long)N * sizeof(T) * 2 + (long long)(l + 1) * N * sizeof(T));
     if (!dots(W, N, l)) return false;
     ph(PH_RM_GRAM1);
-    const double rr = red_s[l + 2], naz2 = red_s[l];
-    if (sc.first) {
-      sc.rnorm = sqrt(rr);
-      sc.eps = C.rtol * sc.rnorm;
-      sc.first = 0;
-    }
     // w_hat = w - W W^T w: its norm by Pythagoras; another pass whenever that cancelled
     // more than half of it (classical Gram-Schmidt, "twice is enough")
     double* Rc = R + l * (l - 1) / 2;
-    for (int i = threadIdx.x; i < l; i += blockDim.x) Rc[i] = 0.0;
-    bool discard = !isfinite(naz2) || !(naz2 > 0.0);
-    const double tiny = a.brk * a.brk * naz2;
-    double nw2 = 0.0, wr = 0.0;
     for (int pass = 0;; ++pass) {
-      double hh = 0.0;
-      for (int i = 0; i < l; ++i) hh += red_s[i] * red_s[i];
-      const double n2 = red_s[l];
-      nw2 = n2 - hh;
-      wr = red_s[l + 1];
-      __syncthreads();
+      judge(l, pass);
       for (int i = threadIdx.x; i < l; i += blockDim.x) {
         cf[i] = red_s[i];
-        Rc[i] += red_s[i];
+        Rc[i] = pass == 0 ? red_s[i] : Rc[i] + red_s[i];
       }
       __syncthreads();
-      if (discard || l == 0 || nw2 >= 0.25 * n2 || pass == 3) break;
-      if (pass > 0 && !(nw2 > tiny)) break;   // nothing left: linearly dependent
+      if (pass == 0 && sc.first) {
+        sc.r2 = rms->rr;
+        sc.eps2 = C.rtol * C.rtol * sc.r2;
+        sc.first = 0;
+      }
+      if (rms->verdict != 1) break;
       project(W, N, l, w, [&](int lr, T v) { w[lr] = v; });
-      count((double)(l + 2) * N * sizeof(T) + (double)(l + 1) * N * sizeof(T));   // apply + second dots
+      count((long long)(l + 2) * N * sizeof(T) + (long long)(l + 1) * N * sizeof(T));   // apply + second dots
       if (!dots(W, N, l)) return false;
       ph(PH_RM_REORTH);
     }
-    if (!isfinite(nw2) || !(nw2 > tiny)) discard = true;
-    if (discard) {
-      sc.rnorm = sqrt(rr);
+    if (rms->verdict == 2) {
+      sc.r2 = rms->rr;
       return true;
     }
-    const double gam = 1.0 / sqrt(nw2), alp = gam * wr;   // alpha = w_hat . r (r is orthogonal to W)
-    const T g = (T)gam, al_t = (T)alp;
+    const T g = (T)rms->gam, al_t = (T)rms->alp;   // alpha = w_hat . r (r is orthogonal to W)
     T* Wl = W + (size_t)l * N + row0;
     T* Zl = vec(C.Z) + (size_t)l * N + row0;
     project(W, N, l, w, [&](int lr, T v) {
@@ -589,34 +646,60 @@ struct CoarseCycle {
       rs[lr] = fma(-al_t, wv, rs[lr]);
     });
     if (threadIdx.x == 0) {
-      gm[l] = gam;
-      al[l] = alp;
+      gm[l] = rms->gam;
+      al[l] = rms->alp;
     }
-    count((double)(l + 4) * N * sizeof(T));   // W columns; w, r in; new columns and r out
+    count((long long)(l + 4) * N * sizeof(T));   // W columns; w, r in; new columns and r out
     // ||r - alpha w||^2 = ||r||^2 - alpha^2 for unit w with alpha = w . r; reduce the
     // updated vector explicitly only if that cancels more than four digits
-    const double r2new = rr - alp * alp;
     sc.l++;
-    if (r2new > 1e-4 * rr) {
-      sc.rnorm = sqrt(r2new);
-    } else {
-      if (!residual_norm(sc)) return false;
-    }
+    sc.r2 = rms->r2new;
+    if (!(sc.r2 > 1e-4 * rms->rr) && !residual_norm(sc)) return false;
     ph(PH_RM_UPDATE);
     return true;
   }
 
-  // sc.rnorm = ||r|| from the own rows of every block
+  // warp 0: the scalars of a Gram pass with l columns from red_s into rms (the caller's
+  // __syncthreads publishes them)
+  __device__ void judge(int l, int pass) {
+    if (threadIdx.x >= 32) return;
+    double hh = 0.0;
+    for (int i = threadIdx.x; i < l; i += 32) hh = fma(red_s[i], red_s[i], hh);
+    if (l > 0)
+#pragma unroll
+      for (int o = 16; o; o >>= 1) hh += __shfl_xor_sync(0xffffffffu, hh, o);
+    if (threadIdx.x != 0) return;
+    const double n2 = red_s[l], nw2 = n2 - hh;
+    if (pass == 0) {
+      rms->naz2 = n2;
+      rms->rr = red_s[l + 2];
+    }
+    const double tiny = a.brk * a.brk * rms->naz2;
+    int v = 0;
+    if (!isfinite(n2) || !(n2 > 0.0)) v = 2;
+    else if (l > 0 && nw2 < 0.25 * n2 && pass < 3 && (pass == 0 || nw2 > tiny)) v = 1;
+    else if (!isfinite(nw2) || !(nw2 > tiny)) v = 2;
+    rms->verdict = v;
+    if (v == 0) {
+      const double gam = rsqrt(nw2), alp = gam * red_s[l + 1];
+      rms->gam = gam;
+      rms->alp = alp;
+      rms->r2new = rms->rr - alp * alp;
+    }
+  }
+
+  // sc.r2 = ||r||^2 from the own rows of every block
   __device__ bool residual_norm(LvScal& sc) {
     double* pt = next_partial();
     double s = 0.0;
+    const T* rs = rs_();
     for (int j = threadIdx.x; j < rows; j += blockDim.x) s = fma((double)rs[j], (double)rs[j], s);
     double v[1] = {s};
     __syncthreads();
     bsum_n<1>(v, sh);
     if (threadIdx.x == 0) (gridDim.x == 1 ? red_s : pt)[blockIdx.x] = v[0];
     if (!reduce_cols(pt, 1)) return false;
-    sc.rnorm = sqrt(red_s[0]);
+    sc.r2 = red_s[0];
     return true;
   }
 
@@ -650,7 +733,7 @@ struct CoarseCycle {
       for (; i < l; ++i) s[0] = fma((T)cf[i], Z[(size_t)i * N + row0 + lr], s[0]);
       x[row0 + lr] = ldv(x + row0 + lr) + ((s[0] + s[1]) + (s[2] + s[3]));
     }
-    count((double)(l + 2) * N * sizeof(T));
+    count((long long)(l + 2) * N * sizeof(T));
   }
 
   // ---------------------------------------------------------------- transfers
@@ -658,7 +741,7 @@ struct CoarseCycle {
   // C.r of this level complete in global memory.
   __device__ void restrict_(bool start) {
     const CoarseLevel &F = L(lev), &C = L(lev + 1);
-    count((double)F.N * sizeof(T) + (double)C.N * sizeof(T) * (start ? 3 : 1));
+    count((long long)F.N * sizeof(T) + (long long)C.N * sizeof(T) * (start ? 3 : 1));
     const int cells = C.N / NP;
     const int J0 = first_cell(cells, blockIdx.x), nJ = first_cell(cells, blockIdx.x + 1) - J0;
     const T* rf = vec(F.r);
@@ -670,7 +753,7 @@ struct CoarseCycle {
       stage[i] = ldv(rf + (size_t)(fx + F.n[0] * (fy + F.n[1] * fz)) * NP + q);
     }
     __syncthreads();
-    T* rc = start ? reinterpret_cast<T*>(smem + C.sm_r) : nullptr;
+    T* rc = reinterpret_cast<T*>(smem_cc + C.sm_r);
     for (int lr = threadIdx.x; lr < nJ * NP; lr += blockDim.x) {
       const int c = lr / NP, i = lr - c * NP;
       T s[NCH];
@@ -695,10 +778,10 @@ struct CoarseCycle {
   // z = P x_{lev + 1} on the own rows: zsV() and C.z
   __device__ void prolong() {
     const CoarseLevel &F = L(lev), &C = L(lev + 1);
-    count((double)F.N * sizeof(T) + (double)C.N * sizeof(T));
+    count((long long)F.N * sizeof(T) + (long long)C.N * sizeof(T));
     const T* xc = vec(C.x);
     T* zf = vec(F.z);
-    T* own = zsV() + NP;
+    T* own = zsV() + own0;
     for (int lr = threadIdx.x; lr < rows; lr += blockDim.x) {
       const int K = K0 + lr / NP, q = lr % NP;
       const int ix = K % F.n[0], iy = (K / F.n[0]) % F.n[1], iz = DIM == 3 ? K / (F.n[0] * F.n[1]) : 0;
@@ -718,7 +801,7 @@ struct CoarseCycle {
   // x_c = A_c^{-1} b_c (FP64 dense inverse), one warp per row, rows over blocks first
   __device__ void coarse_solve(int l) {
     const CoarseLevel& C = L(l);
-    count((double)a.Nc * a.Nc * 8 + (double)a.Nc * 2 * sizeof(T));
+    count((long long)a.Nc * a.Nc * 8 + (long long)a.Nc * 2 * sizeof(T));
     const T* bc = vec(C.b);
     T* xc = vec(C.x);
     const int nw = blockDim.x >> 5, warp = threadIdx.x >> 5, ln = threadIdx.x & 31;
@@ -738,25 +821,21 @@ struct CoarseCycle {
   }
 
   // ---------------------------------------------------------------- timing
-  // time attribution per phase kind (thread 0 of block 0; the interval since the previous
-  // phase boundary, closing barrier included)
-  unsigned long long t_ph = 0;
+  // SM clocks per phase kind (the interval since the previous phase boundary, closing barrier
+  // included) and per level, by thread 0 of block 0; the clock counter is read in a few cycles,
+  // the global timer only at the kernel's ends, which give the scale
+  long long t_ph = 0, t_mark = 0;
   __device__ void ph(int kind) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-      unsigned long long t;
-      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-      if (t_ph) atomicAdd(a.stat_phase_ns + kind, t - t_ph);
+      const long long t = clock64();
+      if (t_ph) tph[kind] += t - t_ph;
       t_ph = t;
     }
   }
-
-  // time attribution per level (thread 0 of block 0)
-  unsigned long long t_mark = 0;
   __device__ void mark(int l) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-      unsigned long long t;
-      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-      if (t_mark) atomicAdd(a.stat_level_ns + l, t - t_mark);
+      const long long t = clock64();
+      if (t_mark) tph[kCoarsePhases + l] += t - t_mark;
       t_mark = t;
     }
   }
@@ -772,8 +851,8 @@ struct CoarseCycle {
     sc.l = 0;
     sc.it = 0;
     sc.first = 1;
-    sc.rnorm = rtol < 1.0 ? 1.0 : 0.0;   // stands for ||b|| > rtol ||b|| until ||b|| is known
-    sc.eps = 0.0;
+    sc.r2 = rtol < 1.0 ? 1.0 : 0.0;   // stands for ||b|| > rtol ||b|| until ||b|| is known
+    sc.eps2 = 0.0;
   }
 
   __device__ void run(int lev0) {
@@ -796,7 +875,7 @@ struct CoarseCycle {
         ph(PH_TRANSFER);
       } else {
         // while ||r|| > eps (level-local criteria of Sec. 4.2)
-        if (phase[lev] == PRE && !(s.rnorm > s.eps && s.it < C.maxit && guard[lev] < (1 << 24))) {
+        if (phase[lev] == PRE && !(s.r2 > s.eps2 && s.it < C.maxit && guard[lev] < (1 << 24))) {
           if (blockIdx.x == 0 && threadIdx.x == 0 && C.st) {
             C.st->iters_total += s.it;
             C.st->nrestart += restarts[lev];
@@ -816,12 +895,12 @@ struct CoarseCycle {
       if (!(ok = rm(s))) break;
       if (phase[lev] == PRE) {
         ++guard[lev];
-        if (s.it == 0 && s.l == 0 && !(s.rnorm > 0.0)) {           // b = 0 (or not finite): x = 0
-          s.rnorm = 0.0;
+        if (s.it == 0 && s.l == 0 && !(s.r2 > 0.0)) {              // b = 0 (or not finite): x = 0
+          s.r2 = 0.0;
           continue;
         }
         T* rg = vec(C.r);
-        for (int lr = threadIdx.x; lr < rows; lr += blockDim.x) rg[row0 + lr] = rs[lr];
+        for (int lr = threadIdx.x; lr < rows; lr += blockDim.x) rg[row0 + lr] = rs_()[lr];
         if (!(ok = bar())) break;                                  // r complete everywhere
         const bool direct = (lev + 1 == a.nlev - 1);
         restrict_(!direct);                                        // r_c = R r
@@ -851,8 +930,8 @@ struct CoarseCycle {
           if (!(ok = bar())) break;
           load_slabs<T>(vec(C.x), zsV(), true);
           const T* b = vec(C.b);
-          for_rows<T, 0>(C.A, zsV(), [&](int lr, T v) { rs[lr] = ldv(b + row0 + lr) - v; });
-          count(opbytes(C, S, sizeof(T)) + (double)C.N * sizeof(T) * 3);
+          for_rows<T, 0>(C.A, zsV(), [&](int lr, T v) { rs_()[lr] = ldv(b + row0 + lr) - v; });
+          count(opbytes(C, S, sizeof(T)) + (long long)C.N * sizeof(T) * 3);
           s.l = 0;
           if (!(ok = residual_norm(s))) break;
           ph(PH_RESTART);
@@ -864,41 +943,49 @@ struct CoarseCycle {
   }
 };
 
-// Resident blocks per SM the register allocation must allow.  With 2, level-0 kernels of the
-// task-parallel cycle can run on its SMs beside it.
-#ifndef KCMG_CC_MINBLOCKS
-#define KCMG_CC_MINBLOCKS 2
-#endif
+// Registers: a bound of 512 threads allows 128, with which nothing spills; 320 threads then take
+// under two thirds of the register file, so that level-0 kernels of the task-parallel cycle run
+// on the same SMs beside this one.
 template <typename TV, typename TS, typename TI, int NP, int DIM>
-__global__ void __launch_bounds__(320, KCMG_CC_MINBLOCKS) k_coarse_cycle(const __grid_constant__ CoarseArgs a) {
+__global__ void __launch_bounds__(512) k_coarse_cycle(const __grid_constant__ CoarseArgs a) {
   using T = TV;
-  extern __shared__ __align__(16) unsigned char smem_cc[];
   __shared__ double sh[32 * 8];
   __shared__ double red_s[kCoarseMaxCols + 4];
   __shared__ double cf[kCoarseMaxCols];
+  __shared__ RmScal rms;
+  __shared__ int nbs[2 * DIM + 1];
+  __shared__ long long tph[kCoarsePhases + KCMG_MAX_LEVELS];
+  if (threadIdx.x < kCoarsePhases + KCMG_MAX_LEVELS) tph[threadIdx.x] = 0;
   constexpr int NCH = 1 << DIM;
   T* Ps = reinterpret_cast<T*>(smem_cc);   // prolongation matrices first
   const double* P = static_cast<const double*>(a.P);   // FP64 prolongation matrices
   for (int i = threadIdx.x; i < NCH * NP * NP; i += blockDim.x) Ps[i] = (T)P[i];
-  CoarseCycle<TV, TS, TI, NP, DIM> cc{a, smem_cc, sh, red_s, cf, Ps};
+  CoarseCycle<TV, TS, TI, NP, DIM> cc{a, sh, red_s, cf, &rms, nbs, tph, Ps};
   unsigned long long t0 = 0;
-  if (blockIdx.x == 0 && threadIdx.x == 0) asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
-  for (int l = a.lev0; l < a.nlev - 1; ++l) cc.build_mask(l);
+  long long c0 = 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+    c0 = clock64();
+  }
   // start of MG on the first coarse level: b, r, x were set by the restriction kernel
   cc.enter(a.lev0);
   for (int lr = threadIdx.x; lr < cc.rows; lr += blockDim.x)
-    cc.rs[lr] = ldv(static_cast<const T*>(a.lv[a.lev0].b) + cc.row0 + lr);
+    cc.rs_()[lr] = ldv(static_cast<const T*>(a.lv[a.lev0].b) + cc.row0 + lr);
   __syncthreads();
-  cc.count((double)a.lv[a.lev0].N * sizeof(T));
+  cc.count((long long)a.lv[a.lev0].N * sizeof(T));
   cc.run(a.lev0);
   // device time of this launch: every block has passed the last barrier of the cycle
   if (cc.ok) cc.ok = cc.bar();
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     unsigned long long t1;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
+    const double scale = (double)(t1 - t0) / (double)max(1ll, clock64() - c0);   // ns per clock
+    for (int k = 0; k < kCoarsePhases; ++k) atomicAdd(a.stat_phase_ns + k, (unsigned long long)(tph[k] * scale));
+    for (int l = 0; l < a.nlev; ++l)
+      atomicAdd(a.stat_level_ns + l, (unsigned long long)(tph[kCoarsePhases + l] * scale));
     atomicAdd(a.stat_ns, t1 - t0);
     atomicAdd(a.stat_launches, 1ull);
-    atomicAdd(a.stat_bytes, cc.bytes);
+    atomicAdd(a.stat_bytes, (double)cc.bytes);
   }
   cc_leave(a);
 }

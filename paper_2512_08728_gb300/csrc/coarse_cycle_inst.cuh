@@ -58,12 +58,12 @@ static void coarse_cycle_layout(CoarseArgs* a, int grid) {
     const size_t rows = (size_t)own * a->np;
     if (l > a->lev0) slab = std::max(slab, rows * nch);                   // children of the own cells
     if (l == a->nlev - 1) break;
-    slab = std::max(slab, (size_t)(own + 2 + (grid > 1 ? segs * own : 0)) * a->np);
+    const int pad = a->dim == 2 ? L.n[0] : L.n[0] * L.n[1];   // one block: zeros on both sides
+    slab = std::max(slab, (size_t)(grid > 1 ? own + 2 + segs * own : own + 2 * pad) * a->np);
     rows_max = std::max(rows_max, rows);
     L.sm_r = take(rows * sizeof(CC_TV));
     L.coef_len = 2 * L.lcap + L.lcap * (L.lcap - 1) / 2;
     L.sm_gm = L.lcap <= kCoarseCoefMax ? take((size_t)L.coef_len * sizeof(double)) : -1;
-    L.sm_mask = take(own);
   }
   a->sm_zv = take(slab * sizeof(CC_TV));
   a->sm_zs = sizeof(CC_TV) == sizeof(CC_T) ? a->sm_zv : take(slab * sizeof(CC_T));

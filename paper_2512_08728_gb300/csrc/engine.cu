@@ -1260,6 +1260,7 @@ kcmg_ctx* build_ctx(const kcmg_params* p, cudaStream_t user, const double* block
       a.np = ctx->np;
       a.P = ctx->P64;
       a.omega = p->omega;
+      a.omega1 = 1.0 - p->omega;
       a.sweeps = p->sweeps;
       a.lmax = p->lmax;
       a.brk = 1e-14;

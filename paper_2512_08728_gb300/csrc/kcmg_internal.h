@@ -223,8 +223,8 @@ struct CoarseLevel {
   const void *as_inv0, *as_inv1;
   void *as_z, *as_r;
   // a block's share in dynamic shared memory (byte offsets): residual of the own rows; gamma,
-  // alpha and the packed coefficients of Alg. 1; neighbour masks of the own cells
-  int sm_r, sm_gm, sm_mask;
+  // alpha and the packed coefficients of Alg. 1
+  int sm_r, sm_gm;
   // gamma, alpha and coefficients in global memory (coef_len doubles a block) where sm_gm < 0:
   // bases so long that they do not fit
   double* coef;
@@ -237,7 +237,7 @@ struct CoarseArgs {
   const void* P;               // prolongation matrices (FP64; the kernel converts them)
   const double* Ainv;          // dense inverse of the coarsest operator
   int Nc;
-  double omega;
+  double omega, omega1;        // damping, 1 - damping
   int sweeps, lmax;
   double brk;                  // breakdown threshold of Alg. 1
   // dynamic shared memory (byte offsets): iterate slabs in the vector type and in the smoother's

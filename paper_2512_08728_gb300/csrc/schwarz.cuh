@@ -87,6 +87,30 @@ __device__ __forceinline__ void as_patch_solve_warp(const int* n, int part, int 
   __syncwarp();
 }
 
+// rows 32 t .. of one patch only (as as_patch_solve_warp): the coarse levels' patches are few, so
+// several warps share one
+template <typename T, typename TI, int NP, int DIM>
+__device__ __forceinline__ void as_patch_rows_warp(const int* n, int part, int pi, int t, const TI* invT,
+                                                   const T* r, T* z, T* rs) {
+  constexpr int NCH = 1 << DIM, M = NCH * NP;
+  const int lane = threadIdx.x & 31, j = 32 * t + lane;
+  int cell[NCH];
+  as_members<DIM>(n, part, pi, cell);
+  for (int e = lane; e < M; e += 32) {
+    const int a = e / NP, q = e - a * NP;
+    rs[e] = cell[a] >= 0 ? __ldcg(r + (size_t)cell[a] * NP + q) : T(0);
+  }
+  __syncwarp();
+  const TI* Ai = invT + (size_t)pi * M * M + j;
+  if (j < M) {
+    T acc = T(0);
+#pragma unroll 8
+    for (int q = 0; q < M; ++q) acc = fma(AsLoad<T, TI>::get(Ai + (size_t)q * M), rs[q], acc);
+    z[(size_t)pi * M + j] = acc;
+  }
+  __syncwarp();
+}
+
 // x_new (DOF row) = x_old + omega (z_0 + z_1) (first sweep from x = 0: omega (z_0 + z_1));
 // zP holds partition 0's patches first, then partition 1's
 template <typename T, int NP, int DIM>
