@@ -20,11 +20,15 @@
 //
 // Control runs on the host: per loop test the engine reads three flags of the level's
 // device state (any active, any restart due, any convergence claim).  Per-right-hand-side
-// decisions (reorthogonalisation, discard, alpha, masks) are taken on the device by
-// one-warp control kernels.
+// decisions (reorthogonalisation, discard, alpha, masks) are taken on the device by the last
+// block of the reduction whose sums they need, loop tests included: a residual minimisation is
+// eight launches (five on small levels), and the flags go straight to pinned host memory, so a
+// loop test costs no launch and no copy of its own.  On small levels, where every launch is
+// latency, a thread takes one entry (row, right-hand side) of a cell instead of a column of it.
 #include "kcmg_internal.h"
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -45,8 +49,10 @@ enum : int { MF_REORTH = 1, MF_DISCARD = 2 };
 
 // Device state of one level (one MG call is active per level at any time).
 struct MState {
-  int any, any_restart, any_claim, any_reorth;   // flags the host reads (first 32 bytes)
-  int nact, pad_f0, pad_f1, pad_f2;              // active columns after the last test
+  int any, any_restart, any_claim, any_reorth;   // flags of the last loop test and Gram pass
+  int nact;                                      // active columns after the last test
+  unsigned int ticket;                           // last-block counter of the reductions
+  int pad_f1, pad_f2;
   int R, lcap, maxit, it;
   int iters_total, nrestart, status, guard;
   int guard_cap, level, per_cycle, cap;    // restart when l + per_cycle > cap
@@ -55,17 +61,33 @@ struct MState {
   double rnorm[kMaxRhs], rnorm0[kMaxRhs], eps[kMaxRhs], naz2[kMaxRhs], gam[kMaxRhs], alp[kMaxRhs];
 };
 
-enum CtlKind : int {
+// Control steps; up to eight run one after another at the end of a reduction (packed, 4 bits each)
+enum CtlKind : unsigned {
+  CTL_NONE = 0,
   CTL_INIT0,    // level 0 start: sums = ||b - A x0||^2
   CTL_BEGIN,    // level >= 1 start: sums = ||b_c||^2 (restricted residual)
-  CTL_TEST,     // loop test (level-local criteria); restart / claim flags
-  CTL_GRAM1,    // sums = W^T w (columns < l) and ||w||^2 (column lcap)
-  CTL_GRAM2,    // sums = W^T w' (reorthogonalisation pass)
-  CTL_UPDATE,   // sums = ||w_hat||^2, w_hat . r
+  CTL_TEST,     // loop test (level-local criteria); restart / claim flags, to the host as well
+  CTL_GRAM1,    // sums = W^T w (columns < l), ||w||^2 (column lcap), w . r (column lcap + 1)
+  CTL_GRAM2,    // sums = W^T w' and so on (reorthogonalisation pass)
   CTL_FINISH,   // sums = ||r||^2 after the update
   CTL_RESTART,  // sums = ||b - A x||^2 for the restarting right-hand sides
   CTL_CONFIRM,  // level 0: sums = true ||b - A x||^2 of the claiming right-hand sides
   CTL_ITEND     // end of an iteration
+};
+constexpr unsigned ctl_seq(unsigned a, unsigned b = 0, unsigned c = 0) { return a | (b << 4) | (c << 8); }
+
+// what the host reads of a loop test (pinned memory that the device writes)
+struct HostFlags { volatile int any, any_restart, any_claim, nact; volatile unsigned int seq; };
+
+// The control that follows a reduction: state, parent level's state (CTL_BEGIN), steps, the
+// coefficient arrays, the host's flags and the sequence number that marks them written.
+struct CtlArgs {
+  MState* st;
+  const MState* parent;
+  unsigned steps;
+  double *sums, *cw, *cz;
+  HostFlags* host;
+  unsigned seq;
 };
 
 // ------------------------------------------------------------------ small helpers
@@ -99,11 +121,251 @@ __device__ __forceinline__ void tf32_split(float x, uint32_t& hi, uint32_t& lo) 
 template <typename TI> __device__ __forceinline__ float to_f(TI v);
 template <> __device__ __forceinline__ float to_f<float>(float v) { return v; }
 template <> __device__ __forceinline__ float to_f<__nv_bfloat16>(__nv_bfloat16 v) { return __bfloat162float(v); }
+__device__ __forceinline__ double to_f_or_d(double v) { return v; }
+__device__ __forceinline__ float to_f_or_d(float v) { return v; }
+__device__ __forceinline__ float to_f_or_d(__nv_bfloat16 v) { return __bfloat162float(v); }
 
 __device__ __forceinline__ int max_l(const MState* st) {
   int m = 0;
   for (int r = 0; r < st->R; ++r) m = max(m, st->l[r]);
   return m;
+}
+
+// ------------------------------------------------------------------ control (one warp)
+__device__ void mctl_step(const CtlArgs& c, unsigned kind) {
+  MState* st = c.st;
+  const MState* parent = c.parent;
+  const double* sums = c.sums;   // written by other threads or blocks of this kernel: read through L2
+  double *cw = c.cw, *cz = c.cz;
+  const int r = threadIdx.x;
+  const int R = st->R, lcap = st->lcap;
+  bool f_any = false, f_restart = false, f_claim = false, f_reorth = false;
+  if (r < R) {
+    switch (kind) {
+      case CTL_INIT0: {
+        const double n0 = sqrt(__ldcg(sums + r));
+        st->rnorm0[r] = n0;
+        st->rnorm[r] = n0;
+        st->eps[r] = fmax(st->rtol * n0, st->atol);
+        st->act[r] = n0 > st->eps[r] && isfinite(n0);
+        if (!isfinite(n0)) st->status = KCMG_NONFINITE;
+        st->l[r] = 0;
+        st->flags[r] = 0;
+        st->brk[r] = 0;
+        st->claim[r] = 0;
+        st->restart[r] = 0;
+        break;
+      }
+      case CTL_BEGIN: {
+        const double n0 = sqrt(__ldcg(sums + r));
+        st->rnorm0[r] = n0;
+        st->rnorm[r] = n0;
+        st->eps[r] = st->rtol * n0;
+        st->act[r] = parent->act[r] && n0 > 0.0;
+        st->l[r] = 0;
+        st->flags[r] = 0;
+        st->restart[r] = 0;
+        break;
+      }
+      case CTL_TEST: {
+        const bool active = st->act[r] != 0;
+        const bool conv = !(st->rnorm[r] > st->eps[r]);
+        if (st->level == 0) {
+          st->claim[r] = active && conv;    // confirmed by a true residual first
+          f_claim = active && conv;
+        } else if (active && conv) {
+          st->act[r] = 0;
+        }
+        st->restart[r] = st->act[r] && !st->claim[r] && st->l[r] > 0 && st->l[r] + st->per_cycle > st->cap;
+        f_restart = st->restart[r] != 0;
+        f_any = st->act[r] != 0;
+        break;
+      }
+      // the norm of w_hat = w - W h by Pythagoras (used where it did not cancel below a quarter
+      // of ||w||^2; else a second pass is requested), alpha = w_hat . r = w . r (r is orthogonal
+      // to W)
+      case CTL_GRAM1: {
+        const int l = st->l[r];
+        double hh = 0.0;
+#pragma unroll 8
+        for (int i = 0; i < l; ++i) {
+          const double h = __ldcg(sums + (size_t)i * 32 + r);
+          hh += h * h;
+          cw[(size_t)i * 32 + r] = h;
+          cz[(size_t)i * 32 + r] = h;
+        }
+        const double naz2 = __ldcg(sums + (size_t)lcap * 32 + r), nw2 = naz2 - hh;
+        st->naz2[r] = naz2;
+        const bool discard = !st->act[r] || !isfinite(naz2) || !(naz2 > 0.0);
+        const bool reorth = !discard && l > 0 && nw2 < 0.25 * naz2;
+        st->flags[r] = (discard ? MF_DISCARD : 0) | (reorth ? MF_REORTH : 0);
+        st->gam[r] = st->alp[r] = 0.0;
+        if (!discard && !reorth) {
+          st->gam[r] = 1.0 / sqrt(nw2);
+          st->alp[r] = st->gam[r] * __ldcg(sums + (size_t)(lcap + 1) * 32 + r);
+        }
+        f_reorth = reorth;
+        break;
+      }
+      // w' = w - W h: one that loses most of its norm again, or falls below brk_tol relative to
+      // ||A z||, is rounding noise (linear dependence)
+      case CTL_GRAM2: {
+        if (st->flags[r] & MF_REORTH) {
+          const int l = st->l[r];
+          double hh = 0.0;
+#pragma unroll 8
+          for (int i = 0; i < l; ++i) {
+            const double h2 = __ldcg(sums + (size_t)i * 32 + r);
+            hh += h2 * h2;
+            cz[(size_t)i * 32 + r] += h2;
+            cw[(size_t)i * 32 + r] = h2;
+          }
+          const double n2 = __ldcg(sums + (size_t)lcap * 32 + r), nw2 = n2 - hh;
+          if (!isfinite(nw2) || !(nw2 >= 0.25 * n2) || !(nw2 > st->brk_tol * st->brk_tol * st->naz2[r])) {
+            st->flags[r] |= MF_DISCARD;
+          } else {
+            st->gam[r] = 1.0 / sqrt(nw2);
+            st->alp[r] = st->gam[r] * __ldcg(sums + (size_t)(lcap + 1) * 32 + r);
+          }
+        }
+        f_reorth = (st->flags[r] & MF_REORTH) != 0;
+        break;
+      }
+      case CTL_FINISH: {
+        const bool discard = (st->flags[r] & MF_DISCARD) != 0;
+        if (!discard) {
+          st->l[r] += 1;
+          st->rnorm[r] = sqrt(__ldcg(sums + r));
+          st->brk[r] = 0;
+        } else if (st->act[r]) {
+          if (++st->brk[r] >= 2 && st->level == 0) {   // two consecutive discards
+            st->status = KCMG_BREAKDOWN;
+            st->act[r] = 0;
+          }
+        }
+        if (!isfinite(st->rnorm[r])) {
+          st->status = KCMG_NONFINITE;
+          st->act[r] = 0;
+        }
+        break;
+      }
+      case CTL_RESTART: {
+        if (st->restart[r]) {
+          st->rnorm[r] = sqrt(__ldcg(sums + r));
+          st->l[r] = 0;
+          st->restart[r] = 0;
+        }
+        break;
+      }
+      case CTL_CONFIRM: {
+        if (st->claim[r]) {
+          const double rn = sqrt(__ldcg(sums + r));
+          st->rnorm[r] = rn;
+          st->l[r] = 0;
+          st->act[r] = rn > st->eps[r];
+          st->claim[r] = 0;
+        }
+        break;
+      }
+      case CTL_ITEND:
+        break;
+    }
+  }
+  const int nact = __popc(__ballot_sync(0xffffffffu, r < R && st->act[r]));
+  f_any = __any_sync(0xffffffffu, f_any);
+  f_restart = __any_sync(0xffffffffu, f_restart);
+  f_claim = __any_sync(0xffffffffu, f_claim);
+  f_reorth = __any_sync(0xffffffffu, f_reorth);
+  if (r == 0) {
+    switch (kind) {
+      case CTL_TEST: {
+        const bool go = f_any && st->it < st->maxit && st->guard < st->guard_cap;
+        st->any = go;
+        st->any_restart = go && f_restart;
+        st->any_claim = f_claim;
+        st->nact = nact;
+        if (go && !f_restart && !f_claim) st->guard++;
+        if (c.host) {
+          c.host->any = go;
+          c.host->any_restart = go && f_restart;
+          c.host->any_claim = f_claim;
+          c.host->nact = nact;
+          __threadfence_system();
+          c.host->seq = c.seq;
+        }
+        break;
+      }
+      case CTL_GRAM1:
+      case CTL_GRAM2:
+        st->any_reorth = f_reorth;
+        break;
+      case CTL_RESTART:
+        st->nrestart++;
+        break;
+      case CTL_CONFIRM:
+        st->nrestart++;
+        break;
+      case CTL_ITEND:
+        st->it++;
+        st->iters_total++;
+        break;
+      case CTL_BEGIN:
+        st->it = 0;
+        break;
+      case CTL_INIT0:
+        st->it = 0;
+        break;
+      default:
+        break;
+    }
+  }
+}
+// the steps of c in turn, by warp 0 of the calling block
+__device__ void mctl_run(const CtlArgs& c) {
+  if (threadIdx.x >= 32) return;
+  for (unsigned k = c.steps; k; k >>= 4) {
+    mctl_step(c, k & 15u);
+    __threadfence_block();
+    __syncwarp();
+  }
+}
+
+// True in every thread of the block that finished last (all other blocks' writes visible).
+__device__ __forceinline__ bool mlast_block(unsigned int* ticket) {
+  __shared__ int s_last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = (atomicAdd(ticket, 1u) == gridDim.x - 1);
+  __syncthreads();
+  if (s_last) __threadfence();
+  return s_last != 0;
+}
+
+// sums[c][32] = sum over nblk blocks of part[blk][c][32] for the column, by one warp
+__device__ __forceinline__ void mreduce_col(const double* part, int nblk, int pstride, int c, double* sums) {
+  const int lane = threadIdx.x & 31;
+  double s0 = 0.0, s1 = 0.0;
+  int b = 0;
+  for (; b + 1 < nblk; b += 2) {
+    s0 += __ldcg(part + ((size_t)b * pstride + c) * 32 + lane);
+    s1 += __ldcg(part + ((size_t)(b + 1) * pstride + c) * 32 + lane);
+  }
+  if (b < nblk) s0 += __ldcg(part + ((size_t)b * pstride + c) * 32 + lane);
+  sums[(size_t)c * 32 + lane] = s0 + s1;
+}
+
+// End of a reduction kernel whose blocks wrote part[blk][c][32]: with c.steps the last block sums
+// the columns (c < L, and the ones from lcap on) and runs the control; without, a k_mreduce
+// launch does.
+__device__ __forceinline__ void mfinish_reduction(const double* part, int pstride, int L, int lcap, const CtlArgs& c) {
+  if (!c.steps) return;
+  if (!mlast_block(&c.st->ticket)) return;
+  const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5, n = L + pstride - lcap;
+  for (int k = warp; k < n; k += nw) mreduce_col(part, gridDim.x, pstride, k < L ? k : lcap + k - L, c.sums);
+  if (threadIdx.x == 0) c.st->ticket = 0u;
+  __threadfence_block();
+  __syncthreads();
+  mctl_run(c);
 }
 
 // ------------------------------------------------------------------ operator (FP64)
@@ -382,7 +644,8 @@ template <int NP, int DIM>
 __global__ void __launch_bounds__(256) k_mrestrict(const double* __restrict__ rf, int nfx, int nfy, int ncx,
                                                    int ncy, int Cc, const double* __restrict__ P, int R,
                                                    double* __restrict__ bc, double* __restrict__ rc,
-                                                   double* __restrict__ xc, double* __restrict__ part) {
+                                                   double* __restrict__ xc, double* __restrict__ part,
+                                                   CtlArgs ctl) {
   constexpr int NCH = 1 << DIM;
   __shared__ double Ps[NCH * NP * NP];
   __shared__ double red[8][32];
@@ -423,6 +686,146 @@ __global__ void __launch_bounds__(256) k_mrestrict(const double* __restrict__ rf
     for (int w = 0; w < wpb; ++w) t += red[w][threadIdx.x];
     part[(size_t)blockIdx.x * 32 + threadIdx.x] = t;
   }
+  mfinish_reduction(part, 1, 0, 0, ctl);
+}
+
+// ---- one entry (row, right-hand side) of a cell per thread: small levels, where the mappings
+// above leave a few warps with a long serial chain each (64 cells x 8 columns: sweep 42 us, w = A z
+// 47, restriction 55, coarsest solve 22 on eight warps a block of eight cells).  A block holds
+// whole cells.  The sums run in the same order, so results are the same.
+template <int NP>
+__device__ __forceinline__ bool mrow_entry(int C, int R, int& cell, int& i, int& r, int& c) {
+  c = threadIdx.x / (NP * R);
+  const int rem = threadIdx.x - c * NP * R;
+  i = rem / R;
+  r = rem - i * R;
+  cell = blockIdx.x * (blockDim.x / (NP * R)) + c;
+  return c < (int)blockDim.x / (NP * R) && cell < C;
+}
+
+// y = A x or (RESID) b - A x
+template <int NP, int S, bool RESID>
+__global__ void __launch_bounds__(640) k_mrow_spmm(const double* __restrict__ A, const int* __restrict__ nbr, int C,
+                                                   int R, const double* __restrict__ x, double* __restrict__ y,
+                                                   const double* __restrict__ b) {
+  int K, i, r, c;
+  if (!mrow_entry<NP>(C, R, K, i, r, c)) return;
+  double acc = 0.0;
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    const int J = s == 0 ? K : __ldg(nbr + (size_t)K * (S - 1) + s - 1);
+    const double* Ab = A + (((size_t)s * C + K) * NP + i) * NP;
+    const double* xp = x + (size_t)(J < 0 ? K : J) * NP * R + r;
+#pragma unroll
+    for (int q = 0; q < NP; ++q) {
+      const double av = __ldg(Ab + q), xv = __ldg(xp + (size_t)q * R);
+      if (J >= 0) acc = fma(av, xv, acc);
+    }
+  }
+  const size_t o = ((size_t)K * NP + i) * R + r;
+  y[o] = RESID ? __ldg(b + o) - acc : acc;
+}
+
+// one block-Jacobi sweep; FP64 sums from r (as k_msweep64), FP32 from zero and adds r (as
+// k_msweep_simt).  TR, TZ as in k_mpat_sweep: the first sweep converts, the last writes FP64.
+template <typename T, typename TI, typename TR, typename TZ, int NP, int S>
+__global__ void __launch_bounds__(640) k_mrow_sweep(const T* __restrict__ A, size_t slot_stride, size_t cell_stride,
+                                                    const TI* __restrict__ D, const int* __restrict__ nbr, int C,
+                                                    int R, const TR* __restrict__ rv, T* __restrict__ r_lo,
+                                                    const T* __restrict__ zo, TZ* __restrict__ zn, T om, int first) {
+  extern __shared__ __align__(16) unsigned char smem_mrow[];
+  T* ts = reinterpret_cast<T*>(smem_mrow);   // [cell][row][R]
+  int K, i, r, c;
+  const bool act = mrow_entry<NP>(C, R, K, i, r, c);
+  const size_t o = ((size_t)K * NP + i) * R + r;
+  T d[NP];
+  if (act) {
+    const T rr = (T)__ldg(rv + o);
+    T t = rr;
+    if (first) {
+      if constexpr (!std::is_same<T, TR>::value) r_lo[o] = t;
+    } else {
+      if (!std::is_same<T, double>::value) t = T(0);
+#pragma unroll
+      for (int s = 1; s < S; ++s) {
+        const int J = __ldg(nbr + (size_t)K * (S - 1) + s - 1);
+        const T* Ab = A + s * slot_stride + K * cell_stride + i * NP;
+        const T* zp = zo + (size_t)(J < 0 ? K : J) * NP * R + r;
+#pragma unroll
+        for (int q = 0; q < NP; ++q) {
+          const T av = __ldg(Ab + q), zv = __ldg(zp + (size_t)q * R);
+          if (J >= 0) t = fma(-av, zv, t);
+        }
+      }
+      if (!std::is_same<T, double>::value) t += rr;
+    }
+    ts[threadIdx.x] = t;
+#pragma unroll
+    for (int q = 0; q < NP; ++q) d[q] = (T)to_f_or_d(D[(size_t)K * NP * NP + i * NP + q]);
+  }
+  __syncthreads();
+  if (!act) return;
+  T e = T(0);
+#pragma unroll
+  for (int q = 0; q < NP; ++q) e = fma(d[q], ts[(c * NP + q) * R + r], e);
+  zn[o] = (TZ)(first ? om * e : fma(T(1) - om, __ldg(zo + o), om * e));
+}
+
+// b_c = P^T r_f as k_mrestrict, one coarse cell per block; part[blk][32]: sum of b_c^2
+template <int NP, int DIM>
+__global__ void __launch_bounds__(640) k_mrow_restrict(const double* __restrict__ rf, int nfx, int nfy, int ncx,
+                                                       int ncy, const double* __restrict__ P, int R,
+                                                       double* __restrict__ bc, double* __restrict__ rc,
+                                                       double* __restrict__ xc, double* __restrict__ part,
+                                                       CtlArgs ctl) {
+  constexpr int NCH = 1 << DIM;
+  extern __shared__ __align__(16) unsigned char smem_mrow[];
+  double* sq = reinterpret_cast<double*>(smem_mrow);   // [NP][R]
+  const int J = blockIdx.x, i = threadIdx.x / R, r = threadIdx.x - i * R;
+  if (i < NP) {
+    const int jx = J % ncx, jy = (J / ncx) % ncy, jz = DIM == 3 ? J / (ncx * ncy) : 0;
+    double s = 0.0;
+#pragma unroll 2
+    for (int k = 0; k < NCH; ++k) {
+      const int fx = 2 * jx + (k & 1), fy = 2 * jy + ((k >> 1) & 1), fz = DIM == 3 ? 2 * jz + ((k >> 2) & 1) : 0;
+      const double* rp = rf + (size_t)(fx + nfx * (fy + nfy * fz)) * NP * R + r;
+#pragma unroll
+      for (int q = 0; q < NP; ++q) s = fma(__ldg(P + (k * NP + q) * NP + i), __ldg(rp + (size_t)q * R), s);
+    }
+    const size_t o = ((size_t)J * NP + i) * R + r;
+    bc[o] = s;
+    if (rc) {
+      rc[o] = s;
+      xc[o] = 0.0;
+    }
+    sq[i * R + r] = s * s;
+  }
+  if (!part) return;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    double t = 0.0;
+    if ((int)threadIdx.x < R)
+      for (int q = 0; q < NP; ++q) t += sq[q * R + threadIdx.x];
+    part[(size_t)blockIdx.x * 32 + threadIdx.x] = t;
+  }
+  mfinish_reduction(part, 1, 0, 0, ctl);
+}
+
+// z_f = P x_c, one entry per thread
+template <int NP, int DIM>
+__global__ void __launch_bounds__(256) k_mrow_prolong(const double* __restrict__ xc, int nfx, int nfy, int Cf,
+                                                      int ncx, int ncy, const double* __restrict__ P, int R,
+                                                      double* __restrict__ zf) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= Cf * NP * R) return;
+  const int r = e % R, q = (e / R) % NP, K = e / (R * NP);
+  const int ix = K % nfx, iy = (K / nfx) % nfy, iz = DIM == 3 ? K / (nfx * nfy) : 0;
+  const int k = (ix & 1) | ((iy & 1) << 1) | (DIM == 3 ? ((iz & 1) << 2) : 0);
+  const double* xp = xc + (size_t)((ix >> 1) + ncx * ((iy >> 1) + ncy * (iz >> 1))) * NP * R + r;
+  double s = 0.0;
+#pragma unroll
+  for (int i = 0; i < NP; ++i) s = fma(__ldg(P + (k * NP + q) * NP + i), __ldg(xp + (size_t)i * R), s);
+  zf[e] = s;
 }
 
 // z_f = P x_c (warp per fine cell, lane = RHS)
@@ -453,21 +856,28 @@ __global__ void __launch_bounds__(256) k_mprolong(const double* __restrict__ xc,
   }
 }
 
-// x_c = A_c^{-1} b_c, warp per row, lane = RHS
+// x_c = A_c^{-1} b_c, one row per block, the row's products split over its warps, lane = RHS
 __global__ void __launch_bounds__(256) k_mcoarse(const double* __restrict__ Ainv, int n, int R,
                                                  const double* __restrict__ bc, double* __restrict__ xc) {
-  const int wpb = blockDim.x >> 5, r = threadIdx.x & 31;
-  for (int row = blockIdx.x * wpb + (threadIdx.x >> 5); row < n; row += gridDim.x * wpb) {
-    if (r >= R) continue;
+  __shared__ double red[8][32];
+  const int warp = threadIdx.x >> 5, r = threadIdx.x & 31, row = blockIdx.x;
+  double s0 = 0.0, s1 = 0.0;
+  if (r < R) {
     const double* a = Ainv + (size_t)row * n;
-    double s0 = 0.0, s1 = 0.0;
-    int j = 0;
-    for (; j + 1 < n; j += 2) {
+    int j = warp;
+    for (; j + 8 < n; j += 16) {
       s0 = fma(__ldg(a + j), __ldg(bc + (size_t)j * R + r), s0);
-      s1 = fma(__ldg(a + j + 1), __ldg(bc + (size_t)(j + 1) * R + r), s1);
+      s1 = fma(__ldg(a + j + 8), __ldg(bc + (size_t)(j + 8) * R + r), s1);
     }
     if (j < n) s0 = fma(__ldg(a + j), __ldg(bc + (size_t)j * R + r), s0);
-    xc[(size_t)row * R + r] = s0 + s1;
+  }
+  red[warp][r] = s0 + s1;
+  __syncthreads();
+  if (warp == 0 && r < R) {
+    double t = 0.0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) t += red[w][r];
+    xc[(size_t)row * R + r] = t;
   }
 }
 
@@ -490,59 +900,68 @@ __device__ __forceinline__ void block_cols(const double (&v)[NC], double* red /*
   }
 }
 
-// part[blk][c][32] = sum over the block's rows of W[c] . w (c < l_r); part[blk][lcap] = ||w||^2.
-// gated: return at once unless some right-hand side reorthogonalises (second pass).
+// part[blk][c][32] = sum over the block's rows of W[c] . w (c < l_r); [lcap]: ||w||^2, [lcap + 1]:
+// w . r.  gated: return at once unless some right-hand side reorthogonalises (second pass).
 __global__ void __launch_bounds__(256) k_mdots(const double* __restrict__ W, const double* __restrict__ w,
-                                               int N, int R, int lcap, const MState* __restrict__ st,
-                                               double* __restrict__ part, int gated) {
-  __shared__ double red[kGramWarps * 9 * 32];
+                                               const double* __restrict__ rv, int N, int R, int lcap,
+                                               double* __restrict__ part, int gated, CtlArgs ctl) {
+  __shared__ double red[kGramWarps * 8 * 32];
+  const MState* st = ctl.st;
   if (gated && !st->any_reorth) return;
   const int L = max_l(st);
   const int wpb = blockDim.x >> 5, lane = threadIdx.x & 31;
   const int lr = lane < R ? st->l[lane] : 0;
   const bool use = lane < R && (!gated || (st->flags[lane] & MF_REORTH));
   for (int c0 = 0; c0 == 0 || c0 < L; c0 += 8) {
-    double acc[9];
+    double acc[8], ww = 0.0, wr = 0.0;
 #pragma unroll
-    for (int c = 0; c < 9; ++c) acc[c] = 0.0;
+    for (int c = 0; c < 8; ++c) acc[c] = 0.0;
     if (use) {
       for (int j = blockIdx.x * wpb + (threadIdx.x >> 5); j < N; j += gridDim.x * wpb) {
         const double wv = __ldg(w + (size_t)j * R + lane);
-        if (c0 == 0) acc[8] = fma(wv, wv, acc[8]);
+        if (c0 == 0) {
+          ww = fma(wv, wv, ww);
+          wr = fma(wv, __ldg(rv + (size_t)j * R + lane), wr);
+        }
 #pragma unroll
         for (int c = 0; c < 8; ++c)
           if (c0 + c < lr) acc[c] = fma(__ldg(W + ((size_t)(c0 + c) * N + j) * R + lane), wv, acc[c]);
       }
     }
-    double v8[8];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) v8[c] = acc[c];
-    block_cols<8>(v8, red, part, lcap + 1, c0, min(8, lcap - c0));
+    block_cols<8>(acc, red, part, lcap + 2, c0, min(8, lcap - c0));
     if (c0 == 0) {
-      double vn[1] = {acc[8]};
-      block_cols<1>(vn, red, part, lcap + 1, lcap, 1);
+      double vn[2] = {ww, wr};
+      block_cols<2>(vn, red, part, lcap + 2, lcap, 2);
     }
   }
+  mfinish_reduction(part, lcap + 2, L, lcap, ctl);
 }
 
-// out[c][32] = sum over blocks of part[blk][c][32] for c < ncols (columns c < lcols-limit
-// with c >= max l are skipped when limit is set: they are unused)
-__global__ void __launch_bounds__(256) k_mreduce(const double* __restrict__ part, int nblk, int ncols,
-                                                 const MState* __restrict__ st, int limit,
-                                                 double* __restrict__ out) {
+// sums[c][32] = sum over blocks of part[blk][c][32], one block per column (c < max l, and from
+// lcap on); the last block runs the control.  gated: nothing to do without reorthogonalisation.
+__global__ void __launch_bounds__(256) k_mreduce(const double* __restrict__ part, int nblk, int pstride, int lcap,
+                                                 int gated, CtlArgs ctl) {
   __shared__ double red[8][32];
+  MState* st = ctl.st;
+  if (gated && !st->any_reorth) return;
   const int c = blockIdx.x;
-  if (limit && c < ncols - 1 && c >= max_l(st)) return;
-  const int wpb = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double s = 0.0;
-  for (int b = warp; b < nblk; b += wpb) s += part[((size_t)b * ncols + c) * 32 + lane];
-  red[warp][lane] = s;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double t = 0.0;
-    for (int w = 0; w < wpb; ++w) t += red[w][threadIdx.x];
-    out[(size_t)c * 32 + threadIdx.x] = t;
+  if (c >= lcap || c < max_l(st)) {
+    const int wpb = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double s = 0.0;
+    for (int b = warp; b < nblk; b += wpb) s += __ldcg(part + ((size_t)b * pstride + c) * 32 + lane);
+    red[warp][lane] = s;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      double t = 0.0;
+      for (int w = 0; w < wpb; ++w) t += red[w][threadIdx.x];
+      ctl.sums[(size_t)c * 32 + threadIdx.x] = t;
+    }
   }
+  if (!mlast_block(&st->ticket)) return;
+  if (threadIdx.x == 0) st->ticket = 0u;
+  __threadfence_block();
+  __syncthreads();
+  mctl_run(ctl);
 }
 
 // w' = w - W h (reorthogonalising right-hand sides only)
@@ -555,74 +974,62 @@ __global__ void __launch_bounds__(256) k_mapply(const double* __restrict__ W, co
   const int lr = st->l[lane];
   for (int j = blockIdx.x * wpb + (threadIdx.x >> 5); j < N; j += gridDim.x * wpb) {
     double s = __ldg(w + (size_t)j * R + lane);
+#pragma unroll 4
     for (int i = 0; i < lr; ++i) s = fma(-h[(size_t)i * 32 + lane], __ldg(W + ((size_t)i * N + j) * R + lane), s);
     wre[(size_t)j * R + lane] = s;
   }
 }
 
-// w_hat = wsrc - W cw, z_hat = z - Z cz into column l_r; part[blk][0..1][32] = ||w_hat||^2, w_hat . r
+// The step of Alg. 1 per right-hand side: w_l = gamma (wsrc - W cw), z_l = gamma (z - Z cz) into
+// column l_r, x += alpha z_l, r -= alpha w_l (gamma, alpha from the Gram pass; discarded
+// corrections change nothing); part[blk][32] = ||r||^2.
 __global__ void __launch_bounds__(256) k_mupdate(double* __restrict__ W, double* __restrict__ Z, int N, int R,
                                                  const double* __restrict__ w, const double* __restrict__ wre,
-                                                 const double* __restrict__ z, const double* __restrict__ rv,
-                                                 const MState* __restrict__ st, const double* __restrict__ cw,
-                                                 const double* __restrict__ cz, double* __restrict__ part) {
-  __shared__ double red[kGramWarps * 2 * 32];
-  const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
-  double v[2] = {0.0, 0.0};
-  if (lane < R && !(st->flags[lane] & MF_DISCARD)) {
-    const int lr = st->l[lane];
-    const double* wsrc = (st->flags[lane] & MF_REORTH) ? wre : w;
-    double* Wl = W + (size_t)lr * N * R;
-    double* Zl = Z + (size_t)lr * N * R;
-    for (int j = blockIdx.x * wpb + (threadIdx.x >> 5); j < N; j += gridDim.x * wpb) {
-      const size_t o = (size_t)j * R + lane;
-      double av = wsrc[o], zv = __ldg(z + o);
-      for (int i = 0; i < lr; ++i) {
-        const size_t oi = ((size_t)i * N + j) * R + lane;
-        av = fma(-cw[(size_t)i * 32 + lane], __ldg(W + oi), av);
-        zv = fma(-cz[(size_t)i * 32 + lane], __ldg(Z + oi), zv);
-      }
-      Wl[o] = av;
-      Zl[o] = zv;
-      v[0] = fma(av, av, v[0]);
-      v[1] = fma(av, __ldg(rv + o), v[1]);
-    }
-  }
-  block_cols<2>(v, red, part, 2, 0, 2);
-}
-
-// normalise the new columns and update x, r; part[blk][32] = ||r||^2
-__global__ void __launch_bounds__(256) k_mfinish(double* __restrict__ W, double* __restrict__ Z, int N, int R,
-                                                 double* __restrict__ x, double* __restrict__ rv,
-                                                 const MState* __restrict__ st, double* __restrict__ part) {
+                                                 const double* __restrict__ z, double* __restrict__ x,
+                                                 double* __restrict__ rv, const double* __restrict__ cw,
+                                                 const double* __restrict__ cz, double* __restrict__ part,
+                                                 CtlArgs ctl) {
   __shared__ double red[kGramWarps * 32];
+  const MState* st = ctl.st;
   const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
   double v[1] = {0.0};
   if (lane < R) {
     const bool upd = !(st->flags[lane] & MF_DISCARD);
     const int lr = st->l[lane];
     const double g = st->gam[lane], al = st->alp[lane];
+    const double* wsrc = (st->flags[lane] & MF_REORTH) ? wre : w;
     double* Wl = W + (size_t)lr * N * R;
     double* Zl = Z + (size_t)lr * N * R;
     for (int j = blockIdx.x * wpb + (threadIdx.x >> 5); j < N; j += gridDim.x * wpb) {
       const size_t o = (size_t)j * R + lane;
       double r_ = rv[o];
       if (upd) {
-        const double wv = Wl[o] * g, zv = Zl[o] * g;
-        Wl[o] = wv;
+        double av = wsrc[o], zv = __ldg(z + o);
+        const double xo = x[o];
+#pragma unroll 4
+        for (int i = 0; i < lr; ++i) {
+          const size_t oi = ((size_t)i * N + j) * R + lane;
+          av = fma(-cw[(size_t)i * 32 + lane], __ldg(W + oi), av);
+          zv = fma(-cz[(size_t)i * 32 + lane], __ldg(Z + oi), zv);
+        }
+        av *= g;
+        zv *= g;
+        Wl[o] = av;
         Zl[o] = zv;
-        x[o] = fma(al, zv, x[o]);
-        r_ = fma(-al, wv, r_);
+        x[o] = fma(al, zv, xo);
+        r_ = fma(-al, av, r_);
         rv[o] = r_;
       }
       v[0] = fma(r_, r_, v[0]);
     }
   }
   block_cols<1>(v, red, part, 1, 0, 1);
+  mfinish_reduction(part, 1, 0, 0, ctl);
 }
 
 // part[blk][32] = sum of v^2 per right-hand side
-__global__ void __launch_bounds__(256) k_mnorm(const double* __restrict__ v, int N, int R, double* __restrict__ part) {
+__global__ void __launch_bounds__(256) k_mnorm(const double* __restrict__ v, int N, int R, double* __restrict__ part,
+                                               CtlArgs ctl) {
   __shared__ double red[kGramWarps * 32];
   const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
   double a[1] = {0.0};
@@ -632,6 +1039,7 @@ __global__ void __launch_bounds__(256) k_mnorm(const double* __restrict__ v, int
       a[0] = fma(t, t, a[0]);
     }
   block_cols<1>(a, red, part, 1, 0, 1);
+  mfinish_reduction(part, 1, 0, 0, ctl);
 }
 
 // dst = src for the right-hand sides flagged in mask[] (restart / confirmation)
@@ -660,174 +1068,6 @@ template <typename T>
 __global__ void k_narrow(const double* __restrict__ src, T* __restrict__ dst, size_t n) {
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     dst[i] = (T)src[i];
-}
-
-// ------------------------------------------------------------------ control (one warp)
-__global__ void k_mctl(MState* st, const MState* parent, const double* __restrict__ sums, double* cw,
-                       double* cz, int kind) {
-  const int r = threadIdx.x;
-  const int R = st->R, lcap = st->lcap;
-  bool f_any = false, f_restart = false, f_claim = false, f_reorth = false;
-  if (r < R) {
-    switch (kind) {
-      case CTL_INIT0: {
-        const double n0 = sqrt(sums[r]);
-        st->rnorm0[r] = n0;
-        st->rnorm[r] = n0;
-        st->eps[r] = fmax(st->rtol * n0, st->atol);
-        st->act[r] = n0 > st->eps[r] && isfinite(n0);
-        if (!isfinite(n0)) st->status = KCMG_NONFINITE;
-        st->l[r] = 0;
-        st->flags[r] = 0;
-        st->brk[r] = 0;
-        st->claim[r] = 0;
-        st->restart[r] = 0;
-        break;
-      }
-      case CTL_BEGIN: {
-        const double n0 = sqrt(sums[r]);
-        st->rnorm0[r] = n0;
-        st->rnorm[r] = n0;
-        st->eps[r] = st->rtol * n0;
-        st->act[r] = parent->act[r] && n0 > 0.0;
-        st->l[r] = 0;
-        st->flags[r] = 0;
-        st->restart[r] = 0;
-        break;
-      }
-      case CTL_TEST: {
-        const bool active = st->act[r] != 0;
-        const bool conv = !(st->rnorm[r] > st->eps[r]);
-        if (st->level == 0) {
-          st->claim[r] = active && conv;    // confirmed by a true residual first
-          f_claim = active && conv;
-        } else if (active && conv) {
-          st->act[r] = 0;
-        }
-        st->restart[r] = st->act[r] && !st->claim[r] && st->l[r] > 0 && st->l[r] + st->per_cycle > st->cap;
-        f_restart = st->restart[r] != 0;
-        f_any = st->act[r] != 0;
-        break;
-      }
-      case CTL_GRAM1: {
-        const int l = st->l[r];
-        double hh = 0.0;
-        for (int i = 0; i < l; ++i) {
-          const double h = sums[(size_t)i * 32 + r];
-          hh += h * h;
-          cw[(size_t)i * 32 + r] = h;
-          cz[(size_t)i * 32 + r] = h;
-        }
-        const double naz2 = sums[(size_t)lcap * 32 + r];
-        st->naz2[r] = naz2;
-        const bool discard = !st->act[r] || !isfinite(naz2) || !(naz2 > 0.0);
-        const bool reorth = !discard && l > 0 && (naz2 - hh < 0.25 * naz2);
-        st->flags[r] = (discard ? MF_DISCARD : 0) | (reorth ? MF_REORTH : 0);
-        f_reorth = reorth;
-        break;
-      }
-      case CTL_GRAM2: {
-        if (st->flags[r] & MF_REORTH) {
-          for (int i = 0; i < st->l[r]; ++i) {
-            const double h2 = sums[(size_t)i * 32 + r];
-            cz[(size_t)i * 32 + r] += h2;
-            cw[(size_t)i * 32 + r] = h2;
-          }
-        }
-        f_reorth = (st->flags[r] & MF_REORTH) != 0;
-        break;
-      }
-      case CTL_UPDATE: {
-        const double nw = sqrt(sums[r]);
-        bool discard = (st->flags[r] & MF_DISCARD) != 0;
-        if (!isfinite(nw) || !(nw > st->brk_tol * sqrt(st->naz2[r]))) discard = true;
-        st->gam[r] = discard ? 0.0 : 1.0 / nw;
-        st->alp[r] = discard ? 0.0 : sums[32 + r] / nw;
-        if (discard) st->flags[r] |= MF_DISCARD;
-        f_reorth = (st->flags[r] & MF_REORTH) != 0;
-        break;
-      }
-      case CTL_FINISH: {
-        const bool discard = (st->flags[r] & MF_DISCARD) != 0;
-        if (!discard) {
-          st->l[r] += 1;
-          st->rnorm[r] = sqrt(sums[r]);
-          st->brk[r] = 0;
-        } else if (st->act[r]) {
-          if (++st->brk[r] >= 2 && st->level == 0) {   // two consecutive discards
-            st->status = KCMG_BREAKDOWN;
-            st->act[r] = 0;
-          }
-        }
-        if (!isfinite(st->rnorm[r])) {
-          st->status = KCMG_NONFINITE;
-          st->act[r] = 0;
-        }
-        break;
-      }
-      case CTL_RESTART: {
-        if (st->restart[r]) {
-          st->rnorm[r] = sqrt(sums[r]);
-          st->l[r] = 0;
-          st->restart[r] = 0;
-        }
-        break;
-      }
-      case CTL_CONFIRM: {
-        if (st->claim[r]) {
-          const double rn = sqrt(sums[r]);
-          st->rnorm[r] = rn;
-          st->l[r] = 0;
-          st->act[r] = rn > st->eps[r];
-          st->claim[r] = 0;
-        }
-        break;
-      }
-      case CTL_ITEND:
-        break;
-    }
-  }
-  const int nact = __popc(__ballot_sync(0xffffffffu, r < R && st->act[r]));
-  f_any = __any_sync(0xffffffffu, f_any);
-  f_restart = __any_sync(0xffffffffu, f_restart);
-  f_claim = __any_sync(0xffffffffu, f_claim);
-  f_reorth = __any_sync(0xffffffffu, f_reorth);
-  if (r == 0) {
-    switch (kind) {
-      case CTL_TEST: {
-        const bool go = f_any && st->it < st->maxit && st->guard < st->guard_cap;
-        st->any = go;
-        st->any_restart = go && f_restart;
-        st->any_claim = f_claim;
-        st->nact = nact;
-        if (go && !f_restart && !f_claim) st->guard++;
-        break;
-      }
-      case CTL_GRAM1:
-      case CTL_GRAM2:
-      case CTL_UPDATE:
-        st->any_reorth = f_reorth;
-        break;
-      case CTL_RESTART:
-        st->nrestart++;
-        break;
-      case CTL_CONFIRM:
-        st->nrestart++;
-        break;
-      case CTL_ITEND:
-        st->it++;
-        st->iters_total++;
-        break;
-      case CTL_BEGIN:
-        st->it = 0;
-        break;
-      case CTL_INIT0:
-        st->it = 0;
-        break;
-      default:
-        break;
-    }
-  }
 }
 
 // restart mask for the confirmation of claims: the masked copy reads st->claim
@@ -1164,13 +1404,15 @@ struct MrhsEngine {
   double *part = nullptr, *sums = nullptr, *cw = nullptr, *cz = nullptr;
   size_t part_len = 0;
   int* mask = nullptr;
-  MState* hst = nullptr;  // pinned host copy of the flags
+  HostFlags* hst = nullptr;   // pinned: the flags of the last loop test
+  unsigned seq = 0;           // its sequence number
   long long launches = 0;
   std::vector<int> hist_act;   // active columns at each level-0 loop test
   std::string* err = nullptr;
   cudaStream_t s = nullptr;
   // autotuner record: per level 0 the chosen shapes and their times
   double tune[16] = {};
+  bool forced_sweep = false;   // KCMG_SWEEP names the FP32 sweep kernel of every level
   int* tc_err = nullptr;  // set by the bulk-copy sweep when a copy did not complete in time
 };
 
@@ -1217,9 +1459,46 @@ int grid_for(size_t items, int per_block, int cap) {
   }
 
 // ---------------------------------------------------------------- launch wrappers
+// Levels on the entry-per-thread kernels (k_mrow_*): with a warp per cell and column lanes the
+// chip needs about 16 warps an SM to reach the FMA rate, and one entry per thread gives np times
+// the threads; from there on the column mapping's fewer loads win.
+bool mrow_level(const MrhsEngine* E, const MLev& L) { return L.C <= 16 * E->nsm && !E->forced_sweep; }
+// whole cells of a block: about 128 threads
+int mrow_cells(const MrhsEngine* E) { return std::max(1, 128 / (E->v.np * E->R)); }
+
+template <typename T, typename TI, typename TR, typename TZ>
+void sweep_mrow(MrhsEngine* E, const MLev& L, const T* A, bool cell_major, const TI* D, const TR* r, T* r_lo,
+                const T* zo, TZ* zn, int first) {
+  const int cpb = mrow_cells(E);
+  MRHS_ND_SWITCH(E->v.np, E->v.dim, {
+    constexpr int S = 2 * DIM + 1;
+    const size_t bs = (size_t)NP * NP, slot = cell_major ? bs : (size_t)L.C * bs, cell = cell_major ? S * bs : bs;
+    const int t = cpb * NP * E->R;
+    k_mrow_sweep<T, TI, TR, TZ, NP, S><<<grid_for(L.C, cpb, 1 << 30), t, t * sizeof(T), E->s>>>(
+        A, slot, cell, D, L.nbr, L.C, E->R, r, r_lo, zo, zn, (T)E->v.omega, first);
+  });
+  E->launches++;
+}
+template <typename TR, typename TZ>
+void sweep_mrow32(MrhsEngine* E, const MLev& L, const TR* r, const float* zo, TZ* zn, int first) {
+  if (L.D16) sweep_mrow<float, __nv_bfloat16, TR, TZ>(E, L, L.Acm, true, L.D16, r, L.r32, zo, zn, first);
+  else sweep_mrow<float, float, TR, TZ>(E, L, L.Acm, true, L.D32, r, L.r32, zo, zn, first);
+}
+
 void spmm64(MrhsEngine* E, const MLev& L, const double* x, double* y, const double* b, int mode) {
   if (L.V64 && mode != 1) {
     launch_mpattern_spmm(E->v.np, E->v.dim, L.n, E->R, L.V64, x, y, b, mode, E->s);
+    E->launches++;
+    return;
+  }
+  if (mrow_level(E, L) && mode != 2) {
+    const int cpb = mrow_cells(E);
+    MRHS_ND_SWITCH(E->v.np, E->v.dim, {
+      constexpr int S = 2 * DIM + 1;
+      const int g = grid_for(L.C, cpb, 1 << 30), t = cpb * NP * E->R;
+      if (mode == 0) k_mrow_spmm<NP, S, false><<<g, t, 0, E->s>>>(L.A64, L.nbr, L.C, E->R, x, y, b);
+      else k_mrow_spmm<NP, S, true><<<g, t, 0, E->s>>>(L.A64, L.nbr, L.C, E->R, x, y, b);
+    });
     E->launches++;
     return;
   }
@@ -1323,29 +1602,55 @@ void sweep64(MrhsEngine* E, const MLev& L, const double* rv, const double* zo, d
   E->launches++;
 }
 
-int gram_grid(const MLev& L) { return grid_for((size_t)L.N, kGramWarps, kGramBlocks); }
+// blocks of the Gram and vector kernels: four rows a warp on small levels (fewer partial sums)
+int gram_grid(const MLev& L) { return grid_for((size_t)L.N, 4 * kGramWarps, kGramBlocks); }
 
-void ctl(MrhsEngine* E, int lev, int kind, const MState* parent = nullptr) {
-  k_mctl<<<1, 32, 0, E->s>>>(E->lv[lev].st, parent, E->sums, E->cw, E->cz, kind);
+// steps after the reduction, on level lev; a loop test among them gets the next sequence number
+CtlArgs ctl_args(MrhsEngine* E, int lev, unsigned steps, const MState* parent = nullptr) {
+  CtlArgs c{E->lv[lev].st, parent, steps, E->sums, E->cw, E->cz, E->hst, 0u};
+  for (unsigned k = steps; k; k >>= 4)
+    if ((k & 15u) == CTL_TEST) c.seq = ++E->seq;
+  return c;
+}
+
+// Small reductions end in the kernel itself (its last block sums at most this many values: a few
+// microseconds for one SM); larger ones in a k_mreduce launch with a block per column.
+constexpr size_t kInKernelSums = 65536;
+bool in_kernel(int nblk, int cols) { return (size_t)nblk * cols * 32 <= kInKernelSums; }
+
+void reduce(MrhsEngine* E, int nblk, int pstride, int lcap, int gated, const CtlArgs& c) {
+  k_mreduce<<<pstride, 256, 0, E->s>>>(E->part, nblk, pstride, lcap, gated, c);
   E->launches++;
 }
 
-void reduce(MrhsEngine* E, int nblk, int ncols, const MState* st, int limit) {
-  k_mreduce<<<ncols, 256, 0, E->s>>>(E->part, nblk, ncols, st, limit, E->sums);
-  E->launches++;
-}
-
-// per-RHS ||v||^2 -> sums[0..R)
-void norms(MrhsEngine* E, const MLev& L, const double* vv) {
+// per-RHS ||v||^2 -> sums[0..R), then the control steps on level lev
+void norms(MrhsEngine* E, int lev, const double* vv, unsigned steps) {
+  const MLev& L = E->lv[lev];
   const int g = gram_grid(L);
-  k_mnorm<<<g, kGramWarps * 32, 0, E->s>>>(vv, L.N, E->R, E->part);
+  const CtlArgs c = ctl_args(E, lev, steps);
+  const bool in = in_kernel(g, 1) && steps;
+  CtlArgs none = c;
+  none.steps = 0;
+  k_mnorm<<<g, kGramWarps * 32, 0, E->s>>>(vv, L.N, E->R, E->part, in ? c : none);
   E->launches++;
-  reduce(E, g, 1, nullptr, 0);
+  if (!in) reduce(E, g, 1, 0, 0, c);
 }
 
-void read_flags(MrhsEngine* E, int lev) {
-  MCK(cudaMemcpyAsync(E->hst, E->lv[lev].st, 32, cudaMemcpyDeviceToHost, E->s));
-  MCK(cudaStreamSynchronize(E->s));
+// The flags of the loop test with sequence number E->seq: the device writes them to pinned memory,
+// the number last.  The wait is bounded by the stream: once that has drained or failed without
+// the number, the run failed.
+void read_flags(MrhsEngine* E) {
+  for (unsigned spins = 0; E->hst->seq != E->seq; ++spins) {
+    if ((spins & 4095u) != 4095u) continue;
+    const cudaError_t q = cudaStreamQuery(E->s);
+    if (q == cudaErrorNotReady) continue;
+    MCK(q);
+    if (E->hst->seq != E->seq) {
+      if (E->err) *E->err = "batched solve: a loop test's flags did not arrive";
+      throw Fail2{KCMG_CUDA_ERROR};
+    }
+  }
+  std::atomic_thread_fence(std::memory_order_acquire);
 }
 
 // ---------------------------------------------------------------- cycle pieces
@@ -1376,6 +1681,8 @@ void smooth(MrhsEngine* E, int lev, const double* rr = nullptr, double* zz = nul
         launch_mpattern_sweep<double, double, double, double>(E->v.np, E->v.dim, L.n, E->R, L.V64, L.D64, rr, nullptr,
                                                               zo, zn, E->v.omega, k == 0, E->s);
         E->launches++;
+      } else if (mrow_level(E, L)) {
+        sweep_mrow<double, double, double, double>(E, L, L.A64, false, L.D64, rr, nullptr, zo, zn, k == 0);
       } else {
         sweep64(E, L, rr, zo, zn, k == 0);
       }
@@ -1387,6 +1694,13 @@ void smooth(MrhsEngine* E, int lev, const double* rr = nullptr, double* zz = nul
     sweep_pattern32<double, float>(E, L, rr, L.r32, nullptr, buf[0], true);
     for (int k = 1; k < sw - 1; ++k) sweep_pattern32<float, float>(E, L, L.r32, nullptr, buf[(k + 1) & 1], buf[k & 1], false);
     sweep_pattern32<float, double>(E, L, L.r32, nullptr, buf[sw & 1], zz, false);
+    return;
+  }
+  if (mrow_level(E, L) && sw > 1) {
+    float* buf[2] = {L.s0, L.s1};
+    sweep_mrow32<double, float>(E, L, rr, nullptr, buf[0], 1);
+    for (int k = 1; k < sw - 1; ++k) sweep_mrow32<float, float>(E, L, L.r32, buf[(k + 1) & 1], buf[k & 1], 0);
+    sweep_mrow32<float, double>(E, L, L.r32, buf[sw & 1], zz, 0);
     return;
   }
   const size_t n = (size_t)L.N * E->R;
@@ -1427,41 +1741,50 @@ void smooth(MrhsEngine* E, int lev, const double* rr = nullptr, double* zz = nul
   }
 }
 
-// Alg. 1 for every right-hand side at once on the correction zcor (default: L.z)
-void rm(MrhsEngine* E, int lev, const double* zcor = nullptr) {
+// Alg. 1 for every right-hand side at once on the correction zcor (default: L.z); tail: control
+// steps after it
+void rm(MrhsEngine* E, int lev, const double* zcor = nullptr, unsigned tail = 0) {
   MLev& L = E->lv[lev];
-  const int R = E->R, g = gram_grid(L), thr = kGramWarps * 32;
+  const int R = E->R, g = gram_grid(L), thr = kGramWarps * 32, ps = L.lcap + 2;
   const double* zz = zcor ? zcor : L.z;
+  const bool in = in_kernel(g, ps), in1 = in_kernel(g, 1);
+  const CtlArgs none = ctl_args(E, lev, CTL_NONE);
+  const CtlArgs g1 = ctl_args(E, lev, CTL_GRAM1), g2 = ctl_args(E, lev, CTL_GRAM2);
+  const CtlArgs fin = ctl_args(E, lev, ctl_seq(CTL_FINISH) | (tail << 4));
   spmm64(E, L, zz, L.w, nullptr, 0);                                     // w = A z
-  k_mdots<<<g, thr, 0, E->s>>>(L.W, L.w, L.N, R, L.lcap, L.st, E->part, 0);
-  reduce(E, g, L.lcap + 1, L.st, 1);
-  ctl(E, lev, CTL_GRAM1);
-  k_mapply<<<g, thr, 0, E->s>>>(L.W, L.w, L.wre, L.N, R, L.st, E->sums);   // sums = h (pass 1)
-  k_mdots<<<g, thr, 0, E->s>>>(L.W, L.wre, L.N, R, L.lcap, L.st, E->part, 1);
-  E->launches += 3;
-  // pass 2 results: the reduce reads only when some right-hand side reorthogonalised;
-  // otherwise the partials are stale but CTL_GRAM2 ignores them (no REORTH flags)
-  reduce(E, g, L.lcap + 1, L.st, 1);
-  ctl(E, lev, CTL_GRAM2);
-  k_mupdate<<<g, thr, 0, E->s>>>(L.W, L.Z, L.N, R, L.w, L.wre, zz, L.r, L.st, E->cw, E->cz, E->part);
-  E->launches++;
-  reduce(E, g, 2, nullptr, 0);
-  ctl(E, lev, CTL_UPDATE);
-  k_mfinish<<<g, thr, 0, E->s>>>(L.W, L.Z, L.N, R, L.x, L.r, L.st, E->part);
-  E->launches++;
-  reduce(E, g, 1, nullptr, 0);
-  ctl(E, lev, CTL_FINISH);
+  k_mdots<<<g, thr, 0, E->s>>>(L.W, L.w, L.r, L.N, R, L.lcap, E->part, 0, in ? g1 : none);
+  if (!in) reduce(E, g, ps, L.lcap, 0, g1);
+  k_mapply<<<g, thr, 0, E->s>>>(L.W, L.w, L.wre, L.N, R, L.st, E->cw);      // cw = h (pass 1)
+  k_mdots<<<g, thr, 0, E->s>>>(L.W, L.wre, L.r, L.N, R, L.lcap, E->part, 1, in ? g2 : none);
+  if (!in) reduce(E, g, ps, L.lcap, 1, g2);
+  k_mupdate<<<g, thr, 0, E->s>>>(L.W, L.Z, L.N, R, L.w, L.wre, zz, L.x, L.r, E->cw, E->cz, E->part, in1 ? fin : none);
+  if (!in1) reduce(E, g, 1, 0, 0, fin);
+  E->launches += 4;
 }
 
+// b_{lev+1} = R r_lev; start: also r = b, x = 0 and the state of level lev + 1, with its first
+// loop test
 void restrict_to(MrhsEngine* E, int lev, bool start) {
   MLev &F = E->lv[lev], &C = E->lv[lev + 1];
-  const int g = grid_for(C.C, 8, 4096);
+  CtlArgs c{}, none{};
+  if (start) c = ctl_args(E, lev + 1, ctl_seq(CTL_BEGIN, CTL_TEST), F.st);
+  none.st = c.st;
+  double *rc = start ? C.r : nullptr, *xc = start ? C.x : nullptr, *part = start ? E->part : nullptr;
+  const bool row = C.C <= 16 * E->nsm;
+  const int g = row ? C.C : grid_for(C.C, 8, 4096);
+  const bool in = in_kernel(g, 1);
   MRHS_ND_SWITCH(E->v.np, E->v.dim, {
-    k_mrestrict<NP, DIM><<<g, 256, 0, E->s>>>(F.r, F.n[0], F.n[1], C.n[0], C.n[1], C.C, E->v.P, E->R, C.b,
-                                              start ? C.r : nullptr, start ? C.x : nullptr, start ? E->part : nullptr);
+    if (row) {
+      const int t = (NP * E->R + 31) / 32 * 32;
+      k_mrow_restrict<NP, DIM><<<g, t, NP * E->R * sizeof(double), E->s>>>(
+          F.r, F.n[0], F.n[1], C.n[0], C.n[1], E->v.P, E->R, C.b, rc, xc, part, in ? c : none);
+    } else {
+      k_mrestrict<NP, DIM><<<g, 256, 0, E->s>>>(F.r, F.n[0], F.n[1], C.n[0], C.n[1], C.C, E->v.P, E->R, C.b, rc, xc,
+                                                part, in ? c : none);
+    }
   });
   E->launches++;
-  if (start) reduce(E, g, 1, nullptr, 0);
+  if (start && !in) reduce(E, g, 1, 0, 0, c);
 }
 
 void prolong_from(MrhsEngine* E, int lev, double* target = nullptr) {
@@ -1469,6 +1792,10 @@ void prolong_from(MrhsEngine* E, int lev, double* target = nullptr) {
   const int g = grid_for(F.C, 8, 1 << 30);
   double* zf = target ? target : F.z;
   MRHS_ND_SWITCH(E->v.np, E->v.dim, {
+    if (F.C <= 16 * E->nsm)
+      k_mrow_prolong<NP, DIM><<<grid_for((size_t)F.N * E->R, 256, 1 << 30), 256, 0, E->s>>>(
+          C.x, F.n[0], F.n[1], F.C, C.n[0], C.n[1], E->v.P, E->R, zf);
+    else
     k_mprolong<NP, DIM><<<g, 256, 0, E->s>>>(C.x, F.n[0], F.n[1], F.C, C.n[0], C.n[1], E->v.P, E->R, zf);
   });
   E->launches++;
@@ -1476,7 +1803,7 @@ void prolong_from(MrhsEngine* E, int lev, double* target = nullptr) {
 
 void coarse_solve(MrhsEngine* E) {
   MLev& C = E->lv[E->v.nlev - 1];
-  k_mcoarse<<<grid_for(E->v.Nc, 8, 1 << 30), 256, 0, E->s>>>(E->v.Ainv, E->v.Nc, E->R, C.b, C.x);
+  k_mcoarse<<<E->v.Nc, 256, 0, E->s>>>(E->v.Ainv, E->v.Nc, E->R, C.b, C.x);
   E->launches++;
 }
 
@@ -1489,18 +1816,17 @@ void restart(MrhsEngine* E, int lev, bool confirm) {
   const size_t n = (size_t)L.N * E->R;
   k_mcopy_masked<<<grid_for(n, 256, E->nsm * 16), 256, 0, E->s>>>(L.t, L.r, L.N, E->R, E->mask);
   E->launches += 2;
-  norms(E, L, L.t);
-  ctl(E, lev, confirm ? CTL_CONFIRM : CTL_RESTART);
+  norms(E, lev, L.t, ctl_seq(confirm ? CTL_CONFIRM : CTL_RESTART, CTL_TEST));
 }
 
-// MG(lev) of Alg. 2 for all right-hand sides; on entry b, r, x and the state are set
+// MG(lev) of Alg. 2 for all right-hand sides; on entry b, r, x and the state are set and the
+// first loop test is issued
 void mg(MrhsEngine* E, int lev) {
   MLev& L = E->lv[lev];
   const int nlev = E->v.nlev;
   for (;;) {
-    ctl(E, lev, CTL_TEST);
-    read_flags(E, lev);
-    if (lev == 0) E->hist_act.push_back(E->hst->nact);
+    read_flags(E);
+    if (lev == 0) E->hist_act.push_back((int)E->hst->nact);
     if (E->hst->any_claim) { restart(E, lev, true); continue; }
     if (!E->hst->any) break;
     if (E->hst->any_restart) { restart(E, lev, false); continue; }
@@ -1511,14 +1837,12 @@ void mg(MrhsEngine* E, int lev) {
       coarse_solve(E);
     } else {
       restrict_to(E, lev, true);
-      ctl(E, lev + 1, CTL_BEGIN, L.st);
       mg(E, lev + 1);
     }
     prolong_from(E, lev);                             // coarse correction
     rm(E, lev);
     smooth(E, lev);                                   // post-smoother
-    rm(E, lev);
-    ctl(E, lev, CTL_ITEND);
+    rm(E, lev, nullptr, ctl_seq(CTL_ITEND, CTL_TEST));
   }
 }
 
@@ -1532,9 +1856,8 @@ void mg_async0(MrhsEngine* E) {
   MLev& L = E->lv[0];
   const int nlev = E->v.nlev;
   for (;;) {
-    ctl(E, 0, CTL_TEST);
-    read_flags(E, 0);
-    E->hist_act.push_back(E->hst->nact);
+    read_flags(E);
+    E->hist_act.push_back((int)E->hst->nact);
     if (E->hst->any_claim) { restart(E, 0, true); continue; }
     if (!E->hst->any) break;
     if (E->hst->any_restart) { restart(E, 0, false); continue; }
@@ -1543,7 +1866,6 @@ void mg_async0(MrhsEngine* E) {
       coarse_solve(E);
     } else {
       restrict_to(E, 0, true);
-      ctl(E, 1, CTL_BEGIN, L.st);
       mg(E, 1);
     }
     prolong_from(E, 0, L.zc);
@@ -1551,8 +1873,7 @@ void mg_async0(MrhsEngine* E) {
       smooth(E, 0);
       rm(E, 0);
     }
-    rm(E, 0, L.zc);                                   // the synchronisation
-    ctl(E, 0, CTL_ITEND);
+    rm(E, 0, L.zc, ctl_seq(CTL_ITEND, CTL_TEST));     // the synchronisation
   }
 }
 
@@ -1620,7 +1941,7 @@ void autotune(MrhsEngine* E) {
       E->tune[0] = L.sp_wpb;
       if (L.V32 && E->v.sweeps > 1) E->tune[2] = 4, E->tune[8] = 3;
     }
-    if (L.C < 256) continue;                        // small levels: defaults
+    if (L.C < 256 || (!L.V64 && mrow_level(E, L))) continue;   // small levels: one shape
     const int reps = lev == 0 ? 3 : 5;
     // FP64 operator: warps per block (the pattern kernels have one shape)
     float best = 1e30f;
@@ -1724,6 +2045,7 @@ void build(MrhsEngine* E, const MrhsView& v, int R) {
   E->precision = v.precision;
   E->mixed = v.precision != KCMG_FP64;
   E->s = v.s;
+  E->forced_sweep = getenv("KCMG_SWEEP") != nullptr;
   int dev = 0;
   MCK(cudaGetDevice(&dev));
   MCK(cudaDeviceGetAttribute(&E->nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -1754,7 +2076,7 @@ void build(MrhsEngine* E, const MrhsView& v, int R) {
       const size_t nv = mpattern_values(np, v.dim, L.C);
       L.V64 = malloc_dev<double>(E, nv);
       launch_mpattern_pack<double>(np, v.dim, L.A64, L.nbr, L.C, L.V64, E->s);
-      if (E->mixed && !getenv("KCMG_SWEEP")) {   // a forced sweep kernel runs on every level
+      if (E->mixed && !E->forced_sweep) {   // a forced sweep kernel runs on every level
         L.V32 = malloc_dev<float>(E, nv);
         launch_mpattern_pack<float>(np, v.dim, L.A64, L.nbr, L.C, L.V32, E->s);
       }
@@ -1823,16 +2145,17 @@ void build(MrhsEngine* E, const MrhsView& v, int R) {
     throw Fail2{KCMG_SINGULAR};
   }
   int maxcols = 2;
-  for (int l = 0; l < v.nlev - 1; ++l) maxcols = std::max(maxcols, E->lv[l].lcap + 1);
+  for (int l = 0; l < v.nlev - 1; ++l) maxcols = std::max(maxcols, E->lv[l].lcap + 2);
   E->part_len = (size_t)kGramBlocks * maxcols * 32;
-  const size_t rblocks = (size_t)grid_for(E->lv[1].C, 8, 4096);
+  const size_t rblocks = (size_t)std::max(grid_for(E->lv[1].C, 8, 4096), 16 * E->nsm);
   E->part_len = std::max(E->part_len, rblocks * 32);
   E->part = malloc_dev<double>(E, E->part_len);
   E->sums = malloc_dev<double>(E, (size_t)maxcols * 32);
   E->cw = malloc_dev<double>(E, (size_t)maxcols * 32);
   E->cz = malloc_dev<double>(E, (size_t)maxcols * 32);
   E->mask = malloc_dev<int>(E, kMaxRhs);
-  MCK(cudaMallocHost(&E->hst, sizeof(MState)));
+  MCK(cudaHostAlloc((void**)&E->hst, sizeof(HostFlags), cudaHostAllocDefault));
+  E->hst->seq = 0;
   if (E->mixed) tc_prepare(E);
   autotune(E);
 }
@@ -1913,13 +2236,12 @@ kcmg_status mrhs_solve(MrhsEngine** peng, const MrhsView& v, const double* b, do
     }
     // r0 = b - A x0 (compensated), ||r0|| per right-hand side
     spmm64(E, L, L.x, L.r, L.b, 2);
-    norms(E, L, L.r);
-    ctl(E, 0, CTL_INIT0);
+    norms(E, 0, L.r, ctl_seq(CTL_INIT0, CTL_TEST));
     if (v.async_smooth > 0) mg_async0(E);
     else mg(E, 0);
     // final true residual
     spmm64(E, L, L.x, L.t, L.b, 2);
-    norms(E, L, L.t);
+    norms(E, 0, L.t, CTL_NONE);
     std::vector<double> rn2(R);
     MCK(cudaMemcpyAsync(rn2.data(), E->sums, R * sizeof(double), cudaMemcpyDeviceToHost, E->s));
     std::vector<MState> hs(v.nlev - 1);

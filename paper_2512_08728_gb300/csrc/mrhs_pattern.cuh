@@ -10,7 +10,7 @@
 // sweep; np = 10, 3-D) where the dense kernels do 700; the FP32 sweep by HBM and L2.
 // Measured (GB300): one level-0 cycle of 13 minimisations at 32^3 x 32 columns, FP64, 133 -> 61 ms;
 // five FP32/BF16 sweeps at 48^3 x 32 as a whole call 1232 -> 788 us (staging copies and conversion
-// passes gone as well).
+// passes gone as well), 666 us with four columns a lane (k_mpat_sweep4).
 // Results are those of the dense kernels (k_mspmm64, k_msweep64, k_msweep_simt) bit for bit: a
 // row sees its entries in the same order, and poison_rows() keeps what an infinity or NaN does to
 // the dense kernels' zero products.
@@ -194,6 +194,153 @@ k_mpat_sweep(const T* __restrict__ V, const TI* __restrict__ D, PatGrid g, int R
   }
 }
 
+// The FP32 sweep for column counts that are a multiple of four (16 to 32): a lane owns four
+// columns, so 32 columns are eight lanes and a warp takes four cells, and the entries and
+// inverses of a block's cells are staged in shared memory, the inverses as FP32.  With a column a
+// lane (above) the sweep is bound by L1: 200 load instructions a cell, 110 of them one address for
+// the whole warp.  Here a row of the iterate is one 16-byte load a lane and an entry pair one
+// conflict-free shared-memory read for four cells: about 100 L1 accesses a cell.
+template <int NP, int DIM, int LPC> struct MSweep4 {
+  static constexpr int CELLS = kMpatThreads / LPC;            // cells of a block
+  static constexpr int VS = MPattern<NP, DIM>::STRIDE;        // floats of a cell's entries
+  static constexpr int DR = (NP + 3) / 4 * 4;                 // floats of an inverse row
+  static constexpr int BYTES = CELLS * (VS + NP * DR) * 4;
+};
+
+template <typename Part, int E>
+static __device__ __forceinline__ void m4_entry(const float* Vc, const float4& x, float4 (&t)[Part::ROWS]) {
+  constexpr int I = Part::tab.i[E];
+  if constexpr (I >= 0) {
+    const float v = Vc[E];
+    t[I].x = fmaf(-v, x.x, t[I].x);
+    t[I].y = fmaf(-v, x.y, t[I].y);
+    t[I].z = fmaf(-v, x.z, t[I].z);
+    t[I].w = fmaf(-v, x.w, t[I].w);
+  }
+}
+template <typename Part, int B, int NP, int... E>
+static __device__ __forceinline__ void m4_entries(std::integer_sequence<int, E...>, const float* Vc,
+                                                  const float4 (&x)[NP], float4 (&t)[Part::ROWS]) {
+  (m4_entry<Part, B + E>(Vc, x[Part::tab.j[B + E]], t), ...);
+}
+static __device__ __forceinline__ float4 ld4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+static __device__ __forceinline__ float4 ld4(const double* p) {
+  const double2 a = __ldg(reinterpret_cast<const double2*>(p)), b = __ldg(reinterpret_cast<const double2*>(p) + 1);
+  return make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
+}
+static __device__ __forceinline__ void st4(float* p, const float4& v) { *reinterpret_cast<float4*>(p) = v; }
+static __device__ __forceinline__ void st4(double* p, const float4& v) {
+  *reinterpret_cast<double2*>(p) = make_double2(v.x, v.y);
+  *reinterpret_cast<double2*>(p + 2) = make_double2(v.z, v.w);
+}
+
+template <typename TI, typename TR, typename TZ, int NP, int DIM, int LPC, bool FIRST>
+__global__ void __launch_bounds__(kMpatThreads)
+k_mpat_sweep4(const float* __restrict__ V, const TI* __restrict__ D, PatGrid g, int R, const TR* __restrict__ r,
+              float* __restrict__ r_lo, const float* __restrict__ zo, TZ* __restrict__ zn, float om) {
+  using MP = MPattern<NP, DIM>;
+  using Part = typename MP::Part;
+  using Sh = MSweep4<NP, DIM, LPC>;
+  extern __shared__ __align__(16) float smem_m4[];
+  float* Vs = smem_m4;
+  float* Ds = smem_m4 + Sh::CELLS * Sh::VS;
+  const int K0 = blockIdx.x * Sh::CELLS, nk = min(Sh::CELLS, g.C - K0);
+  if (!FIRST) {
+    const float4* src = reinterpret_cast<const float4*>(V + (size_t)K0 * Sh::VS);
+    for (int q = threadIdx.x; q < nk * (Sh::VS / 4); q += kMpatThreads) reinterpret_cast<float4*>(Vs)[q] = __ldg(src + q);
+  }
+  for (int q = threadIdx.x; q < nk * NP * NP; q += kMpatThreads) {
+    const int c = q / (NP * NP), e = q - c * NP * NP;
+    Ds[(c * NP + e / NP) * Sh::DR + e % NP] = (float)D[(size_t)K0 * NP * NP + q];
+  }
+  __syncthreads();
+  const int c = threadIdx.x / LPC, K = K0 + c, col = (threadIdx.x % LPC) * 4;
+  if (c >= nk || col >= R) return;
+  const size_t o0 = (size_t)K * NP * R + col;
+  float4 t[NP];
+  if constexpr (FIRST) {
+#pragma unroll
+    for (int i = 0; i < NP; ++i) t[i] = ld4(r + o0 + (size_t)i * R);
+    if constexpr (!std::is_same<float, TR>::value) {
+#pragma unroll
+      for (int i = 0; i < NP; ++i) st4(r_lo + o0 + (size_t)i * R, t[i]);
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < NP; ++i) t[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float* Vc = Vs + c * Sh::VS;
+    const int q0 = (unsigned)K / (unsigned)g.n0, c0 = K - q0 * g.n0;
+    const int c2 = DIM == 3 ? (unsigned)q0 / (unsigned)g.n1 : 0, c1 = DIM == 3 ? q0 - c2 * g.n1 : q0;
+    int mag = 0;
+    auto slot = [&](auto sc) {
+      constexpr int s = decltype(sc)::value;
+      if constexpr (s < MP::TP::S) {
+        const int J = pat_neighbour<DIM>(g, K, c0, c1, c2, s);
+        if (J >= 0) {
+          float4 x[NP];
+#pragma unroll
+          for (int j = 0; j < NP; ++j) x[j] = ld4(zo + (size_t)J * NP * R + col + (size_t)j * R);
+#pragma unroll
+          for (int j = 0; j < NP; ++j)
+            mag = max(max(mag, max(mag_bits(x[j].x), mag_bits(x[j].y))), max(mag_bits(x[j].z), mag_bits(x[j].w)));
+          constexpr int B = Part::tab.begin[s], N = Part::tab.begin[s + 1] - B;
+          m4_entries<Part, B>(std::make_integer_sequence<int, N>{}, Vc, x, t);
+        }
+      }
+    };
+    slot(std::integral_constant<int, 1>{});
+    slot(std::integral_constant<int, 2>{});
+    slot(std::integral_constant<int, 3>{});
+    slot(std::integral_constant<int, 4>{});
+    slot(std::integral_constant<int, 5>{});
+    slot(std::integral_constant<int, 6>{});
+    if (mag >= Nonfinite<float>::FROM) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const unsigned rows = mpat_poison<float, NP, DIM, 1>(zo + col + k, g, K, c0, c1, c2, R);
+#pragma unroll
+        for (int i = 0; i < NP; ++i)
+          if ((rows >> i) & 1u) poison(k == 0 ? t[i].x : k == 1 ? t[i].y : k == 2 ? t[i].z : t[i].w);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      const float4 b = ld4(r + o0 + (size_t)i * R);
+      t[i].x += b.x;
+      t[i].y += b.y;
+      t[i].z += b.z;
+      t[i].w += b.w;
+    }
+  }
+  const float* Dc = Ds + c * NP * Sh::DR;
+#pragma unroll
+  for (int i = 0; i < NP; ++i) {
+    float4 e = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+      const float d = Dc[i * Sh::DR + j];
+      e.x = fmaf(d, t[j].x, e.x);
+      e.y = fmaf(d, t[j].y, e.y);
+      e.z = fmaf(d, t[j].z, e.z);
+      e.w = fmaf(d, t[j].w, e.w);
+    }
+    const size_t o = o0 + (size_t)i * R;
+    if constexpr (FIRST) {
+      e.x *= om;
+      e.y *= om;
+      e.z *= om;
+      e.w *= om;
+    } else {
+      const float4 z = ld4(zo + o);
+      e.x = fmaf(1.f - om, z.x, om * e.x);
+      e.y = fmaf(1.f - om, z.y, om * e.y);
+      e.z = fmaf(1.f - om, z.z, om * e.z);
+      e.w = fmaf(1.f - om, z.w, om * e.w);
+    }
+    st4(zn + o, e);
+  }
+}
+
 namespace {
 
 
@@ -267,6 +414,29 @@ template <typename T, typename TI, typename TR, typename TZ>
 void launch_mpattern_sweep(int np, int dim, const int* n, int R, const T* V, const TI* D, const TR* r, T* r_lo,
                            const T* zo, TZ* zn, double omega, int first, cudaStream_t s) {
   const PatGrid g = mpat_dims(n, dim);
+  if constexpr (std::is_same<T, float>::value) {
+    // four columns a lane: rows on 16-byte boundaries and at least four lanes a cell (fewer columns
+    // stage more cells than they keep busy); np = 20 would need 80 sums a lane
+    if (R % 4 == 0 && R >= 16 && np <= 10) {
+      mpat_switch(np, dim, [&](auto NPc, auto DIMc) {
+        constexpr int NP = decltype(NPc)::value, DIM = decltype(DIMc)::value;
+        auto go = [&](auto LPCc) {
+          constexpr int LPC = decltype(LPCc)::value;
+          using Sh = MSweep4<NP, DIM, LPC>;
+          const int grid = (g.C + Sh::CELLS - 1) / Sh::CELLS;
+          if constexpr (std::is_same<TZ, T>::value && !std::is_same<TR, T>::value)
+            if (first) k_mpat_sweep4<TI, TR, TZ, NP, DIM, LPC, true><<<grid, kMpatThreads, Sh::BYTES, s>>>(V, D, g, R, r, r_lo, zo, zn, (T)omega);
+          if constexpr (std::is_same<TR, T>::value)
+            if (!first) k_mpat_sweep4<TI, TR, TZ, NP, DIM, LPC, false><<<grid, kMpatThreads, Sh::BYTES, s>>>(V, D, g, R, r, r_lo, zo, zn, (T)omega);
+        };
+        if constexpr (NP <= 10) {
+          if (R > 16) go(std::integral_constant<int, 8>{});
+          else go(std::integral_constant<int, 4>{});
+        }
+      });
+      return;
+    }
+  }
   mpat_switch(np, dim, [&](auto NPc, auto DIMc) {
     rp_switch<std::is_same<T, float>::value>(R, [&](auto RPc) {
       constexpr int NP = decltype(NPc)::value, DIM = decltype(DIMc)::value, RP = decltype(RPc)::value;
