@@ -220,7 +220,7 @@ void alloc_cycle_vectors(kcmg_ctx* ctx, Level& L, int lcap) {
   L.h = dalloc<double>(ctx, lcap);
   L.h2 = dalloc<double>(ctx, lcap);
   const size_t spmv_blocks = L.rows_pad / L.block_rows;
-  size_t plen = (size_t)kDotBlocksMax * (lcap + 1);
+  size_t plen = (size_t)kDotBlocksMax * (lcap + 2);
   if (spmv_blocks > plen) plen = spmv_blocks;
   if (L.pat) plen = std::max(plen, (size_t)pattern_blocks(ctx->np, ctx->dim, L.ncell));
   if ((size_t)4 * 65536 > plen) plen = 4 * 65536;
@@ -551,20 +551,16 @@ struct Cycle {
     V* Z = static_cast<V*>(L.Z);
     V* w = static_cast<V*>(L.w);
     V* wre = static_cast<V*>(L.wre);
-    EpiArgs none = epi(lev, EPI_NONE);
-    launches += 6;
-    apply_op<V>(ctx, L, z, w,
-                   nullptr, L.partial, none, 0, s);
-    launch_gram_dots<V>(W, L.N, w, L.lcap, L.nblk, L.partial, epi(lev, EPI_GRAM1), 0, s);
+    V* r = static_cast<V*>(L.r);
+    launches += 5;
+    apply_op<V>(ctx, L, z, w, nullptr, L.partial, epi(lev, EPI_NONE), 0, s);
+    launch_gram_dots<V>(W, L.N, w, r, L.lcap, L.nblk, L.partial, epi(lev, EPI_GRAM1), 0, s);
     launch_gram_apply<V>(W, L.N, w, wre, L.lcap, L.nblk2, L.st, L.h, s);
-    launch_gram_dots<V>(W, L.N, wre, L.lcap, L.nblk, L.partial, epi(lev, EPI_GRAM2), 1, s);
-    launch_gram_update<V>(W, Z, L.N, w, wre, z, static_cast<V*>(L.r), L.lcap, L.nblk2, L.partial,
-                          epi(lev, EPI_UPDATE), s);
+    launch_gram_dots<V>(W, L.N, wre, r, L.lcap, L.nblk, L.partial, epi(lev, EPI_GRAM2), 1, s);
     EpiArgs fin = epi(lev, EPI_FINISH);
     fin.end_iter = end_iter;
     fin.hist_type = htype;
-    launch_rm_finish<V>(W, Z, L.N, static_cast<V*>(L.x), static_cast<V*>(L.r), L.nblk2, L.partial,
-                        fin, s);
+    launch_gram_update<V>(W, Z, L.N, w, wre, z, static_cast<V*>(L.x), r, L.lcap, L.nblk2, L.partial, fin, s);
   }
 
   // one pass of the while body of Alg. 2 on level lev; V is the level's vector type
@@ -1851,16 +1847,16 @@ kcmg_status kcmg_kernel_report(kcmg_ctx* ctx, int reps, double* out, int nout) {
         g1.h = L.h;
         g1.h2 = L.h2;
         EpiArgs up = g1;
-        up.kind = EPI_UPDATE;
+        up.kind = EPI_NONE;
         float ms = 0;
         CK(cudaEventRecord(e0, ctx->s));
         for (int k = 0; k < reps; ++k) {
           if (ctx->ir)
-            launch_gram_dots<float>(static_cast<float*>(L.W), L.N, static_cast<float*>(L.w), L.lcap, L.nblk,
-                                    L.partial, g1, 0, ctx->s);
+            launch_gram_dots<float>(static_cast<float*>(L.W), L.N, static_cast<float*>(L.w), static_cast<float*>(L.r),
+                                    L.lcap, L.nblk, L.partial, g1, 0, ctx->s);
           else
-            launch_gram_dots<double>(static_cast<double*>(L.W), L.N, static_cast<double*>(L.w), L.lcap, L.nblk,
-                                     L.partial, g1, 0, ctx->s);
+            launch_gram_dots<double>(static_cast<double*>(L.W), L.N, static_cast<double*>(L.w),
+                                     static_cast<double*>(L.r), L.lcap, L.nblk, L.partial, g1, 0, ctx->s);
         }
         CK(cudaEventRecord(e1, ctx->s));
         CK(cudaEventSynchronize(e1));
@@ -1868,20 +1864,21 @@ kcmg_status kcmg_kernel_report(kcmg_ctx* ctx, int reps, double* out, int nout) {
         out[o1 + 4] = ms / reps;
         out[o1 + 5] = 2.0 * (lt + 1) * L.N;
         // the first pass set the flags from zero vectors: clear them for a plain update
-        h.flags = 0;
-        CK(cudaMemcpyAsync(&L.st->flags, &h.flags, sizeof(int), cudaMemcpyHostToDevice, ctx->s));
+        h.gamma = 1.0;
+        h.alpha = 0.0;
+        CK(cudaMemcpyAsync(L.st, &h, sizeof h, cudaMemcpyHostToDevice, ctx->s));
         CK(cudaEventRecord(e0, ctx->s));
         for (int k = 0; k < reps; ++k) {
           if (ctx->ir)
             launch_gram_update<float>(static_cast<float*>(L.W), static_cast<float*>(L.Z), L.N,
                                       static_cast<float*>(L.w), static_cast<float*>(L.wre),
-                                      static_cast<float*>(L.z), static_cast<float*>(L.r), L.lcap, L.nblk2,
-                                      L.partial, up, ctx->s);
+                                      static_cast<float*>(L.z), static_cast<float*>(L.x), static_cast<float*>(L.r),
+                                      L.lcap, L.nblk2, L.partial, up, ctx->s);
           else
             launch_gram_update<double>(static_cast<double*>(L.W), static_cast<double*>(L.Z), L.N,
                                        static_cast<double*>(L.w), static_cast<double*>(L.wre),
-                                       static_cast<double*>(L.z), static_cast<double*>(L.r), L.lcap, L.nblk2,
-                                       L.partial, up, ctx->s);
+                                       static_cast<double*>(L.z), static_cast<double*>(L.x),
+                                       static_cast<double*>(L.r), L.lcap, L.nblk2, L.partial, up, ctx->s);
         }
         CK(cudaEventRecord(e1, ctx->s));
         CK(cudaEventSynchronize(e1));

@@ -82,30 +82,35 @@ static __device__ void epilogue(const EpiArgs& e, const double* sums) {
       record(e, 0);
       set_cond(e, more_cycles(st));
     } break;
+    // W^T w, ||w||^2 and w . r decide the whole step: the norm of w_hat = w - W h by Pythagoras
+    // (reliable, as it is only used when it did not cancel below a quarter of ||w||^2; else the
+    // second Gram-Schmidt pass is requested, "twice is enough"), and alpha = w_hat . r = w . r, as
+    // r is orthogonal to W
     case EPI_GRAM1: {
       const int l = st->l;
-      double hh = 0.0;
-      for (int i = 0; i < l; ++i) { e.h[i] = sums[i]; hh += sums[i] * sums[i]; }
-      const double naz2 = sums[l];
+      const double naz2 = sums[l], nw2 = naz2 - sums[l + 2];   // [l + 2]: sum of the squared coefficients
       st->naz2 = naz2;
       int f = 0;
-      // Pythagoras estimate of ||w - W h||^2; reorthogonalise when it fell below a
-      // quarter of ||w||^2 (a second Gram-Schmidt pass, "twice is enough")
-      if (l > 0 && naz2 - hh < 0.25 * naz2) f |= F_REORTH;
       if (!isfinite(naz2) || !(naz2 > 0.0)) f |= F_DISCARD;
+      else if (l > 0 && nw2 < 0.25 * naz2) f |= F_REORTH;
+      else {
+        st->gamma = 1.0 / sqrt(nw2);
+        st->alpha = st->gamma * sums[l + 1];
+      }
+      if (!isfinite(naz2) && st->level == 0) st->status = KCMG_NONFINITE;
       st->flags = f;
     } break;
+    // the second pass: w' = w - W h.  A w' that loses most of its norm again, or falls below brk
+    // relative to ||A z||, is rounding noise: the correction depends linearly on the basis
     case EPI_GRAM2: {
-      for (int i = 0; i < st->l; ++i) e.h2[i] = sums[i];
-    } break;
-    case EPI_UPDATE: {
-      const double nw = sqrt(sums[0]), naz = sqrt(st->naz2);
-      if ((st->flags & F_DISCARD) || !isfinite(nw) || !(nw > st->brk * naz)) {
+      const int l = st->l;
+      const double n2 = sums[l], nw2 = n2 - sums[l + 2];
+      if (!isfinite(nw2) || !(nw2 >= 0.25 * n2) || !(nw2 > st->brk * st->brk * st->naz2)) {
         st->flags |= F_DISCARD;
-        if (!isfinite(nw) && st->level == 0) st->status = KCMG_NONFINITE;
+        if (!isfinite(n2) && st->level == 0) st->status = KCMG_NONFINITE;
       } else {
-        st->gamma = 1.0 / nw;
-        st->alpha = st->gamma * sums[1];   // alpha = (gamma w_hat) . r
+        st->gamma = 1.0 / sqrt(nw2);
+        st->alpha = st->gamma * sums[l + 1];
       }
     } break;
     case EPI_FINISH: {

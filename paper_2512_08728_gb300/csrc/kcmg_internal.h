@@ -49,9 +49,8 @@ struct LevelState {
 enum EpiKind : int {
   EPI_NONE = 0,
   EPI_MG_BEGIN,     // sum = ||r0||^2: start of an MG call on the level
-  EPI_GRAM1,        // sums = W^T w, ||w||^2
-  EPI_GRAM2,        // sums = W^T w' (reorthogonalisation pass)
-  EPI_UPDATE,       // sums = ||w_hat||^2, w_hat . r
+  EPI_GRAM1,        // sums = W^T w, ||w||^2, w . r
+  EPI_GRAM2,        // sums = W^T w', ||w'||^2, w' . r (reorthogonalisation pass)
   EPI_FINISH,       // sum = ||r||^2 after the x, r update
   EPI_RESTART,      // sum = ||b - A x||^2: restart of the level
   EPI_NORM          // sum = ||y||^2 stored into *out (component calls, refinement)
@@ -100,18 +99,14 @@ void launch_prolong(int np, int dim, const int* nf, const int* nc, const T* P, c
 template <typename T>
 void launch_coarse_gemv(const double* Ainv, int n, const T* b, T* x, cudaStream_t s);
 template <typename T>
-void launch_gram_dots(const T* W, int N, const T* w, int lcap, int nblk, double* partial,
+void launch_gram_dots(const T* W, int N, const T* w, const T* r, int lcap, int nblk, double* partial,
                       const EpiArgs& e, int conditional, cudaStream_t s);
 template <typename T>
 void launch_gram_apply(const T* W, int N, const T* w, T* wout, int lcap, int nblk,
                        LevelState* st, const double* h, cudaStream_t s);
 template <typename T>
-void launch_gram_update(const T* W, const T* Z, int N, const T* w, const T* wre, const T* z,
-                        const T* r, int lcap, int nblk, double* partial, const EpiArgs& e,
-                        cudaStream_t s);
-template <typename T>
-void launch_rm_finish(T* W, T* Z, int N, T* x, T* r, int nblk, double* partial,
-                      const EpiArgs& e, cudaStream_t s);
+void launch_gram_update(T* W, T* Z, int N, const T* w, const T* wre, const T* z, T* x, T* r, int lcap, int nblk,
+                        double* partial, const EpiArgs& e, cudaStream_t s);
 template <typename T>
 void launch_norm(const T* v, int N, int nblk, double* partial, const EpiArgs& e,
                  cudaStream_t s);

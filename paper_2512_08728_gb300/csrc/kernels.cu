@@ -267,14 +267,14 @@ __global__ void k_coarse_gemv(const double* __restrict__ Ainv, int n, const T* _
 }
 
 // ------------------------------------------------------------------ Gram / RM (Alg. 1)
-// partial[k][c] = sum over element chunk k of W_c . w for c < l, and ||w||^2 at c = l.
+// partial[k][c] = sum over element chunk k of W_c . w for c < l, ||w||^2 at c = l, w . r at l + 1.
 // Work items are (group of kDotCols columns) x (element chunk); the fixed grid takes them
 // round-robin with K = grid / groups chunks per group, so a block reduces its sums once
 // per item and the reduction order depends only on N, l and the grid.  With PAIR (N even)
 // a thread takes two consecutive elements per step with one 16-byte (FP64) or 8-byte
 // (FP32) load per column.  The last partial column group reads a valid column in place of
 // the missing ones and drops those sums, so every step issues the same FMAs (no
-// predicated arithmetic).  ||w||^2 rides with group 0 as a separate accumulator.
+// predicated arithmetic).  ||w||^2 and w . r ride with group 0 as separate accumulators.
 constexpr int kDotCols = 8;
 
 template <typename T> struct Pair;
@@ -282,8 +282,9 @@ template <> struct Pair<double> { using type = double2; };
 template <> struct Pair<float> { using type = float2; };
 
 template <typename T, bool PAIR, bool NORM>
-__device__ __forceinline__ void dots_item(const T* __restrict__ W, int N, const T* __restrict__ w, int l, int c0,
-                                          int u0, int u1, T (&acc)[kDotCols], T& ww) {
+__device__ __forceinline__ void dots_item(const T* __restrict__ W, int N, const T* __restrict__ w,
+                                          const T* __restrict__ r, int l, int c0, int u0, int u1,
+                                          T (&acc)[kDotCols], T& ww, T& wr) {
   using T2 = typename Pair<T>::type;
   const T* Wc[kDotCols];
 #pragma unroll
@@ -298,28 +299,34 @@ __device__ __forceinline__ void dots_item(const T* __restrict__ W, int N, const 
         acc[c] = fma(a.y, wv.y, acc[c]);
       }
       if (NORM) {
+        const T2 rv = __ldg(reinterpret_cast<const T2*>(r) + u);
         ww = fma(wv.x, wv.x, ww);
         ww = fma(wv.y, wv.y, ww);
+        wr = fma(wv.x, rv.x, wr);
+        wr = fma(wv.y, rv.y, wr);
       }
     } else {
       const T wv = __ldg(w + u);
 #pragma unroll
       for (int c = 0; c < kDotCols; ++c) acc[c] = fma(__ldg(Wc[c] + u), wv, acc[c]);
-      if (NORM) ww = fma(wv, wv, ww);
+      if (NORM) {
+        ww = fma(wv, wv, ww);
+        wr = fma(wv, __ldg(r + u), wr);
+      }
     }
   }
 }
 
 template <typename T, bool PAIR>
 __global__ void __launch_bounds__(kVecThreads)
-k_gram_dots(const T* __restrict__ W, int N, const T* __restrict__ w, double* partial,
+k_gram_dots(const T* __restrict__ W, int N, const T* __restrict__ w, const T* __restrict__ r, double* partial,
             EpiArgs e, int conditional) {
   LevelState* st = e.st;
   if (conditional && !(st->flags & F_REORTH)) return;
   __shared__ double sh[32 * 8];   // bsum_n<NC> needs 32 * NC
   const int l = st->l;
-  const int ncol = l + 1;
-  const int groups = l > 0 ? (l + kDotCols - 1) / kDotCols : 1;   // l = 0: the norm only
+  const int ncol = l + 2;
+  const int groups = l > 0 ? (l + kDotCols - 1) / kDotCols : 1;   // l = 0: ||w||^2 and w . r only
   const int K = max(1, (int)gridDim.x / groups);
   const int units = PAIR ? N / 2 : N;
   const int chunk = (units + K - 1) / K;
@@ -330,22 +337,26 @@ k_gram_dots(const T* __restrict__ W, int N, const T* __restrict__ w, double* par
     T acct[kDotCols];
 #pragma unroll
     for (int c = 0; c < kDotCols; ++c) acct[c] = T(0);
-    T ww = T(0);
+    T ww = T(0), wr = T(0);
     if (l == 0) {
       for (int u = u0 + threadIdx.x; u < u1; u += blockDim.x) {
         if (PAIR) {
-          const typename Pair<T>::type wv = __ldg(reinterpret_cast<const typename Pair<T>::type*>(w) + u);
+          using T2 = typename Pair<T>::type;
+          const T2 wv = __ldg(reinterpret_cast<const T2*>(w) + u), rv = __ldg(reinterpret_cast<const T2*>(r) + u);
           ww = fma(wv.x, wv.x, ww);
           ww = fma(wv.y, wv.y, ww);
+          wr = fma(wv.x, rv.x, wr);
+          wr = fma(wv.y, rv.y, wr);
         } else {
           const T wv = __ldg(w + u);
           ww = fma(wv, wv, ww);
+          wr = fma(wv, __ldg(r + u), wr);
         }
       }
     } else if (g == 0) {
-      dots_item<T, PAIR, true>(W, N, w, l, c0, u0, u1, acct, ww);
+      dots_item<T, PAIR, true>(W, N, w, r, l, c0, u0, u1, acct, ww, wr);
     } else {
-      dots_item<T, PAIR, false>(W, N, w, l, c0, u0, u1, acct, ww);
+      dots_item<T, PAIR, false>(W, N, w, r, l, c0, u0, u1, acct, ww, wr);
     }
     // the block's sums in FP64 (FP32 vectors: FP32 products and per-thread sums)
     double acc[8];
@@ -357,14 +368,17 @@ k_gram_dots(const T* __restrict__ W, int N, const T* __restrict__ w, double* par
       for (int c = 0; c < kDotCols; ++c)
         if (c0 + c < l) partial[(size_t)k * ncol + c0 + c] = acc[c];
     if (g == 0) {
-      double v[1] = {(double)ww};
-      bsum_n<1>(v, sh);
-      if (threadIdx.x == 0) partial[(size_t)k * ncol + l] = v[0];
+      double v[2] = {(double)ww, (double)wr};
+      bsum_n<2>(v, sh);
+      if (threadIdx.x == 0) {
+        partial[(size_t)k * ncol + l] = v[0];
+        partial[(size_t)k * ncol + l + 1] = v[1];
+      }
     }
   }
   if (last_block(&st->ticket)) {
     // one warp per column: lanes read independent partials, then a fixed shuffle tree
-    extern __shared__ double sums[];  // [ncol]
+    extern __shared__ double sums[];  // [ncol], then the sum of the squared coefficients
     const int wid = threadIdx.x >> 5, ln = threadIdx.x & 31, nw = blockDim.x >> 5;
     for (int c = wid; c < ncol; c += nw) {
       double s = 0.0;
@@ -374,9 +388,20 @@ k_gram_dots(const T* __restrict__ W, int N, const T* __restrict__ w, double* par
       if (ln == 0) sums[c] = s;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      epilogue(e, sums);
-      st->ticket = 0u;
+    // the coefficients and the sum of their squares, in parallel: one thread's loop over the basis
+    // would take 60 clocks a column
+    double* h = e.kind == EPI_GRAM2 ? e.h2 : e.h;
+    for (int i = threadIdx.x; i < l; i += blockDim.x) h[i] = sums[i];
+    if (wid == 0) {
+      double hh = 0.0;
+      for (int i = ln; i < l; i += 32) hh = fma(sums[i], sums[i], hh);
+#pragma unroll
+      for (int o = 16; o; o >>= 1) hh += __shfl_xor_sync(0xffffffffu, hh, o);
+      if (ln == 0) {
+        sums[ncol] = hh;
+        epilogue(e, sums);
+        st->ticket = 0u;
+      }
     }
   }
 }
@@ -399,95 +424,90 @@ k_gram_apply(const T* __restrict__ W, int N, const T* __restrict__ w, T* __restr
   }
 }
 
-// w_hat = w_src - W c_w, z_hat = z - Z c_z written to column l of W and Z; partial sums
-// ||w_hat||^2 and w_hat . r.  Without reorthogonalisation w_src = w, c_w = c_z = h; with it
-// w_src = w' = w - W h, c_w = h2, c_z = h + h2.  With PAIR (N even) a thread updates two
-// consecutive elements with one 16-byte (FP64) / 8-byte (FP32) load per column of W and Z.
+// The step of Alg. 1: w_l = gamma (w_src - W c_w), z_l = gamma (z - Z c_z) written to column l
+// of W and Z, x += alpha z_l, r -= alpha w_l; ||r||^2 -> EPI_FINISH.  gamma and alpha are known
+// from the Gram pass, so the column is normalised and applied as it is formed: the pass that read
+// the two new columns again to normalise them, and read and wrote x and r, is gone (8^3 mixed solve
+// 30.1 -> 28.3 ms, 2-D 128 x 96 16.4 -> 16.0, launches being what they spend most on).  Without
+// reorthogonalisation w_src = w, c_w = c_z = h; with it w_src = w' = w - W h, c_w = h2,
+// c_z = h + h2.  A discarded correction leaves W, Z, x, r unchanged.  With PAIR (N even) a thread
+// takes two consecutive elements with one 16-byte (FP64) / 8-byte (FP32) load per column.
 template <typename T, bool PAIR>
 __global__ void __launch_bounds__(kVecThreads)
 k_gram_update(T* W, T* Z, int N, const T* __restrict__ w, const T* __restrict__ wre,
-              const T* __restrict__ z, const T* __restrict__ r, double* partial, EpiArgs e) {
+              const T* __restrict__ z, T* __restrict__ x, T* __restrict__ r, double* partial, EpiArgs e) {
   using T2 = typename Pair<T>::type;
   LevelState* st = e.st;
   extern __shared__ double cs[];  // [2][l]
   __shared__ double sh[32 * 8];   // bsum_n<NC> needs 32 * NC
   const int l = st->l;
-  const bool re = (st->flags & F_REORTH) != 0;
-  for (int i = threadIdx.x; i < l; i += blockDim.x) {
-    cs[i] = re ? e.h2[i] : e.h[i];
-    cs[l + i] = re ? e.h[i] + e.h2[i] : e.h[i];
-  }
+  const bool re = (st->flags & F_REORTH) != 0, keep = !(st->flags & F_DISCARD);
+  const T gam = (T)st->gamma, al = (T)st->alpha;
+  if (keep)
+    for (int i = threadIdx.x; i < l; i += blockDim.x) {
+      cs[i] = re ? e.h2[i] : e.h[i];
+      cs[l + i] = re ? e.h[i] + e.h2[i] : e.h[i];
+    }
   __syncthreads();
   const T* ws = re ? wre : w;
   T* Wl = W + (size_t)l * N;
   T* Zl = Z + (size_t)l * N;
-  T nw2 = T(0), wr = T(0);   // per-thread sums in T, reduced in FP64
+  T r2 = T(0);   // per-thread sums in T, reduced in FP64
   if (PAIR) {
     const int units = N / 2;
     for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < units; u += gridDim.x * blockDim.x) {
-      T2 a = reinterpret_cast<const T2*>(ws)[u], c = reinterpret_cast<const T2*>(z)[u];
+      T2 rv = reinterpret_cast<const T2*>(r)[u];
+      if (keep) {
+        T2 a = __ldg(reinterpret_cast<const T2*>(ws) + u), c = __ldg(reinterpret_cast<const T2*>(z) + u);
+        T2 xv = reinterpret_cast<const T2*>(x)[u];
 #pragma unroll 4
-      for (int i = 0; i < l; ++i) {
-        const T2 wi = __ldg(reinterpret_cast<const T2*>(W + (size_t)i * N) + u);
-        const T2 zi = __ldg(reinterpret_cast<const T2*>(Z + (size_t)i * N) + u);
-        const T cw = (T)(-cs[i]), cz = (T)(-cs[l + i]);
-        a.x = fma(cw, wi.x, a.x);
-        a.y = fma(cw, wi.y, a.y);
-        c.x = fma(cz, zi.x, c.x);
-        c.y = fma(cz, zi.y, c.y);
+        for (int i = 0; i < l; ++i) {
+          const T2 wi = __ldg(reinterpret_cast<const T2*>(W + (size_t)i * N) + u);
+          const T2 zi = __ldg(reinterpret_cast<const T2*>(Z + (size_t)i * N) + u);
+          const T cw = (T)(-cs[i]), cz = (T)(-cs[l + i]);
+          a.x = fma(cw, wi.x, a.x);
+          a.y = fma(cw, wi.y, a.y);
+          c.x = fma(cz, zi.x, c.x);
+          c.y = fma(cz, zi.y, c.y);
+        }
+        a.x *= gam;
+        a.y *= gam;
+        c.x *= gam;
+        c.y *= gam;
+        reinterpret_cast<T2*>(Wl)[u] = a;
+        reinterpret_cast<T2*>(Zl)[u] = c;
+        xv.x = fma(al, c.x, xv.x);
+        xv.y = fma(al, c.y, xv.y);
+        reinterpret_cast<T2*>(x)[u] = xv;
+        rv.x = fma(-al, a.x, rv.x);
+        rv.y = fma(-al, a.y, rv.y);
+        reinterpret_cast<T2*>(r)[u] = rv;
       }
-      reinterpret_cast<T2*>(Wl)[u] = a;
-      reinterpret_cast<T2*>(Zl)[u] = c;
-      const T2 rv = reinterpret_cast<const T2*>(r)[u];
-      nw2 = fma(a.x, a.x, nw2);
-      nw2 = fma(a.y, a.y, nw2);
-      wr = fma(a.x, rv.x, wr);
-      wr = fma(a.y, rv.y, wr);
+      r2 = fma(rv.x, rv.x, r2);
+      r2 = fma(rv.y, rv.y, r2);
     }
   } else {
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < N; j += gridDim.x * blockDim.x) {
-      T a = ws[j], c = z[j];
+      T rv = r[j];
+      if (keep) {
+        T a = ws[j], c = z[j];
 #pragma unroll 4
-      for (int i = 0; i < l; ++i) {
-        a = fma((T)(-cs[i]), __ldg(W + (size_t)i * N + j), a);
-        c = fma((T)(-cs[l + i]), __ldg(Z + (size_t)i * N + j), c);
+        for (int i = 0; i < l; ++i) {
+          a = fma((T)(-cs[i]), __ldg(W + (size_t)i * N + j), a);
+          c = fma((T)(-cs[l + i]), __ldg(Z + (size_t)i * N + j), c);
+        }
+        a *= gam;
+        c *= gam;
+        Wl[j] = a;
+        Zl[j] = c;
+        x[j] = fma(al, c, x[j]);
+        rv = fma(-al, a, rv);
+        r[j] = rv;
       }
-      Wl[j] = a;
-      Zl[j] = c;
-      nw2 = fma(a, a, nw2);
-      wr = fma(a, r[j], wr);
+      r2 = fma(rv, rv, r2);
     }
   }
-  double v[2] = {(double)nw2, (double)wr};
-  finish_reduction<2>(v, partial, e, sh);
-}
-
-// Normalise the new column (gamma) and update x += alpha z_{l+1}, r -= alpha w_{l+1};
-// ||r||^2 -> EPI_FINISH.  A discarded correction leaves W, Z, x, r unchanged.
-template <typename T>
-__global__ void __launch_bounds__(kVecThreads)
-k_rm_finish(T* W, T* Z, int N, T* x, T* r, double* partial, EpiArgs e) {
-  LevelState* st = e.st;
-  __shared__ double sh[32 * 8];   // bsum_n<NC> needs 32 * NC
-  const bool keep = !(st->flags & F_DISCARD);
-  const int l = st->l;
-  const T gam = (T)st->gamma, al = (T)st->alpha;
-  T* Wl = W + (size_t)l * N;
-  T* Zl = Z + (size_t)l * N;
-  double r2 = 0.0;
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < N; j += gridDim.x * blockDim.x) {
-    T rv = r[j];
-    if (keep) {
-      const T wv = Wl[j] * gam, zv = Zl[j] * gam;
-      Wl[j] = wv;
-      Zl[j] = zv;
-      x[j] = fma(al, zv, x[j]);
-      rv = fma(-al, wv, rv);
-      r[j] = rv;
-    }
-    r2 = fma((double)rv, (double)rv, r2);
-  }
-  double v[1] = {r2};
+  double v[1] = {(double)r2};
   finish_reduction<1>(v, partial, e, sh);
 }
 
@@ -933,15 +953,16 @@ void launch_coarse_gemv(const double* Ainv, int n, const T* b, T* x, cudaStream_
   k_coarse_gemv<T><<<(n + rows_per_block - 1) / rows_per_block, 32 * rows_per_block, 0, s>>>(Ainv, n, b, x);
 }
 
-// dynamic shared memory: the final sums (lcap + 1 doubles) or the coefficients
+// dynamic shared memory: the final sums (lcap + 3 doubles) or the coefficients
 // (lcap or 2 lcap doubles); lcap <= kLcapMax keeps it within the default 48 KB
 template <typename T>
-void launch_gram_dots(const T* W, int N, const T* w, int lcap, int nblk, double* partial,
+void launch_gram_dots(const T* W, int N, const T* w, const T* r, int lcap, int nblk, double* partial,
                       const EpiArgs& e, int conditional, cudaStream_t s) {
+  const size_t sm = (lcap + 3) * sizeof(double);
   if (N % 2 == 0)   // pairs of elements: every column base is 16-byte (FP64) / 8-byte (FP32) aligned
-    k_gram_dots<T, true><<<nblk, kVecThreads, (lcap + 1) * sizeof(double), s>>>(W, N, w, partial, e, conditional);
+    k_gram_dots<T, true><<<nblk, kVecThreads, sm, s>>>(W, N, w, r, partial, e, conditional);
   else
-    k_gram_dots<T, false><<<nblk, kVecThreads, (lcap + 1) * sizeof(double), s>>>(W, N, w, partial, e, conditional);
+    k_gram_dots<T, false><<<nblk, kVecThreads, sm, s>>>(W, N, w, r, partial, e, conditional);
 }
 
 template <typename T>
@@ -951,21 +972,13 @@ void launch_gram_apply(const T* W, int N, const T* w, T* wout, int lcap, int nbl
 }
 
 template <typename T>
-void launch_gram_update(const T* W, const T* Z, int N, const T* w, const T* wre, const T* z,
-                        const T* r, int lcap, int nblk, double* partial, const EpiArgs& e,
-                        cudaStream_t s) {
+void launch_gram_update(T* W, T* Z, int N, const T* w, const T* wre, const T* z, T* x, T* r, int lcap, int nblk,
+                        double* partial, const EpiArgs& e, cudaStream_t s) {
+  const size_t sm = 2 * lcap * sizeof(double);
   if (N % 2 == 0)   // pairs of elements (aligned column bases), half the grid
-    k_gram_update<T, true><<<(nblk + 1) / 2, kVecThreads, 2 * lcap * sizeof(double), s>>>(
-        const_cast<T*>(W), const_cast<T*>(Z), N, w, wre, z, r, partial, e);
+    k_gram_update<T, true><<<(nblk + 1) / 2, kVecThreads, sm, s>>>(W, Z, N, w, wre, z, x, r, partial, e);
   else
-    k_gram_update<T, false><<<nblk, kVecThreads, 2 * lcap * sizeof(double), s>>>(
-        const_cast<T*>(W), const_cast<T*>(Z), N, w, wre, z, r, partial, e);
-}
-
-template <typename T>
-void launch_rm_finish(T* W, T* Z, int N, T* x, T* r, int nblk, double* partial, const EpiArgs& e,
-                      cudaStream_t s) {
-  k_rm_finish<T><<<nblk, kVecThreads, 0, s>>>(W, Z, N, x, r, partial, e);
+    k_gram_update<T, false><<<nblk, kVecThreads, sm, s>>>(W, Z, N, w, wre, z, x, r, partial, e);
 }
 
 template <typename T>
@@ -1070,14 +1083,12 @@ void launch_grad_lognu(int np, int dim, const int* n, const double* nu, const do
   template void launch_prolong<T, T>(int, int, const int*, const int*, const T*, const T*, T*,    \
                                      cudaStream_t);                                              \
   template void launch_coarse_gemv<T>(const double*, int, const T*, T*, cudaStream_t);           \
-  template void launch_gram_dots<T>(const T*, int, const T*, int, int, double*, const EpiArgs&,   \
-                                    int, cudaStream_t);                                          \
+  template void launch_gram_dots<T>(const T*, int, const T*, const T*, int, int, double*,          \
+                                    const EpiArgs&, int, cudaStream_t);                          \
   template void launch_gram_apply<T>(const T*, int, const T*, T*, int, int, LevelState*,         \
                                      const double*, cudaStream_t);                               \
-  template void launch_gram_update<T>(const T*, const T*, int, const T*, const T*, const T*,     \
-                                      const T*, int, int, double*, const EpiArgs&, cudaStream_t); \
-  template void launch_rm_finish<T>(T*, T*, int, T*, T*, int, double*, const EpiArgs&,           \
-                                    cudaStream_t);                                               \
+  template void launch_gram_update<T>(T*, T*, int, const T*, const T*, const T*, T*, T*, int,    \
+                                      int, double*, const EpiArgs&, cudaStream_t);               \
   template void launch_norm<T>(const T*, int, int, double*, const EpiArgs&, cudaStream_t);       \
   template void launch_interleave<T>(int, int, const double*, int, int, T*, cudaStream_t);       \
   template void launch_axpy_to_double<T>(const T*, double*, size_t, cudaStream_t);
