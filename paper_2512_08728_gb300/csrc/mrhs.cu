@@ -341,17 +341,17 @@ __device__ __forceinline__ bool mlast_block(unsigned int* ticket) {
   return s_last != 0;
 }
 
-// sums[c][32] = sum over nblk blocks of part[blk][c][32] for the column, by one warp
-__device__ __forceinline__ void mreduce_col(const double* part, int nblk, int pstride, int c, double* sums) {
+// sum over blocks b0..b1 of part[blk][c][lane], eight loads in flight
+__device__ __forceinline__ double mreduce_col(const double* part, int b0, int b1, int pstride, int c) {
   const int lane = threadIdx.x & 31;
-  double s0 = 0.0, s1 = 0.0;
-  int b = 0;
-  for (; b + 1 < nblk; b += 2) {
-    s0 += __ldcg(part + ((size_t)b * pstride + c) * 32 + lane);
-    s1 += __ldcg(part + ((size_t)(b + 1) * pstride + c) * 32 + lane);
+  double s = 0.0;
+  for (int b = b0; b < b1; b += 8) {
+    double v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = b + k < b1 ? __ldcg(part + ((size_t)(b + k) * pstride + c) * 32 + lane) : 0.0;
+    s += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
   }
-  if (b < nblk) s0 += __ldcg(part + ((size_t)b * pstride + c) * 32 + lane);
-  sums[(size_t)c * 32 + lane] = s0 + s1;
+  return s;
 }
 
 // End of a reduction kernel whose blocks wrote part[blk][c][32]: with c.steps the last block sums
@@ -360,8 +360,23 @@ __device__ __forceinline__ void mreduce_col(const double* part, int nblk, int ps
 __device__ __forceinline__ void mfinish_reduction(const double* part, int pstride, int L, int lcap, const CtlArgs& c) {
   if (!c.steps) return;
   if (!mlast_block(&c.st->ticket)) return;
-  const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5, n = L + pstride - lcap;
-  for (int k = warp; k < n; k += nw) mreduce_col(part, gridDim.x, pstride, k < L ? k : lcap + k - L, c.sums);
+  const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5, n = L + pstride - lcap, nblk = gridDim.x;
+  if (n == 1 && nw > 1) {   // one column: the warps take shares of the blocks
+    __shared__ double seg[32][32];
+    const int per = (nblk + nw - 1) / nw;
+    seg[warp][threadIdx.x & 31] = mreduce_col(part, min(nblk, warp * per), min(nblk, (warp + 1) * per), pstride, lcap - L);
+    __syncthreads();
+    if (warp == 0) {
+      double t = 0.0;
+      for (int w = 0; w < nw; ++w) t += seg[w][threadIdx.x];
+      c.sums[(size_t)(lcap - L) * 32 + threadIdx.x] = t;
+    }
+  } else {
+    for (int k = warp; k < n; k += nw) {
+      const int col = k < L ? k : lcap + k - L;
+      c.sums[(size_t)col * 32 + (threadIdx.x & 31)] = mreduce_col(part, 0, nblk, pstride, col);
+    }
+  }
   if (threadIdx.x == 0) c.st->ticket = 0u;
   __threadfence_block();
   __syncthreads();
@@ -785,7 +800,7 @@ __global__ void __launch_bounds__(640) k_mrow_restrict(const double* __restrict_
   if (i < NP) {
     const int jx = J % ncx, jy = (J / ncx) % ncy, jz = DIM == 3 ? J / (ncx * ncy) : 0;
     double s = 0.0;
-#pragma unroll 2
+#pragma unroll 4
     for (int k = 0; k < NCH; ++k) {
       const int fx = 2 * jx + (k & 1), fy = 2 * jy + ((k >> 1) & 1), fz = DIM == 3 ? 2 * jz + ((k >> 2) & 1) : 0;
       const double* rp = rf + (size_t)(fx + nfx * (fy + nfy * fz)) * NP * R + r;
@@ -974,7 +989,7 @@ __global__ void __launch_bounds__(256) k_mapply(const double* __restrict__ W, co
   const int lr = st->l[lane];
   for (int j = blockIdx.x * wpb + (threadIdx.x >> 5); j < N; j += gridDim.x * wpb) {
     double s = __ldg(w + (size_t)j * R + lane);
-#pragma unroll 4
+#pragma unroll 8
     for (int i = 0; i < lr; ++i) s = fma(-h[(size_t)i * 32 + lane], __ldg(W + ((size_t)i * N + j) * R + lane), s);
     wre[(size_t)j * R + lane] = s;
   }
@@ -982,7 +997,10 @@ __global__ void __launch_bounds__(256) k_mapply(const double* __restrict__ W, co
 
 // The step of Alg. 1 per right-hand side: w_l = gamma (wsrc - W cw), z_l = gamma (z - Z cz) into
 // column l_r, x += alpha z_l, r -= alpha w_l (gamma, alpha from the Gram pass; discarded
-// corrections change nothing); part[blk][32] = ||r||^2.
+// corrections change nothing); part[blk][32] = ||r||^2.  UNROLL columns' loads in flight: eight on
+// small levels, where they are what takes the time, four where many warps hide it and the
+// registers cost occupancy (32^3 x 32: eight 60.1, four 57.2 ms a cycle).
+template <int UNROLL>
 __global__ void __launch_bounds__(256) k_mupdate(double* __restrict__ W, double* __restrict__ Z, int N, int R,
                                                  const double* __restrict__ w, const double* __restrict__ wre,
                                                  const double* __restrict__ z, double* __restrict__ x,
@@ -1006,7 +1024,7 @@ __global__ void __launch_bounds__(256) k_mupdate(double* __restrict__ W, double*
       if (upd) {
         double av = wsrc[o], zv = __ldg(z + o);
         const double xo = x[o];
-#pragma unroll 4
+#pragma unroll UNROLL
         for (int i = 0; i < lr; ++i) {
           const size_t oi = ((size_t)i * N + j) * R + lane;
           av = fma(-cw[(size_t)i * 32 + lane], __ldg(W + oi), av);
@@ -1602,8 +1620,10 @@ void sweep64(MrhsEngine* E, const MLev& L, const double* rv, const double* zo, d
   E->launches++;
 }
 
-// blocks of the Gram and vector kernels: four rows a warp on small levels (fewer partial sums)
-int gram_grid(const MLev& L) { return grid_for((size_t)L.N, 4 * kGramWarps, kGramBlocks); }
+// blocks of the Gram kernels: two rows a warp on small levels (fewer partial sums); of the vector
+// kernels: one
+int gram_grid(const MLev& L) { return grid_for((size_t)L.N, 2 * kGramWarps, kGramBlocks); }
+int vec_grid(const MLev& L) { return grid_for((size_t)L.N, kGramWarps, kGramBlocks); }
 
 // steps after the reduction, on level lev; a loop test among them gets the next sequence number
 CtlArgs ctl_args(MrhsEngine* E, int lev, unsigned steps, const MState* parent = nullptr) {
@@ -1745,20 +1765,21 @@ void smooth(MrhsEngine* E, int lev, const double* rr = nullptr, double* zz = nul
 // steps after it
 void rm(MrhsEngine* E, int lev, const double* zcor = nullptr, unsigned tail = 0) {
   MLev& L = E->lv[lev];
-  const int R = E->R, g = gram_grid(L), thr = kGramWarps * 32, ps = L.lcap + 2;
+  const int R = E->R, g = gram_grid(L), gv = vec_grid(L), thr = kGramWarps * 32, ps = L.lcap + 2;
   const double* zz = zcor ? zcor : L.z;
-  const bool in = in_kernel(g, ps), in1 = in_kernel(g, 1);
+  const bool in = in_kernel(g, ps), in1 = in_kernel(gv, 1);
   const CtlArgs none = ctl_args(E, lev, CTL_NONE);
   const CtlArgs g1 = ctl_args(E, lev, CTL_GRAM1), g2 = ctl_args(E, lev, CTL_GRAM2);
   const CtlArgs fin = ctl_args(E, lev, ctl_seq(CTL_FINISH) | (tail << 4));
   spmm64(E, L, zz, L.w, nullptr, 0);                                     // w = A z
   k_mdots<<<g, thr, 0, E->s>>>(L.W, L.w, L.r, L.N, R, L.lcap, E->part, 0, in ? g1 : none);
   if (!in) reduce(E, g, ps, L.lcap, 0, g1);
-  k_mapply<<<g, thr, 0, E->s>>>(L.W, L.w, L.wre, L.N, R, L.st, E->cw);      // cw = h (pass 1)
+  k_mapply<<<gv, thr, 0, E->s>>>(L.W, L.w, L.wre, L.N, R, L.st, E->cw);      // cw = h (pass 1)
   k_mdots<<<g, thr, 0, E->s>>>(L.W, L.wre, L.r, L.N, R, L.lcap, E->part, 1, in ? g2 : none);
   if (!in) reduce(E, g, ps, L.lcap, 1, g2);
-  k_mupdate<<<g, thr, 0, E->s>>>(L.W, L.Z, L.N, R, L.w, L.wre, zz, L.x, L.r, E->cw, E->cz, E->part, in1 ? fin : none);
-  if (!in1) reduce(E, g, 1, 0, 0, fin);
+  auto update = gv < kGramBlocks ? k_mupdate<8> : k_mupdate<4>;
+  update<<<gv, thr, 0, E->s>>>(L.W, L.Z, L.N, R, L.w, L.wre, zz, L.x, L.r, E->cw, E->cz, E->part, in1 ? fin : none);
+  if (!in1) reduce(E, gv, 1, 0, 0, fin);
   E->launches += 4;
 }
 
