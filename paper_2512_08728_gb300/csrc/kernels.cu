@@ -317,8 +317,12 @@ __device__ __forceinline__ void dots_item(const T* __restrict__ W, int N, const 
   }
 }
 
+// At most 64 registers: two of this kernel's warps then fit an SM sub-partition beside three of
+// the coarse cycle's at 128 (64K registers a SM, a quarter to each), so that in the task-parallel
+// cycle it runs beside that kernel; with 68 the whole smoother path waited for its end (24^3,
+// p = 3, Schwarz, m = 12, one cycle: 11.6 -> 10.0 ms).
 template <typename T, bool PAIR>
-__global__ void __launch_bounds__(kVecThreads)
+__global__ void __launch_bounds__(kVecThreads, 4)
 k_gram_dots(const T* __restrict__ W, int N, const T* __restrict__ w, const T* __restrict__ r, double* partial,
             EpiArgs e, int conditional) {
   LevelState* st = e.st;
