@@ -90,7 +90,10 @@ cudaError_t coarse_cycle_prepare<CC_TV, CC_T, CC_TI>(CoarseArgs* a, int* grid) {
   cudaFuncAttributes fa;
   if ((e = cudaFuncGetAttributes(&fa, f)) != cudaSuccess) return e;
   if (a->sm_bytes + (int)fa.sharedSizeBytes > optin) return cudaErrorInvalidConfiguration;
-  if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, a->sm_bytes)) != cudaSuccess) return e;
+  // the limit belongs to the kernel, which contexts of other sizes launch too: the device's, always
+  if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes)) !=
+      cudaSuccess)
+    return e;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, kCoarseThreads, a->sm_bytes)) != cudaSuccess)
     return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
