@@ -153,8 +153,8 @@ struct CoarseCycle {
 
   const CoarseArgs& a;
   double* sh;            // 32 * 8 doubles
-  double* red_s;         // reduced sums, kCoarseMaxCols + 4
-  double* cf;            // coefficients of the minimisation, kCoarseMaxCols
+  double* red_s;         // reduced sums, a.cols + 4
+  double* cf;            // coefficients of the minimisation, a.cols
   RmScal* rms;
   int* nbs;              // neighbour slab of each slot: cell offset in the slab buffer
   long long* tph;        // clocks per phase kind, then per level (thread 0 of block 0)
@@ -164,14 +164,22 @@ struct CoarseCycle {
   bool ok = true;
   long long bytes = 0;   // algorithmic bytes of this launch (kept by thread 0 of block 0)
 
-  // the block's range on the current level (set by enter())
-  int lev = 0, K0 = 0, nc = 0, rows = 0, row0 = 0;
+  // blocks that take part in the current level (all, or block 0 alone on the smallest levels) and
+  // this block's range of it (set by enter())
+  int nblk = 1, lev = 0, K0 = 0, nc = 0, rows = 0, row0 = 0;
   int lpr = 1, part = 0, lrow = 0;   // threads per row; this thread's part and row (rows < blockDim)
   int rs_off = 0;                    // residual, own rows (byte offset)
   int own0 = 0;                      // the own rows' place in the slab buffer
   double *R = nullptr, *gm = nullptr, *al = nullptr;   // packed columns of R, 1 / R_kk, alpha
 
-  __device__ bool bar() { return cc_barrier(a, gen); }
+  __device__ bool grid_bar() { return cc_barrier(a, gen); }
+  // barrier of the blocks that take part in the current level
+  __device__ bool bar() {
+    if (nblk > 1) return grid_bar();
+    __syncthreads();
+    return true;
+  }
+  __device__ int blocks_of(int l) const { return l >= a.solo_from ? 1 : (int)gridDim.x; }
   __device__ void count(long long b) {
     if (blockIdx.x == 0 && threadIdx.x == 0) bytes += b;
   }
@@ -188,15 +196,16 @@ struct CoarseCycle {
   __device__ T* rs_() const { return reinterpret_cast<T*>(smem_cc + rs_off); }
   __device__ double* ps() const { return reinterpret_cast<double*>(smem_cc + a.sm_ps); }
 
-  // first cell of block b on a level of C cells
-  __device__ static int first_cell(int C, int b) { return (int)(((long long)C * b) / gridDim.x); }
+  // first of C cells of block b out of n
+  __device__ static int first_cell(int C, int b, int n) { return (int)(((long long)C * b) / n); }
 
   __device__ void enter(int l) {
     lev = l;
+    nblk = blocks_of(l);
     const CoarseLevel& C = L(l);
     const int cells = C.N / NP;
-    K0 = first_cell(cells, blockIdx.x);
-    nc = first_cell(cells, blockIdx.x + 1) - K0;
+    K0 = first_cell(cells, blockIdx.x, nblk);
+    nc = first_cell(cells, blockIdx.x + 1, nblk) - K0;
     rows = nc * NP;
     row0 = K0 * NP;
     // threads per row: 8, 4, 2 or 1, as many as the block has
@@ -209,19 +218,19 @@ struct CoarseCycle {
       lrow = threadIdx.x - part * rows;
     }
     rs_off = C.sm_r;
-    gm = C.sm_gm >= 0 ? reinterpret_cast<double*>(smem_cc + C.sm_gm) : C.coef + (size_t)blockIdx.x * C.coef_len;
+    gm = C.sm_gm >= 0 ? reinterpret_cast<double*>(smem_cc + C.sm_gm) : C.coef;
     al = gm + C.lcap;
     R = al + C.lcap;
     // slab buffer: [own cells with one more on each side | -y | +y | -z | +z]; one block owns all
     // cells, and its own slab, with the largest stride of zeros on each side, serves every slot
-    const int pad = gridDim.x == 1 ? (DIM == 2 ? C.n[0] : C.n[0] * C.n[1]) : 1;
+    const int pad = nblk == 1 ? (DIM == 2 ? C.n[0] : C.n[0] * C.n[1]) : 1;
     own0 = pad * NP;
     __syncthreads();
     if (threadIdx.x < S) {
       const int s = threadIdx.x, k = (s - 1) / 2, side = (s - 1) & 1;
       const int st = k == 0 ? 1 : k == 1 ? C.n[0] : C.n[0] * C.n[1];
       nbs[s] = s == 0 ? pad
-               : (k == 0 || gridDim.x == 1) ? pad + (side ? st : -st)
+               : (k == 0 || nblk == 1) ? pad + (side ? st : -st)
                                             : (nc + 2) + (2 * (k - 1) + side) * nc;
     }
     __syncthreads();
@@ -238,7 +247,7 @@ struct CoarseCycle {
     constexpr int NS = 2 * DIM - 2;
     if (own)
       for (int i = threadIdx.x; i < rows; i += blockDim.x) buf[own0 + i] = ldv(z + row0 + i);
-    if (gridDim.x > 1) {
+    if (nblk > 1) {
       const int st[2] = {C.n[0] * NP, C.n[0] * C.n[1] * NP};
       for (int i = threadIdx.x; i < rows; i += blockDim.x) {
         TX v[NS];
@@ -431,7 +440,7 @@ struct CoarseCycle {
     // a warp takes 32 rows of a patch; units over blocks first, so that few patches use every SM
     constexpr int JT = (M + 31) / 32;
     const int units = (np0 + np1) * JT;
-    for (int u = blockIdx.x + gridDim.x * warp; u < units; u += gridDim.x * wpb) {
+    for (int u = blockIdx.x + nblk * warp; u < units; u += nblk * wpb) {
       const int w = u / JT, t = u - w * JT;
       if (w < np0) as_patch_rows_warp<TS, TI, NP, DIM>(C.n, 0, w, t, inv0, res, zP, prs);
       else as_patch_rows_warp<TS, TI, NP, DIM>(C.n, 1, w - np0, t, inv1, res, zP + (size_t)np0 * M, prs);
@@ -492,21 +501,21 @@ struct CoarseCycle {
   // partial[c][b] of every block b -> red_s[0..n): few columns are summed by every block, more
   // columns by one owner each (a second barrier)
   __device__ bool reduce_cols(double* pt, int n) {
-    if (gridDim.x == 1) {   // the sums are the block's own, in red_s already
+    if (nblk == 1) {   // the sums are the block's own, in red_s already
       __syncthreads();
       return true;
     }
     if (!bar()) return false;
     const int warp = threadIdx.x >> 5, ln = threadIdx.x & 31, nw = blockDim.x >> 5;
-    if (n * (int)gridDim.x <= 4096) {
+    if (n * nblk <= 4096) {
       // four columns a warp: their loads are in flight together, and the transposed sum takes
       // fewer FP64 additions than one column at a time
       for (int c0 = 4 * warp; c0 < n; c0 += 4 * nw) {
         double v[4] = {0.0, 0.0, 0.0, 0.0};
-        for (int b = ln; b < (int)gridDim.x; b += 32)
+        for (int b = ln; b < nblk; b += 32)
 #pragma unroll
           for (int k = 0; k < 4; ++k)
-            v[k] += c0 + k < n ? __ldcg(pt + (size_t)(c0 + k) * gridDim.x + b) : 0.0;
+            v[k] += c0 + k < n ? __ldcg(pt + (size_t)(c0 + k) * nblk + b) : 0.0;
         int k;
         const double t = warp_sum_t<4>(v, ln, k);
         if ((ln & 7) == 0 && c0 + k < n) red_s[c0 + k] = t;
@@ -514,9 +523,9 @@ struct CoarseCycle {
       __syncthreads();
       return true;
     }
-    for (int c = blockIdx.x + gridDim.x * warp; c < n; c += gridDim.x * nw) {
+    for (int c = blockIdx.x + nblk * warp; c < n; c += nblk * nw) {
       double v = 0.0;
-      for (int b = ln; b < (int)gridDim.x; b += 32) v += __ldcg(pt + (size_t)c * gridDim.x + b);
+      for (int b = ln; b < nblk; b += 32) v += __ldcg(pt + (size_t)c * nblk + b);
 #pragma unroll
       for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
       if (ln == 0) a.red[c] = v;
@@ -527,6 +536,7 @@ struct CoarseCycle {
     return true;
   }
   __device__ double* next_partial() {
+    if (nblk == 1) return nullptr;   // alone: no partial sums, and the others' count must not differ
     double* pt = a.partial + (size_t)(rcount & 1) * a.partial_stride;
     rcount++;
     return pt;
@@ -558,8 +568,8 @@ struct CoarseCycle {
 #pragma unroll
       for (int o = LPC / 2; o; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
       if (lc == 0 && c < n) {
-        if (gridDim.x == 1) red_s[c] = d;
-        else pt[(size_t)c * gridDim.x + blockIdx.x] = d;
+        if (nblk == 1) red_s[c] = d;
+        else pt[(size_t)c * nblk + blockIdx.x] = d;
       }
     }
   }
@@ -597,28 +607,32 @@ struct CoarseCycle {
     __syncthreads();
   }
 
+  // whether this block keeps the level's coefficients: every block in shared memory, block 0 where
+  // a long basis puts them in global memory (read by all after a barrier)
+  __device__ bool own_coef() const { return L(lev).sm_gm >= 0 || blockIdx.x == 0; }
+
   // ---------------------------------------------------------------- Alg. 1
-  // with the correction z: own rows in zsV(), all rows in C.z; returns false on a barrier error
-  __device__ bool rm(LvScal& sc) {
+  // with the correction zg: own rows in zsV(), all rows in zg; returns false on a barrier error
+  __device__ bool rm(LvScal& sc, const T* zg) {
     const CoarseLevel& C = L(lev);
     const int N = C.N, l = sc.l;
     T* W = vec(C.W);
     T* w = ws();
     const T* zown = zsV() + own0;
     T* rs = rs_();
-    load_slabs<T>(vec(C.z), zsV(), false);
+    load_slabs<T>(zg, zsV(), false);
     for_rows<T, 0>(C.A, zsV(), [&](int lr, T v) { w[lr] = v; });
     count(opbytes(C, S, sizeof(T)) + (long long)N * sizeof(T) * 2 + (long long)(l + 1) * N * sizeof(T));
     if (!dots(W, N, l)) return false;
     ph(PH_RM_GRAM1);
     // w_hat = w - W W^T w: its norm by Pythagoras; another pass whenever that cancelled
     // more than half of it (classical Gram-Schmidt, "twice is enough")
-    double* Rc = R + l * (l - 1) / 2;
+    double* Rc = R + (size_t)l * (l - 1) / 2;
     for (int pass = 0;; ++pass) {
       judge(l, pass);
       for (int i = threadIdx.x; i < l; i += blockDim.x) {
         cf[i] = red_s[i];
-        Rc[i] = pass == 0 ? red_s[i] : Rc[i] + red_s[i];
+        if (own_coef()) Rc[i] = pass == 0 ? red_s[i] : Rc[i] + red_s[i];
       }
       __syncthreads();
       if (pass == 0 && sc.first) {
@@ -645,7 +659,7 @@ struct CoarseCycle {
       Zl[lr] = zown[lr];
       rs[lr] = fma(-al_t, wv, rs[lr]);
     });
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && own_coef()) {
       gm[l] = rms->gam;
       al[l] = rms->alp;
     }
@@ -697,26 +711,33 @@ struct CoarseCycle {
     double v[1] = {s};
     __syncthreads();
     bsum_n<1>(v, sh);
-    if (threadIdx.x == 0) (gridDim.x == 1 ? red_s : pt)[blockIdx.x] = v[0];
+    if (threadIdx.x == 0) *(nblk == 1 ? red_s : pt + blockIdx.x) = v[0];
     if (!reduce_cols(pt, 1)) return false;
     sc.r2 = red_s[0];
     return true;
   }
 
   // x += sum_k y_k z_k over the level's corrections, with R y = alpha (back substitution by one
-  // warp of every block)
-  __device__ void update_x(const LvScal& sc) {
+  // warp of every block); returns false on a barrier error
+  __device__ bool update_x(const LvScal& sc) {
     const CoarseLevel& C = L(lev);
     const int l = sc.l, N = C.N;
+    if (C.sm_gm < 0 && !bar()) return false;
     __syncthreads();
     if (threadIdx.x < 32) {
-      for (int i = threadIdx.x; i < l; i += 32) cf[i] = al[i];
+      // coefficients in global memory are another block's: read through L2
+      const bool far = C.sm_gm < 0;
+      auto get = [&](const double* q) { return far ? __ldcg(q) : *q; };
+      for (int i = threadIdx.x; i < l; i += 32) cf[i] = get(al + i);
       __syncwarp();
+      double g = l > 0 ? get(gm + l - 1) : 0.0;
       for (int k = l - 1; k >= 0; --k) {
-        const double y = cf[k] * gm[k];
+        const double y = cf[k] * g;
+        if (k > 0) g = get(gm + k - 1);
         __syncwarp();
-        const double* Rk = R + k * (k - 1) / 2;
-        for (int i = threadIdx.x; i < k; i += 32) cf[i] = fma(-Rk[i], y, cf[i]);
+        const double* Rk = R + (size_t)k * (k - 1) / 2;
+#pragma unroll 4
+        for (int i = threadIdx.x; i < k; i += 32) cf[i] = fma(-get(Rk + i), y, cf[i]);
         if (threadIdx.x == 0) cf[k] = y;
         __syncwarp();
       }
@@ -734,6 +755,7 @@ struct CoarseCycle {
       x[row0 + lr] = ldv(x + row0 + lr) + ((s[0] + s[1]) + (s[2] + s[3]));
     }
     count((long long)(l + 2) * N * sizeof(T));
+    return true;
   }
 
   // ---------------------------------------------------------------- transfers
@@ -743,7 +765,8 @@ struct CoarseCycle {
     const CoarseLevel &F = L(lev), &C = L(lev + 1);
     count((long long)F.N * sizeof(T) + (long long)C.N * sizeof(T) * (start ? 3 : 1));
     const int cells = C.N / NP;
-    const int J0 = first_cell(cells, blockIdx.x), nJ = first_cell(cells, blockIdx.x + 1) - J0;
+    const int nb = blocks_of(lev + 1);
+    const int J0 = first_cell(cells, blockIdx.x, nb), nJ = first_cell(cells, blockIdx.x + 1, nb) - J0;
     const T* rf = vec(F.r);
     T* stage = zsV();   // children of the own coarse cells: [cell][child][NP]
     for (int i = threadIdx.x; i < nJ * NCH * NP; i += blockDim.x) {
@@ -775,12 +798,11 @@ struct CoarseCycle {
     __syncthreads();
   }
 
-  // z = P x_{lev + 1} on the own rows: zsV() and C.z
-  __device__ void prolong() {
+  // z = P x_{lev + 1} on the own rows: zsV() and zf
+  __device__ void prolong(T* zf) {
     const CoarseLevel &F = L(lev), &C = L(lev + 1);
     count((long long)F.N * sizeof(T) + (long long)C.N * sizeof(T));
     const T* xc = vec(C.x);
-    T* zf = vec(F.z);
     T* own = zsV() + own0;
     for (int lr = threadIdx.x; lr < rows; lr += blockDim.x) {
       const int K = K0 + lr / NP, q = lr % NP;
@@ -805,7 +827,7 @@ struct CoarseCycle {
     const T* bc = vec(C.b);
     T* xc = vec(C.x);
     const int nw = blockDim.x >> 5, warp = threadIdx.x >> 5, ln = threadIdx.x & 31;
-    for (int row = blockIdx.x + gridDim.x * warp; row < a.Nc; row += gridDim.x * nw) {
+    for (int row = blockIdx.x + nblk * warp; row < a.Nc; row += nblk * nw) {
       double s[4] = {0.0, 0.0, 0.0, 0.0};
       const double* Ar = a.Ainv + (size_t)row * a.Nc;
       int j = ln;
@@ -845,7 +867,13 @@ struct CoarseCycle {
   // per-level state (the levels form a chain, so a phase per level suffices).  On entry b, r = b
   // and x = 0 of level lev0 are set, r also in shared memory.  ||b|| comes with the first
   // reduction of a visit.
-  enum Phase { PRE, CORRECT, POST };   // the residual minimisation that comes next on the level
+  // Level 0 is part of the kernel when the whole hierarchy is small (a.lev0 == 0): its loop, its
+  // tolerance and iteration cap, the history, restarts on a compensated residual and the
+  // breakdown count follow the per-step kernels (EPI_* in epilogue.cuh); its tolerance and
+  // ||r0|| are set by the residual kernel before the launch.  Alg. AsyncMG's cycle runs its coarse path
+  // first: it reads only the cycle-start residual, so the iterates are those of the concurrent
+  // form.
+  enum Phase { PRE, CORRECT, POST, STEP };   // what comes next on the level
 
   __device__ static void start(LvScal& sc, double rtol) {
     sc.l = 0;
@@ -855,90 +883,195 @@ struct CoarseCycle {
     sc.eps2 = 0.0;
   }
 
+  // level 0's scalars of Alg. 1 and 2 beside LvScal (identical in every block)
+  struct Top { int status, breakdowns, hist_len, bodies, steps; };
+  __device__ void record(Top& t, double r2, int type) {
+    const LevelState* st = L(0).st;
+    if (t.hist_len >= st->hist_cap || !a.hist) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      a.hist[t.hist_len] = sqrt(r2);
+      a.hist_type[t.hist_len] = type;
+    }
+    ++t.hist_len;
+  }
+
+  // r = b - A x on the level (compensated on an FP64 finest level), its norm, empty basis
+  __device__ bool restart(LvScal& s) {
+    const CoarseLevel& C = L(lev);
+    if (!update_x(s) || !bar()) return false;
+    load_slabs<T>(vec(C.x), zsV(), true);
+    const T* b = vec(C.b);
+    if constexpr (sizeof(T) == 8) {
+      if (lev == 0) {
+        for (int lr = threadIdx.x; lr < rows; lr += blockDim.x) rs_()[lr] = row_residual_dd(lr, ldv(b + row0 + lr));
+        __syncthreads();
+      }
+    }
+    if (sizeof(T) != 8 || lev > 0)
+      for_rows<T, 0>(C.A, zsV(), [&](int lr, T v) { rs_()[lr] = ldv(b + row0 + lr) - v; });
+    count(opbytes(C, S, sizeof(T)) + (long long)C.N * sizeof(T) * 3);
+    s.l = 0;
+    return residual_norm(s);
+  }
+  // b - A x of own row lr with products and sums in double-double, rounded once; a missing
+  // neighbour's block is not applied (the finest level's blocks are the caller's)
+  __device__ double row_residual_dd(int lr, double bv) const {
+    const CoarseLevel& C = L(lev);
+    const int c = lr / NP, K = K0 + c, row = row0 + lr, g = row >> 5, lane = row & 31;
+    const double2* Ap = reinterpret_cast<const double2*>(C.A) + (size_t)g * JP * 32 + lane;
+    const double* x = reinterpret_cast<const double*>(smem_cc + a.sm_zv);
+    double hi = 0.0, lo = 0.0;
+    for (int s = 0; s < S; ++s) {
+      if (s > 0 && __ldg(C.nbr + (size_t)K * (S - 1) + s - 1) < 0) continue;
+      const double* xp = x + (nbs[s] + c) * NP;
+      for (int j = 0; j < NP; ++j) {
+        const double2 a2 = __ldg(Ap + ((size_t)s * C.G * JP + j / 2) * 32);
+        const double av = (j & 1) ? a2.y : a2.x, p = av * xp[j], pe = fma(av, xp[j], -p);
+        const double sm = hi + p, bb = sm - hi;
+        lo += ((hi - (sm - bb)) + (p - bb)) + pe;
+        hi = sm;
+      }
+    }
+    const double t = bv - hi, bb = t - bv;
+    return t + (((bv - (t - bb)) + (-hi - bb)) - lo);
+  }
+
   __device__ void run(int lev0) {
     LvScal sc[KCMG_MAX_LEVELS];
     int phase[KCMG_MAX_LEVELS];
     int restarts[KCMG_MAX_LEVELS];
     int guard[KCMG_MAX_LEVELS];
     for (int i = 0; i < KCMG_MAX_LEVELS; ++i) { phase[i] = PRE; restarts[i] = 0; guard[i] = 0; }
-    enter(lev0);
+    Top top{KCMG_OK, 0, 0, 0, 0};
     mark(lev);
     ph(PH_CONTROL);
-    start(sc[lev], L(lev).rtol);
+    start(sc[lev], lev0 == 0 ? 0.0 : L(lev).rtol);
+    int maxit0 = 0;
+    if (lev0 == 0) {
+      const LevelState* st = L(0).st;
+      sc[0].first = 0;
+      sc[0].r2 = st->rnorm * st->rnorm;
+      sc[0].eps2 = st->eps * st->eps;
+      top.status = st->status;
+      top.hist_len = st->hist_len;
+      maxit0 = st->maxit;
+    }
     // one smoother call or prolongation and one residual minimisation per pass
     while (ok) {
       const CoarseLevel& C = L(lev);
       LvScal& s = sc[lev];
+      const bool top0 = lev == 0, async = top0 && a.async_smooth > 0;
+      const T* z = vec(C.z);
+      bool minimise = true;
       if (phase[lev] == CORRECT) {
-        prolong();                                                 // z = P z_c
+        prolong(async ? vec(a.zc) : vec(C.z));                     // z = P z_c
         if (!(ok = bar())) break;
         ph(PH_TRANSFER);
+        if (async) {
+          phase[lev] = STEP;
+          top.steps = 0;
+          continue;
+        }
+      } else if (phase[lev] == STEP && top.steps == a.async_smooth) {
+        z = vec(a.zc);                                             // the coarse correction closes the cycle
+        for (int i = threadIdx.x; i < rows; i += blockDim.x) zsV()[own0 + i] = ldv(z + row0 + i);
       } else {
         // while ||r|| > eps (level-local criteria of Sec. 4.2)
-        if (phase[lev] == PRE && !(s.r2 > s.eps2 && s.it < C.maxit && guard[lev] < (1 << 24))) {
-          if (blockIdx.x == 0 && threadIdx.x == 0 && C.st) {
+        if (phase[lev] == PRE &&
+            !(s.r2 > s.eps2 && s.it < (top0 ? maxit0 : C.maxit) && guard[lev] < (1 << 24) &&
+              (!top0 || top.status == KCMG_OK))) {
+          if (!top0 && blockIdx.x == 0 && threadIdx.x == 0 && C.st) {
             C.st->iters_total += s.it;
             C.st->nrestart += restarts[lev];
           }
-          restarts[lev] = 0;
-          update_x(s);
+          if (!(ok = update_x(s))) break;
           mark(lev);
           if (lev == lev0) break;
-          if (!(ok = bar())) break;                                // x complete everywhere
+          restarts[lev] = 0;
+          // x complete everywhere: the caller's blocks, of which only this one may have been here
+          if (!(ok = blocks_of(lev - 1) > 1 ? grid_bar() : bar())) break;
           ph(PH_CONTROL);
           enter(lev - 1);                                          // return to the caller
           continue;
         }
-        smooth();                                                  // pre- or post-smoother
+        if (phase[lev] == PRE && async) minimise = false;          // the coarse path comes first
+        else smooth();                                             // pre- or post-smoother
         if (!ok) break;
       }
-      if (!(ok = rm(s))) break;
+      if (minimise) {
+        const int l0 = s.l;
+        if (!(ok = rm(s, z))) break;
+        if (top0) {
+          if (s.l > l0) {
+            top.breakdowns = 0;
+          } else {
+            if (!isfinite(rms->naz2) && top.status == KCMG_OK) top.status = KCMG_NONFINITE;
+            if (++top.breakdowns >= 2 && top.status == KCMG_OK) top.status = KCMG_BREAKDOWN;
+          }
+          if (!isfinite(s.r2) && top.status == KCMG_OK) top.status = KCMG_NONFINITE;
+          record(top, s.r2, phase[0] == CORRECT || z != vec(C.z) ? 2 : phase[0] == POST ? 3 : 1);
+        }
+      }
       if (phase[lev] == PRE) {
         ++guard[lev];
-        if (s.it == 0 && s.l == 0 && !(s.r2 > 0.0)) {              // b = 0 (or not finite): x = 0
+        if (!top0 && s.it == 0 && s.l == 0 && !(s.r2 > 0.0)) {     // b = 0 (or not finite): x = 0
           s.r2 = 0.0;
           continue;
         }
         T* rg = vec(C.r);
         for (int lr = threadIdx.x; lr < rows; lr += blockDim.x) rg[row0 + lr] = rs_()[lr];
         if (!(ok = bar())) break;                                  // r complete everywhere
-        const bool direct = (lev + 1 == a.nlev - 1);
-        restrict_(!direct);                                        // r_c = R r
         phase[lev] = CORRECT;
-        if (direct) {
+        const bool direct = (lev + 1 == a.nlev - 1), alone = blocks_of(lev + 1) < nblk;
+        if (!alone || blockIdx.x == 0) restrict_(!direct);         // r_c = R r
+        ph(PH_TRANSFER);
+        mark(lev);
+        if (alone && blockIdx.x != 0) {                            // block 0 solves the rest
+          if (!(ok = grid_bar())) break;
+        } else if (direct) {
+          const int nb = nblk;
+          nblk = blocks_of(lev + 1);
           if (!(ok = bar())) break;
-          ph(PH_TRANSFER);
-          mark(lev);
           coarse_solve(lev + 1);                                   // z_c = A_c \ r_c
+          nblk = nb;
           if (!(ok = bar())) break;
           ph(PH_COARSEST);
           mark(lev + 1);
         } else {
-          ph(PH_TRANSFER);
-          mark(lev);
           enter(lev + 1);                                          // z_c = MG(A_c, r_c, 0)
           start(sc[lev], L(lev).rtol);
           phase[lev] = PRE;
         }
       } else if (phase[lev] == CORRECT) {
         phase[lev] = POST;
+      } else if (phase[lev] == STEP && top.steps < a.async_smooth) {
+        ++top.steps;
       } else {
         s.it++;
-        const int cap = (a.lmax > 0 && a.lmax < C.lcap) ? a.lmax : C.lcap;
-        if (s.l + 3 > cap) {                                       // restart: r = b - A x
-          update_x(s);
-          if (!(ok = bar())) break;
-          load_slabs<T>(vec(C.x), zsV(), true);
-          const T* b = vec(C.b);
-          for_rows<T, 0>(C.A, zsV(), [&](int lr, T v) { rs_()[lr] = ldv(b + row0 + lr) - v; });
-          count(opbytes(C, S, sizeof(T)) + (long long)C.N * sizeof(T) * 3);
-          s.l = 0;
-          if (!(ok = residual_norm(s))) break;
+        const int cap = (a.lmax > 0 && a.lmax < C.lcap) ? a.lmax : C.lcap, per = async ? a.async_smooth + 1 : 3;
+        const bool converged = top0 && !(s.r2 > s.eps2) && s.l > 0;
+        if (s.l + per > cap || converged) {                        // restart: r = b - A x
+          if (!(ok = restart(s))) break;
           ph(PH_RESTART);
           ++restarts[lev];
+          if (top0) {
+            if (!isfinite(s.r2) && top.status == KCMG_OK) top.status = KCMG_NONFINITE;
+            record(top, s.r2, 4);
+          }
         }
         phase[lev] = PRE;
       }
+    }
+    if (lev0 == 0 && ok && blockIdx.x == 0 && threadIdx.x == 0) {
+      LevelState* st = L(0).st;
+      st->it = sc[0].it;
+      st->iters_total += sc[0].it;
+      st->l = sc[0].l;
+      st->rnorm = sqrt(sc[0].r2);
+      st->nrestart += restarts[0];
+      st->status = top.status;
+      st->breakdowns = top.breakdowns;
+      st->hist_len = top.hist_len;
     }
   }
 };
@@ -950,8 +1083,8 @@ template <typename TV, typename TS, typename TI, int NP, int DIM>
 __global__ void __launch_bounds__(512) k_coarse_cycle(const __grid_constant__ CoarseArgs a) {
   using T = TV;
   __shared__ double sh[32 * 8];
-  __shared__ double red_s[kCoarseMaxCols + 4];
-  __shared__ double cf[kCoarseMaxCols];
+  double* red_s = reinterpret_cast<double*>(smem_cc + a.sm_red);   // cols + 4 sums
+  double* cf = red_s + a.cols + 4;                                  // cols coefficients
   __shared__ RmScal rms;
   __shared__ int nbs[2 * DIM + 1];
   __shared__ long long tph[kCoarsePhases + KCMG_MAX_LEVELS];
@@ -967,15 +1100,20 @@ __global__ void __launch_bounds__(512) k_coarse_cycle(const __grid_constant__ Co
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
     c0 = clock64();
   }
-  // start of MG on the first coarse level: b, r, x were set by the restriction kernel
-  cc.enter(a.lev0);
-  for (int lr = threadIdx.x; lr < cc.rows; lr += blockDim.x)
-    cc.rs_()[lr] = ldv(static_cast<const T*>(a.lv[a.lev0].b) + cc.row0 + lr);
-  __syncthreads();
-  cc.count((long long)a.lv[a.lev0].N * sizeof(T));
-  cc.run(a.lev0);
+  // start of MG on the first level: on a coarse level r = b, set by the restriction kernel with
+  // x = 0; on level 0 r = b - A x0 by the residual kernel.  Blocks without a part in the first
+  // level go to the end.
+  if (blockIdx.x < cc.blocks_of(a.lev0)) {
+    cc.enter(a.lev0);
+    const CoarseLevel& C = a.lv[a.lev0];
+    for (int lr = threadIdx.x; lr < cc.rows; lr += blockDim.x)
+      cc.rs_()[lr] = ldv(static_cast<const T*>(a.lev0 == 0 ? C.r : C.b) + cc.row0 + lr);
+    __syncthreads();
+    cc.count((long long)C.N * sizeof(T));
+    cc.run(a.lev0);
+  }
   // device time of this launch: every block has passed the last barrier of the cycle
-  if (cc.ok) cc.ok = cc.bar();
+  if (cc.ok) cc.ok = cc.grid_bar();
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     unsigned long long t1;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));

@@ -26,15 +26,27 @@ static void* coarse_kernel_ptr(int np, int dim) {
   return f;
 }
 
-// Blocks for a hierarchy whose largest level here has N unknowns in cells of np.  One block needs
-// no grid barrier (about 1 us a phase with every SM taking part) but has one SM's FP64 FMA rate,
-// two per clock: it wins while a sweep's FMAs take it less than that.  Otherwise one block per SM,
-// and no more blocks than cells.
+// FMAs of one operator application on a level
+static long long cc_fmas(const CoarseArgs& a, int l) {
+  return (long long)a.lv[l].N * (2 * a.dim + 1) * a.np;
+}
+// One block needs no grid barrier (about 1 us a phase with every SM taking part) but has one SM's
+// FP64 FMA rate, two per clock: it wins while a sweep's FMAs take it less than that.  The same
+// for the dense coarsest solve, which belongs to the block that runs the levels above it.
+constexpr long long kCoarseSoloFmas = 6000, kCoarseSoloCoarsest = 12000;
+
+// first level that block 0 runs alone: every level from there on, the coarsest included, is small
+static int cc_solo_from(const CoarseArgs& a) {
+  if ((long long)a.Nc * a.Nc > kCoarseSoloCoarsest) return a.nlev;
+  int from = a.nlev - 1;
+  while (from > a.lev0 && cc_fmas(a, from - 1) <= kCoarseSoloFmas) --from;
+  return from < a.nlev - 1 ? from : a.nlev;
+}
+
+// blocks: one per SM and no more than the largest level's cells; one if that runs alone
 static int cc_blocks(const CoarseArgs& a, int nsm) {
-  const CoarseLevel& L = a.lv[a.lev0];
-  const long long fmas = (long long)L.N * (2 * a.dim + 1) * a.np;
-  if (fmas <= 6000) return 1;
-  const int cells = L.N / a.np;
+  if (a.solo_from <= a.lev0) return 1;
+  const int cells = a.lv[a.lev0].N / a.np;
   return cells < nsm ? cells : nsm;
 }
 
@@ -52,24 +64,28 @@ static void coarse_cycle_layout(CoarseArgs* a, int grid) {
   const int nch = 1 << a->dim, segs = 2 * a->dim - 2;
   take((size_t)nch * a->np * a->np * sizeof(CC_TV));   // prolongation matrices
   size_t slab = 0, rows_max = 0;
+  a->cols = 1;
   for (int l = a->lev0; l < a->nlev; ++l) {
     CoarseLevel& L = a->lv[l];
-    const int cells = L.N / a->np, own = (cells + grid - 1) / grid;
+    const int parts = l >= a->solo_from ? 1 : grid;
+    const int cells = L.N / a->np, own = (cells + parts - 1) / parts;
     const size_t rows = (size_t)own * a->np;
     if (l > a->lev0) slab = std::max(slab, rows * nch);                   // children of the own cells
     if (l == a->nlev - 1) break;
     const int pad = a->dim == 2 ? L.n[0] : L.n[0] * L.n[1];   // one block: zeros on both sides
-    slab = std::max(slab, (size_t)(grid > 1 ? own + 2 + segs * own : own + 2 * pad) * a->np);
+    slab = std::max(slab, (size_t)(parts > 1 ? own + 2 + segs * own : own + 2 * pad) * a->np);
     rows_max = std::max(rows_max, rows);
+    a->cols = std::max(a->cols, L.lcap);
     L.sm_r = take(rows * sizeof(CC_TV));
-    L.coef_len = 2 * L.lcap + L.lcap * (L.lcap - 1) / 2;
-    L.sm_gm = L.lcap <= kCoarseCoefMax ? take((size_t)L.coef_len * sizeof(double)) : -1;
+    L.coef_len = 2 * (size_t)L.lcap + (size_t)L.lcap * (L.lcap - 1) / 2;
+    L.sm_gm = L.lcap <= kCoarseCoefMax ? take(L.coef_len * sizeof(double)) : -1;
   }
   a->sm_zv = take(slab * sizeof(CC_TV));
   a->sm_zs = sizeof(CC_TV) == sizeof(CC_T) ? a->sm_zv : take(slab * sizeof(CC_T));
   a->sm_ts = take(rows_max * sizeof(CC_T));
   a->sm_ws = take(rows_max * sizeof(CC_TV));
   a->sm_ps = take((size_t)kCoarseThreads * sizeof(double));
+  a->sm_red = take((size_t)(2 * a->cols + 4) * sizeof(double));
   a->sm_as = a->smoother == 1 ? take((size_t)(kCoarseThreads / 32) * nch * a->np * sizeof(CC_T)) : 0;
   a->sm_bytes = top;
 }
@@ -82,6 +98,7 @@ cudaError_t coarse_cycle_prepare<CC_TV, CC_T, CC_TI>(CoarseArgs* a, int* grid) {
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  a->solo_from = cc_solo_from(*a);
   int g = cc_blocks(*a, nsm);
   if (*grid > 0 && *grid < g) g = *grid;   // the caller's cap
   coarse_cycle_layout(a, g);

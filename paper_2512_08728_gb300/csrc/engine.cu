@@ -83,6 +83,7 @@ struct kcmg_ctx {
   // persistent coarse cycle (levels >= 1 in one cooperative launch per level-0 cycle)
   bool coarse_kernel = false;
   int cc_lev0 = 0;   // first level run by the persistent kernel
+  bool whole = false;   // it runs the whole solve, level 0 included
   int cc_grid = 0;
   CoarseArgs cc{};
   long long graph_body_launches = 0;  // kernels per level-0 loop body of the graph
@@ -204,6 +205,13 @@ void setup_level_geometry(kcmg_ctx* ctx, Level& L, int l) {
   launch_build_nbr(ctx->dim, L.n, L.nbr, ctx->s);
 }
 
+// basis capacity of a coarse level: 3 stored corrections a cycle, and the restart length
+int coarse_capacity(const kcmg_params& p, int l) {
+  int cap = 3 * (p.lvl_maxit[l] > 0 ? p.lvl_maxit[l] : 1) + 3;
+  if (p.lmax > 0 && p.lmax + 3 < cap) cap = p.lmax + 3;
+  return cap;
+}
+
 template <typename T>
 void alloc_cycle_vectors(kcmg_ctx* ctx, Level& L, int lcap) {
   const size_t N = L.N;
@@ -227,6 +235,28 @@ void alloc_cycle_vectors(kcmg_ctx* ctx, Level& L, int lcap) {
   L.partial = dalloc<double>(ctx, plen);
   L.st = dalloc<LevelState>(ctx, 1);
   CK(cudaMemsetAsync(L.st, 0, sizeof(LevelState), ctx->s));
+}
+
+// Whether the persistent kernel runs the whole solve.  A step of the finest level is then a phase
+// of it (a grid barrier and an L2 round trip, 3 us, plus the dense FMAs) in place of a kernel in
+// the graph (6 us and up on small problems, with the loop's own nodes); from about kWholeFmas FMAs
+// an application the phase's FP64 time makes up the difference, and the finest level's own
+// kernels skip the zeros of its blocks.  Measured, per-step finest level against whole solve:
+// 16 x 16, p = 1, to 1e-11 20.4 / 13.5 ms; 8^3, p = 2, mixed, to 1e-11 28.3 / 23.1 ms; three
+// cycles at 0.8M FMAs (12 x 12 x 8, p = 2) 5.24 / 5.03 ms, at 1.1M (20 x 20 x 24, p = 1) 2.39 / 2.25.
+// The task-parallel cycle's smoother steps run beside the coarse levels' kernel where there is
+// one, which hides them (16^3, p = 1, three levels, m = 8: 2.25 / 2.66 ms); with two levels there
+// is none (8^3, p = 1: 1.89 / 1.01).
+constexpr long long kWholeFmas = 1200000;
+bool whole_solve(const kcmg_ctx* ctx) {
+  const kcmg_params& p = ctx->p;
+  if (!p.coarse_persistent || p.mf_nu || p.mf_F || getenv("KCMG_PERSISTENT_ROWS")) return false;
+  if (p.async_smooth > 0 && ctx->nlev > 2) return false;
+  long long cells = 1;
+  for (int j = 0; j < ctx->dim; ++j) cells *= p.n[j];
+  for (int l = 1; l < ctx->nlev - 1; ++l)   // longer bases than the kernel keeps on the coarse levels
+    if (coarse_capacity(p, l) + 1 > kCoarseMaxCols) return false;
+  return cells * ctx->np * ctx->np * ctx->S <= kWholeFmas;
 }
 
 // The finest level's blocks and inverses (natural layout) in the pattern kernels' storage, if
@@ -293,23 +323,24 @@ void build_hierarchy(kcmg_ctx* ctx, const double* blocks_src) {
     const size_t invsz = (size_t)L.G * ((np + 1) / 2) * 64;
     const bool bf16 = ctx->p.precision == KCMG_MIXED_BF16INV || ctx->p.precision == KCMG_IR32_BF16INV;
     if (l == 0) store_pattern(ctx, L, inv_nat, bf16);
-    if (!L.pat) {
+    const bool dense = !L.pat || ctx->whole;   // the persistent kernel reads this layout
+    if (dense) {
       L.A64 = dalloc<double>(ctx, opsz);
       L.D64 = dalloc<double>(ctx, invsz);
-      launch_interleave<double>(np, S, L.nat, L.ncell, L.G, L.A64, ctx->s);
-      launch_interleave<double>(np, 1, inv_nat, L.ncell, L.G, L.D64, ctx->s);
+      launch_interleave<double>(np, S, L.nat, L.nbr, L.ncell, L.G, L.A64, ctx->s);
+      launch_interleave<double>(np, 1, inv_nat, nullptr, L.ncell, L.G, L.D64, ctx->s);
     }
-    if (ctx->mixed && !L.pat) {
+    if (ctx->mixed && dense) {
       L.A32 = dalloc<float>(ctx, opsz);
-      launch_interleave<float>(np, S, L.nat, L.ncell, L.G, L.A32, ctx->s);
+      launch_interleave<float>(np, S, L.nat, L.nbr, L.ncell, L.G, L.A32, ctx->s);
     }
-    if (ctx->mixed && (!L.pat || ctx->p.mf_nu)) {   // the matrix-free sweeps read this layout
+    if (ctx->mixed && (dense || ctx->p.mf_nu)) {   // the matrix-free sweeps read this layout
       if (bf16) {
         L.D16 = dalloc<__nv_bfloat16>(ctx, invsz);
-        launch_interleave<__nv_bfloat16>(np, 1, inv_nat, L.ncell, L.G, L.D16, ctx->s);
+        launch_interleave<__nv_bfloat16>(np, 1, inv_nat, nullptr, L.ncell, L.G, L.D16, ctx->s);
       } else {
         L.D32 = dalloc<float>(ctx, invsz);
-        launch_interleave<float>(np, 1, inv_nat, L.ncell, L.G, L.D32, ctx->s);
+        launch_interleave<float>(np, 1, inv_nat, nullptr, L.ncell, L.G, L.D32, ctx->s);
       }
     }
     CK(cudaGetLastError());
@@ -734,7 +765,6 @@ struct Cycle {
   // level 0: r0 = b - A x0 (compensated FP64; FP32 in the inner solve of the
   // iterative-refinement forms), then the level-0 loop
   void run(cudaStream_t s) {
-    Level& L = ctx->lv[0];
     if (capture) {
       cudaGraph_t g;
       cudaStreamCaptureStatus cs;
@@ -745,13 +775,18 @@ struct Cycle {
       CK(cudaStreamGetCaptureInfo(s, &cs, &id, &g, &deps, &ed, &nd));
       CK(cudaGraphConditionalHandleCreate(&handle[0], g, 0, 0));
     }
+    initial_residual(s);
+    loop<T0>(0, s);
+  }
+
+  void initial_residual(cudaStream_t s) {
+    Level& L = ctx->lv[0];
     if (std::is_same<T0, double>::value)
       apply_residual_dd(ctx, L, static_cast<double*>(L.x), static_cast<double*>(L.r), static_cast<double*>(L.b),
                          L.partial, epi(0, EPI_MG_BEGIN), 0, s);
     else
       apply_op<T0>(ctx, L, static_cast<T0*>(L.x), static_cast<T0*>(L.r), static_cast<T0*>(L.b), L.partial,
                       epi(0, EPI_MG_BEGIN), 0, s);
-    loop<T0>(0, s);
   }
 };
 
@@ -789,7 +824,12 @@ void init_states(kcmg_ctx* ctx, double rtol0, double atol0, int maxit0) {
 
 template <typename T0, typename T>
 void run_cycle(kcmg_ctx* ctx) {
-  if (ctx->p.use_graph) {
+  if (ctx->whole) {   // the initial residual, then one kernel (nothing for a graph to save)
+    Cycle<T0, T> cy{ctx};
+    cy.initial_residual(ctx->s);
+    launch_coarse(ctx, ctx->s);
+    ctx->last_launches = 2;
+  } else if (ctx->p.use_graph) {
     if (!ctx->graph_ready) {
       Cycle<T0, T> cy{ctx};
       cy.capture = true;
@@ -1177,6 +1217,7 @@ kcmg_ctx* build_ctx(const kcmg_params* p, cudaStream_t user, const double* block
     copy_in(ctx, ctx->P64, p->prolong, ctx->nch * bs);
     ctx->P32 = dalloc<float>(ctx, ctx->nch * bs);
     launch_convert<double, float>(ctx->P64, ctx->P32, ctx->nch * bs, ctx->s);
+    ctx->whole = whole_solve(ctx);
     build_hierarchy(ctx, blocks_override ? blocks_override : p->blocks);
     if (p->mf_nu || p->mf_F) {   // matrix-free level-0 coupling for the FP32 sweeps
       REQUIRE(p->mf_nu && p->mf_F, "mf_nu and mf_F go together");
@@ -1206,8 +1247,7 @@ kcmg_ctx* build_ctx(const kcmg_params* p, cudaStream_t user, const double* block
       // the task-parallel cycle): the restart test runs at the end of a cycle
       const int per_cycle0 = std::max(3, p->async_smooth + 1);
       if (l == 0) cap = (p->lmax > 0 ? p->lmax : 512 - per_cycle0) + per_cycle0;
-      else cap = 3 * (p->lvl_maxit[l] > 0 ? p->lvl_maxit[l] : 1) + 3;
-      if (p->lmax > 0 && l > 0 && p->lmax + 3 < cap) cap = p->lmax + 3;
+      else cap = coarse_capacity(*p, l);
       if (cap > kLcapMax) cap = kLcapMax;
       // keep the level-0 basis within a third of the free device memory
       if (l == 0) {
@@ -1242,9 +1282,10 @@ kcmg_ctx* build_ctx(const kcmg_params* p, cudaStream_t user, const double* block
       for (int l = 1; l < ctx->nlev - 1; ++l)
         if (ctx->lv[l].N <= rows_max) { ctx->cc_lev0 = l; break; }
     }
-    ctx->coarse_kernel = p->coarse_persistent && ctx->cc_lev0 > 0;
+    if (ctx->whole) ctx->cc_lev0 = 0;
+    ctx->coarse_kernel = p->coarse_persistent && (ctx->cc_lev0 > 0 || ctx->whole);
     if (ctx->coarse_kernel) {
-      for (int l = ctx->cc_lev0; l < ctx->nlev - 1; ++l)
+      for (int l = std::max(1, ctx->cc_lev0); l < ctx->nlev - 1; ++l)
         REQUIRE(ctx->lv[l].lcap + 1 <= kCoarseMaxCols,
                 "level %d keeps %d basis vectors; the persistent coarse cycle supports %d",
                 l, ctx->lv[l].lcap, kCoarseMaxCols - 1);
@@ -1261,12 +1302,11 @@ kcmg_ctx* build_ctx(const kcmg_params* p, cudaStream_t user, const double* block
       a.lmax = p->lmax;
       a.brk = 1e-14;
       a.smoother = p->smoother;
-      a.red = dalloc<double>(ctx, kCoarseMaxCols + 4);
       a.bar_count = dalloc<unsigned int>(ctx, 1);
       a.bar_gen = dalloc<unsigned int>(ctx, 1);
       a.err = dalloc<int>(ctx, 1);
       CK(cudaMemsetAsync(a.bar_gen, 0, sizeof(unsigned int), ctx->s));
-      for (int l = 1; l < ctx->nlev; ++l) {
+      for (int l = ctx->whole ? 0 : 1; l < ctx->nlev; ++l) {
         Level& L = ctx->lv[l];
         CoarseLevel& c = a.lv[l];
         c.A = ctx->ir ? (const void*)L.A32 : (const void*)L.A64;      // Alg. 1 operator
@@ -1310,6 +1350,7 @@ kcmg_ctx* build_ctx(const kcmg_params* p, cudaStream_t user, const double* block
           break;
         }
         cudaGetLastError();
+        ctx->whole = false;
         if (ctx->cc_lev0 + 1 >= ctx->nlev - 1) {
           ctx->coarse_kernel = false;
           break;
@@ -1318,9 +1359,10 @@ kcmg_ctx* build_ctx(const kcmg_params* p, cudaStream_t user, const double* block
       }
       if (!ctx->coarse_kernel) grid = 1;
       for (int l = ctx->cc_lev0; l < ctx->nlev - 1; ++l)
-        if (a.lv[l].sm_gm < 0) a.lv[l].coef = dalloc<double>(ctx, (size_t)grid * a.lv[l].coef_len);
+        if (a.lv[l].sm_gm < 0) a.lv[l].coef = dalloc<double>(ctx, a.lv[l].coef_len);
       ctx->cc_grid = grid;
-      a.partial_stride = (size_t)grid * (kCoarseMaxCols + 4);
+      a.partial_stride = (size_t)grid * (a.cols + 4);
+      a.red = dalloc<double>(ctx, a.cols + 4);
       a.partial = dalloc<double>(ctx, 2 * a.partial_stride);
       ctx->stat_ns = dalloc<unsigned long long>(ctx, 1);
       ctx->stat_launches = dalloc<unsigned long long>(ctx, 1);
@@ -1350,6 +1392,10 @@ kcmg_ctx* build_ctx(const kcmg_params* p, cudaStream_t user, const double* block
     if (p->async_smooth > 0) ctx->zc = dalloc<double>(ctx, N0);
     ctx->hist = dalloc<double>(ctx, ctx->hist_cap);
     ctx->hist_type = dalloc<int>(ctx, ctx->hist_cap);
+    ctx->cc.async_smooth = p->async_smooth;
+    ctx->cc.zc = ctx->zc;
+    ctx->cc.hist = ctx->hist;
+    ctx->cc.hist_type = ctx->hist_type;
     size_t maxN = 0;
     for (auto& L : ctx->lv) maxN = maxN > (size_t)L.N ? maxN : (size_t)L.N;
     ctx->stage_in = dalloc<double>(ctx, maxN);

@@ -174,7 +174,7 @@ void launch_assemble_dense(int np, int dim, const double* blk, const int* nbr, i
                            double* M /*[n][2n]*/, cudaStream_t s);
 void launch_extract_inverse(const double* M, int n, double* Ainv, cudaStream_t s);
 template <typename T>
-void launch_interleave(int np, int nslot, const double* nat, int ncell, int G, T* out,
+void launch_interleave(int np, int nslot, const double* nat, const int* nbr, int ncell, int G, T* out,
                        cudaStream_t s);
 void launch_transpose_blocks(int np, int dim, const double* in, const int* nbr, int ncell,
                              double* out, cudaStream_t s);
@@ -186,7 +186,7 @@ void launch_grad_lognu(int np, int dim, const int* n, const double* nu, const do
                        double* g, cudaStream_t s);
 
 // ---------------------------------------------------------------- coarse cycle kernel
-constexpr int kCoarseMaxCols = 128;   // basis capacity + 1 on the coarse levels
+constexpr int kCoarseMaxCols = 128;   // basis capacity + 1 on the coarse levels (setup refuses more)
 // phase kinds timed inside the persistent coarse cycle (each includes its closing barrier)
 enum CoarsePhase : int {
   PH_SWEEP = 0,      // one block-Jacobi sweep
@@ -220,10 +220,10 @@ struct CoarseLevel {
   // a block's share in dynamic shared memory (byte offsets): residual of the own rows; gamma,
   // alpha and the packed coefficients of Alg. 1
   int sm_r, sm_gm;
-  // gamma, alpha and coefficients in global memory (coef_len doubles a block) where sm_gm < 0:
+  // gamma, alpha and coefficients in global memory (coef_len doubles, one copy) where sm_gm < 0:
   // bases so long that they do not fit
   double* coef;
-  int coef_len;
+  size_t coef_len;
 };
 
 struct CoarseArgs {
@@ -237,10 +237,18 @@ struct CoarseArgs {
   double brk;                  // breakdown threshold of Alg. 1
   // dynamic shared memory (byte offsets): iterate slabs in the vector type and in the smoother's
   // type, t, w, per-thread partial sums, gathered patch residuals; sm_bytes in all
-  int sm_zv, sm_zs, sm_ts, sm_ws, sm_ps, sm_as, sm_bytes;
+  int sm_zv, sm_zs, sm_ts, sm_ws, sm_ps, sm_as, sm_red, sm_bytes;
+  int cols;                    // longest basis of the levels here
+  int solo_from;               // first level that block 0 runs alone (nlev: none)
+  // level 0 in the kernel (lev0 == 0): smoother steps of Alg. AsyncMG (0: Alg. 2), its coarse
+  // correction, the residual history
+  int async_smooth;
+  void* zc;
+  double* hist;
+  int* hist_type;
   double* partial;             // 2 buffers of partial_stride doubles
-  size_t partial_stride;       // grid * (kCoarseMaxCols + 4)
-  double* red;                 // kCoarseMaxCols + 4 reduced sums
+  size_t partial_stride;       // grid * (cols + 4)
+  double* red;                 // cols + 4 reduced sums
   unsigned int* bar_count;     // arrivals at the grid barrier in this launch
   unsigned int* bar_gen;       // blocks that have left the kernel
   int* err;                    // set when a grid barrier timed out

@@ -753,9 +753,11 @@ __global__ void k_extract_inverse(const double* __restrict__ M, int n, double* A
   }
 }
 
-// natural [nslot][C][np][np] FP64 -> row-interleaved T
+// natural [nslot][C][np][np] FP64 -> row-interleaved T; with nbr [C][nslot - 1], blocks towards a
+// missing neighbour become zero (no kernel applies them; some need not test for them then)
 template <typename T>
-__global__ void k_interleave(int np, int nslot, const double* __restrict__ nat, int ncell, int G,
+__global__ void k_interleave(int np, int nslot, const double* __restrict__ nat, const int* __restrict__ nbr,
+                             int ncell, int G,
                              T* __restrict__ out) {
   const int JP = (np + 1) / 2;
   const size_t tot = (size_t)nslot * G * JP * 64;
@@ -771,7 +773,8 @@ __global__ void k_interleave(int np, int nslot, const double* __restrict__ nat, 
     double v = 0.0;
     if (row < ncell * np && j < np) {
       const int K = row / np, i = row % np;
-      v = nat[((size_t)s * ncell + K) * np * np + i * np + j];
+      if (s == 0 || !nbr || nbr[(size_t)K * (nslot - 1) + s - 1] >= 0)
+        v = nat[((size_t)s * ncell + K) * np * np + i * np + j];
     }
     out[idx] = (T)v;
   }
@@ -1047,10 +1050,10 @@ void launch_extract_inverse(const double* M, int n, double* Ainv, cudaStream_t s
 }
 
 template <typename T>
-void launch_interleave(int np, int nslot, const double* nat, int ncell, int G, T* out,
+void launch_interleave(int np, int nslot, const double* nat, const int* nbr, int ncell, int G, T* out,
                        cudaStream_t s) {
   const size_t tot = (size_t)nslot * G * ((np + 1) / 2) * 64;
-  k_interleave<T><<<nblocks(tot, 256, 1 << 16), 256, 0, s>>>(np, nslot, nat, ncell, G, out);
+  k_interleave<T><<<nblocks(tot, 256, 1 << 16), 256, 0, s>>>(np, nslot, nat, nbr, ncell, G, out);
 }
 
 void launch_transpose_blocks(int np, int dim, const double* in, const int* nbr, int ncell,
@@ -1094,7 +1097,7 @@ void launch_grad_lognu(int np, int dim, const int* n, const double* nu, const do
   template void launch_gram_update<T>(T*, T*, int, const T*, const T*, const T*, T*, T*, int,    \
                                       int, double*, const EpiArgs&, cudaStream_t);               \
   template void launch_norm<T>(const T*, int, int, double*, const EpiArgs&, cudaStream_t);       \
-  template void launch_interleave<T>(int, int, const double*, int, int, T*, cudaStream_t);       \
+  template void launch_interleave<T>(int, int, const double*, const int*, int, int, T*, cudaStream_t); \
   template void launch_axpy_to_double<T>(const T*, double*, size_t, cudaStream_t);
 
 KCMG_INST_T(double)
@@ -1108,7 +1111,7 @@ template void launch_bj_sweep<float, float>(int, int, const float*, const float*
 template void launch_bj_sweep<float, __nv_bfloat16>(int, int, const float*, const __nv_bfloat16*,
                                                     const int*, int, int, int, int, const float*,
                                                     const float*, float*, double, int, cudaStream_t);
-template void launch_interleave<__nv_bfloat16>(int, int, const double*, int, int, __nv_bfloat16*,
+template void launch_interleave<__nv_bfloat16>(int, int, const double*, const int*, int, int, __nv_bfloat16*,
                                                cudaStream_t);
 template void launch_restrict<float, double>(int, int, const int*, const int*, const float*,
                                              const double*, float*, float*, float*, double*,
