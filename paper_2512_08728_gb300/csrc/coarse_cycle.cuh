@@ -196,8 +196,11 @@ struct CoarseCycle {
   __device__ T* rs_() const { return reinterpret_cast<T*>(smem_cc + rs_off); }
   __device__ double* ps() const { return reinterpret_cast<double*>(smem_cc + a.sm_ps); }
 
-  // first of C cells of block b out of n
-  __device__ static int first_cell(int C, int b, int n) { return (int)(((long long)C * b) / n); }
+  // first of C cells of block b out of n; with fewer cells than blocks the first C have one each
+  __device__ static int first_cell(int C, int b, int n) {
+    n = min(n, C);
+    return b >= n ? C : (int)(((long long)C * b) / n);
+  }
 
   __device__ void enter(int l) {
     lev = l;
@@ -506,16 +509,16 @@ struct CoarseCycle {
       return true;
     }
     if (!bar()) return false;
-    const int warp = threadIdx.x >> 5, ln = threadIdx.x & 31, nw = blockDim.x >> 5;
-    if (n * nblk <= 4096) {
+    const int warp = threadIdx.x >> 5, ln = threadIdx.x & 31, nw = blockDim.x >> 5, nsum = summands();
+    if (n * nsum <= 4096) {
       // four columns a warp: their loads are in flight together, and the transposed sum takes
       // fewer FP64 additions than one column at a time
       for (int c0 = 4 * warp; c0 < n; c0 += 4 * nw) {
         double v[4] = {0.0, 0.0, 0.0, 0.0};
-        for (int b = ln; b < nblk; b += 32)
+        for (int b = ln; b < nsum; b += 32)
 #pragma unroll
           for (int k = 0; k < 4; ++k)
-            v[k] += c0 + k < n ? __ldcg(pt + (size_t)(c0 + k) * nblk + b) : 0.0;
+            v[k] += c0 + k < n ? __ldcg(pt + (size_t)(c0 + k) * nsum + b) : 0.0;
         int k;
         const double t = warp_sum_t<4>(v, ln, k);
         if ((ln & 7) == 0 && c0 + k < n) red_s[c0 + k] = t;
@@ -525,7 +528,7 @@ struct CoarseCycle {
     }
     for (int c = blockIdx.x + nblk * warp; c < n; c += nblk * nw) {
       double v = 0.0;
-      for (int b = ln; b < nblk; b += 32) v += __ldcg(pt + (size_t)c * nblk + b);
+      for (int b = ln; b < nsum; b += 32) v += __ldcg(pt + (size_t)c * nsum + b);
 #pragma unroll
       for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
       if (ln == 0) a.red[c] = v;
@@ -535,6 +538,8 @@ struct CoarseCycle {
     __syncthreads();
     return true;
   }
+  // blocks with cells of the level, the first of all: the others only keep step
+  __device__ int summands() const { return min(nblk, L(lev).N / NP); }
   __device__ double* next_partial() {
     if (nblk == 1) return nullptr;   // alone: no partial sums, and the others' count must not differ
     double* pt = a.partial + (size_t)(rcount & 1) * a.partial_stride;
@@ -548,7 +553,7 @@ struct CoarseCycle {
   __device__ void dots_lpc(const T* W, int N, int l, double* pt) {
     constexpr int CPW = 32 / LPC;
     const int warp = threadIdx.x >> 5, ln = threadIdx.x & 31, nw = blockDim.x >> 5;
-    const int sub = ln / LPC, lc = ln - sub * LPC, n = l + 3;
+    const int sub = ln / LPC, lc = ln - sub * LPC, n = l + 3, nsum = summands();
     const T* w = ws();
     const T* rs = rs_();
     for (int c0 = warp * CPW; c0 < n; c0 += nw * CPW) {
@@ -569,7 +574,7 @@ struct CoarseCycle {
       for (int o = LPC / 2; o; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
       if (lc == 0 && c < n) {
         if (nblk == 1) red_s[c] = d;
-        else pt[(size_t)c * nblk + blockIdx.x] = d;
+        else if (rows > 0) pt[(size_t)c * nsum + blockIdx.x] = d;
       }
     }
   }
@@ -711,7 +716,7 @@ struct CoarseCycle {
     double v[1] = {s};
     __syncthreads();
     bsum_n<1>(v, sh);
-    if (threadIdx.x == 0) *(nblk == 1 ? red_s : pt + blockIdx.x) = v[0];
+    if (threadIdx.x == 0 && rows > 0) *(nblk == 1 ? red_s : pt + blockIdx.x) = v[0];
     if (!reduce_cols(pt, 1)) return false;
     sc.r2 = red_s[0];
     return true;
