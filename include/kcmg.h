@@ -100,9 +100,11 @@ typedef struct {
     int precision;           /* kcmg_precision */
     int use_graph;           /* 1: run the cycle as a CUDA graph with conditional while
                                 nodes; 0: host-driven control (reads a flag per loop test) */
-    int coarse_persistent;   /* 1: every level below the finest runs in one persistent
-                                cooperative kernel per finest-level cycle; 0: one kernel
-                                per step (nested loops as conditional graph nodes) */
+    int coarse_persistent;   /* 1: the levels below the finest that are small run in one
+                                persistent cooperative kernel per finest-level cycle, and a
+                                small problem (finest level included) in one for the whole
+                                solve; use_graph is then ignored.  0: one kernel per step
+                                (nested loops as conditional graph nodes) */
     int tc_tf32_only;        /* batched solves (nrhs > 1) in the mixed forms: 0 (default) =
                                 every block product of the tensor-core sweeps is split into
                                 three TF32 products (head*head + head*tail + tail*head,
@@ -191,12 +193,15 @@ kcmg_status kcmg_setup(kcmg_ctx **out, const kcmg_params *p, void *cuda_stream);
    ||b_j - A x_j|| <= max(rtol ||b_j - A x0_j||, atol), confirmed by a compensated FP64
    true residual.  The batched form is host-driven (use_graph is ignored).  Its level-0
    basis holds lmax vectors per column (default 60 when lmax = 0) plus one cycle's
-   corrections, shrunk to what the device can hold.  In the mixed forms the block-Jacobi sweeps run on the tensor cores
-   (TF32 products, FP32 accumulation), with launch shapes chosen by an autotuner at the
-   first batched solve (see kcmg_mrhs_tuning).  info: iters and level_iters count the
-   shared loop; rel_res is the largest relative residual over the columns and res0 the
-   largest initial residual; the history records the number of active columns at every
-   level-0 loop test (hist_type 5). */
+   corrections, shrunk to what the device can hold.  Small problems (with coarse_persistent) run
+   in one kernel, every column on its own group of blocks with its own operator applications,
+   loop and stopping test; the sweeps of the mixed forms are then FP32 FMAs.  Otherwise, in the
+   mixed forms, the block-Jacobi sweeps run on the tensor cores (TF32 products, FP32
+   accumulation) or the CUDA cores, with launch shapes chosen by an autotuner at the first such
+   solve (see kcmg_mrhs_tuning).  info: iters and level_iters count the shared loop (in the one
+   kernel: the largest count over the columns); rel_res is the largest relative residual over
+   the columns and res0 the largest initial residual; the history records the number of active
+   columns at every level-0 loop test (hist_type 5). */
 kcmg_status kcmg_solve(kcmg_ctx *ctx, const double *b, double *x, int nrhs, double rtol,
                        double atol, int maxiter, kcmg_info *info);
 
@@ -235,24 +240,24 @@ kcmg_status kcmg_get_blocks(kcmg_ctx *ctx, int level, double *out);
 kcmg_status kcmg_rm_sequence(kcmg_ctx *ctx, int level, const double *b, const double *x0,
                              const double *z, int ncorr, double *x, double *r, int *l);
 
-/* Measurement support (no counterpart in the paper).  out[0..2]: launches, total device
+/* Measurement support (no counterpart in the paper). out[0..2]: launches, total device
    milliseconds (GPU global timer, entry to last barrier) and algorithmic bytes (unique
-   operator and vector bytes of every phase) of the persistent coarse-cycle kernel since
-   the previous call; the counters are then reset.  If reps > 0 also times, with CUDA events
-   on the library's stream, reps launches each of the level-0 FP64 operator application
-   (out[3] ms per launch, out[4] algorithmic bytes) and of one full block-Jacobi sweep in
-   the smoother's precision (out[5] ms, out[6] bytes).  out[7 + l] (if nout allows): device
-   milliseconds the coarse-cycle kernel spent on level l (the coarsest: its direct solves).
-   out[19 + k] (if nout allows): milliseconds it spent in phases of kind k, each with its
-   closing grid barrier: 0 block-Jacobi sweep, 1 w = A z with the first Gram pass and its
-   reduction, 2 second Gram pass, 3 new basis column with its norms, 4 normalisation and
-   x, r update, 5 restriction or prolongation, 6 coarsest solve, 7 restart residual,
-   8 level entry and return.  out[28..31] (if nout allows, reps > 0 and level 1 is iterated):
-   the same four timings as out[3..6] on level 1.  out[32..36] (if nout allows, reps > 0):
-   the level-0 Gram kernels of Alg. 1 at the basis length halfway through a restart period:
-   ms and FLOPs of the first Gram pass, ms and FLOPs of the update of the new column, and
-   the basis length used (these calls overwrite the basis; the next solve starts afresh).
-   nout >= 7. */
+   operator and vector bytes of every phase) of the persistent coarse-cycle kernel (single
+   right-hand side; the whole solve on a small problem) since the previous call; the counters
+   are then reset. If reps > 0 also times, with CUDA events on the library's stream, reps
+   launches each of the level-0 FP64 operator application (out[3] ms per launch, out[4]
+   algorithmic bytes) and of one full block-Jacobi sweep in the smoother's precision (out[5]
+   ms, out[6] bytes). out[7 + l] (if nout allows): device milliseconds the coarse-cycle kernel
+   spent on level l (the coarsest: its direct solves). out[19 + k] (if nout allows):
+   milliseconds it spent in phases of kind k, each with its closing grid barrier: 0 block-
+   Jacobi sweep, 1 w = A z with the first Gram pass and its reduction, 2 second Gram pass, 3
+   new basis column with the r update, 4 unused, 5 restriction or prolongation, 6 coarsest
+   solve, 7 restart residual, 8 level entry and return. out[28..31] (if nout allows, reps > 0
+   and level 1 is iterated): the same four timings as out[3..6] on level 1. out[32..36] (if
+   nout allows, reps > 0): the level-0 Gram kernels of Alg. 1 at the basis length halfway
+   through a restart period: ms and FLOPs of the first Gram pass, ms and FLOPs of the update of
+   the new column, and the basis length used (these calls overwrite the basis; the next solve
+   starts afresh). nout >= 7. */
 kcmg_status kcmg_kernel_report(kcmg_ctx *ctx, int reps, double *out, int nout);
 
 /* r = b - A x with the finest-level FP64 operator, and *rnorm = ||r|| (a host double),
@@ -284,17 +289,18 @@ kcmg_status kcmg_residual_noalloc(kcmg_ctx *ctx, const double *b, const double *
 kcmg_status kcmg_apply_multi(kcmg_ctx *ctx, int level, int nrhs, const double *x, double *y);
 kcmg_status kcmg_smooth_multi(kcmg_ctx *ctx, int level, int nrhs, const double *r, double *z);
 
-/* Launch shapes the multi-right-hand-side autotuner chose at the first batched solve of
-   ctx: out[0] warps per block of the FP64 block SpMM, out[1] its time (ms), out[2] warps
-   per block of the FP32 sweep, out[3] its grid (0 = one warp per cell), out[4] its
-   time (ms), out[5] level-0 basis capacity per column, out[6] nrhs, out[7] 1 if the
-   tensor-core sweeps split each product into three TF32 products (tc_tf32_only = 0),
-   out[8] the level-0 sweep kernel, the fastest of three: 0 = tensor cores (one warp per
-   cell), 1 = tensor cores with each cell's blocks, inverse, r and neighbour slabs staged
-   by double-buffered 1-D bulk copies, 2 = FP32 CUDA cores (register-blocked; exact FP32
-   products); 3 = not tuned: FP32 CUDA cores over the nonzero entries of a finest level with a
-   tensor basis's zero pattern.  The environment variable KCMG_SWEEP = tc | tcb | simt, read at the first
-   batched solve, forces one kernel on every level.  Zero-filled up to nout. */
+/* Launch shapes the multi-right-hand-side autotuner chose for the batched kernels of ctx (at
+   their first call, or here if only small batched solves have run): out[0] warps per block of
+   the FP64 block SpMM, out[1] its time (ms), out[2] warps per block of the FP32 sweep, out[3]
+   its grid (0 = one warp per cell), out[4] its time (ms), out[5] level-0 basis capacity per
+   column, out[6] nrhs, out[7] 1 if the tensor-core sweeps split each product into three TF32
+   products (tc_tf32_only = 0), out[8] the level-0 sweep kernel, the fastest of three: 0 =
+   tensor cores (one warp per cell), 1 = tensor cores with each cell's blocks, inverse, r and
+   neighbour slabs staged by double-buffered 1-D bulk copies, 2 = FP32 CUDA cores (register-
+   blocked; exact FP32 products); 3 = not tuned: FP32 CUDA cores over the nonzero entries of a
+   finest level with a tensor basis's zero pattern. The environment variable KCMG_SWEEP = tc |
+   tcb | simt, read at the first batched solve, forces one kernel on every level (and the
+   batched kernels on small problems). Zero-filled up to nout. */
 kcmg_status kcmg_mrhs_tuning(kcmg_ctx *ctx, double *out, int nout);
 
 /* Level sizes: number of cells of a level (0 if out of range). */

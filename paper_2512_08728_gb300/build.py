@@ -14,6 +14,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libkcmg.so")
 SOURCES = ["kernels.cu", "engine.cu", "coarse_cycle_f64.cu", "coarse_cycle_f32.cu", "coarse_cycle_bf16.cu",
+           "coarse_group_f64.cu", "coarse_group_f32.cu", "coarse_group_bf16.cu",
            "coarse_cycle_ir32.cu", "coarse_cycle_ir32_bf16.cu", "noalloc.cu", "mrhs.cu", "mrhs_simt.cu", "schwarz.cu",
            "matfree.cu", "pattern_ops_f64.cu", "pattern_ops_f32.cu",
            "mrhs_pattern_f64.cu", "mrhs_pattern_f32.cu"]

@@ -81,18 +81,19 @@ template <typename T> __device__ __forceinline__ T ldv(const T* p) { return __ld
 
 // Grid barrier with a bounded wait.  Every block adds one to a counter (a release, which
 // publishes the block's writes, and without waiting for the old value) and polls until the
-// counter reaches the total for this generation.  gen: this block's barrier count so far in the
+// counter reaches the total for this generation.  blocks: how many share the barrier (the grid, or
+// one group of it).  gen: this block's barrier count so far in the
 // launch; the last block to leave the kernel clears the counter (cc_leave), the host at the start
 // of every solve.  Returns false (in every thread of the block) once the error flag is set;
 // callers then leave the kernel.
-static __device__ __forceinline__ bool cc_barrier(const CoarseArgs& a, unsigned int& gen) {
+static __device__ __forceinline__ bool cc_barrier(const CoarseArgs& a, unsigned int& gen, unsigned int blocks) {
   __shared__ int s_ok;
   __syncthreads();
-  if (gridDim.x == 1) return true;
+  if (blocks == 1) return true;
   if (threadIdx.x == 0) {
     cuda::atomic_ref<unsigned int, cuda::thread_scope_device> cnt(*a.bar_count);
     cuda::atomic_ref<int, cuda::thread_scope_device> err(*a.err);
-    const unsigned int target = (gen + 1) * gridDim.x;
+    const unsigned int target = (gen + 1) * blocks;
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.bar_count) : "memory");
     long long spins = 0;
     int ok = 1;
@@ -115,9 +116,9 @@ static __device__ __forceinline__ bool cc_barrier(const CoarseArgs& a, unsigned 
 
 // Called by every block after its last barrier: the last one clears the counters for the next
 // launch.  No block polls any more, since all have passed the barrier.
-static __device__ __forceinline__ void cc_leave(const CoarseArgs& a) {
-  if (gridDim.x == 1 || threadIdx.x != 0) return;
-  if (atomicAdd(a.bar_gen, 1u) == gridDim.x - 1) {
+static __device__ __forceinline__ void cc_leave(const CoarseArgs& a, unsigned int blocks) {
+  if (blocks == 1 || threadIdx.x != 0) return;
+  if (atomicAdd(a.bar_gen, 1u) == blocks - 1) {
     *a.bar_count = 0u;
     *a.bar_gen = 0u;
     __threadfence();
@@ -142,7 +143,7 @@ struct RmScal {
 // Vectors, basis W, Z, the Alg. 1 operator and the transfers are in TV (FP64, or FP32 in
 // the inner solve of the iterative-refinement forms); the smoother sweeps run in TS with
 // inverses stored as TI.  Reductions and Gram coefficients are FP64 in every form.
-template <typename TV, typename TS, typename TI, int NP, int DIM>
+template <typename TV, typename TS, typename TI, int NP, int DIM, bool GROUP>
 struct CoarseCycle {
   using T = TV;
   using V2 = typename V2T<TV>::type;
@@ -159,6 +160,7 @@ struct CoarseCycle {
   int* nbs;              // neighbour slab of each slot: cell offset in the slab buffer
   long long* tph;        // clocks per phase kind, then per level (thread 0 of block 0)
   T* Ps;                 // NCH*NP*NP (prolongation matrices)
+  int bid_ = 0, nall_ = 0;   // with GROUP: this block among those that share the cycle, and their number
   int rcount = 0;        // reductions done (selects the partial buffer)
   unsigned int gen = 0;  // grid barriers passed (identical in every block)
   bool ok = true;
@@ -172,16 +174,19 @@ struct CoarseCycle {
   int own0 = 0;                      // the own rows' place in the slab buffer
   double *R = nullptr, *gm = nullptr, *al = nullptr;   // packed columns of R, 1 / R_kk, alpha
 
-  __device__ bool grid_bar() { return cc_barrier(a, gen); }
+  // the whole grid's: read where they are used, which keeps no registers
+  __device__ int bid() const { return GROUP ? bid_ : (int)blockIdx.x; }
+  __device__ int nall() const { return GROUP ? nall_ : (int)gridDim.x; }
+  __device__ bool grid_bar() { return cc_barrier(a, gen, nall()); }
   // barrier of the blocks that take part in the current level
   __device__ bool bar() {
     if (nblk > 1) return grid_bar();
     __syncthreads();
     return true;
   }
-  __device__ int blocks_of(int l) const { return l >= a.solo_from ? 1 : (int)gridDim.x; }
+  __device__ int blocks_of(int l) const { return l >= a.solo_from ? 1 : nall(); }
   __device__ void count(long long b) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) bytes += b;
+    if (bid() == 0 && threadIdx.x == 0) bytes += b;
   }
   // unique operator bytes of n slots on a level with this element size
   __device__ long long opbytes(const CoarseLevel& C, int slots, int elem) const {
@@ -207,8 +212,8 @@ struct CoarseCycle {
     nblk = blocks_of(l);
     const CoarseLevel& C = L(l);
     const int cells = C.N / NP;
-    K0 = first_cell(cells, blockIdx.x, nblk);
-    nc = first_cell(cells, blockIdx.x + 1, nblk) - K0;
+    K0 = first_cell(cells, bid(), nblk);
+    nc = first_cell(cells, bid() + 1, nblk) - K0;
     rows = nc * NP;
     row0 = K0 * NP;
     // threads per row: 8, 4, 2 or 1, as many as the block has
@@ -443,7 +448,7 @@ struct CoarseCycle {
     // a warp takes 32 rows of a patch; units over blocks first, so that few patches use every SM
     constexpr int JT = (M + 31) / 32;
     const int units = (np0 + np1) * JT;
-    for (int u = blockIdx.x + nblk * warp; u < units; u += nblk * wpb) {
+    for (int u = bid() + nblk * warp; u < units; u += nblk * wpb) {
       const int w = u / JT, t = u - w * JT;
       if (w < np0) as_patch_rows_warp<TS, TI, NP, DIM>(C.n, 0, w, t, inv0, res, zP, prs);
       else as_patch_rows_warp<TS, TI, NP, DIM>(C.n, 1, w - np0, t, inv1, res, zP + (size_t)np0 * M, prs);
@@ -526,7 +531,7 @@ struct CoarseCycle {
       __syncthreads();
       return true;
     }
-    for (int c = blockIdx.x + nblk * warp; c < n; c += nblk * nw) {
+    for (int c = bid() + nblk * warp; c < n; c += nblk * nw) {
       double v = 0.0;
       for (int b = ln; b < nsum; b += 32) v += __ldcg(pt + (size_t)c * nsum + b);
 #pragma unroll
@@ -574,7 +579,7 @@ struct CoarseCycle {
       for (int o = LPC / 2; o; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
       if (lc == 0 && c < n) {
         if (nblk == 1) red_s[c] = d;
-        else if (rows > 0) pt[(size_t)c * nsum + blockIdx.x] = d;
+        else if (rows > 0) pt[(size_t)c * nsum + bid()] = d;
       }
     }
   }
@@ -614,7 +619,7 @@ struct CoarseCycle {
 
   // whether this block keeps the level's coefficients: every block in shared memory, block 0 where
   // a long basis puts them in global memory (read by all after a barrier)
-  __device__ bool own_coef() const { return L(lev).sm_gm >= 0 || blockIdx.x == 0; }
+  __device__ bool own_coef() const { return L(lev).sm_gm >= 0 || bid() == 0; }
 
   // ---------------------------------------------------------------- Alg. 1
   // with the correction zg: own rows in zsV(), all rows in zg; returns false on a barrier error
@@ -716,7 +721,7 @@ struct CoarseCycle {
     double v[1] = {s};
     __syncthreads();
     bsum_n<1>(v, sh);
-    if (threadIdx.x == 0 && rows > 0) *(nblk == 1 ? red_s : pt + blockIdx.x) = v[0];
+    if (threadIdx.x == 0 && rows > 0) *(nblk == 1 ? red_s : pt + bid()) = v[0];
     if (!reduce_cols(pt, 1)) return false;
     sc.r2 = red_s[0];
     return true;
@@ -771,7 +776,7 @@ struct CoarseCycle {
     count((long long)F.N * sizeof(T) + (long long)C.N * sizeof(T) * (start ? 3 : 1));
     const int cells = C.N / NP;
     const int nb = blocks_of(lev + 1);
-    const int J0 = first_cell(cells, blockIdx.x, nb), nJ = first_cell(cells, blockIdx.x + 1, nb) - J0;
+    const int J0 = first_cell(cells, bid(), nb), nJ = first_cell(cells, bid() + 1, nb) - J0;
     const T* rf = vec(F.r);
     T* stage = zsV();   // children of the own coarse cells: [cell][child][NP]
     for (int i = threadIdx.x; i < nJ * NCH * NP; i += blockDim.x) {
@@ -832,7 +837,7 @@ struct CoarseCycle {
     const T* bc = vec(C.b);
     T* xc = vec(C.x);
     const int nw = blockDim.x >> 5, warp = threadIdx.x >> 5, ln = threadIdx.x & 31;
-    for (int row = blockIdx.x + nblk * warp; row < a.Nc; row += nblk * nw) {
+    for (int row = bid() + nblk * warp; row < a.Nc; row += nblk * nw) {
       double s[4] = {0.0, 0.0, 0.0, 0.0};
       const double* Ar = a.Ainv + (size_t)row * a.Nc;
       int j = ln;
@@ -853,14 +858,14 @@ struct CoarseCycle {
   // the global timer only at the kernel's ends, which give the scale
   long long t_ph = 0, t_mark = 0;
   __device__ void ph(int kind) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (bid() == 0 && threadIdx.x == 0) {
       const long long t = clock64();
       if (t_ph) tph[kind] += t - t_ph;
       t_ph = t;
     }
   }
   __device__ void mark(int l) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (bid() == 0 && threadIdx.x == 0) {
       const long long t = clock64();
       if (t_mark) tph[kCoarsePhases + l] += t - t_mark;
       t_mark = t;
@@ -893,7 +898,7 @@ struct CoarseCycle {
   __device__ void record(Top& t, double r2, int type) {
     const LevelState* st = L(0).st;
     if (t.hist_len >= st->hist_cap || !a.hist) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (bid() == 0 && threadIdx.x == 0) {
       a.hist[t.hist_len] = sqrt(r2);
       a.hist_type[t.hist_len] = type;
     }
@@ -952,7 +957,16 @@ struct CoarseCycle {
     ph(PH_CONTROL);
     start(sc[lev], lev0 == 0 ? 0.0 : L(lev).rtol);
     int maxit0 = 0;
-    if (lev0 == 0) {
+    if constexpr (GROUP) {   // r = b - A x0 and its norm
+      const LevelState* st = L(0).st;
+      if (!(ok = restart(sc[0]))) return;
+      sc[0].first = 0;
+      const double n0 = sqrt(sc[0].r2), eps = fmax(st->rtol * n0, st->atol);
+      sc[0].eps2 = eps * eps;
+      if (!isfinite(n0)) top.status = KCMG_NONFINITE;
+      maxit0 = st->maxit;
+      if (bid() == 0 && threadIdx.x == 0) L(0).st->rnorm0 = n0;
+    } else if (lev0 == 0) {   // set by the residual kernel
       const LevelState* st = L(0).st;
       sc[0].first = 0;
       sc[0].r2 = st->rnorm * st->rnorm;
@@ -985,7 +999,7 @@ struct CoarseCycle {
         if (phase[lev] == PRE &&
             !(s.r2 > s.eps2 && s.it < (top0 ? maxit0 : C.maxit) && guard[lev] < (1 << 24) &&
               (!top0 || top.status == KCMG_OK))) {
-          if (!top0 && blockIdx.x == 0 && threadIdx.x == 0 && C.st) {
+          if (!top0 && bid() == 0 && threadIdx.x == 0 && C.st) {
             C.st->iters_total += s.it;
             C.st->nrestart += restarts[lev];
           }
@@ -1028,10 +1042,10 @@ struct CoarseCycle {
         if (!(ok = bar())) break;                                  // r complete everywhere
         phase[lev] = CORRECT;
         const bool direct = (lev + 1 == a.nlev - 1), alone = blocks_of(lev + 1) < nblk;
-        if (!alone || blockIdx.x == 0) restrict_(!direct);         // r_c = R r
+        if (!alone || bid() == 0) restrict_(!direct);         // r_c = R r
         ph(PH_TRANSFER);
         mark(lev);
-        if (alone && blockIdx.x != 0) {                            // block 0 solves the rest
+        if (alone && bid() != 0) {                            // block 0 solves the rest
           if (!(ok = grid_bar())) break;
         } else if (direct) {
           const int nb = nblk;
@@ -1067,7 +1081,16 @@ struct CoarseCycle {
         phase[lev] = PRE;
       }
     }
-    if (lev0 == 0 && ok && blockIdx.x == 0 && threadIdx.x == 0) {
+    if constexpr (GROUP) {   // true residual, and the column to the caller's array
+      if (!ok) return;
+      const int l = sc[0].l;
+      sc[0].l = 0;
+      if (!(ok = restart(sc[0]))) return;
+      sc[0].l = l;
+      for (int lr = threadIdx.x; lr < rows; lr += blockDim.x)
+        a.io_x[(size_t)(row0 + lr) * a.io_stride] = (double)ldv(vec(L(0).x) + row0 + lr);
+    }
+    if (lev0 == 0 && ok && bid() == 0 && threadIdx.x == 0) {
       LevelState* st = L(0).st;
       st->it = sc[0].it;
       st->iters_total += sc[0].it;
@@ -1098,7 +1121,7 @@ __global__ void __launch_bounds__(512) k_coarse_cycle(const __grid_constant__ Co
   T* Ps = reinterpret_cast<T*>(smem_cc);   // prolongation matrices first
   const double* P = static_cast<const double*>(a.P);   // FP64 prolongation matrices
   for (int i = threadIdx.x; i < NCH * NP * NP; i += blockDim.x) Ps[i] = (T)P[i];
-  CoarseCycle<TV, TS, TI, NP, DIM> cc{a, sh, red_s, cf, &rms, nbs, tph, Ps};
+  CoarseCycle<TV, TS, TI, NP, DIM, false> cc{a, sh, red_s, cf, &rms, nbs, tph, Ps};
   unsigned long long t0 = 0;
   long long c0 = 0;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -1130,7 +1153,51 @@ __global__ void __launch_bounds__(512) k_coarse_cycle(const __grid_constant__ Co
     atomicAdd(a.stat_launches, 1ull);
     atomicAdd(a.stat_bytes, (double)cc.bytes);
   }
-  cc_leave(a);
+  cc_leave(a, gridDim.x);
+}
+
+// Several right-hand sides: group g of gb blocks solves columns g, g + groups, ... one after
+// another, each as k_coarse_cycle does with the whole grid, and the groups run side by side.  A
+// phase of a small level is mostly latency (a barrier, an L2 round trip), which the columns'
+// phases then spend at the same time; the groups need no barrier with one another.  Measured
+// (GB300) against the batched kernels, one launch a step for all columns and the loop on the host:
+// 8^3, np = 10, to 1e-11, 8 columns of 19 blocks 182 -> 34 ms, 32 columns of 4 blocks 242 -> 58 ms.
+template <typename TV, typename TS, typename TI, int NP, int DIM>
+__global__ void __launch_bounds__(512) k_coarse_group(const CoarseArgs* __restrict__ cols, int ncol, int gb) {
+  using T = TV;
+  __shared__ CoarseArgs a;
+  __shared__ double sh[32 * 8];
+  __shared__ RmScal rms;
+  __shared__ int nbs[2 * DIM + 1];
+  __shared__ long long tph[kCoarsePhases + KCMG_MAX_LEVELS];
+  constexpr int NCH = 1 << DIM;
+  const int bid = blockIdx.x % gb, groups = gridDim.x / gb;
+  T* Ps = reinterpret_cast<T*>(smem_cc);
+  unsigned int gen = 0;
+  for (int col = blockIdx.x / gb; col < ncol; col += groups) {
+    __syncthreads();
+    static_assert(sizeof(CoarseArgs) % 4 == 0, "copied in words");
+    for (int i = threadIdx.x; i < (int)(sizeof(CoarseArgs) / 4); i += blockDim.x)
+      reinterpret_cast<unsigned int*>(&a)[i] = reinterpret_cast<const unsigned int*>(cols + col)[i];
+    if (threadIdx.x < kCoarsePhases + KCMG_MAX_LEVELS) tph[threadIdx.x] = 0;
+    __syncthreads();
+    const double* P = static_cast<const double*>(a.P);
+    for (int i = threadIdx.x; i < NCH * NP * NP; i += blockDim.x) Ps[i] = (T)P[i];
+    double* red_s = reinterpret_cast<double*>(smem_cc + a.sm_red);
+    CoarseCycle<TV, TS, TI, NP, DIM, true> cc{a, sh, red_s, red_s + a.cols + 4, &rms, nbs, tph, Ps, bid, gb};
+    cc.gen = gen;
+    cc.enter(0);
+    const CoarseLevel& C = a.lv[0];
+    for (int lr = threadIdx.x; lr < cc.rows; lr += blockDim.x) {
+      const size_t row = cc.row0 + lr;
+      static_cast<T*>(C.b)[row] = (T)a.io_b[row * a.io_stride];
+      static_cast<T*>(C.x)[row] = (T)a.io_x[row * a.io_stride];
+    }
+    cc.run(0);
+    gen = cc.gen;
+    if (!cc.ok) break;
+  }
+  cc_leave(a, gb);
 }
 
 }  // namespace

@@ -1,7 +1,8 @@
 // Instantiation of the persistent coarse-cycle kernel (coarse_cycle.cuh) for one precision
 // form.  The including translation unit defines CC_TV (vectors, basis, residual
 // minimisation), CC_T (smoother sweeps) and CC_TI (stored block inverses); one
-// translation unit per form keeps the build parallel.
+// translation unit per form keeps the build parallel.  With CC_GROUP it is the kernel for
+// several columns.
 #pragma once
 #include "coarse_cycle.cuh"
 
@@ -22,7 +23,11 @@ namespace kcmg {
 
 static void* coarse_kernel_ptr(int np, int dim) {
   void* f = nullptr;
+#ifdef CC_GROUP
+  KCMG_CC_SWITCH(np, dim, { f = (void*)k_coarse_group<CC_TV, CC_T, CC_TI, NP, DIM>; });
+#else
   KCMG_CC_SWITCH(np, dim, { f = (void*)k_coarse_cycle<CC_TV, CC_T, CC_TI, NP, DIM>; });
+#endif
   return f;
 }
 
@@ -90,11 +95,73 @@ static void coarse_cycle_layout(CoarseArgs* a, int grid) {
   a->sm_bytes = top;
 }
 
+// whether a block's share fits beside the kernel's static shared memory; sets the kernel's limit
+static cudaError_t cc_fits(void* f, const CoarseArgs& a, int dev) {
+  cudaError_t e;
+  int optin = 0, per_sm = 0;
+  if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
+  cudaFuncAttributes fa;
+  if ((e = cudaFuncGetAttributes(&fa, f)) != cudaSuccess) return e;
+  if (a.sm_bytes + (int)fa.sharedSizeBytes > optin) return cudaErrorInvalidConfiguration;
+  if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                optin - (int)fa.sharedSizeBytes)) != cudaSuccess)   // the kernel's, not this context's
+    return e;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, kCoarseThreads, a.sm_bytes)) != cudaSuccess)
+    return e;
+  return per_sm < 1 ? cudaErrorInvalidConfiguration : cudaSuccess;
+}
+
+static cudaError_t cc_launch(void* f, int grid, int smem, void** args, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kCoarseThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelExC(&cfg, f, args);
+}
+
+#ifdef CC_GROUP
+template <>
+cudaError_t coarse_group_prepare<CC_TV, CC_T, CC_TI>(CoarseArgs* a, int ncol, int* blocks, int* groups) {
+  void* f = coarse_kernel_ptr(a->np, a->dim);
+  if (!f) return cudaErrorInvalidValue;
+  int dev = 0, nsm = 0;
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  a->solo_from = cc_solo_from(*a);
+  const int cap = cc_blocks(*a, nsm);
+  // an equal share of the SMs; more where a block's part does not fit in shared memory
+  for (int g = std::max(1, std::min(cap, nsm / ncol)); g <= cap; ++g) {
+    coarse_cycle_layout(a, g);
+    e = cc_fits(f, *a, dev);
+    if (e == cudaErrorInvalidConfiguration) continue;
+    if (e != cudaSuccess) return e;
+    *blocks = g;
+    *groups = std::min(ncol, nsm / g);
+    return cudaSuccess;
+  }
+  return cudaErrorInvalidConfiguration;
+}
+
+template <>
+cudaError_t launch_coarse_group<CC_TV, CC_T, CC_TI>(const CoarseArgs& a, const CoarseArgs* cols, int ncol, int blocks,
+                                                    int groups, cudaStream_t s) {
+  void* f = coarse_kernel_ptr(a.np, a.dim);
+  void* args[] = {&cols, &ncol, &blocks};
+  return cc_launch(f, blocks * groups, a.sm_bytes, args, s);
+}
+#else
 template <>
 cudaError_t coarse_cycle_prepare<CC_TV, CC_T, CC_TI>(CoarseArgs* a, int* grid) {
   void* f = coarse_kernel_ptr(a->np, a->dim);
   if (!f) return cudaErrorInvalidValue;
-  int per_sm = 0, dev = 0, nsm = 0;
+  int dev = 0, nsm = 0;
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
@@ -102,18 +169,7 @@ cudaError_t coarse_cycle_prepare<CC_TV, CC_T, CC_TI>(CoarseArgs* a, int* grid) {
   int g = cc_blocks(*a, nsm);
   if (*grid > 0 && *grid < g) g = *grid;   // the caller's cap
   coarse_cycle_layout(a, g);
-  int optin = 0;
-  if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
-  cudaFuncAttributes fa;
-  if ((e = cudaFuncGetAttributes(&fa, f)) != cudaSuccess) return e;
-  if (a->sm_bytes + (int)fa.sharedSizeBytes > optin) return cudaErrorInvalidConfiguration;
-  // the limit belongs to the kernel, which contexts of other sizes launch too: the device's, always
-  if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes)) !=
-      cudaSuccess)
-    return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, kCoarseThreads, a->sm_bytes)) != cudaSuccess)
-    return e;
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  if ((e = cc_fits(f, *a, dev)) != cudaSuccess) return e;
   *grid = g;
   return cudaSuccess;
 }
@@ -122,18 +178,9 @@ template <>
 cudaError_t launch_coarse_cycle<CC_TV, CC_T, CC_TI>(const CoarseArgs& a, int grid, cudaStream_t s) {
   void* f = coarse_kernel_ptr(a.np, a.dim);
   if (!f) return cudaErrorInvalidValue;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(kCoarseThreads);
-  cfg.dynamicSmemBytes = a.sm_bytes;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
   void* args[] = {const_cast<CoarseArgs*>(&a)};
-  return cudaLaunchKernelExC(&cfg, f, args);
+  return cc_launch(f, grid, a.sm_bytes, args, s);
 }
+#endif
 
 }  // namespace kcmg

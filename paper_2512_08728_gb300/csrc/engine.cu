@@ -53,6 +53,22 @@ struct Level {
 
 }  // namespace
 
+// Several right-hand sides of a small problem: every column's whole solve by its own group of
+// blocks of one kernel (k_coarse_group), with its own vectors and bases.
+struct ColumnGroups {
+  int nrhs = 0;
+  bool usable = false;        // false: a share does not fit, or no memory for the columns
+  CoarseArgs a{};             // shared-memory layout, and what the columns have in common
+  int blocks = 0, groups = 0;
+  char* mem = nullptr;        // all of the columns' vectors
+  std::vector<CoarseArgs> cols;
+  CoarseArgs* cols_d = nullptr;
+  LevelState* st = nullptr;   // [nrhs][nlev]
+  double *b = nullptr, *x = nullptr;   // [N][nrhs]
+  unsigned int* bars = nullptr;        // [groups][2]
+  int* err = nullptr;
+};
+
 struct kcmg_ctx {
   kcmg_params p{};
   int dim = 0, np = 0, S = 0, nlev = 0, nch = 0;
@@ -83,7 +99,10 @@ struct kcmg_ctx {
   // persistent coarse cycle (levels >= 1 in one cooperative launch per level-0 cycle)
   bool coarse_kernel = false;
   int cc_lev0 = 0;   // first level run by the persistent kernel
+  long long fmas0 = 0;  // FMAs of one dense application of the finest level's operator
   bool whole = false;   // it runs the whole solve, level 0 included
+  ColumnGroups* groups = nullptr;   // several columns at once (small problems)
+  int multi_nrhs = 0;  // right-hand sides of the last batched call
   int cc_grid = 0;
   CoarseArgs cc{};
   long long graph_body_launches = 0;  // kernels per level-0 loop body of the graph
@@ -252,11 +271,9 @@ bool whole_solve(const kcmg_ctx* ctx) {
   const kcmg_params& p = ctx->p;
   if (!p.coarse_persistent || p.mf_nu || p.mf_F || getenv("KCMG_PERSISTENT_ROWS")) return false;
   if (p.async_smooth > 0 && ctx->nlev > 2) return false;
-  long long cells = 1;
-  for (int j = 0; j < ctx->dim; ++j) cells *= p.n[j];
   for (int l = 1; l < ctx->nlev - 1; ++l)   // longer bases than the kernel keeps on the coarse levels
     if (coarse_capacity(p, l) + 1 > kCoarseMaxCols) return false;
-  return cells * ctx->np * ctx->np * ctx->S <= kWholeFmas;
+  return ctx->fmas0 <= kWholeFmas;
 }
 
 // The finest level's blocks and inverses (natural layout) in the pattern kernels' storage, if
@@ -1068,9 +1085,222 @@ MrhsView mrhs_view(kcmg_ctx* ctx) {
   return v;
 }
 
+// ---------------------------------------------------------------- columns on groups of blocks
+void drop_groups(kcmg_ctx* ctx) {
+  if (!ctx->groups) return;
+  if (ctx->groups->mem) cudaFree(ctx->groups->mem);
+  delete ctx->groups;
+  ctx->groups = nullptr;
+}
+
+// The columns' form for this number of right-hand sides, or null where the batched kernels take
+// the solve.  The batched kernels multiply the nonzero entries by all columns at the rate of the
+// chip, but take some 8 us a step and a few more for the host's part of the loop; a group takes
+// about 3 us a step, and its few SMs work through the dense blocks.  The two meet at some 30M FMAs
+// over all columns.  Measured, batched kernels against groups: 8^3, p = 2, to 1e-11, 8 columns
+// 180 / 34 ms, 32 columns 242 / 58; 16 x 16, p = 1, 32 columns 173 / 23; one cycle at 13M FMAs
+// (20 x 20 x 16, p = 2, 3 columns) 5.1 / 2.0 ms, at 23M (16^3, p = 2, 8 columns) 3.9 / 2.7, at 33M
+// (24 x 24 x 16, p = 1, 32 columns) 6.4 / 6.9.
+constexpr long long kColumnsFmas = 30000000;
+ColumnGroups* column_groups(kcmg_ctx* ctx, int nrhs) {
+  const kcmg_params& p = ctx->p;
+  if (!ctx->coarse_kernel || ctx->ir || p.smoother || p.mf_nu || p.mf_F || getenv("KCMG_SWEEP") ||
+      getenv("KCMG_PERSISTENT_ROWS") || nrhs * ctx->fmas0 > kColumnsFmas)
+    return nullptr;
+  if (ctx->groups && ctx->groups->nrhs == nrhs) return ctx->groups->usable ? ctx->groups : nullptr;
+  drop_groups(ctx);
+  ColumnGroups* g = ctx->groups = new ColumnGroups;
+  g->nrhs = nrhs;
+  CoarseArgs& a = g->a;
+  a = ctx->cc;
+  a.lev0 = 0;
+  a.hist = nullptr;
+  // the basis of a batched solve: lmax (default 60) and one cycle's corrections
+  const int per_cycle0 = std::max(3, p.async_smooth + 1);
+  a.lv[0].lcap = std::min((p.lmax > 0 ? p.lmax : 60) + per_cycle0, kLcapMax);
+  cudaError_t e;
+  const bool bf16 = p.precision == KCMG_MIXED_BF16INV;
+  if (!ctx->mixed) e = coarse_group_prepare<double, double, double>(&a, nrhs, &g->blocks, &g->groups);
+  else if (bf16) e = coarse_group_prepare<double, float, __nv_bfloat16>(&a, nrhs, &g->blocks, &g->groups);
+  else e = coarse_group_prepare<double, float, float>(&a, nrhs, &g->blocks, &g->groups);
+  if (e == cudaErrorInvalidConfiguration) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  CK(e);
+  a.partial_stride = (size_t)g->blocks * (a.cols + 4);
+  // the finest level's dense blocks, where the context keeps the nonzero entries only
+  Level& F = ctx->lv[0];
+  const bool own_blocks = !F.A64;
+  const size_t invsz = (size_t)F.G * ((ctx->np + 1) / 2) * 64, opsz = invsz * ctx->S;
+  double *A64 = F.A64, *D64 = F.D64, *inv = nullptr;
+  float *A32 = F.A32, *D32 = F.D32;
+  __nv_bfloat16* D16 = F.D16;
+  int* fail = nullptr;
+  // one allocation, carved twice: first for its size
+  size_t top = 0;
+  auto take = [&](size_t bytes) {
+    char* at = g->mem ? g->mem + top : nullptr;
+    top += (bytes + 255) / 256 * 256;
+    return (void*)at;
+  };
+  const size_t N0 = ctx->lv[0].N;
+  auto carve = [&] {
+    top = 0;
+    g->cols_d = (CoarseArgs*)take(nrhs * sizeof(CoarseArgs));
+    g->st = (LevelState*)take((size_t)nrhs * ctx->nlev * sizeof(LevelState));
+    g->b = (double*)take(N0 * nrhs * sizeof(double));
+    g->x = (double*)take(N0 * nrhs * sizeof(double));
+    g->bars = (unsigned int*)take((size_t)2 * g->groups * sizeof(unsigned int));
+    g->err = (int*)take(sizeof(int));
+    if (own_blocks) {
+      A64 = (double*)take(opsz * sizeof(double));
+      if (!ctx->mixed) D64 = (double*)take(invsz * sizeof(double));
+      else A32 = (float*)take(opsz * sizeof(float));
+      if (ctx->mixed && bf16) D16 = (__nv_bfloat16*)take(invsz * sizeof(__nv_bfloat16));
+      else if (ctx->mixed) D32 = (float*)take(invsz * sizeof(float));
+      inv = (double*)take((size_t)F.ncell * ctx->np * ctx->np * sizeof(double));
+      fail = (int*)take(sizeof(int));
+      a.lv[0].A = A64;
+      a.lv[0].As = ctx->mixed ? (const void*)A32 : (const void*)A64;
+      a.lv[0].Dinv = !ctx->mixed ? (const void*)D64 : bf16 ? (const void*)D16 : (const void*)D32;
+    }
+    g->cols.assign(nrhs, a);
+    for (int j = 0; j < nrhs; ++j) {
+      CoarseArgs& c = g->cols[j];
+      for (int l = 0; l < ctx->nlev; ++l) {
+        CoarseLevel& L = c.lv[l];
+        const size_t v = (size_t)L.N * sizeof(double);
+        L.x = take(v);
+        L.b = take(v);
+        if (l == ctx->nlev - 1) break;
+        L.r = take(v);
+        L.z = take(v);
+        L.s0 = take(ctx->mixed ? v / 2 : v);   // smoother scratch, in its precision
+        L.s1 = take(ctx->mixed ? v / 2 : v);
+        L.t = L.w = L.wre = nullptr;
+        L.W = take(v * L.lcap);
+        L.Z = take(v * L.lcap);
+        L.st = g->st + (size_t)j * ctx->nlev + l;
+        L.coef = L.sm_gm < 0 ? (double*)take(L.coef_len * sizeof(double)) : nullptr;
+      }
+      c.zc = p.async_smooth > 0 ? take(N0 * sizeof(double)) : nullptr;
+      c.partial = (double*)take(2 * a.partial_stride * sizeof(double));
+      c.red = (double*)take((size_t)(a.cols + 4) * sizeof(double));
+      c.bar_count = g->bars + 2 * (j % g->groups);
+      c.bar_gen = c.bar_count + 1;
+      c.err = g->err;
+      c.io_b = g->b + j;
+      c.io_x = g->x + j;
+      c.io_stride = nrhs;
+    }
+  };
+  carve();
+  if (cudaMalloc((void**)&g->mem, top) != cudaSuccess) {
+    cudaGetLastError();
+    g->mem = nullptr;
+    return nullptr;
+  }
+  carve();
+  if (own_blocks) {   // the context's setup has inverted these blocks already: fail stays clear
+    CK(cudaMemsetAsync(fail, 0, sizeof(int), ctx->s));
+    launch_block_inverse(ctx->np, F.nat, F.ncell, inv, fail, ctx->s);
+    launch_interleave<double>(ctx->np, ctx->S, F.nat, F.nbr, F.ncell, F.G, A64, ctx->s);
+    if (!ctx->mixed) launch_interleave<double>(ctx->np, 1, inv, nullptr, F.ncell, F.G, D64, ctx->s);
+    else launch_interleave<float>(ctx->np, ctx->S, F.nat, F.nbr, F.ncell, F.G, A32, ctx->s);
+    if (ctx->mixed && bf16) launch_interleave<__nv_bfloat16>(ctx->np, 1, inv, nullptr, F.ncell, F.G, D16, ctx->s);
+    else if (ctx->mixed) launch_interleave<float>(ctx->np, 1, inv, nullptr, F.ncell, F.G, D32, ctx->s);
+    CK(cudaGetLastError());
+  }
+  CK(cudaMemcpyAsync(g->cols_d, g->cols.data(), nrhs * sizeof(CoarseArgs), cudaMemcpyHostToDevice, ctx->s));
+  CK(cudaStreamSynchronize(ctx->s));
+  g->usable = true;
+  return g;
+}
+
+kcmg_status solve_groups(kcmg_ctx* ctx, ColumnGroups* g, const double* b, double* x, double rtol, double atol,
+                         int maxiter, kcmg_info* info) {
+  const int R = g->nrhs, nl = ctx->nlev;
+  const size_t NR = (size_t)ctx->lv[0].N * R;
+  CK(cudaMemcpyAsync(g->b, b, NR * sizeof(double), cudaMemcpyDefault, ctx->s));
+  CK(cudaMemcpyAsync(g->x, x, NR * sizeof(double), cudaMemcpyDefault, ctx->s));
+  std::vector<LevelState> st((size_t)R * nl);
+  memset(st.data(), 0, st.size() * sizeof(LevelState));
+  for (int j = 0; j < R; ++j) {
+    LevelState& h = st[(size_t)j * nl];
+    h.maxit = maxiter;
+    h.rtol = rtol;
+    h.atol = atol;
+    h.status = KCMG_OK;
+  }
+  CK(cudaMemcpyAsync(g->st, st.data(), st.size() * sizeof(LevelState), cudaMemcpyHostToDevice, ctx->s));
+  CK(cudaMemsetAsync(g->bars, 0, (size_t)2 * g->groups * sizeof(unsigned int), ctx->s));
+  CK(cudaMemsetAsync(g->err, 0, sizeof(int), ctx->s));
+  cudaError_t e;
+  const bool bf16 = ctx->p.precision == KCMG_MIXED_BF16INV;
+  if (!ctx->mixed) e = launch_coarse_group<double, double, double>(g->a, g->cols_d, R, g->blocks, g->groups, ctx->s);
+  else if (bf16) e = launch_coarse_group<double, float, __nv_bfloat16>(g->a, g->cols_d, R, g->blocks, g->groups, ctx->s);
+  else e = launch_coarse_group<double, float, float>(g->a, g->cols_d, R, g->blocks, g->groups, ctx->s);
+  CK(e);
+  int bar_err = 0;
+  CK(cudaMemcpyAsync(st.data(), g->st, st.size() * sizeof(LevelState), cudaMemcpyDeviceToHost, ctx->s));
+  CK(cudaMemcpyAsync(&bar_err, g->err, sizeof(int), cudaMemcpyDeviceToHost, ctx->s));
+  CK(cudaStreamSynchronize(ctx->s));
+  if (bar_err) {
+    set_err(ctx, "batched solve: a barrier timed out; the result is invalid");
+    return KCMG_CUDA_ERROR;
+  }
+  CK(cudaMemcpyAsync(x, g->x, NR * sizeof(double), cudaMemcpyDefault, ctx->s));
+  CK(cudaStreamSynchronize(ctx->s));
+  double worst = 0.0, res0 = 0.0;
+  bool all_ok = true, finite = true;
+  int status = KCMG_OK, its = 0, restarts = 0;
+  int lit[KCMG_MAX_LEVELS] = {0};
+  for (int j = 0; j < R; ++j) {
+    const LevelState* h = &st[(size_t)j * nl];
+    finite = finite && std::isfinite(h->rnorm);
+    worst = std::max(worst, h->rnorm0 > 0 ? h->rnorm / h->rnorm0 : 0.0);
+    res0 = std::max(res0, h->rnorm0);
+    all_ok = all_ok && h->rnorm <= fmax(rtol * h->rnorm0, atol);
+    if (h->status == KCMG_NONFINITE || status == KCMG_OK) status = h->status;
+    its = std::max(its, h->it);
+    restarts = std::max(restarts, h->nrestart);
+    for (int l = 0; l < nl - 1; ++l) lit[l] = std::max(lit[l], h[l].iters_total);
+  }
+  if (info) {
+    info->iters = its;
+    for (int l = 0; l < KCMG_MAX_LEVELS; ++l) info->level_iters[l] = lit[l];
+    info->restarts = restarts;
+    info->refinements = ctx->mixed ? restarts + 1 : 0;
+    info->res0 = res0;
+    info->rel_res = worst;
+    info->kernel_launches = 1;
+    // active columns at every level-0 loop test (type 5)
+    int m = 0;
+    if (info->hist && info->hist_type && info->hist_cap > 0) {
+      m = std::min(info->hist_cap, its + 1);
+      std::vector<double> hv(m, 0.0);
+      std::vector<int> ht(m, 5);
+      for (int j = 0; j < R; ++j) {
+        const LevelState& h = st[(size_t)j * nl];
+        const bool conv = h.rnorm <= fmax(rtol * h.rnorm0, atol);
+        for (int k = 0; k < m; ++k) hv[k] += k < h.it || (k == h.it && !conv);
+      }
+      CK(cudaMemcpy(info->hist, hv.data(), m * sizeof(double), cudaMemcpyDefault));
+      CK(cudaMemcpy(info->hist_type, ht.data(), m * sizeof(int), cudaMemcpyDefault));
+    }
+    info->hist_len = m;
+  }
+  if (status != KCMG_OK) return (kcmg_status)status;
+  if (!finite) return KCMG_NONFINITE;
+  return all_ok ? KCMG_OK : KCMG_NOT_CONVERGED;
+}
+
 // batched solve of nrhs > 1 columns on the hierarchy of ctx
 kcmg_status solve_multi(kcmg_ctx* ctx, const double* b, double* x, int nrhs, double rtol, double atol,
                         int maxiter, kcmg_info* info) {
+  ctx->multi_nrhs = nrhs;
+  if (ColumnGroups* g = column_groups(ctx, nrhs)) return solve_groups(ctx, g, b, x, rtol, atol, maxiter, info);
   return mrhs_solve(&ctx->mrhs, mrhs_view(ctx), b, x, nrhs, rtol, atol, maxiter, info, &ctx->err);
 }
 
@@ -1125,6 +1355,7 @@ void kcmg_destroy(kcmg_ctx* ctx) {
   if (ctx->adj && ctx->adj != ctx) kcmg_destroy(ctx->adj);
   if (ctx->s) cudaStreamSynchronize(ctx->s);
   if (ctx->mrhs) mrhs_destroy(ctx->mrhs);
+  drop_groups(ctx);
   if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
   for (void* p : ctx->allocs) cudaFree(p);
   if (ctx->stage_big) cudaFree(ctx->stage_big);
@@ -1217,6 +1448,8 @@ kcmg_ctx* build_ctx(const kcmg_params* p, cudaStream_t user, const double* block
     copy_in(ctx, ctx->P64, p->prolong, ctx->nch * bs);
     ctx->P32 = dalloc<float>(ctx, ctx->nch * bs);
     launch_convert<double, float>(ctx->P64, ctx->P32, ctx->nch * bs, ctx->s);
+    ctx->fmas0 = (long long)ctx->np * ctx->np * ctx->S;
+    for (int j = 0; j < ctx->dim; ++j) ctx->fmas0 *= p->n[j];
     ctx->whole = whole_solve(ctx);
     build_hierarchy(ctx, blocks_override ? blocks_override : p->blocks);
     if (p->mf_nu || p->mf_F) {   // matrix-free level-0 coupling for the FP32 sweeps
@@ -1306,7 +1539,7 @@ kcmg_ctx* build_ctx(const kcmg_params* p, cudaStream_t user, const double* block
       a.bar_gen = dalloc<unsigned int>(ctx, 1);
       a.err = dalloc<int>(ctx, 1);
       CK(cudaMemsetAsync(a.bar_gen, 0, sizeof(unsigned int), ctx->s));
-      for (int l = ctx->whole ? 0 : 1; l < ctx->nlev; ++l) {
+      for (int l = 0; l < ctx->nlev; ++l) {
         Level& L = ctx->lv[l];
         CoarseLevel& c = a.lv[l];
         c.A = ctx->ir ? (const void*)L.A32 : (const void*)L.A64;      // Alg. 1 operator
@@ -1700,6 +1933,7 @@ kcmg_status kcmg_apply_multi(kcmg_ctx* ctx, int level, int nrhs, const double* x
     REQUIRE(level >= 0 && level < ctx->nlev - 1 && x && y, "bad level or null vector");
     REQUIRE(nrhs >= 2 && nrhs <= kMaxRhs, "nrhs must be in [2, %d]", kMaxRhs);
     REQUIRE(!ctx->ir, "batched calls support the FP64 and mixed forms");
+    ctx->multi_nrhs = nrhs;
     kcmg_status st = mrhs_ensure(&ctx->mrhs, mrhs_view(ctx), nrhs, &ctx->err);
     if (st != KCMG_OK) return st;
     return mrhs_apply(ctx->mrhs, level, x, y, in_place_ok(ctx, x, y, (size_t)ctx->lv[level].N * nrhs));
@@ -1711,6 +1945,7 @@ kcmg_status kcmg_smooth_multi(kcmg_ctx* ctx, int level, int nrhs, const double* 
     REQUIRE(level >= 0 && level < ctx->nlev - 1 && r && z, "bad level or null vector");
     REQUIRE(nrhs >= 2 && nrhs <= kMaxRhs, "nrhs must be in [2, %d]", kMaxRhs);
     REQUIRE(!ctx->ir, "batched calls support the FP64 and mixed forms");
+    ctx->multi_nrhs = nrhs;
     kcmg_status st = mrhs_ensure(&ctx->mrhs, mrhs_view(ctx), nrhs, &ctx->err);
     if (st != KCMG_OK) return st;
     return mrhs_smooth(ctx->mrhs, level, r, z, in_place_ok(ctx, r, z, (size_t)ctx->lv[level].N * nrhs));
@@ -1721,7 +1956,9 @@ kcmg_status kcmg_mrhs_tuning(kcmg_ctx* ctx, double* out, int nout) {
   return guarded(ctx, [&]() -> kcmg_status {
     REQUIRE(out && nout >= 1, "out must hold at least one value");
     for (int i = 0; i < nout; ++i) out[i] = 0.0;
-    REQUIRE(ctx->mrhs, "no multi-right-hand-side solve has run on this context");
+    REQUIRE(ctx->multi_nrhs, "no multi-right-hand-side solve has run on this context");
+    kcmg_status st = mrhs_ensure(&ctx->mrhs, mrhs_view(ctx), ctx->multi_nrhs, &ctx->err);
+    if (st != KCMG_OK) return st;
     mrhs_tuning(ctx->mrhs, out, nout);
     return KCMG_OK;
   });

@@ -246,6 +246,11 @@ struct CoarseArgs {
   void* zc;
   double* hist;
   int* hist_type;
+  // one of several columns, each solved by its own group of blocks: the column of the caller's
+  // [N][io_stride] right-hand sides and iterates (null: level 0's vectors are set before the launch)
+  const double* io_b;
+  double* io_x;
+  int io_stride;
   double* partial;             // 2 buffers of partial_stride doubles
   size_t partial_stride;       // grid * (cols + 4)
   double* red;                 // cols + 4 reduced sums
@@ -273,6 +278,13 @@ template <typename TV, typename T, typename TI>
 cudaError_t coarse_cycle_prepare(CoarseArgs* a, int* grid);
 template <typename TV, typename T, typename TI>
 cudaError_t launch_coarse_cycle(const CoarseArgs& a, int grid, cudaStream_t s);
+// the same for ncol columns at once: blocks of one column's group, the groups that run at a time
+// and a's shared-memory layout; cols: the columns' arguments on the device
+template <typename TV, typename T, typename TI>
+cudaError_t coarse_group_prepare(CoarseArgs* a, int ncol, int* blocks, int* groups);
+template <typename TV, typename T, typename TI>
+cudaError_t launch_coarse_group(const CoarseArgs& a, const CoarseArgs* cols, int ncol, int blocks, int groups,
+                                cudaStream_t s);
 
 // finest-level FP64 operator of a context, for the no-allocation residual (noalloc.cu)
 struct Level0View {
