@@ -100,12 +100,13 @@ static __device__ void epilogue(const EpiArgs& e, const double* sums) {
       if (!isfinite(naz2) && st->level == 0) st->status = KCMG_NONFINITE;
       st->flags = f;
     } break;
-    // the second pass: w' = w - W h.  A w' that loses most of its norm again, or falls below brk
-    // relative to ||A z||, is rounding noise: the correction depends linearly on the basis
+    // the second pass: w' = w - W h.  What is left of it after this pass is kept, however much of
+    // its norm it loses again (in FP32 often most of it), while the norm can be told from rounding
+    // and is above brk relative to ||A z||
     case EPI_GRAM2: {
       const int l = st->l;
       const double n2 = sums[l], nw2 = n2 - sums[l + 2];
-      if (!isfinite(nw2) || !(nw2 >= 0.25 * n2) || !(nw2 > st->brk * st->brk * st->naz2)) {
+      if (!isfinite(nw2) || !(nw2 > e.dep * n2) || !(nw2 > st->brk * st->brk * st->naz2)) {
         st->flags |= F_DISCARD;
         if (!isfinite(n2) && st->level == 0) st->status = KCMG_NONFINITE;
       } else {

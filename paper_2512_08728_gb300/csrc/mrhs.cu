@@ -207,8 +207,8 @@ __device__ void mctl_step(const CtlArgs& c, unsigned kind) {
         f_reorth = reorth;
         break;
       }
-      // w' = w - W h: one that loses most of its norm again, or falls below brk_tol relative to
-      // ||A z||, is rounding noise (linear dependence)
+      // w' = w - W h: kept while what this pass leaves can be told from rounding and is above
+      // brk_tol relative to ||A z||
       case CTL_GRAM2: {
         if (st->flags[r] & MF_REORTH) {
           const int l = st->l[r];
@@ -221,7 +221,7 @@ __device__ void mctl_step(const CtlArgs& c, unsigned kind) {
             cw[(size_t)i * 32 + r] = h2;
           }
           const double n2 = __ldcg(sums + (size_t)lcap * 32 + r), nw2 = n2 - hh;
-          if (!isfinite(nw2) || !(nw2 >= 0.25 * n2) || !(nw2 > st->brk_tol * st->brk_tol * st->naz2[r])) {
+          if (!isfinite(nw2) || !(nw2 > kDependent64 * n2) || !(nw2 > st->brk_tol * st->brk_tol * st->naz2[r])) {
             st->flags[r] |= MF_DISCARD;
           } else {
             st->gam[r] = 1.0 / sqrt(nw2);
