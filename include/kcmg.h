@@ -277,7 +277,8 @@ kcmg_status kcmg_kernel_report(kcmg_ctx *ctx, int reps, double *out, int nout);
    scratch and it keeps the last call's contents (the reduction counter is cleared at every
    call): calls that overlap on the GPU (other streams, other host threads, other contexts
    on the same device) race and must not be issued.  Stream-ordered on the context's
-   stream; it copies ||r|| to host memory and synchronises that stream before returning. */
+   stream; the kernel writes ||r|| to host memory that kcmg_setup allocated, and the call
+   synchronises that stream before returning. */
 kcmg_status kcmg_residual_noalloc(kcmg_ctx *ctx, const double *b, const double *x, double *r,
                                   double *rnorm);
 

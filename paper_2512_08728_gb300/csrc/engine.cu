@@ -76,6 +76,7 @@ struct kcmg_ctx {
   bool ir = false;                    // FP64 iterative refinement around an FP32 inner solve
   double *xo = nullptr, *bo = nullptr, *xt = nullptr;   // its FP64 outer x, b and trial x
   double* na_scratch = nullptr;       // static scratch of kcmg_residual_noalloc on dev
+  double* na_norm = nullptr;          // and its norm's place in host memory
   bool mixed = false;
   cudaStream_t user = nullptr, s = nullptr;
   cudaStream_t cap[KCMG_MAX_LEVELS + 2] = {};
@@ -1635,7 +1636,7 @@ kcmg_ctx* build_ctx(const kcmg_params* p, cudaStream_t user, const double* block
     ctx->stage_in = dalloc<double>(ctx, maxN);
     ctx->stage_out = dalloc<double>(ctx, maxN);
     // the no-allocation residual's static scratch on this device (address and kernels)
-    CK(noalloc_prepare(dev, &ctx->na_scratch));
+    CK(noalloc_prepare(dev, &ctx->na_scratch, &ctx->na_norm));
     if (ctx->lv[0].pat) CK(pattern_residual_load(ctx->np, ctx->dim));
     CK(cudaStreamSynchronize(ctx->s));
     *out_status = KCMG_OK;
@@ -2192,7 +2193,7 @@ kcmg_status kcmg_residual_noalloc(kcmg_ctx* ctx, const double* b, const double* 
     }
     const Level& L = ctx->lv[0];
     Level0View v{L.pat ? L.V64 : L.A64, L.nbr, L.N, L.G, L.rows_pad, L.block_rows, ctx->np, ctx->dim, ctx->s,
-                 ctx->na_scratch, L.pat, {L.n[0], L.n[1], L.n[2]}};
+                 ctx->na_scratch, ctx->na_norm, L.pat, {L.n[0], L.n[1], L.n[2]}};
     // run on the context's device (its scratch address, operator and stream live there)
     int cur = 0;
     CK(cudaGetDevice(&cur));

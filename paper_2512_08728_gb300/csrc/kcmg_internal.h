@@ -151,7 +151,7 @@ template <typename T, typename TI, typename TR, typename TZ>
 void launch_pattern_sweep(int np, int dim, const int* n, const T* V, const TI* D, const TR* r, T* r_lo, const T* zold,
                           TZ* znew, double omega, int first, cudaStream_t s);
 void launch_pattern_residual_scratch(int np, int dim, const int* n, const double* V, const double* x, const double* b,
-                                     double* r, double* scratch, int norm_at, cudaStream_t s);
+                                     double* r, double* scratch, int count_at, double* norm, cudaStream_t s);
 cudaError_t pattern_residual_load(int np, int dim);       // load that kernel's code now
 
 // additive Schwarz smoother on cell patches (schwarz.cu, schwarz.cuh)
@@ -301,12 +301,13 @@ struct Level0View {
   int N, G, rows_pad, block_rows, np, dim;
   cudaStream_t stream;
   double* scratch;   // device address of the static scratch (from noalloc_prepare)
+  double* norm;      // the norm's place in page-locked host memory (from noalloc_prepare)
   bool pat;          // A holds the pattern kernels' storage
   int n[3];
 };
 // With device dev current: look up the static scratch's device address (once per device)
 // and load the no-allocation kernels.  Called by kcmg_setup.
-cudaError_t noalloc_prepare(int dev, double** scratch);
+cudaError_t noalloc_prepare(int dev, double** scratch, double** norm);
 cudaError_t residual_noalloc(const Level0View& v, const double* b, const double* x, double* r,
                              double* rnorm_host, int* too_large);
 

@@ -12,9 +12,9 @@
 // in buffers the context allocates.  This variant keeps them in one file-scope static
 // device array instead, so the call itself allocates nothing (no cudaMalloc, no cudaFree,
 // no allocating library routine).  kcmg_setup looks up the array's device address (with
-// the context's device current) and loads this file's kernels, so that a later call does
-// no set-up of its own.  The call reads ||r|| into host memory and synchronises the
-// context's stream before it returns.
+// the context's device current), allocates the norm's place in page-locked host memory (once a
+// device) and loads this file's kernels, so that a later call does no set-up of its own.  The
+// kernel writes ||r|| there and the call synchronises its stream before it returns.
 #include "kcmg_internal.h"
 
 #include <mutex>
@@ -22,7 +22,7 @@
 namespace kcmg {
 
 // Scratch of the no-allocation residual: [0, kNoallocMaxBlocks) block partial sums, then
-// the norm, then the reduction counter.  Every GPU that loads the library holds it (257 KB)
+// the reduction counter.  Every GPU that loads the library holds it (257 KB)
 // until the process exits.  All calls share it and it keeps the last call's contents.
 constexpr int kNoallocMaxBlocks = 32768;
 constexpr int kNoallocDoubles = kNoallocMaxBlocks + 64;
@@ -54,7 +54,7 @@ template <int NP, int S>
 __global__ void __launch_bounds__(320)
 k_residual_noalloc(const double* __restrict__ A, const int* __restrict__ nbr, int N, int G,
                    const double* __restrict__ x, const double* __restrict__ b, double* __restrict__ r,
-                   double* scratch) {
+                   double* scratch, double* norm) {
   constexpr int JP = (NP + 1) / 2;
   constexpr int NF = S - 1;
   __shared__ double sh[32];
@@ -82,7 +82,7 @@ k_residual_noalloc(const double* __restrict__ A, const int* __restrict__ nbr, in
     r[row] = out;
   }
   const double part = na_block_sum(out * out, sh);
-  unsigned int* counter = reinterpret_cast<unsigned int*>(scratch + kNoallocMaxBlocks + 1);
+  unsigned int* counter = reinterpret_cast<unsigned int*>(scratch + kNoallocMaxBlocks);
   if (threadIdx.x == 0) {
     scratch[blockIdx.x] = part;
     __threadfence();
@@ -94,7 +94,7 @@ k_residual_noalloc(const double* __restrict__ A, const int* __restrict__ nbr, in
     for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) t += __ldcg(scratch + i);
     t = na_block_sum(t, sh);
     if (threadIdx.x == 0) {
-      scratch[kNoallocMaxBlocks] = sqrt(t);
+      *norm = sqrt(t);
       *counter = 0u;
     }
   }
@@ -103,10 +103,11 @@ k_residual_noalloc(const double* __restrict__ A, const int* __restrict__ nbr, in
 // device address of the scratch, looked up once per device
 std::mutex g_na_mutex;
 void* g_na_ptr[256] = {};
+double* g_na_norm[256] = {};   // the norm of each device's calls, in page-locked host memory
 
 }  // namespace
 
-cudaError_t noalloc_prepare(int dev, double** scratch) {
+cudaError_t noalloc_prepare(int dev, double** scratch, double** norm) {
   std::lock_guard<std::mutex> lock(g_na_mutex);
   if (dev < 0 || dev >= 256) return cudaErrorInvalidDevice;
   int cur = -1;
@@ -124,9 +125,13 @@ cudaError_t noalloc_prepare(int dev, double** scratch) {
                          (const void*)k_residual_noalloc<10, 7>, (const void*)k_residual_noalloc<20, 7>};
     for (const void* f : fns)
       if ((e = cudaFuncGetAttributes(&fa, f)) != cudaSuccess) return e;
+    if (!g_na_norm[dev] &&
+        (e = cudaHostAlloc((void**)&g_na_norm[dev], sizeof(double), cudaHostAllocPortable)) != cudaSuccess)
+      return e;
     g_na_ptr[dev] = p;
   }
   *scratch = static_cast<double*>(g_na_ptr[dev]);
+  *norm = g_na_norm[dev];
   return cudaSuccess;
 }
 
@@ -139,23 +144,24 @@ cudaError_t residual_noalloc(const Level0View& v, const double* b, const double*
   if (!scratch) return cudaErrorInvalidValue;
   cudaError_t e;
   // the counter must start at zero (the previous call may have been interrupted)
-  if ((e = cudaMemsetAsync(scratch + kNoallocMaxBlocks + 1, 0, sizeof(double), v.stream)) != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(scratch + kNoallocMaxBlocks, 0, sizeof(double), v.stream)) != cudaSuccess) return e;
   if (v.pat)
-    launch_pattern_residual_scratch(v.np, v.dim, v.n, v.A, x, b, r, scratch, kNoallocMaxBlocks, v.stream);
+    launch_pattern_residual_scratch(v.np, v.dim, v.n, v.A, x, b, r, scratch, kNoallocMaxBlocks, v.norm,
+                                    v.stream);
   else switch (v.np * 10 + v.dim) {
-    case 32: k_residual_noalloc<3, 5><<<grid, v.block_rows, 0, v.stream>>>(v.A, v.nbr, v.N, v.G, x, b, r, scratch); break;
-    case 62: k_residual_noalloc<6, 5><<<grid, v.block_rows, 0, v.stream>>>(v.A, v.nbr, v.N, v.G, x, b, r, scratch); break;
-    case 102: k_residual_noalloc<10, 5><<<grid, v.block_rows, 0, v.stream>>>(v.A, v.nbr, v.N, v.G, x, b, r, scratch); break;
-    case 43: k_residual_noalloc<4, 7><<<grid, v.block_rows, 0, v.stream>>>(v.A, v.nbr, v.N, v.G, x, b, r, scratch); break;
-    case 103: k_residual_noalloc<10, 7><<<grid, v.block_rows, 0, v.stream>>>(v.A, v.nbr, v.N, v.G, x, b, r, scratch); break;
-    case 203: k_residual_noalloc<20, 7><<<grid, v.block_rows, 0, v.stream>>>(v.A, v.nbr, v.N, v.G, x, b, r, scratch); break;
+    case 32: k_residual_noalloc<3, 5><<<grid, v.block_rows, 0, v.stream>>>(v.A, v.nbr, v.N, v.G, x, b, r, scratch, v.norm); break;
+    case 62: k_residual_noalloc<6, 5><<<grid, v.block_rows, 0, v.stream>>>(v.A, v.nbr, v.N, v.G, x, b, r, scratch, v.norm); break;
+    case 102: k_residual_noalloc<10, 5><<<grid, v.block_rows, 0, v.stream>>>(v.A, v.nbr, v.N, v.G, x, b, r, scratch, v.norm); break;
+    case 43: k_residual_noalloc<4, 7><<<grid, v.block_rows, 0, v.stream>>>(v.A, v.nbr, v.N, v.G, x, b, r, scratch, v.norm); break;
+    case 103: k_residual_noalloc<10, 7><<<grid, v.block_rows, 0, v.stream>>>(v.A, v.nbr, v.N, v.G, x, b, r, scratch, v.norm); break;
+    case 203: k_residual_noalloc<20, 7><<<grid, v.block_rows, 0, v.stream>>>(v.A, v.nbr, v.N, v.G, x, b, r, scratch, v.norm); break;
     default: return cudaErrorInvalidValue;
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if ((e = cudaMemcpyAsync(rnorm_host, scratch + kNoallocMaxBlocks, sizeof(double), cudaMemcpyDeviceToHost,
-                           v.stream)) != cudaSuccess)
-    return e;
-  return cudaStreamSynchronize(v.stream);
+  // the norm is in host memory when the kernel is done: no copy after it
+  if ((e = cudaStreamSynchronize(v.stream)) != cudaSuccess) return e;
+  *rnorm_host = *static_cast<volatile double*>(v.norm);
+  return cudaSuccess;
 }
 
 }  // namespace kcmg

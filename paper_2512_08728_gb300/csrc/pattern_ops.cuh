@@ -166,12 +166,13 @@ k_pat_sweep(const T* __restrict__ V, const TI* __restrict__ D, PatGrid gr, const
   });
 }
 
-// residual of the no-allocation call (noalloc.cu): r = b - A x, ||r||^2 through the caller's
-// scratch: [0, blocks) partial sums, then the norm at norm_at, a counter at norm_at + 1
+// residual of the no-allocation call (noalloc.cu): r = b - A x, ||r|| to *norm through the
+// caller's scratch: [0, blocks) partial sums, a counter at count_at
 template <int NP, int DIM, bool VEC>
 __global__ void __launch_bounds__(kPatThreads)
 k_pat_residual_scratch(const double* __restrict__ V, PatGrid gr, const double* __restrict__ x,
-                       const double* __restrict__ b, double* __restrict__ r, double* scratch, int norm_at) {
+                       const double* __restrict__ b, double* __restrict__ r, double* scratch, int count_at,
+                       double* norm) {
   constexpr int PARTS = TensorPattern<NP, DIM>::PARTS;
   __shared__ double sh[32 * 8];
   __shared__ int s_last;
@@ -195,7 +196,7 @@ k_pat_residual_scratch(const double* __restrict__ V, PatGrid gr, const double* _
     }
   });
   bsum_n<1>(nrm, sh);
-  unsigned int* counter = reinterpret_cast<unsigned int*>(scratch + norm_at + 1);
+  unsigned int* counter = reinterpret_cast<unsigned int*>(scratch + count_at);
   if (threadIdx.x == 0) {
     scratch[blockIdx.x] = nrm[0];
     __threadfence();
@@ -207,7 +208,7 @@ k_pat_residual_scratch(const double* __restrict__ V, PatGrid gr, const double* _
     for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) t[0] += __ldcg(scratch + i);
     bsum_n<1>(t, sh);
     if (threadIdx.x == 0) {
-      scratch[norm_at] = sqrt(t[0]);
+      *norm = sqrt(t[0]);
       *counter = 0u;
     }
   }

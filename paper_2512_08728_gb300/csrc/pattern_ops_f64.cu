@@ -51,14 +51,14 @@ void launch_pattern_residual_dd(int np, int dim, const int* n, const double* V, 
 }
 
 void launch_pattern_residual_scratch(int np, int dim, const int* n, const double* V, const double* x, const double* b,
-                                     double* r, double* scratch, int norm_at, cudaStream_t s) {
+                                     double* r, double* scratch, int count_at, double* norm, cudaStream_t s) {
   const PatGrid g = pat_grid(n, dim);
   KCMG_PAT(np, dim, {
     const int grid = pattern_blocks(np, dim, g.C);
     if (((uintptr_t)x & 15) == 0)
-      k_pat_residual_scratch<NP, DIM, true><<<grid, kPatThreads, 0, s>>>(V, g, x, b, r, scratch, norm_at);
+      k_pat_residual_scratch<NP, DIM, true><<<grid, kPatThreads, 0, s>>>(V, g, x, b, r, scratch, count_at, norm);
     else   // a caller's vector that does not start on the vector loads' boundary
-      k_pat_residual_scratch<NP, DIM, false><<<grid, kPatThreads, 0, s>>>(V, g, x, b, r, scratch, norm_at);
+      k_pat_residual_scratch<NP, DIM, false><<<grid, kPatThreads, 0, s>>>(V, g, x, b, r, scratch, count_at, norm);
   });
 }
 
