@@ -1,5 +1,5 @@
 // Persistent cooperative kernel for the coarse part of the K-cycle: MG(lambda) of Alg. 2
-// on every level below the finest, with the block-Jacobi smoother (Alg. BJ), residual
+// on the small levels below the finest (and, for small problems, on all levels), with the block-Jacobi smoother (Alg. BJ), residual
 // minimisation (Alg. 1), transfers, the level-local criteria of Sec. 4.2 and the dense
 // coarsest solve, all in one launch per finest-level cycle.
 //
@@ -21,15 +21,19 @@
 //   - Corrections are stored as they come; x = sum_k y_k z_k with R y = alpha (R: the
 //     orthogonalisation coefficients) is formed when the level returns or restarts, so Alg. 1's
 //     second recurrence costs one pass over the corrections per visit, not one per correction.
-//   - A level set too small to pay for a grid barrier runs in one block (cc_blocks()).
+//   - Levels too small to pay for a grid barrier run in one block while the others wait for it
+//     (cc_solo_from()); a reduction sums over the blocks that have cells of the level.
+//   - A small problem's finest level is part of the launch too (Alg. 2 on level 0, below), and
+//     several columns of one run side by side (k_coarse_group).
 //   - FP64 instructions are scarce (one of a warp takes its SM 16 clocks), so scalars are computed
 //     by one warp, sums over lanes are transposed (several columns at a time) and bytes are
 //     counted in integers.
 // Measured (GB300, one launch; first the kernel whose blocks took whole 320-row tiles, read every
 // neighbour value through L2 and reduced three times a minimisation): levels 16^3 and 8^3 at
 // np = 10 beside the finest level's kernels 971 -> 553 us; 64 x 48 and two levels below at
-// np = 10, 2-D, 16.7 -> 8.4 ms; 16^3 and 8^3 alone, 16 visits, 5.0 -> 2.7 ms; 192 unknowns
-// 749 -> 257 us.
+// np = 10, 2-D, 16.7 -> 8.2 ms; 16^3 and 8^3 alone, 16 visits, 5.0 -> 2.7 ms; 192 unknowns
+// 749 -> 257 us.  Whole solves to 1e-11, finest level on a kernel a step before: 16 x 16, np = 3,
+// 20.4 -> 13.5 ms; 8^3, np = 10, mixed, 28.3 -> 21.5 ms.
 // Every control decision is taken by all blocks from the same reduced values (fixed reduction
 // order), so all blocks follow the same path.  The grid barrier spins with a bound: if it ever
 // times out it raises an error flag and every block leaves the kernel, so a fault becomes a
@@ -639,7 +643,7 @@ struct CoarseCycle {
     // more than half of it (classical Gram-Schmidt, "twice is enough")
     double* Rc = R + (size_t)l * (l - 1) / 2;
     for (int pass = 0;; ++pass) {
-      judge(l, pass);
+      decide(l, pass);
       for (int i = threadIdx.x; i < l; i += blockDim.x) {
         cf[i] = red_s[i];
         if (own_coef()) Rc[i] = pass == 0 ? red_s[i] : Rc[i] + red_s[i];
@@ -685,7 +689,7 @@ struct CoarseCycle {
 
   // warp 0: the scalars of a Gram pass with l columns from red_s into rms (the caller's
   // __syncthreads publishes them)
-  __device__ void judge(int l, int pass) {
+  __device__ void decide(int l, int pass) {
     if (threadIdx.x >= 32) return;
     double hh = 0.0;
     for (int i = threadIdx.x; i < l; i += 32) hh = fma(red_s[i], red_s[i], hh);
@@ -872,7 +876,7 @@ struct CoarseCycle {
     }
   }
 
-  // ---------------------------------------------------------------- Alg. 2 on lev >= 1
+  // ---------------------------------------------------------------- Alg. 2
   // The recursion MG(lev) -> MG(lev + 1) of Alg. 2 runs as a loop over an explicit
   // per-level state (the levels form a chain, so a phase per level suffices).  On entry b, r = b
   // and x = 0 of level lev0 are set, r also in shared memory.  ||b|| comes with the first

@@ -39,7 +39,8 @@ struct Level {
   // matrix-free level-0 coupling (FP32 sweeps): coefficient per cell, face matrices
   float *mf_nu = nullptr, *mf_F = nullptr;
   // finest level with a tensor basis's zero pattern: the nonzero entries and the inverses in the
-  // pattern kernels' layout (pattern_ops.cuh); A64, D64, A32, D32, D16 are then not stored
+  // pattern kernels' layout (pattern_ops.cuh); A64, D64, A32, D32, D16 are then not stored, unless
+  // the persistent kernel runs this level too
   bool pat = false;
   double *V64 = nullptr, *PD64 = nullptr;
   float *V32 = nullptr, *PD32 = nullptr;
@@ -1197,7 +1198,6 @@ ColumnGroups* column_groups(kcmg_ctx* ctx, int nrhs) {
         L.z = take(v);
         L.s0 = take(ctx->mixed ? v / 2 : v);   // smoother scratch, in its precision
         L.s1 = take(ctx->mixed ? v / 2 : v);
-        L.t = L.w = L.wre = nullptr;
         L.W = take(v * L.lcap);
         L.Z = take(v * L.lcap);
         L.st = g->st + (size_t)j * ctx->nlev + l;
@@ -1572,7 +1572,7 @@ kcmg_ctx* build_ctx(const kcmg_params* p, cudaStream_t user, const double* block
         c.N = L.N;
         c.G = L.G;
         c.rows_pad = L.rows_pad;
-        c.x = L.x; c.r = L.r; c.b = L.b; c.z = L.z; c.t = L.t; c.w = L.w; c.wre = L.wre;
+        c.x = L.x; c.r = L.r; c.b = L.b; c.z = L.z;
         c.W = L.W; c.Z = L.Z;
         c.lcap = L.lcap;
         c.maxit = p->lvl_maxit[l];

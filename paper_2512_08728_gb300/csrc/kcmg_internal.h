@@ -227,7 +227,7 @@ struct CoarseLevel {
   const int* nbr;
   int n[3];
   int N, G, rows_pad;
-  void *x, *r, *b, *z, *t, *w, *wre, *W, *Z;
+  void *x, *r, *b, *z, *W, *Z;
   int lcap, maxit;
   double rtol;
   LevelState* st;       // iteration/restart counters for the report
