@@ -49,6 +49,7 @@ struct Level {
   int nblk = 1;                     // blocks of the multi-column dot kernels
   int nblk2 = 1;                    // blocks of the update / finish / norm kernels
   double *h = nullptr, *h2 = nullptr, *partial = nullptr;
+  RmCoef co{};
   LevelState* st = nullptr;
 };
 
@@ -248,6 +249,10 @@ void alloc_cycle_vectors(kcmg_ctx* ctx, Level& L, int lcap) {
   L.Z = dalloc<T>(ctx, N * lcap);
   L.h = dalloc<double>(ctx, lcap);
   L.h2 = dalloc<double>(ctx, lcap);
+  L.co.gm = dalloc<double>(ctx, 3 * (size_t)lcap + (size_t)lcap * (lcap - 1) / 2);
+  L.co.al = L.co.gm + lcap;
+  L.co.y = L.co.al + lcap;
+  L.co.R = L.co.y + lcap;
   const size_t spmv_blocks = L.rows_pad / L.block_rows;
   size_t plen = (size_t)kDotBlocksMax * (lcap + 2);
   if (spmv_blocks > plen) plen = spmv_blocks;
@@ -611,7 +616,15 @@ struct Cycle {
     EpiArgs fin = epi(lev, EPI_FINISH);
     fin.end_iter = end_iter;
     fin.hist_type = htype;
-    launch_gram_update<V>(W, Z, L.N, w, wre, z, static_cast<V*>(L.x), r, L.lcap, L.nblk2, L.partial, fin, s);
+    launch_gram_update<V>(W, Z, L.N, w, wre, z, L.co, r, L.lcap, L.nblk2, L.partial, fin, s);
+  }
+
+  // x of the level from its corrections: before a restart (conditional), or when its loop is over
+  template <typename V>
+  void update_x(int lev, int conditional, cudaStream_t s) {
+    Level& L = ctx->lv[lev];
+    launches += 2;
+    launch_x_update<V>(static_cast<V*>(L.Z), L.N, static_cast<V*>(L.x), L.st, L.co, L.lcap, L.nblk2, conditional, s);
   }
 
   // one pass of the while body of Alg. 2 on level lev; V is the level's vector type
@@ -654,6 +667,7 @@ struct Cycle {
     rm<V>(lev, static_cast<V*>(L.z), 0, 2, s);
     z = smooth<V>(lev, static_cast<V*>(L.r), s);                           // post-smoother
     rm<V>(lev, z, 1, 3, s);
+    update_x<V>(lev, 1, s);
     // restart check: r = b - A x on request, then the loop condition of this level
     // (compensated on level 0, where the tolerance can sit near the attainable accuracy)
     if (lev == 0 && std::is_same<V, double>::value)
@@ -722,6 +736,7 @@ struct Cycle {
     CK(cudaEventRecord(ctx->join_ev, cs));                               // join
     CK(cudaStreamWaitEvent(s, ctx->join_ev, 0));
     rm<V>(0, reinterpret_cast<const V*>(ctx->zc), 1, 2, s);
+    update_x<V>(0, 1, s);
     launches += 1;                                                       // restart check
     if (std::is_same<V, double>::value)
       apply_residual_dd(ctx, L, (const double*)L.x, (double*)L.r, (const double*)L.b, L.partial,
@@ -752,6 +767,7 @@ struct Cycle {
         if (task_parallel) body_async<V>(s);
         else body<V>(lev, s);
       }
+      update_x<V>(lev, 0, s);
       return;
     }
     cudaGraph_t g;
@@ -780,6 +796,7 @@ struct Cycle {
     body_kernels[lev] = loop_total[lev] - loop_total[lev + 1];
     if (lev == 0) body_launches = launches - before;
     CK(cudaStreamEndCapture(bs, nullptr));
+    update_x<V>(lev, 0, s);
   }
 
   // level 0: r0 = b - A x0 (compensated FP64; FP32 in the inner solve of the
@@ -913,7 +930,7 @@ void read_states(kcmg_ctx* ctx, StateReport& rep) {
 // kernels of one run of the cycle, from the loop-body counts and the executed bodies
 long long cycle_launches(const kcmg_ctx* ctx, const StateReport& rep) {
   if (ctx->last_launches != -2) return ctx->last_launches + 1;
-  long long n = 2;                  // initial and final residual
+  long long n = 4;                  // initial and final residual, x from the last basis
   for (int l = 0; l < ctx->nlev; ++l) n += (long long)rep.st[l].guard * ctx->graph_body_kernels[l];
   return n;
 }
@@ -1901,6 +1918,7 @@ void rm_sequence_impl(kcmg_ctx* ctx, int level, const double* z, int ncorr) {
     load_vec(ctx, level, L.z, z + (size_t)k * L.N, L.N);
     cy.template rm<V>(level, static_cast<V*>(L.z), 0, 1, ctx->s);
   }
+  cy.template update_x<V>(level, 0, ctx->s);
 }
 }  // namespace
 
@@ -2157,19 +2175,17 @@ kcmg_status kcmg_kernel_report(kcmg_ctx* ctx, int reps, double* out, int nout) {
           if (ctx->ir)
             launch_gram_update<float>(static_cast<float*>(L.W), static_cast<float*>(L.Z), L.N,
                                       static_cast<float*>(L.w), static_cast<float*>(L.wre),
-                                      static_cast<float*>(L.z), static_cast<float*>(L.x), static_cast<float*>(L.r),
-                                      L.lcap, L.nblk2, L.partial, up, ctx->s);
+                                      static_cast<float*>(L.z), L.co, static_cast<float*>(L.r), L.lcap, L.nblk2, L.partial, up, ctx->s);
           else
             launch_gram_update<double>(static_cast<double*>(L.W), static_cast<double*>(L.Z), L.N,
                                        static_cast<double*>(L.w), static_cast<double*>(L.wre),
-                                       static_cast<double*>(L.z), static_cast<double*>(L.x),
-                                       static_cast<double*>(L.r), L.lcap, L.nblk2, L.partial, up, ctx->s);
+                                       static_cast<double*>(L.z), L.co, static_cast<double*>(L.r), L.lcap, L.nblk2, L.partial, up, ctx->s);
         }
         CK(cudaEventRecord(e1, ctx->s));
         CK(cudaEventSynchronize(e1));
         CK(cudaEventElapsedTime(&ms, e0, e1));
         out[o1 + 6] = ms / reps;
-        out[o1 + 7] = 4.0 * lt * L.N;
+        out[o1 + 7] = 2.0 * lt * L.N;
         out[o1 + 8] = lt;
       }
       CK(cudaGetLastError());

@@ -46,6 +46,12 @@ struct LevelState {
   double brk;       // breakdown threshold relative to ||A z||
 };
 
+// Coefficients of Alg. 1 for a level's whole basis, A Z = W R: R's columns above the diagonal
+// (column k at k (k - 1) / 2), its diagonal's inverse gm, alpha = W^T r0 and y = R^{-1} alpha
+struct RmCoef {
+  double *gm, *al, *y, *R;
+};
+
 enum EpiKind : int {
   EPI_NONE = 0,
   EPI_MG_BEGIN,     // sum = ||r0||^2: start of an MG call on the level
@@ -113,8 +119,12 @@ template <typename T>
 void launch_gram_apply(const T* W, int N, const T* w, T* wout, int lcap, int nblk,
                        LevelState* st, const double* h, cudaStream_t s);
 template <typename T>
-void launch_gram_update(T* W, T* Z, int N, const T* w, const T* wre, const T* z, T* x, T* r, int lcap, int nblk,
-                        double* partial, const EpiArgs& e, cudaStream_t s);
+void launch_gram_update(T* W, T* Z, int N, const T* w, const T* wre, const T* z, const RmCoef& co, T* r, int lcap,
+                        int nblk, double* partial, const EpiArgs& e, cudaStream_t s);
+// x += Z y with R y = alpha; conditional: only if the level restarts
+template <typename T>
+void launch_x_update(const T* Z, int N, T* x, const LevelState* st, const RmCoef& co, int lcap, int nblk,
+                     int conditional, cudaStream_t s);
 template <typename T>
 void launch_norm(const T* v, int N, int nblk, double* partial, const EpiArgs& e,
                  cudaStream_t s);

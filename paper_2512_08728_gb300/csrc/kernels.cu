@@ -428,21 +428,22 @@ k_gram_apply(const T* __restrict__ W, int N, const T* __restrict__ w, T* __restr
   }
 }
 
-// The step of Alg. 1: w_l = gamma (w_src - W c_w), z_l = gamma (z - Z c_z) written to column l
-// of W and Z, x += alpha z_l, r -= alpha w_l; ||r||^2 -> EPI_FINISH.  gamma and alpha are known
-// from the Gram pass, so the column is normalised and applied as it is formed: the pass that read
-// the two new columns again to normalise them, and read and wrote x and r, is gone (8^3 mixed solve
-// 30.1 -> 28.3 ms, 2-D 128 x 96 16.4 -> 16.0, launches being what they spend most on).  Without
-// reorthogonalisation w_src = w, c_w = c_z = h; with it w_src = w' = w - W h, c_w = h2,
-// c_z = h + h2.  A discarded correction leaves W, Z, x, r unchanged.  With PAIR (N even) a thread
-// takes two consecutive elements with one 16-byte (FP64) / 8-byte (FP32) load per column.
+// The step of Alg. 1: w_l = gamma (w_src - W c) as column l of W, r -= alpha w_l; ||r||^2 ->
+// EPI_FINISH.  gamma and alpha are known from the Gram pass, so the column is normalised and applied
+// as it is formed.  Without reorthogonalisation w_src = w, c = h; with it w_src = w' = w - W h,
+// c = h2.  The correction itself is stored as it comes, with its column of R (h, or h + h2):
+// A Z = W R with R_ll = 1 / gamma_l, so x follows from R y = alpha when it is needed (k_solve_y,
+// k_x_update), and the second recurrence z - Z h of Alg. 1, as much FP64 work as the first, is
+// gone: 64^3, np = 10, m = 12, five cycles 195.4 -> 182.7 ms.
+// A discarded correction leaves W, Z, r unchanged.  With PAIR (N even) a thread takes two
+// consecutive elements with one 16-byte (FP64) / 8-byte (FP32) load per column.
 template <typename T, bool PAIR>
 __global__ void __launch_bounds__(kVecThreads)
 k_gram_update(T* W, T* Z, int N, const T* __restrict__ w, const T* __restrict__ wre,
-              const T* __restrict__ z, T* __restrict__ x, T* __restrict__ r, double* partial, EpiArgs e) {
+              const T* __restrict__ z, RmCoef co, T* __restrict__ r, double* partial, EpiArgs e) {
   using T2 = typename Pair<T>::type;
   LevelState* st = e.st;
-  extern __shared__ double cs[];  // [2][l]
+  extern __shared__ double cs[];  // [l]
   __shared__ double sh[32 * 8];   // bsum_n<NC> needs 32 * NC
   const int l = st->l;
   const bool re = (st->flags & F_REORTH) != 0, keep = !(st->flags & F_DISCARD);
@@ -450,8 +451,12 @@ k_gram_update(T* W, T* Z, int N, const T* __restrict__ w, const T* __restrict__ 
   if (keep)
     for (int i = threadIdx.x; i < l; i += blockDim.x) {
       cs[i] = re ? e.h2[i] : e.h[i];
-      cs[l + i] = re ? e.h[i] + e.h2[i] : e.h[i];
+      if (blockIdx.x == 0) co.R[(size_t)l * (l - 1) / 2 + i] = re ? e.h[i] + e.h2[i] : e.h[i];
     }
+  if (keep && blockIdx.x == 0 && threadIdx.x == 0) {
+    co.gm[l] = st->gamma;
+    co.al[l] = st->alpha;
+  }
   __syncthreads();
   const T* ws = re ? wre : w;
   T* Wl = W + (size_t)l * N;
@@ -462,27 +467,18 @@ k_gram_update(T* W, T* Z, int N, const T* __restrict__ w, const T* __restrict__ 
     for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < units; u += gridDim.x * blockDim.x) {
       T2 rv = reinterpret_cast<const T2*>(r)[u];
       if (keep) {
-        T2 a = __ldg(reinterpret_cast<const T2*>(ws) + u), c = __ldg(reinterpret_cast<const T2*>(z) + u);
-        T2 xv = reinterpret_cast<const T2*>(x)[u];
+        T2 a = __ldg(reinterpret_cast<const T2*>(ws) + u);
+        reinterpret_cast<T2*>(Zl)[u] = __ldg(reinterpret_cast<const T2*>(z) + u);
 #pragma unroll 4
         for (int i = 0; i < l; ++i) {
           const T2 wi = __ldg(reinterpret_cast<const T2*>(W + (size_t)i * N) + u);
-          const T2 zi = __ldg(reinterpret_cast<const T2*>(Z + (size_t)i * N) + u);
-          const T cw = (T)(-cs[i]), cz = (T)(-cs[l + i]);
+          const T cw = (T)(-cs[i]);
           a.x = fma(cw, wi.x, a.x);
           a.y = fma(cw, wi.y, a.y);
-          c.x = fma(cz, zi.x, c.x);
-          c.y = fma(cz, zi.y, c.y);
         }
         a.x *= gam;
         a.y *= gam;
-        c.x *= gam;
-        c.y *= gam;
         reinterpret_cast<T2*>(Wl)[u] = a;
-        reinterpret_cast<T2*>(Zl)[u] = c;
-        xv.x = fma(al, c.x, xv.x);
-        xv.y = fma(al, c.y, xv.y);
-        reinterpret_cast<T2*>(x)[u] = xv;
         rv.x = fma(-al, a.x, rv.x);
         rv.y = fma(-al, a.y, rv.y);
         reinterpret_cast<T2*>(r)[u] = rv;
@@ -494,17 +490,12 @@ k_gram_update(T* W, T* Z, int N, const T* __restrict__ w, const T* __restrict__ 
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < N; j += gridDim.x * blockDim.x) {
       T rv = r[j];
       if (keep) {
-        T a = ws[j], c = z[j];
+        T a = ws[j];
+        Zl[j] = z[j];
 #pragma unroll 4
-        for (int i = 0; i < l; ++i) {
-          a = fma((T)(-cs[i]), __ldg(W + (size_t)i * N + j), a);
-          c = fma((T)(-cs[l + i]), __ldg(Z + (size_t)i * N + j), c);
-        }
+        for (int i = 0; i < l; ++i) a = fma((T)(-cs[i]), __ldg(W + (size_t)i * N + j), a);
         a *= gam;
-        c *= gam;
         Wl[j] = a;
-        Zl[j] = c;
-        x[j] = fma(al, c, x[j]);
         rv = fma(-al, a, rv);
         r[j] = rv;
       }
@@ -513,6 +504,79 @@ k_gram_update(T* W, T* Z, int N, const T* __restrict__ w, const T* __restrict__ 
   }
   double v[1] = {(double)r2};
   finish_reduction<1>(v, partial, e, sh);
+}
+
+// R y = alpha by back substitution, one block; conditional: only if the level restarts.  One column
+// of R a step, the next one's entries loaded meanwhile: about an L2 round trip a step.
+constexpr int kSolveThreads = 512;
+__global__ void __launch_bounds__(kSolveThreads) k_solve_y(const LevelState* st, RmCoef co, int conditional) {
+  if (conditional && !st->restart_req) return;
+  extern __shared__ double cf[];
+  constexpr int PER = kLcapMax / kSolveThreads;
+  const int l = st->l;
+  for (int i = threadIdx.x; i < l; i += kSolveThreads) cf[i] = co.al[i];
+  double nx[PER], g = l > 0 ? co.gm[l - 1] : 0.0;
+  auto column = [&](int k) {
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+      const int i = threadIdx.x + p * kSolveThreads;
+      nx[p] = i < k ? co.R[(size_t)k * (k - 1) / 2 + i] : 0.0;
+    }
+  };
+  if (l > 0) column(l - 1);
+  __syncthreads();
+  for (int k = l - 1; k >= 0; --k) {
+    const double y = cf[k] * g;
+    double cur[PER];
+#pragma unroll
+    for (int p = 0; p < PER; ++p) cur[p] = nx[p];
+    if (k > 0) {
+      g = co.gm[k - 1];
+      column(k - 1);
+    }
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+      const int i = threadIdx.x + p * kSolveThreads;
+      if (i < k) cf[i] = fma(-cur[p], y, cf[i]);
+    }
+    if (threadIdx.x == 0) co.y[k] = y;
+    __syncthreads();
+  }
+}
+
+// x += Z y (FP64 coefficients, vectors in T)
+template <typename T, bool PAIR>
+__global__ void __launch_bounds__(kVecThreads)
+k_x_update(const T* __restrict__ Z, int N, T* __restrict__ x, const LevelState* st, RmCoef co, int conditional) {
+  using T2 = typename Pair<T>::type;
+  if (conditional && !st->restart_req) return;
+  extern __shared__ double ys[];
+  const int l = st->l;
+  if (l == 0) return;
+  for (int i = threadIdx.x; i < l; i += blockDim.x) ys[i] = co.y[i];
+  __syncthreads();
+  const int units = PAIR ? N / 2 : N;
+  for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < units; u += gridDim.x * blockDim.x) {
+    if (PAIR) {
+      T2 s = {T(0), T(0)};
+#pragma unroll 4
+      for (int i = 0; i < l; ++i) {
+        const T2 zi = __ldg(reinterpret_cast<const T2*>(Z + (size_t)i * N) + u);
+        const T y = (T)ys[i];
+        s.x = fma(y, zi.x, s.x);
+        s.y = fma(y, zi.y, s.y);
+      }
+      T2 xv = reinterpret_cast<const T2*>(x)[u];
+      xv.x += s.x;
+      xv.y += s.y;
+      reinterpret_cast<T2*>(x)[u] = xv;
+    } else {
+      T s = T(0);
+#pragma unroll 4
+      for (int i = 0; i < l; ++i) s = fma((T)ys[i], __ldg(Z + (size_t)i * N + u), s);
+      x[u] += s;
+    }
+  }
 }
 
 template <typename T>
@@ -979,13 +1043,24 @@ void launch_gram_apply(const T* W, int N, const T* w, T* wout, int lcap, int nbl
 }
 
 template <typename T>
-void launch_gram_update(T* W, T* Z, int N, const T* w, const T* wre, const T* z, T* x, T* r, int lcap, int nblk,
-                        double* partial, const EpiArgs& e, cudaStream_t s) {
-  const size_t sm = 2 * lcap * sizeof(double);
+void launch_gram_update(T* W, T* Z, int N, const T* w, const T* wre, const T* z, const RmCoef& co, T* r, int lcap,
+                        int nblk, double* partial, const EpiArgs& e, cudaStream_t s) {
+  const size_t sm = lcap * sizeof(double);
   if (N % 2 == 0)   // pairs of elements (aligned column bases), half the grid
-    k_gram_update<T, true><<<(nblk + 1) / 2, kVecThreads, sm, s>>>(W, Z, N, w, wre, z, x, r, partial, e);
+    k_gram_update<T, true><<<(nblk + 1) / 2, kVecThreads, sm, s>>>(W, Z, N, w, wre, z, co, r, partial, e);
   else
-    k_gram_update<T, false><<<nblk, kVecThreads, sm, s>>>(W, Z, N, w, wre, z, x, r, partial, e);
+    k_gram_update<T, false><<<nblk, kVecThreads, sm, s>>>(W, Z, N, w, wre, z, co, r, partial, e);
+}
+
+template <typename T>
+void launch_x_update(const T* Z, int N, T* x, const LevelState* st, const RmCoef& co, int lcap, int nblk,
+                     int conditional, cudaStream_t s) {
+  const size_t sm = lcap * sizeof(double);
+  k_solve_y<<<1, kSolveThreads, sm, s>>>(st, co, conditional);
+  if (N % 2 == 0)
+    k_x_update<T, true><<<(nblk + 1) / 2, kVecThreads, sm, s>>>(Z, N, x, st, co, conditional);
+  else
+    k_x_update<T, false><<<nblk, kVecThreads, sm, s>>>(Z, N, x, st, co, conditional);
 }
 
 template <typename T>
@@ -1094,8 +1169,9 @@ void launch_grad_lognu(int np, int dim, const int* n, const double* nu, const do
                                     const EpiArgs&, int, cudaStream_t);                          \
   template void launch_gram_apply<T>(const T*, int, const T*, T*, int, int, LevelState*,         \
                                      const double*, cudaStream_t);                               \
-  template void launch_gram_update<T>(T*, T*, int, const T*, const T*, const T*, T*, T*, int,    \
+  template void launch_gram_update<T>(T*, T*, int, const T*, const T*, const T*, const RmCoef&, T*, int, \
                                       int, double*, const EpiArgs&, cudaStream_t);               \
+  template void launch_x_update<T>(const T*, int, T*, const LevelState*, const RmCoef&, int, int, int, cudaStream_t); \
   template void launch_norm<T>(const T*, int, int, double*, const EpiArgs&, cudaStream_t);       \
   template void launch_interleave<T>(int, int, const double*, const int*, int, int, T*, cudaStream_t); \
   template void launch_axpy_to_double<T>(const T*, double*, size_t, cudaStream_t);
