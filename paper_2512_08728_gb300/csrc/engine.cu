@@ -1782,6 +1782,10 @@ kcmg_status kcmg_solve_adjoint(kcmg_ctx* ctx, const double* g, double* lambda, i
     kcmg_status st = ensure_adjoint(ctx);
     if (st != KCMG_OK) return st;
     kcmg_ctx* a = ctx->adj;
+    if (a != ctx) {   // its stream waits for the caller's work, as this context's does
+      CK(cudaEventRecord(ctx->ev, ctx->s));
+      CK(cudaStreamWaitEvent(a->s, ctx->ev, 0));
+    }
     kcmg_status s2 = nrhs > 1 ? solve_multi(a, g, lambda, nrhs, rtol, atol, maxiter, info)
                               : solve_impl(a, g, lambda, rtol, atol, maxiter, info);
     if (a == ctx) return s2;
