@@ -1779,6 +1779,7 @@ kcmg_status kcmg_solve_adjoint(kcmg_ctx* ctx, const double* g, double* lambda, i
     REQUIRE(nrhs >= 1 && nrhs <= kMaxRhs, "nrhs must be in [1, %d]", kMaxRhs);
     REQUIRE(rtol >= 0 && atol >= 0 && maxiter >= 0, "negative tolerance or maxiter");
     REQUIRE(nrhs == 1 || !ctx->ir, "batched solves (nrhs > 1) support the FP64 and mixed forms");
+    REQUIRE(nrhs == 1 || ctx->p.smoother == 0, "batched solves (nrhs > 1) use the block-Jacobi smoother");
     kcmg_status st = ensure_adjoint(ctx);
     if (st != KCMG_OK) return st;
     kcmg_ctx* a = ctx->adj;
