@@ -1455,10 +1455,8 @@ kcmg_ctx* build_ctx(const kcmg_params* p, cudaStream_t user, const double* block
     CK(cudaEventCreateWithFlags(&ctx->ev, cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&ctx->fork_ev, cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&ctx->join_ev, cudaEventDisableTiming));
-    if (user) {
-      CK(cudaEventRecord(ctx->ev, user));
-      CK(cudaStreamWaitEvent(ctx->s, ctx->ev, 0));
-    }
+    CK(cudaEventRecord(ctx->ev, user));
+    CK(cudaStreamWaitEvent(ctx->s, ctx->ev, 0));
     ctx->lv.resize(ctx->nlev);
     ctx->dflag = dalloc<int>(ctx, 4);
     ctx->scal = dalloc<double>(ctx, 8);
@@ -1705,15 +1703,13 @@ template <typename F>
 kcmg_status guarded(kcmg_ctx* ctx, F&& f) {
   if (!ctx) return KCMG_INVALID_ARG;
   try {
-    if (ctx->user) {
-      CK(cudaEventRecord(ctx->ev, ctx->user));
-      CK(cudaStreamWaitEvent(ctx->s, ctx->ev, 0));
-    }
+    // also where the caller's stream is the default one (null): the library's own stream does not
+    // wait for that by itself
+    CK(cudaEventRecord(ctx->ev, ctx->user));
+    CK(cudaStreamWaitEvent(ctx->s, ctx->ev, 0));
     kcmg_status st = f();
-    if (ctx->user) {
-      CK(cudaEventRecord(ctx->ev, ctx->s));
-      CK(cudaStreamWaitEvent(ctx->user, ctx->ev, 0));
-    }
+    CK(cudaEventRecord(ctx->ev, ctx->s));
+    CK(cudaStreamWaitEvent(ctx->user, ctx->ev, 0));
     return st;
   } catch (Fail& e) {
     return e.st;
@@ -1741,7 +1737,7 @@ kcmg_status ensure_adjoint(kcmg_ctx* ctx) {
     kcmg_params pa = ctx->p;
     pa.prolong = ctx->P64;   // the caller's setup arrays may be gone by now
     pa.blocks = tr;
-    kcmg_ctx* a = build_ctx(&pa, nullptr, tr, &st, &msg);
+    kcmg_ctx* a = build_ctx(&pa, ctx->user, tr, &st, &msg);
     if (st != KCMG_OK) {
       set_err(ctx, "adjoint setup failed: %s", msg.c_str());
       kcmg_destroy(a);

@@ -47,3 +47,27 @@ def test_adjoint_of_a_nonsymmetric_operator(nrhs, kw):
     torch.cuda.synchronize()
     s.close()
     assert torch.equal(first, second)
+
+
+@pytest.mark.parametrize("own", [False, True], ids=["default", "own"])
+@pytest.mark.parametrize("call", ["solve", "solve_multi", "adjoint", "apply", "smooth", "restrict", "apply_multi",
+                                  "residual"])
+def test_every_call_waits(call, own):
+    pr = make_problem(3, 1, (8, 4, 4), 3, seed=1)
+    stream = torch.cuda.Stream() if own else torch.cuda.default_stream()
+    s = pkg.KCycleSolver(pr, stream=stream.cuda_stream or None)
+    multi = call in ("solve_multi", "apply_multi")
+    v = torch.from_numpy(np.random.default_rng(4).uniform(-1, 1, (pr.ndof, 3) if multi else pr.ndof)).cuda()
+    f = {"solve": lambda a: s.solve(a, maxiter=2)[0], "solve_multi": lambda a: s.solve(a, maxiter=2)[0],
+         "adjoint": lambda a: s.solve(a, maxiter=2, adjoint=True)[0], "apply": lambda a: s.apply(0, a),
+         "smooth": lambda a: s.smooth(0, a), "restrict": lambda a: s.restrict(0, a),
+         "apply_multi": lambda a: s.apply_multi(0, a),
+         "residual": lambda a: torch.tensor(pkg.kcmg_residual_noalloc(s.ctx, a, torch.zeros_like(a),
+                                                                      torch.empty_like(a)))}[call]
+    with torch.cuda.stream(stream):
+        torch.cuda.synchronize()
+        want = f(v)
+        got = f(_late(v))
+    torch.cuda.synchronize()
+    s.close()
+    assert want.abs().max() > 0 and torch.equal(want, got)
