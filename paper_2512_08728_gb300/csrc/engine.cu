@@ -145,6 +145,7 @@ void set_err(kcmg_ctx* c, const char* fmt, ...) {
     if (e_ != cudaSuccess) {                                                         \
       set_err(ctx, "%s failed at %s:%d: %s", #call, __FILE__, __LINE__,              \
               cudaGetErrorString(e_));                                               \
+      cudaGetLastError();   /* reported here: not for a later call to find */        \
       throw Fail{e_ == cudaErrorMemoryAllocation ? KCMG_OOM : KCMG_CUDA_ERROR};      \
     }                                                                                \
   } while (0)

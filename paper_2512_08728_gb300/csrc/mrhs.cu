@@ -1446,6 +1446,7 @@ namespace {
                  cudaGetErrorString(e_));                                             \
         *E->err = b_;                                                                 \
       }                                                                               \
+      cudaGetLastError();   /* reported here: not for a later call to find */         \
       throw Fail2{e_ == cudaErrorMemoryAllocation ? KCMG_OOM : KCMG_CUDA_ERROR};      \
     }                                                                                 \
   } while (0)
@@ -2189,21 +2190,22 @@ kcmg_status mrhs_ensure(MrhsEngine** peng, const MrhsView& v, int R, std::string
     mrhs_destroy(E);
     E = *peng = nullptr;
   }
-  try {
-    if (!E) {
-      E = new MrhsEngine();
-      E->err = err;
-      *peng = E;
-      E->x3 = v.tc_tf32_only == 0;
-      build(E, v, R);
-    }
+  if (!E) {
+    E = new MrhsEngine();
     E->err = err;
     E->x3 = v.tc_tf32_only == 0;
-    E->v.tc_tf32_only = v.tc_tf32_only;
-    return KCMG_OK;
-  } catch (Fail2& f) {
-    return f.st;
+    try {
+      build(E, v, R);
+    } catch (Fail2& f) {   // half an engine is of no use, and its memory may be what a retry lacks
+      mrhs_destroy(E);
+      return f.st;
+    }
+    *peng = E;
   }
+  E->err = err;
+  E->x3 = v.tc_tf32_only == 0;
+  E->v.tc_tf32_only = v.tc_tf32_only;
+  return KCMG_OK;
 }
 
 kcmg_status mrhs_apply(MrhsEngine* E, int level, const double* x, double* y, bool direct) {

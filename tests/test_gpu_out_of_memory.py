@@ -1,0 +1,53 @@
+"""Calls that meet a full device: they say so, and work once there is room."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import paper_2512_08728_gb300 as pkg
+from workloads import make_problem
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    pkg.build()
+
+
+def _leave(gib):
+    """Holds all of the device's free memory but this much."""
+    torch.cuda.empty_cache()
+    free, _ = torch.cuda.mem_get_info()
+    return torch.empty(max(0, free - int(gib * 2**30)), dtype=torch.uint8, device="cuda")
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_batched_solve_after_one_that_found_no_memory(precision):
+    # 32 columns of 32^3 cells, p = 2: 84 MB a vector, 20 of them at least
+    pr = make_problem(3, 2, (32, 32, 32), 4, nu_kind="jump", seed=1)
+    b = torch.from_numpy(np.random.default_rng(3).uniform(-1, 1, (pr.ndof, 32))).cuda()
+    s = pkg.KCycleSolver(pr, precision=precision)
+    x0 = torch.zeros_like(b)
+    hold = _leave(0.75)
+    for _ in range(2):                      # the second finds nothing of the first
+        with pytest.raises(pkg.KcmgError) as e:
+            s.solve(b, x0=x0, maxiter=1)
+        assert e.value.status == 6
+    with pytest.raises(pkg.KcmgError) as e:
+        s.smooth_multi(0, b)
+    assert e.value.status == 6
+    y, _ = s.solve(b[:, 0].contiguous(), x0=x0[:, 0].contiguous(), maxiter=1)   # one column has its memory
+    del hold
+    torch.cuda.empty_cache()
+    x, info = s.solve(b, maxiter=1)
+    s.close()
+    assert info["status"] == 1 and info["iters"] == 1
+    other = pkg.KCycleSolver(pr, precision=precision)
+    want, _ = other.solve(b, maxiter=1)
+    other.close()
+    # the FP32 sweep kernel of the level between is the tuner's choice: 1e-4 as for FP32 sweeps
+    assert torch.linalg.norm(x - want) <= (0 if precision == "fp64" else 1e-4) * torch.linalg.norm(want)
+    assert torch.isfinite(y).all()
