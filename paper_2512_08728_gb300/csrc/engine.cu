@@ -1216,6 +1216,11 @@ ColumnGroups* column_groups(kcmg_ctx* ctx, int nrhs) {
     }
   };
   carve();
+  // the same share of the free memory as the batched engine's bases take (mrhs.cu); that engine
+  // shortens its bases where lmax asks for more
+  size_t fr = 0, tot = 0;
+  CK(cudaMemGetInfo(&fr, &tot));
+  if (top > batched_budget(fr)) return nullptr;
   if (cudaMalloc((void**)&g->mem, top) != cudaSuccess) {
     cudaGetLastError();
     g->mem = nullptr;

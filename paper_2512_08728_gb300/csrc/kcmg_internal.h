@@ -348,6 +348,13 @@ struct MrhsView {               // the context's hierarchy, as the batched solve
   cudaStream_t s;
 };
 
+// bytes of the free device memory that a batched solve's bases may take: the rest is for the coarse
+// levels' bases (an eighth per level) and the caller
+inline size_t batched_budget(size_t free_bytes) {
+  const size_t margin = (size_t)4 << 30;
+  return free_bytes > margin ? (size_t)((free_bytes - margin) * 0.8) : free_bytes / 2;
+}
+
 struct MrhsEngine;
 // Solve A X = B for R = nrhs columns (X holds X0 on entry).  Returns the status; on a
 // failure *err receives a message.

@@ -2138,10 +2138,8 @@ void build(MrhsEngine* E, const MrhsView& v, int R) {
     else cap = 3 * std::max(1, v.lvl_maxit[l]) + 3;
     if (v.lmax > 0 && l > 0) cap = std::min(cap, v.lmax + 3);
     if (l == 0) {
-      // reserve the coarse levels' bases (an eighth per level) and a margin
       MCK(cudaMemGetInfo(&free_b, &tot_b));
-      const size_t per = 2 * NR * sizeof(double);
-      const size_t budget = free_b > ((size_t)4 << 30) ? (size_t)((free_b - ((size_t)4 << 30)) * 0.8) : free_b / 2;
+      const size_t per = 2 * NR * sizeof(double), budget = batched_budget(free_b);
       while (cap > 6 && (size_t)cap * per > budget) cap = cap * 3 / 4;
       if (cap < per_cycle0 + 3) cap = per_cycle0 + 3;   // one cycle must always fit
     }
