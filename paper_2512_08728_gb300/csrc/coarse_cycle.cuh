@@ -39,6 +39,7 @@
 // times out it raises an error flag and every block leaves the kernel, so a fault becomes a
 // status, not a hang.
 #pragma once
+#include "barrier_count.h"
 #include "kcmg_internal.h"
 #include "reduce.cuh"
 #include "schwarz.cuh"
@@ -101,7 +102,7 @@ static __device__ __forceinline__ bool cc_barrier(const CoarseArgs& a, unsigned 
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.bar_count) : "memory");
     long long spins = 0;
     int ok = 1;
-    while (cnt.load(cuda::memory_order_acquire) < target) {
+    while (!count_reached(cnt.load(cuda::memory_order_acquire), target)) {
       if ((++spins & 1023) == 0) {
         if (err.load(cuda::memory_order_relaxed)) { ok = 0; break; }
         if (spins > (1LL << 23)) {   // seconds: far beyond any legitimate wait
