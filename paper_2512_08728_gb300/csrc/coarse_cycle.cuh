@@ -100,12 +100,13 @@ static __device__ __forceinline__ bool cc_barrier(const CoarseArgs& a, unsigned 
     cuda::atomic_ref<int, cuda::thread_scope_device> err(*a.err);
     const unsigned int target = (gen + 1) * blocks;
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.bar_count) : "memory");
-    long long spins = 0;
+    cuda::atomic_ref<unsigned int, cuda::thread_scope_device> progress(*a.bar_progress);
+    unsigned int polls = 0, seen = 0;
     int ok = 1;
     while (!count_reached(cnt.load(cuda::memory_order_acquire), target)) {
-      if ((++spins & 1023) == 0) {
+      if ((++polls & 1023) == 0) {
         if (err.load(cuda::memory_order_relaxed)) { ok = 0; break; }
-        if (spins > (1LL << 23)) {   // seconds: far beyond any legitimate wait
+        if (give_up(polls, seen, progress.load(cuda::memory_order_relaxed))) {
           err.store(1, cuda::memory_order_relaxed);
           ok = 0;
           break;
@@ -867,6 +868,7 @@ struct CoarseCycle {
       const long long t = clock64();
       if (t_ph) tph[kind] += t - t_ph;
       t_ph = t;
+      if (nblk < nall()) *static_cast<volatile unsigned int*>(a.bar_progress) = (unsigned int)t;   // the others wait
     }
   }
   __device__ void mark(int l) {

@@ -67,7 +67,7 @@ struct ColumnGroups {
   CoarseArgs* cols_d = nullptr;
   LevelState* st = nullptr;   // [nrhs][nlev]
   double *b = nullptr, *x = nullptr;   // [N][nrhs]
-  unsigned int* bars = nullptr;        // [groups][2]
+  unsigned int* bars = nullptr;        // [groups][3]
   int* err = nullptr;
 };
 
@@ -1172,7 +1172,7 @@ ColumnGroups* column_groups(kcmg_ctx* ctx, int nrhs) {
     g->st = (LevelState*)take((size_t)nrhs * ctx->nlev * sizeof(LevelState));
     g->b = (double*)take(N0 * nrhs * sizeof(double));
     g->x = (double*)take(N0 * nrhs * sizeof(double));
-    g->bars = (unsigned int*)take((size_t)2 * g->groups * sizeof(unsigned int));
+    g->bars = (unsigned int*)take((size_t)3 * g->groups * sizeof(unsigned int));
     g->err = (int*)take(sizeof(int));
     if (own_blocks) {
       A64 = (double*)take(opsz * sizeof(double));
@@ -1207,8 +1207,9 @@ ColumnGroups* column_groups(kcmg_ctx* ctx, int nrhs) {
       c.zc = p.async_smooth > 0 ? take(N0 * sizeof(double)) : nullptr;
       c.partial = (double*)take(2 * a.partial_stride * sizeof(double));
       c.red = (double*)take((size_t)(a.cols + 4) * sizeof(double));
-      c.bar_count = g->bars + 2 * (j % g->groups);
+      c.bar_count = g->bars + 3 * (j % g->groups);
       c.bar_gen = c.bar_count + 1;
+      c.bar_progress = c.bar_count + 2;
       c.err = g->err;
       c.io_b = g->b + j;
       c.io_x = g->x + j;
@@ -1259,7 +1260,7 @@ kcmg_status solve_groups(kcmg_ctx* ctx, ColumnGroups* g, const double* b, double
     h.status = KCMG_OK;
   }
   CK(cudaMemcpyAsync(g->st, st.data(), st.size() * sizeof(LevelState), cudaMemcpyHostToDevice, ctx->s));
-  CK(cudaMemsetAsync(g->bars, 0, (size_t)2 * g->groups * sizeof(unsigned int), ctx->s));
+  CK(cudaMemsetAsync(g->bars, 0, (size_t)3 * g->groups * sizeof(unsigned int), ctx->s));
   CK(cudaMemsetAsync(g->err, 0, sizeof(int), ctx->s));
   cudaError_t e;
   const bool bf16 = ctx->p.precision == KCMG_MIXED_BF16INV;
@@ -1560,8 +1561,10 @@ kcmg_ctx* build_ctx(const kcmg_params* p, cudaStream_t user, const double* block
       a.smoother = p->smoother;
       a.bar_count = dalloc<unsigned int>(ctx, 1);
       a.bar_gen = dalloc<unsigned int>(ctx, 1);
+      a.bar_progress = dalloc<unsigned int>(ctx, 1);
       a.err = dalloc<int>(ctx, 1);
       CK(cudaMemsetAsync(a.bar_gen, 0, sizeof(unsigned int), ctx->s));
+      CK(cudaMemsetAsync(a.bar_progress, 0, sizeof(unsigned int), ctx->s));
       for (int l = 0; l < ctx->nlev; ++l) {
         Level& L = ctx->lv[l];
         CoarseLevel& c = a.lv[l];

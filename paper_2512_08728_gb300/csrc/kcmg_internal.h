@@ -274,6 +274,7 @@ struct CoarseArgs {
   double* red;                 // cols + 4 reduced sums
   unsigned int* bar_count;     // arrivals at the grid barrier in this launch
   unsigned int* bar_gen;       // blocks that have left the kernel
+  unsigned int* bar_progress;  // block 0's clock at its last phase on a level that it runs alone
   int* err;                    // set when a grid barrier timed out
   // measurement: launches, device nanoseconds and algorithmic bytes of every launch
   unsigned long long* stat_ns;

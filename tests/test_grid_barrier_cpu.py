@@ -1,4 +1,4 @@
-"""The rule of the persistent kernel's grid barrier (csrc/barrier_count.h), run on the CPU: blocks
+"""The rules of the persistent kernel's grid barrier (csrc/barrier_count.h), run on the CPU: blocks
 that arrive and poll in random order, over the point where the 32-bit counter wraps."""
 import os
 import subprocess
@@ -47,3 +47,25 @@ int main(int, char** v) {
 def test_nobody_passes_early_or_stays_when_the_counter_wraps(tmp_path, blocks):
     early, passed = _run(tmp_path, WRAP, blocks)
     assert (int(early), int(passed)) == (0, 8 * blocks)
+
+
+LIMIT = r"""
+#include "barrier_count.h"
+#include <cstdio>
+#include <cstdlib>
+int main(int, char** v) {   // polls until a block gives up, with a step of block 0 every so many polls
+  const unsigned every = atoi(v[1]);
+  unsigned polls = 0, seen = 0, n = 0;
+  while (n < (1u << 27)) {
+    ++n;
+    if ((++polls & 1023) == 0 && kcmg::give_up(polls, seen, every ? n / every : 7)) break;
+  }
+  printf("%u\n", n);
+}
+"""
+
+
+@pytest.mark.parametrize("every", [0, 1, 1 << 16, 1 << 22])
+def test_a_block_waits_as_long_as_block_0_reports_progress(tmp_path, every):
+    n = int(_run(tmp_path, LIMIT, every)[0])
+    assert n == 1 << 27 if every else 1 << 23 < n <= (1 << 23) + 2048
