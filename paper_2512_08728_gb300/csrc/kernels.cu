@@ -461,7 +461,7 @@ k_gram_update(T* W, T* Z, int N, const T* __restrict__ w, const T* __restrict__ 
   const T* ws = re ? wre : w;
   T* Wl = W + (size_t)l * N;
   T* Zl = Z + (size_t)l * N;
-  T r2 = T(0);   // per-thread sums in T, reduced in FP64
+  double r2 = 0.0;   // FP64 products and sums also of FP32 vectors: two FMAs a pair beside l
   if (PAIR) {
     const int units = N / 2;
     for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < units; u += gridDim.x * blockDim.x) {
@@ -483,8 +483,8 @@ k_gram_update(T* W, T* Z, int N, const T* __restrict__ w, const T* __restrict__ 
         rv.y = fma(-al, a.y, rv.y);
         reinterpret_cast<T2*>(r)[u] = rv;
       }
-      r2 = fma(rv.x, rv.x, r2);
-      r2 = fma(rv.y, rv.y, r2);
+      r2 = fma((double)rv.x, (double)rv.x, r2);
+      r2 = fma((double)rv.y, (double)rv.y, r2);
     }
   } else {
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < N; j += gridDim.x * blockDim.x) {
@@ -499,10 +499,10 @@ k_gram_update(T* W, T* Z, int N, const T* __restrict__ w, const T* __restrict__ 
         rv = fma(-al, a, rv);
         r[j] = rv;
       }
-      r2 = fma(rv, rv, r2);
+      r2 = fma((double)rv, (double)rv, r2);
     }
   }
-  double v[1] = {(double)r2};
+  double v[1] = {r2};
   finish_reduction<1>(v, partial, e, sh);
 }
 
