@@ -559,7 +559,8 @@ struct CoarseCycle {
   }
 
   // this block's sums of column c < l: W_c . w, l: w . w, l + 1: w . r, l + 2: r . r over the own
-  // rows; LPC lanes of a warp share a column.  Per-thread sums in T, then FP64.
+  // rows; LPC lanes of a warp share a column.  The columns' per-thread sums are in T (coefficients of
+  // the size of ||w||); those of norms and w . r are FP64 products and sums in every form.
   template <int LPC>
   __device__ void dots_lpc(const T* W, int N, int l, double* pt) {
     constexpr int CPW = 32 / LPC;
@@ -570,7 +571,12 @@ struct CoarseCycle {
     for (int c0 = warp * CPW; c0 < n; c0 += nw * CPW) {
       const int c = c0 + sub;
       T s0 = T(0), s1 = T(0);
-      if (c < n) {
+      double d = 0.0;
+      if (sizeof(T) == 4 && c >= l && c < n) {
+        const T* u = c == l + 2 ? rs : w;
+        const T* v = c == l ? w : rs;
+        for (int j = lc; j < rows; j += LPC) d = fma((double)u[j], (double)v[j], d);
+      } else if (c < n) {
         const T* u = c < l ? W + (size_t)c * N + row0 : c == l + 2 ? rs : w;
         const T* v = c <= l ? w : rs;
         int j = lc;
@@ -580,7 +586,7 @@ struct CoarseCycle {
         }
         if (j < rows) s0 = fma(u[j], v[j], s0);
       }
-      double d = (double)(s0 + s1);
+      d += (double)(s0 + s1);
 #pragma unroll
       for (int o = LPC / 2; o; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
       if (lc == 0 && c < n) {

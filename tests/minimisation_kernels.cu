@@ -1,5 +1,6 @@
 // Single steps of the residual minimisation (Alg. 1) for test_gpu_minimisation_kernels.py: the
 // library's kernels on vectors and a level state that the test sets.  Host pointers throughout.
+#include "coarse_cycle.cuh"
 #include "kcmg_internal.h"
 
 #include <cmath>
@@ -50,11 +51,53 @@ int update(int N, int l, T* W, const T* w, const T* z, const double* h, double g
   return st.l == l + 1 ? 0 : 2;
 }
 
+// the persistent kernel's sums over a block that is alone on its level: W^T w, w . w, w . r, r . r
+constexpr int kNP = 3;
+template <typename T>
+__global__ void k_dots(const __grid_constant__ CoarseArgs a, const T* W, int N, int l, const T* w, const T* r,
+                       double* out) {
+  __shared__ double sh[32 * 8];
+  __shared__ RmScal rms;
+  __shared__ int nbs[5];
+  __shared__ long long tph[kCoarsePhases + KCMG_MAX_LEVELS];
+  double* red_s = reinterpret_cast<double*>(smem_cc + a.sm_red);
+  CoarseCycle<T, T, T, kNP, 2, false> cc{a, sh, red_s, red_s + a.cols + 4, &rms, nbs, tph, nullptr};
+  cc.rows = N;
+  cc.rs_off = a.lv[0].sm_r;
+  for (int i = threadIdx.x; i < N; i += blockDim.x) {
+    cc.ws()[i] = w[i];
+    cc.rs_()[i] = r[i];
+  }
+  __syncthreads();
+  cc.dots(W, N, l);
+  for (int i = threadIdx.x; i < l + 3; i += blockDim.x) out[i] = red_s[i];
+}
+
+template <typename T>
+int dots(int N, int l, const T* W, const T* w, const T* r, double* out) {
+  Dev<T> dW(W, (size_t)(l + 1) * N), dw(w, N), dr(r, N);
+  Dev<double> dout(nullptr, l + 3);
+  CoarseArgs a{};
+  a.nlev = 2;
+  a.cols = l + 1;
+  a.lv[0].N = N;
+  a.lv[0].sm_r = (int)(N * sizeof(T) + 15) / 16 * 16;
+  a.sm_red = 2 * a.lv[0].sm_r;
+  a.sm_bytes = a.sm_red + (int)((2 * a.cols + 4) * sizeof(double));
+  k_dots<T><<<1, kCoarseThreads, a.sm_bytes>>>(a, dW.p, N, l, dw.p, dr.p, dout.p);
+  if (cudaDeviceSynchronize() != cudaSuccess) return 1;
+  dout.get(out);
+  return 0;
+}
+
 }  // namespace step_test
 
 using namespace step_test;
 
 extern "C" {
+
+int dots_f32(int N, int l, const float* W, const float* w, const float* r, double* out) { return dots<float>(N, l, W, w, r, out); }
+int dots_f64(int N, int l, const double* W, const double* w, const double* r, double* out) { return dots<double>(N, l, W, w, r, out); }
 
 int update_f32(int N, int l, float* W, const float* w, const float* z, const double* h, double gamma, double alpha,
                float* r, int nblk, double* rnorm) {

@@ -49,3 +49,25 @@ def test_residual_norm_of_an_update_sums_in_fp64(lib, t, N):
     assert getattr(lib, "update_" + t)(N, 0, _p(W), _p(w), _p(z), _p(h), C.c_double(1.0), C.c_double(0.0), _p(r), 1,
                                        C.byref(rn)) == 0
     assert abs(rn.value - want) <= 450 * 2.0**-53 * want
+
+
+# the same for the persistent kernel's sums: eight lanes a sum, so the first 16 entries of every
+# vector are the ones that the others vanish beside; FP64 sums of N / 8 terms a lane
+@pytest.mark.parametrize("t", ["f32", "f64"])
+@pytest.mark.parametrize("N,l", [(2400, 0), (2400, 5), (2400, 20), (27, 2)])
+def test_norms_of_the_persistent_kernel_sum_in_fp64(lib, t, N, l):
+    T = TYPES[t]
+    w, r = np.full(N, 2.0**-13, dtype=T), np.full(N, -(2.0**-13), dtype=T)
+    w[:16], r[:16] = 1.0, 1.0
+    W = np.random.default_rng(1).standard_normal((l + 1, N)).astype(T)
+    out = np.zeros(l + 3)
+    assert getattr(lib, "dots_" + t)(N, l, _p(W), _p(w), _p(r), _p(out)) == 0
+    tol = (N / 8 + 5) * 2.0**-53
+    for got, a, b in ((out[l], w, w), (out[l + 1], w, r), (out[l + 2], r, r)):
+        terms = a.astype(np.float64) * b.astype(np.float64)
+        assert abs(got - math.fsum(terms)) <= tol * np.abs(terms).sum()
+    # the columns' sums are in the vectors' type: N / 16 terms an accumulator
+    eps = 2.0**-24 if t == "f32" else 2.0**-53
+    for c in range(l):
+        terms = W[c].astype(np.float64) * w.astype(np.float64)
+        assert abs(out[c] - math.fsum(terms)) <= (N / 16 + 8) * eps * np.abs(terms).sum()
