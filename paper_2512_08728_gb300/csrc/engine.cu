@@ -477,7 +477,6 @@ struct Cycle {
     e.kind = kind;
     e.h = L.h;
     e.h2 = L.h2;
-    e.dep = ctx->ir ? kDependent32 : kDependent64;
     if (lev == 0) {
       e.hist = ctx->hist;
       e.hist_type_buf = ctx->hist_type;

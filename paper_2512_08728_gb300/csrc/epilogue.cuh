@@ -83,16 +83,15 @@ static __device__ void epilogue(const EpiArgs& e, const double* sums) {
       set_cond(e, more_cycles(st));
     } break;
     // W^T w, ||w||^2 and w . r decide the whole step: the norm of w_hat = w - W h by Pythagoras
-    // (reliable, as it is only used when it did not cancel below a quarter of ||w||^2; else the
-    // second Gram-Schmidt pass is requested, "twice is enough"), and alpha = w_hat . r = w . r, as
-    // r is orthogonal to W
+    // (kPythagoras; else the second Gram-Schmidt pass is requested, "twice is enough"), and
+    // alpha = w_hat . r = w . r, as r is orthogonal to W
     case EPI_GRAM1: {
       const int l = st->l;
       const double naz2 = sums[l], nw2 = naz2 - sums[l + 2];   // [l + 2]: sum of the squared coefficients
       st->naz2 = naz2;
       int f = 0;
       if (!isfinite(naz2) || !(naz2 > 0.0)) f |= F_DISCARD;
-      else if (l > 0 && nw2 < 0.25 * naz2) f |= F_REORTH;
+      else if (l > 0 && nw2 < kPythagoras * naz2) f |= F_REORTH;
       else {
         st->gamma = 1.0 / sqrt(nw2);
         st->alpha = st->gamma * sums[l + 1];
@@ -100,15 +99,17 @@ static __device__ void epilogue(const EpiArgs& e, const double* sums) {
       if (!isfinite(naz2) && st->level == 0) st->status = KCMG_NONFINITE;
       st->flags = f;
     } break;
-    // the second pass: w' = w - W h.  What is left of it after this pass is kept, however much of
-    // its norm it loses again (in FP32 often most of it), while the norm can be told from rounding
-    // and is above brk relative to ||A z||
+    // the second pass: w' = w - W h
     case EPI_GRAM2: {
       const int l = st->l;
       const double n2 = sums[l], nw2 = n2 - sums[l + 2];
-      if (!isfinite(nw2) || !(nw2 > e.dep * n2) || !(nw2 > st->brk * st->brk * st->naz2)) {
+      if (!isfinite(nw2)) {
         st->flags |= F_DISCARD;
         if (!isfinite(n2) && st->level == 0) st->status = KCMG_NONFINITE;
+      } else if (nw2 < kPythagoras * n2) {
+        st->flags |= F_OWN_NORM;
+      } else if (!(nw2 > st->brk * st->brk * st->naz2)) {
+        st->flags |= F_DISCARD;
       } else {
         st->gamma = 1.0 / sqrt(nw2);
         st->alpha = st->gamma * sums[l + 1];

@@ -19,7 +19,7 @@ constexpr int kLcapMax = 2048;     // basis capacity cap per level (shared-memor
 constexpr int kMaxChild = 8;
 
 // flags of the RM call in flight
-enum : int { F_REORTH = 1, F_DISCARD = 2 };
+enum : int { F_REORTH = 1, F_DISCARD = 2, F_OWN_NORM = 4 };
 
 // Device-resident scalar state of one level of the cycle.  One MG call is active per
 // level at any time (Alg. 2 recursion), so one state per level suffices.
@@ -62,19 +62,19 @@ enum EpiKind : int {
   EPI_NORM          // sum = ||y||^2 stored into *out (component calls, refinement)
 };
 
-// After the second Gram-Schmidt pass ||w_hat||^2 = ||w'||^2 - ||h2||^2 is off by the rounding of the
-// sums and of W^T W = I, some 1e-14 ||w'||^2 with FP64 vectors and 1e-6 with FP32 ones.  It serves
-// as the column's norm down to where that is 1e-4 and 1e-2 of it; what is smaller depends linearly
-// on the basis.  (w' is what the first pass left: h2 is its rounding, and a w_hat far below that
-// does not come up but for exact dependence.)
-constexpr double kDependent64 = 1e-10, kDependent32 = 1e-4;
+// ||w_hat||^2 = ||w||^2 - ||h||^2 is off by the rounding of the sums and of W^T W = I, so it serves as
+// the new column's norm while at least this share of ||w||^2 is left.  Less after the first
+// Gram-Schmidt pass asks for the second; less after that one, too, and the norm and alpha come from
+// the column itself (F_OWN_NORM): it is kept while it is above brk relative to ||A z||.
+constexpr double kPythagoras = 0.25;
+// batched solves: a column of which the second pass leaves less than this is discarded
+constexpr double kDependent64 = 1e-10;
 
 struct EpiArgs {
   LevelState* st = nullptr;
   int kind = EPI_NONE;
   int end_iter = 0;      // EPI_FINISH: last RM of the cycle
   int hist_type = 0;     // EPI_FINISH: 1 pre, 2 coarse, 3 post
-  double dep = kDependent64;   // EPI_GRAM2: below this share of ||w'||^2 the norm of w_hat is rounding
   int use_handle = 0;
   cudaGraphConditionalHandle handle = 0;
   double* h = nullptr;   // Gram coefficients, pass 1 [lcap]

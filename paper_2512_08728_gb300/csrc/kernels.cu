@@ -437,6 +437,46 @@ k_gram_apply(const T* __restrict__ W, int N, const T* __restrict__ w, T* __restr
 // gone: 64^3, np = 10, m = 12, five cycles 195.4 -> 182.7 ms.
 // A discarded correction leaves W, Z, r unchanged.  With PAIR (N even) a thread takes two
 // consecutive elements with one 16-byte (FP64) / 8-byte (FP32) load per column.
+// With F_OWN_NORM the column is formed as it is, and the last block takes its norm and w_hat . r
+// from it, normalises and applies it (own_norm): one block's bandwidth, which is rare enough not to
+// matter, in place of two more launches in every minimisation.
+template <typename T>
+__device__ __noinline__ void own_norm(T* Wl, int N, T* r, const RmCoef& co, LevelState* st, double* r2, double* sh) {
+  __shared__ double sc[2];
+  double v[2] = {0.0, 0.0};
+  for (int j = threadIdx.x; j < N; j += blockDim.x) {   // written by other blocks: through L2
+    const double a = __ldcg(Wl + j);
+    v[0] = fma(a, a, v[0]);
+    v[1] = fma(a, (double)__ldcg(r + j), v[1]);
+  }
+  bsum_n<2>(v, sh);
+  if (threadIdx.x == 0) {
+    const double nw = sqrt(v[0]);
+    sc[0] = sc[1] = 0.0;
+    if (!isfinite(nw) || !(nw > st->brk * sqrt(st->naz2))) {
+      st->flags |= F_DISCARD;
+      if (!isfinite(nw) && st->level == 0) st->status = KCMG_NONFINITE;
+    } else {
+      st->gamma = sc[0] = 1.0 / nw;
+      st->alpha = sc[1] = v[1] / nw;
+      co.gm[st->l] = sc[0];
+      co.al[st->l] = sc[1];
+    }
+  }
+  __syncthreads();
+  if (sc[0] == 0.0) return;   // discarded: r and its norm stay
+  const T gam = (T)sc[0], al = (T)sc[1];
+  double s[1] = {0.0};
+  for (int j = threadIdx.x; j < N; j += blockDim.x) {
+    const T a = __ldcg(Wl + j) * gam, rv = fma(-al, a, __ldcg(r + j));
+    Wl[j] = a;
+    r[j] = rv;
+    s[0] = fma((double)rv, (double)rv, s[0]);
+  }
+  bsum_n<1>(s, sh);
+  if (threadIdx.x == 0) *r2 = s[0];
+}
+
 template <typename T, bool PAIR>
 __global__ void __launch_bounds__(kVecThreads)
 k_gram_update(T* W, T* Z, int N, const T* __restrict__ w, const T* __restrict__ wre,
@@ -446,8 +486,8 @@ k_gram_update(T* W, T* Z, int N, const T* __restrict__ w, const T* __restrict__ 
   extern __shared__ double cs[];  // [l]
   __shared__ double sh[32 * 8];   // bsum_n<NC> needs 32 * NC
   const int l = st->l;
-  const bool re = (st->flags & F_REORTH) != 0, keep = !(st->flags & F_DISCARD);
-  const T gam = (T)st->gamma, al = (T)st->alpha;
+  const bool re = (st->flags & F_REORTH) != 0, keep = !(st->flags & F_DISCARD), own = (st->flags & F_OWN_NORM) != 0;
+  const T gam = own ? T(1) : (T)st->gamma, al = own ? T(0) : (T)st->alpha;
   if (keep)
     for (int i = threadIdx.x; i < l; i += blockDim.x) {
       cs[i] = re ? e.h2[i] : e.h[i];
@@ -479,9 +519,11 @@ k_gram_update(T* W, T* Z, int N, const T* __restrict__ w, const T* __restrict__ 
         a.x *= gam;
         a.y *= gam;
         reinterpret_cast<T2*>(Wl)[u] = a;
-        rv.x = fma(-al, a.x, rv.x);
-        rv.y = fma(-al, a.y, rv.y);
-        reinterpret_cast<T2*>(r)[u] = rv;
+        if (!own) {
+          rv.x = fma(-al, a.x, rv.x);
+          rv.y = fma(-al, a.y, rv.y);
+          reinterpret_cast<T2*>(r)[u] = rv;
+        }
       }
       r2 = fma((double)rv.x, (double)rv.x, r2);
       r2 = fma((double)rv.y, (double)rv.y, r2);
@@ -496,14 +538,26 @@ k_gram_update(T* W, T* Z, int N, const T* __restrict__ w, const T* __restrict__ 
         for (int i = 0; i < l; ++i) a = fma((T)(-cs[i]), __ldg(W + (size_t)i * N + j), a);
         a *= gam;
         Wl[j] = a;
-        rv = fma(-al, a, rv);
-        r[j] = rv;
+        if (!own) {
+          rv = fma(-al, a, rv);
+          r[j] = rv;
+        }
       }
       r2 = fma((double)rv, (double)rv, r2);
     }
   }
   double v[1] = {r2};
-  finish_reduction<1>(v, partial, e, sh);
+  bsum_n<1>(v, sh);
+  if (threadIdx.x == 0) partial[blockIdx.x] = v[0];
+  if (last_block(&st->ticket)) {
+    __shared__ double sums[1];
+    reduce_few(partial, gridDim.x, 1, sums, sh);
+    if (own && keep) own_norm<T>(Wl, N, r, co, st, sums, sh);
+    if (threadIdx.x == 0) {
+      epilogue(e, sums);
+      st->ticket = 0u;
+    }
+  }
 }
 
 // R y = alpha by back substitution, one block; conditional: only if the level restarts.  One column

@@ -51,6 +51,43 @@ int update(int N, int l, T* W, const T* w, const T* z, const double* h, double g
   return st.l == l + 1 ? 0 : 2;
 }
 
+// a second Gram-Schmidt pass over w' and the step after it; returns the new column's gamma and alpha
+template <typename T>
+int second_pass(int N, int l, T* W, const T* w, const T* z, double naz2, T* r, int nblk, double* gamma, double* alpha,
+                double* rnorm) {
+  const int lcap = l + 1;
+  Dev<T> dW(W, (size_t)lcap * N), dZ(nullptr, (size_t)lcap * N), dw(w, N), dz(z, N), dr(r, N);
+  Dev<double> h(nullptr, lcap), h2(nullptr, lcap), part(nullptr, (size_t)(nblk + 1) * (lcap + 8)), gm(nullptr, lcap),
+      al(nullptr, lcap), y(nullptr, lcap), R(nullptr, (size_t)lcap * lcap + 1);
+  LevelState st{};
+  st.l = l;
+  st.lcap = lcap;
+  st.naz2 = naz2;
+  st.brk = 1e-14;
+  st.flags = F_REORTH;
+  Dev<LevelState> ds(&st, 1);
+  EpiArgs e;
+  e.st = ds.p;
+  e.kind = EPI_GRAM2;
+  e.h = h.p;
+  e.h2 = h2.p;
+  launch_gram_dots<T>(dW.p, N, dw.p, dr.p, lcap, nblk, part.p, e, 1, 0);
+  e.kind = EPI_FINISH;
+  const RmCoef co{gm.p, al.p, y.p, R.p};
+  launch_gram_update<T>(dW.p, dZ.p, N, dw.p, dw.p, dz.p, co, dr.p, lcap, nblk, part.p, e, 0);
+  if (cudaDeviceSynchronize() != cudaSuccess) return 1;
+  ds.get(&st);
+  dW.get(W);
+  dr.get(r);
+  std::vector<double> g(lcap), a(lcap);
+  gm.get(g.data());
+  al.get(a.data());
+  *gamma = g[l];
+  *alpha = a[l];
+  *rnorm = st.rnorm;
+  return st.l == l + 1 ? 0 : 2;
+}
+
 // the persistent kernel's sums over a block that is alone on its level: W^T w, w . w, w . r, r . r
 constexpr int kNP = 3;
 template <typename T>
@@ -99,6 +136,14 @@ extern "C" {
 int dots_f32(int N, int l, const float* W, const float* w, const float* r, double* out) { return dots<float>(N, l, W, w, r, out); }
 int dots_f64(int N, int l, const double* W, const double* w, const double* r, double* out) { return dots<double>(N, l, W, w, r, out); }
 
+int second_pass_f32(int N, int l, float* W, const float* w, const float* z, double naz2, float* r, int nblk,
+                    double* gamma, double* alpha, double* rnorm) {
+  return second_pass<float>(N, l, W, w, z, naz2, r, nblk, gamma, alpha, rnorm);
+}
+int second_pass_f64(int N, int l, double* W, const double* w, const double* z, double naz2, double* r, int nblk,
+                    double* gamma, double* alpha, double* rnorm) {
+  return second_pass<double>(N, l, W, w, z, naz2, r, nblk, gamma, alpha, rnorm);
+}
 int update_f32(int N, int l, float* W, const float* w, const float* z, const double* h, double gamma, double alpha,
                float* r, int nblk, double* rnorm) {
   return update<float>(N, l, W, w, z, h, gamma, alpha, r, nblk, rnorm);

@@ -71,3 +71,49 @@ def test_norms_of_the_persistent_kernel_sum_in_fp64(lib, t, N, l):
     for c in range(l):
         terms = W[c].astype(np.float64) * w.astype(np.float64)
         assert abs(out[c] - math.fsum(terms)) <= (N / 16 + 8) * eps * np.abs(terms).sum()
+
+
+def _basis(T, N, l, left, seed=3):
+    """l orthonormal columns, a vector with the share ``left`` of its square outside them, and a residual
+    orthogonal to them, all rounded to T."""
+    rng = np.random.default_rng(seed)
+    Q = np.linalg.qr(rng.standard_normal((N, l + 2)))[0].T
+    c = rng.standard_normal(l)
+    w = math.sqrt(1 - left) * (c / np.linalg.norm(c)) @ Q[:l] + math.sqrt(left) * Q[l]
+    W = np.zeros((l + 1, N), T)
+    W[:l] = Q[:l]
+    return W, w.astype(T), (0.6 * Q[l] + 0.8 * Q[l + 1]).astype(T)
+
+
+# After the second pass the new column has unit length and r is orthogonal to it, to the rounding of the
+# sums in the vectors' type: 13 units for a thread's products and sums (12 terms at most), 16 with the
+# normalisation and the storing, times 4 where the norm is ||w'||^2 - ||h2||^2 with a quarter left.
+@pytest.mark.parametrize("t", ["f32", "f64"])
+@pytest.mark.parametrize("N,nblk", [(3000, 1), (3000, 7), (5001, 4)])
+@pytest.mark.parametrize("left", [0.9, 0.3, 0.2, 1e-2, 2e-4])
+def test_column_after_the_second_pass(lib, t, N, nblk, left):
+    T, l = TYPES[t], 9
+    eps = np.finfo(T).eps / 2
+    W, w, r = _basis(T, N, l, left)
+    rn0 = np.linalg.norm(r.astype(np.float64))
+    g, a, rn = C.c_double(), C.c_double(), C.c_double()
+    assert getattr(lib, "second_pass_" + t)(N, l, _p(W), _p(w), _p(w), C.c_double(4.0), _p(r), nblk, C.byref(g),
+                                            C.byref(a), C.byref(rn)) == 0
+    wl, rl = W[l].astype(np.float64), r.astype(np.float64)
+    tol = 4 * 16 * eps
+    assert abs(np.linalg.norm(wl) - 1) <= tol
+    assert abs(rl @ wl) <= tol * rn0
+    assert abs(rn.value - np.linalg.norm(rl)) <= 64 * 2.0**-53
+    assert abs(g.value * math.sqrt(left) - 1) <= 32 * eps / left and abs(a.value - 0.6) <= 32 * eps / left
+
+
+# what is left is below brk = 1e-14 of ||A z||: discarded, the residual as it was
+@pytest.mark.parametrize("t", ["f32", "f64"])
+def test_dependent_after_the_second_pass(lib, t):
+    T, N, l = TYPES[t], 3000, 9
+    W, w, r = _basis(T, N, l, 1e-2)
+    before = r.copy()
+    g, a, rn = C.c_double(), C.c_double(), C.c_double()
+    assert getattr(lib, "second_pass_" + t)(N, l, _p(W), _p(w), _p(w), C.c_double(1e28), _p(r), 3, C.byref(g),
+                                            C.byref(a), C.byref(rn)) == 2
+    assert np.array_equal(r, before) and abs(rn.value - np.linalg.norm(r.astype(np.float64))) <= 64 * 2.0**-53
