@@ -67,8 +67,6 @@ enum EpiKind : int {
 // Gram-Schmidt pass asks for the second; less after that one, too, and the norm and alpha come from
 // the column itself (F_OWN_NORM): it is kept while it is above brk relative to ||A z||.
 constexpr double kPythagoras = 0.25;
-// batched solves: a column of which the second pass leaves less than this is discarded
-constexpr double kDependent64 = 1e-10;
 
 struct EpiArgs {
   LevelState* st = nullptr;

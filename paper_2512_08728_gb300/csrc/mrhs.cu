@@ -45,14 +45,14 @@ constexpr int kGramWarps = 8;      // warps per block of the Gram / vector kerne
 // flight; one block per SM left these kernels latency-bound at 15-27 % of the FP64 rate
 constexpr int kGramBlocks = 4 * 152;
 
-enum : int { MF_REORTH = 1, MF_DISCARD = 2 };
+enum : int { MF_REORTH = 1, MF_DISCARD = 2, MF_OWN_NORM = 4 };
 
 // Device state of one level (one MG call is active per level at any time).
 struct MState {
   int any, any_restart, any_claim, any_reorth;   // flags of the last loop test and Gram pass
   int nact;                                      // active columns after the last test
   unsigned int ticket;                           // last-block counter of the reductions
-  int pad_f1, pad_f2;
+  int any_own, pad_f2;                           // some column's norm is taken from itself
   int R, lcap, maxit, it;
   int iters_total, nrestart, status, guard;
   int guard_cap, level, per_cycle, cap;    // restart when l + per_cycle > cap
@@ -79,8 +79,12 @@ constexpr unsigned ctl_seq(unsigned a, unsigned b = 0, unsigned c = 0) { return 
 // what the host reads of a loop test (pinned memory that the device writes)
 struct HostFlags { volatile int any, any_restart, any_claim, nact; volatile unsigned int seq; };
 
+// a level's basis and vectors, for own_columns()
+struct MColumns { double *W, *Z, *x, *r; int N; };
+
 // The control that follows a reduction: state, parent level's state (CTL_BEGIN), steps, the
-// coefficient arrays, the host's flags and the sequence number that marks them written.
+// coefficient arrays, the host's flags, the sequence number that marks them written, and the vectors
+// that CTL_FINISH may need.
 struct CtlArgs {
   MState* st;
   const MState* parent;
@@ -88,6 +92,7 @@ struct CtlArgs {
   double *sums, *cw, *cz;
   HostFlags* host;
   unsigned seq;
+  MColumns col;
 };
 
 // ------------------------------------------------------------------ small helpers
@@ -139,7 +144,7 @@ __device__ void mctl_step(const CtlArgs& c, unsigned kind) {
   double *cw = c.cw, *cz = c.cz;
   const int r = threadIdx.x;
   const int R = st->R, lcap = st->lcap;
-  bool f_any = false, f_restart = false, f_claim = false, f_reorth = false;
+  bool f_any = false, f_restart = false, f_claim = false, f_reorth = false, f_own = false;
   if (r < R) {
     switch (kind) {
       case CTL_INIT0: {
@@ -181,9 +186,8 @@ __device__ void mctl_step(const CtlArgs& c, unsigned kind) {
         f_any = st->act[r] != 0;
         break;
       }
-      // the norm of w_hat = w - W h by Pythagoras (used where it did not cancel below a quarter
-      // of ||w||^2; else a second pass is requested), alpha = w_hat . r = w . r (r is orthogonal
-      // to W)
+      // the norm of w_hat = w - W h by Pythagoras (kPythagoras; else a second pass is requested),
+      // alpha = w_hat . r = w . r (r is orthogonal to W)
       case CTL_GRAM1: {
         const int l = st->l[r];
         double hh = 0.0;
@@ -197,7 +201,7 @@ __device__ void mctl_step(const CtlArgs& c, unsigned kind) {
         const double naz2 = __ldcg(sums + (size_t)lcap * 32 + r), nw2 = naz2 - hh;
         st->naz2[r] = naz2;
         const bool discard = !st->act[r] || !isfinite(naz2) || !(naz2 > 0.0);
-        const bool reorth = !discard && l > 0 && nw2 < 0.25 * naz2;
+        const bool reorth = !discard && l > 0 && nw2 < kPythagoras * naz2;
         st->flags[r] = (discard ? MF_DISCARD : 0) | (reorth ? MF_REORTH : 0);
         st->gam[r] = st->alp[r] = 0.0;
         if (!discard && !reorth) {
@@ -207,8 +211,7 @@ __device__ void mctl_step(const CtlArgs& c, unsigned kind) {
         f_reorth = reorth;
         break;
       }
-      // w' = w - W h: kept while what this pass leaves can be told from rounding and is above
-      // brk_tol relative to ||A z||
+      // w' = w - W h
       case CTL_GRAM2: {
         if (st->flags[r] & MF_REORTH) {
           const int l = st->l[r];
@@ -221,7 +224,12 @@ __device__ void mctl_step(const CtlArgs& c, unsigned kind) {
             cw[(size_t)i * 32 + r] = h2;
           }
           const double n2 = __ldcg(sums + (size_t)lcap * 32 + r), nw2 = n2 - hh;
-          if (!isfinite(nw2) || !(nw2 > kDependent64 * n2) || !(nw2 > st->brk_tol * st->brk_tol * st->naz2[r])) {
+          if (!isfinite(nw2)) {
+            st->flags[r] |= MF_DISCARD;
+          } else if (nw2 < kPythagoras * n2) {
+            st->flags[r] |= MF_OWN_NORM;
+            f_own = true;
+          } else if (!(nw2 > st->brk_tol * st->brk_tol * st->naz2[r])) {
             st->flags[r] |= MF_DISCARD;
           } else {
             st->gam[r] = 1.0 / sqrt(nw2);
@@ -276,6 +284,7 @@ __device__ void mctl_step(const CtlArgs& c, unsigned kind) {
   f_restart = __any_sync(0xffffffffu, f_restart);
   f_claim = __any_sync(0xffffffffu, f_claim);
   f_reorth = __any_sync(0xffffffffu, f_reorth);
+  f_own = __any_sync(0xffffffffu, f_own);
   if (r == 0) {
     switch (kind) {
       case CTL_TEST: {
@@ -298,6 +307,7 @@ __device__ void mctl_step(const CtlArgs& c, unsigned kind) {
       case CTL_GRAM1:
       case CTL_GRAM2:
         st->any_reorth = f_reorth;
+        st->any_own = f_own;
         break;
       case CTL_RESTART:
         st->nrestart++;
@@ -330,6 +340,69 @@ __device__ void mctl_run(const CtlArgs& c) {
   }
 }
 
+// The columns whose norm is taken from themselves (MF_OWN_NORM; k_mupdate has formed them and left x
+// and r): gamma, alpha, x and r as k_mupdate does for the others, by one block, which is rare enough
+// not to matter.  sums: the ||r||^2 of these right-hand sides.
+__device__ __noinline__ void own_columns(MState* st, MColumns col, double* sums) {
+  __shared__ double red[2][kGramWarps][32], sc[2][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5, R = st->R, N = col.N;
+  const bool own = lane < R && (st->flags[lane] & MF_OWN_NORM) && !(st->flags[lane] & MF_DISCARD);
+  double *Wl = col.W, *Zl = col.Z;
+  if (own) {
+    Wl += (size_t)st->l[lane] * N * R + lane;
+    Zl += (size_t)st->l[lane] * N * R + lane;
+  }
+  double *x = col.x + lane, *rv = col.r + lane, nn = 0.0, wr = 0.0;
+  if (own)
+    for (int j = warp; j < N; j += nw) {
+      const double a = __ldcg(Wl + (size_t)j * R);
+      nn = fma(a, a, nn);
+      wr = fma(a, __ldcg(rv + (size_t)j * R), wr);
+    }
+  red[0][warp][lane] = nn;
+  red[1][warp][lane] = wr;
+  __syncthreads();
+  if (warp == 0) {
+    nn = wr = 0.0;
+    for (int w = 0; w < nw; ++w) {
+      nn += red[0][w][lane];
+      wr += red[1][w][lane];
+    }
+    const double n = sqrt(nn);
+    sc[0][lane] = sc[1][lane] = 0.0;
+    if (own) {
+      if (!isfinite(n) || !(n > st->brk_tol * sqrt(st->naz2[lane]))) {
+        st->flags[lane] |= MF_DISCARD;
+      } else {
+        st->gam[lane] = sc[0][lane] = 1.0 / n;
+        st->alp[lane] = sc[1][lane] = wr / n;
+      }
+    }
+  }
+  __syncthreads();
+  const double g = sc[0][lane], al = sc[1][lane];
+  double r2 = 0.0;
+  if (g != 0.0)
+    for (int j = warp; j < N; j += nw) {
+      const size_t o = (size_t)j * R;
+      const double wv = __ldcg(Wl + o) * g, zv = __ldcg(Zl + o) * g, r_ = fma(-al, wv, __ldcg(rv + o));
+      Wl[o] = wv;
+      Zl[o] = zv;
+      x[o] = fma(al, zv, __ldcg(x + o));
+      rv[o] = r_;
+      r2 = fma(r_, r_, r2);
+    }
+  red[0][warp][lane] = r2;
+  __syncthreads();
+  if (warp == 0 && g != 0.0) {
+    r2 = 0.0;
+    for (int w = 0; w < nw; ++w) r2 += red[0][w][lane];
+    sums[lane] = r2;
+  }
+  __threadfence_block();
+  __syncthreads();
+}
+
 // True in every thread of the block that finished last (all other blocks' writes visible).
 __device__ __forceinline__ bool mlast_block(unsigned int* ticket) {
   __shared__ int s_last;
@@ -357,6 +430,7 @@ __device__ __forceinline__ double mreduce_col(const double* part, int b0, int b1
 // End of a reduction kernel whose blocks wrote part[blk][c][32]: with c.steps the last block sums
 // the columns (c < L, and the ones from lcap on) and runs the control; without, a k_mreduce
 // launch does.
+template <bool FINISH = false>
 __device__ __forceinline__ void mfinish_reduction(const double* part, int pstride, int L, int lcap, const CtlArgs& c) {
   if (!c.steps) return;
   if (!mlast_block(&c.st->ticket)) return;
@@ -380,6 +454,7 @@ __device__ __forceinline__ void mfinish_reduction(const double* part, int pstrid
   if (threadIdx.x == 0) c.st->ticket = 0u;
   __threadfence_block();
   __syncthreads();
+  if (FINISH && c.st->any_own) own_columns(c.st, c.col, c.sums);
   mctl_run(c);
 }
 
@@ -976,6 +1051,7 @@ __global__ void __launch_bounds__(256) k_mreduce(const double* __restrict__ part
   if (threadIdx.x == 0) st->ticket = 0u;
   __threadfence_block();
   __syncthreads();
+  if ((ctl.steps & 15u) == CTL_FINISH && st->any_own) own_columns(st, ctl.col, ctl.sums);
   mctl_run(ctl);
 }
 
@@ -996,8 +1072,8 @@ __global__ void __launch_bounds__(256) k_mapply(const double* __restrict__ W, co
 }
 
 // The step of Alg. 1 per right-hand side: w_l = gamma (wsrc - W cw), z_l = gamma (z - Z cz) into
-// column l_r, x += alpha z_l, r -= alpha w_l (gamma, alpha from the Gram pass; discarded
-// corrections change nothing); part[blk][32] = ||r||^2.  UNROLL columns' loads in flight: eight on
+// column l_r, x += alpha z_l, r -= alpha w_l (gamma, alpha from the Gram pass, or own_columns() does
+// that part; discarded corrections change nothing); part[blk][32] = ||r||^2.  UNROLL columns' loads in flight: eight on
 // small levels, where they are what takes the time, four where many warps hide it and the
 // registers cost occupancy (32^3 x 32: eight 60.1, four 57.2 ms a cycle).
 template <int UNROLL>
@@ -1012,9 +1088,9 @@ __global__ void __launch_bounds__(256) k_mupdate(double* __restrict__ W, double*
   const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
   double v[1] = {0.0};
   if (lane < R) {
-    const bool upd = !(st->flags[lane] & MF_DISCARD);
+    const bool upd = !(st->flags[lane] & MF_DISCARD), own = (st->flags[lane] & MF_OWN_NORM) != 0;
     const int lr = st->l[lane];
-    const double g = st->gam[lane], al = st->alp[lane];
+    const double g = own ? 1.0 : st->gam[lane], al = st->alp[lane];
     const double* wsrc = (st->flags[lane] & MF_REORTH) ? wre : w;
     double* Wl = W + (size_t)lr * N * R;
     double* Zl = Z + (size_t)lr * N * R;
@@ -1034,15 +1110,17 @@ __global__ void __launch_bounds__(256) k_mupdate(double* __restrict__ W, double*
         zv *= g;
         Wl[o] = av;
         Zl[o] = zv;
-        x[o] = fma(al, zv, xo);
-        r_ = fma(-al, av, r_);
-        rv[o] = r_;
+        if (!own) {
+          x[o] = fma(al, zv, xo);
+          r_ = fma(-al, av, r_);
+          rv[o] = r_;
+        }
       }
       v[0] = fma(r_, r_, v[0]);
     }
   }
   block_cols<1>(v, red, part, 1, 0, 1);
-  mfinish_reduction(part, 1, 0, 0, ctl);
+  mfinish_reduction<true>(part, 1, 0, 0, ctl);
 }
 
 // part[blk][32] = sum of v^2 per right-hand side
@@ -1628,7 +1706,8 @@ int vec_grid(const MLev& L) { return grid_for((size_t)L.N, kGramWarps, kGramBloc
 
 // steps after the reduction, on level lev; a loop test among them gets the next sequence number
 CtlArgs ctl_args(MrhsEngine* E, int lev, unsigned steps, const MState* parent = nullptr) {
-  CtlArgs c{E->lv[lev].st, parent, steps, E->sums, E->cw, E->cz, E->hst, 0u};
+  const MLev& L = E->lv[lev];
+  CtlArgs c{L.st, parent, steps, E->sums, E->cw, E->cz, E->hst, 0u, {L.W, L.Z, L.x, L.r, L.N}};
   for (unsigned k = steps; k; k >>= 4)
     if ((k & 15u) == CTL_TEST) c.seq = ++E->seq;
   return c;

@@ -18,17 +18,26 @@ pytestmark = pytest.mark.gpu
 TYPES = {"f32": np.float32, "f64": np.float64}
 
 
-@pytest.fixture(scope="module")
-def lib(tmp_path_factory):
+def _compile(source, folder, *flags):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     path = pkg.build()
-    so = str(tmp_path_factory.mktemp("kernels") / "minimisation_kernels.so")
+    so = str(folder.mktemp("kernels") / (source + ".so"))
     here = os.path.dirname(os.path.abspath(__file__))
-    subprocess.run([B._nvcc(), *B.ARCH, *B.FLAGS, "-I", B.CSRC, "-shared", "-o", so,
-                    os.path.join(here, "minimisation_kernels.cu")], check=True)
+    subprocess.run([B._nvcc(), *B.ARCH, *B.FLAGS, *flags, "-I", B.CSRC, "-shared", "-o", so,
+                    os.path.join(here, source + ".cu")], check=True)
     C.CDLL(path, mode=C.RTLD_GLOBAL)
     return C.CDLL(so)
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    return _compile("minimisation_kernels", tmp_path_factory)
+
+
+@pytest.fixture(scope="module")
+def batched(tmp_path_factory):
+    return _compile("batched_minimisation_kernels", tmp_path_factory, "-Xptxas", "-O1")
 
 
 def _p(a):
@@ -117,3 +126,32 @@ def test_dependent_after_the_second_pass(lib, t):
     assert getattr(lib, "second_pass_" + t)(N, l, _p(W), _p(w), _p(w), C.c_double(1e28), _p(r), 3, C.byref(g),
                                             C.byref(a), C.byref(rn)) == 2
     assert np.array_equal(r, before) and abs(rn.value - np.linalg.norm(r.astype(np.float64))) <= 64 * 2.0**-53
+
+
+# the batched kernels: every right-hand side has its own basis and its own share left; one takes no part
+# (its correction is discarded already).  A thread sums N / (8 blocks) rows.
+@pytest.mark.parametrize("blocks,in_kernel", [(1, 1), (5, 1), (5, 0)])
+def test_columns_after_the_second_pass(batched, blocks, in_kernel):
+    N, l, left = 3000, 9, [0.9, 0.3, 0.2, 1e-3, 1e-6, 0.5]
+    R, part = len(left), np.array([1, 1, 1, 1, 1, 0], dtype=np.int32)
+    cols = [_basis(np.float64, N, l, s, seed=k) for k, s in enumerate(left)]
+    W, w, r = (np.ascontiguousarray(np.stack([c[k] for c in cols], axis=-1)) for k in range(3))
+    rng = np.random.default_rng(11)
+    Z, z, x = rng.standard_normal((l + 1, N, R)), rng.standard_normal((N, R)), rng.standard_normal((N, R))
+    W0, r0, x0 = W.copy(), r.copy(), x.copy()
+    ln, rn = np.zeros(R, dtype=np.int32), np.zeros(R)
+    assert batched.batched_second_pass(N, R, l, _p(W), _p(Z), _p(w), _p(z), C.c_double(4.0), _p(x), _p(r), _p(part),
+                                       in_kernel, blocks, _p(ln), _p(rn)) == 0
+    tol = 4 * (N / (8 * blocks) + 16) * 2.0**-53
+    for k in range(R):
+        if not part[k]:
+            assert ln[k] == l and np.array_equal(r[:, k], r0[:, k]) and np.array_equal(x[:, k], x0[:, k])
+            continue
+        wl = W[l, :, k]
+        assert ln[k] == l + 1 and abs(np.linalg.norm(wl) - 1) <= tol and abs(r[:, k] @ wl) <= tol
+        assert abs(rn[k] - np.linalg.norm(r[:, k])) <= 2 * tol
+        h = W0[:l, :, k] @ w[:, k]
+        g, al = 1.0 / np.linalg.norm(w[:, k] - h @ W0[:l, :, k]), (r0[:, k] - r[:, k]) @ wl
+        zl = g * (z[:, k] - h @ Z[:l, :, k])
+        assert np.abs(Z[l, :, k] - zl).max() <= tol / left[k] * np.abs(zl).max()
+        assert np.abs(x[:, k] - x0[:, k] - al * Z[l, :, k]).max() <= tol * np.abs(zl).max()
