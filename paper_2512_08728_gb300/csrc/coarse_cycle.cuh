@@ -647,8 +647,8 @@ struct CoarseCycle {
     count(opbytes(C, S, sizeof(T)) + (long long)N * sizeof(T) * 2 + (long long)(l + 1) * N * sizeof(T));
     if (!dots(W, N, l)) return false;
     ph(PH_RM_GRAM1);
-    // w_hat = w - W W^T w: its norm by Pythagoras; another pass whenever that cancelled
-    // more than half of it (classical Gram-Schmidt, "twice is enough")
+    // w_hat = w - W W^T w: its norm by Pythagoras; another pass whenever that leaves too little
+    // of it (kPythagoras; classical Gram-Schmidt, "twice is enough" but for a few columns of FP32 forms)
     double* Rc = R + (size_t)l * (l - 1) / 2;
     for (int pass = 0;; ++pass) {
       decide(l, pass);
@@ -695,6 +695,7 @@ struct CoarseCycle {
     return true;
   }
 
+  static constexpr int kMaxPasses = 48;   // 4^-48 < brk^2 = 1e-28
   // warp 0: the scalars of a Gram pass with l columns from red_s into rms (the caller's
   // __syncthreads publishes them)
   __device__ void decide(int l, int pass) {
@@ -711,10 +712,12 @@ struct CoarseCycle {
       rms->rr = red_s[l + 2];
     }
     const double tiny = a.brk * a.brk * rms->naz2;
+    // n2 is the sum over the vector as the passes have left it, so it tells what is rounding; every
+    // pass takes at least 1 - kPythagoras of it, which ends within kMaxPasses
     int v = 0;
-    if (!isfinite(n2) || !(n2 > 0.0)) v = 2;
-    else if (l > 0 && nw2 < 0.25 * n2 && pass < 3 && (pass == 0 || nw2 > tiny)) v = 1;
-    else if (!isfinite(nw2) || !(nw2 > tiny)) v = 2;
+    if (!isfinite(nw2) || !(n2 > (pass > 0 ? tiny : 0.0))) v = 2;
+    else if (l > 0 && nw2 < kPythagoras * n2) v = pass < kMaxPasses ? 1 : 2;
+    else if (!(nw2 > tiny)) v = 2;
     rms->verdict = v;
     if (v == 0) {
       const double gam = rsqrt(nw2), alp = gam * red_s[l + 1];

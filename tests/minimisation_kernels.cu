@@ -110,6 +110,28 @@ __global__ void k_dots(const __grid_constant__ CoarseArgs a, const T* W, int N, 
   for (int i = threadIdx.x; i < l + 3; i += blockDim.x) out[i] = red_s[i];
 }
 
+// what the persistent kernel does after a Gram pass with these sums (l coefficients, the last of them h)
+__global__ void k_decide(const __grid_constant__ CoarseArgs a, int l, int pass, double naz2, double n2, double h,
+                         int* verdict) {
+  __shared__ double red_s[64];
+  __shared__ RmScal rms;
+  CoarseCycle<double, double, double, kNP, 2, false> cc{a, nullptr, red_s, nullptr, &rms, nullptr, nullptr, nullptr};
+  for (int p = 0; p <= pass; p += max(1, pass)) {   // the first pass leaves ||A z||^2
+    __syncthreads();
+    for (int i = threadIdx.x; i < l + 3; i += blockDim.x) red_s[i] = 0.0;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      red_s[l] = p == 0 && pass > 0 ? naz2 : n2;
+      red_s[l + 1] = red_s[l + 2] = 1.0;
+      if (l > 0) red_s[l - 1] = h;
+    }
+    __syncthreads();
+    cc.decide(l, p);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) *verdict = rms.verdict;
+}
+
 template <typename T>
 int dots(int N, int l, const T* W, const T* w, const T* r, double* out) {
   Dev<T> dW(W, (size_t)(l + 1) * N), dw(w, N), dr(r, N);
@@ -133,6 +155,15 @@ using namespace step_test;
 
 extern "C" {
 
+int decide(int l, int pass, double naz2, double n2, double h) {
+  Dev<int> v(nullptr, 1);
+  CoarseArgs a{};
+  a.brk = 1e-14;
+  k_decide<<<1, 64>>>(a, l, pass, naz2, n2, h, v.p);
+  int r = -1;
+  if (cudaDeviceSynchronize() == cudaSuccess) v.get(&r);
+  return r;
+}
 int dots_f32(int N, int l, const float* W, const float* w, const float* r, double* out) { return dots<float>(N, l, W, w, r, out); }
 int dots_f64(int N, int l, const double* W, const double* w, const double* r, double* out) { return dots<double>(N, l, W, w, r, out); }
 

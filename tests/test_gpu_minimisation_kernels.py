@@ -155,3 +155,19 @@ def test_columns_after_the_second_pass(batched, blocks, in_kernel):
         zl = g * (z[:, k] - h @ Z[:l, :, k])
         assert np.abs(Z[l, :, k] - zl).max() <= tol / left[k] * np.abs(zl).max()
         assert np.abs(x[:, k] - x0[:, k] - al * Z[l, :, k]).max() <= tol * np.abs(zl).max()
+
+
+# The persistent kernel makes further passes until at least a quarter of the square is left, and discards
+# what the passes have brought down to brk = 1e-14 of ||A z||; no norm is a difference of less.
+TAKE, AGAIN, DISCARD = 0, 1, 2
+
+
+@pytest.mark.parametrize("l,passes,n2,left,want", [
+    (0, 0, 1.0, 1.0, TAKE), (5, 0, 1.0, 0.26, TAKE), (5, 0, 1.0, 0.24, AGAIN), (5, 0, 0.0, 0.0, DISCARD),
+    (5, 0, math.nan, 1.0, DISCARD), (5, 0, 1.0, -1e-15, AGAIN), (5, 1, 1e-20, 0.9, TAKE), (5, 1, 1e-20, 0.1, AGAIN),
+    (5, 1, 1e-20, -1e-7, AGAIN), (5, 1, 1e-29, 1.0, DISCARD), (5, 2, 1e-10, 0.1, AGAIN), (5, 3, 1e-10, 0.1, AGAIN),
+    (5, 3, 1e-10, 0.3, TAKE), (5, 3, 1e-29, 0.1, DISCARD), (5, 48, 1e-10, 0.1, DISCARD), (5, 48, 1e-10, 0.3, TAKE)])
+def test_what_follows_a_pass(lib, l, passes, n2, left, want):
+    h = math.sqrt(n2 * (1.0 - left)) if n2 == n2 else 0.0
+    f = lib.decide
+    assert f(l, passes, C.c_double(1.0), C.c_double(n2), C.c_double(h if l else 0.0)) == want
