@@ -2092,7 +2092,7 @@ kcmg_status kcmg_kernel_report(kcmg_ctx* ctx, int reps, double* out, int nout) {
           out[o + 2] = ms / reps;
           // operator and r, x, residual; patch inverses and their gathered/solved vectors;
           // the combination reads both patch solutions and x, writes x
-          out[o + 3] = (double)S * L.N * np * sb + 3.0 * L.N * sb + npat * m * m * ib + npat * m * 2 * sb +
+          out[o + 3] = ents * sb + 3.0 * L.N * sb + npat * m * m * ib + npat * m * 2 * sb +
                        4.0 * L.N * sb;
           return;
         }
