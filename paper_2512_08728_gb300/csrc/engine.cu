@@ -2178,6 +2178,7 @@ kcmg_status kcmg_kernel_report(kcmg_ctx* ctx, int reps, double* out, int nout) {
         // the first pass set the flags from zero vectors: clear them for a plain update
         h.gamma = 1.0;
         h.alpha = 0.0;
+        h.left = 0.0;
         CK(cudaMemcpyAsync(L.st, &h, sizeof h, cudaMemcpyHostToDevice, ctx->s));
         CK(cudaEventRecord(e0, ctx->s));
         for (int k = 0; k < reps; ++k) {

@@ -77,14 +77,17 @@ static __device__ void epilogue(const EpiArgs& e, const double* sums) {
     case EPI_MG_BEGIN: {
       st->rnorm0 = st->rnorm = sqrt(sums[0]);
       st->eps = fmax(st->rtol * st->rnorm0, st->atol);
-      st->l = 0; st->it = 0; st->flags = 0; st->breakdowns = 0; st->restart_req = 0;
+      st->l = 0; st->it = 0; st->flags = 0; st->breakdowns = 0; st->restart_req = 0; st->left = 0.0;
       if (!isfinite(st->rnorm)) st->status = KCMG_NONFINITE;
       record(e, 0);
       set_cond(e, more_cycles(st));
     } break;
     // W^T w, ||w||^2 and w . r decide the whole step: the norm of w_hat = w - W h by Pythagoras
     // (kPythagoras; else the second Gram-Schmidt pass is requested, "twice is enough"), and
-    // alpha = w_hat . r = w . r, as r is orthogonal to W
+    // alpha = w_hat . r = w . r - h . (W^T r).  r is orthogonal to W but for what its last update has
+    // left of the last column: alpha of that step was taken this way, too, and its error would come
+    // back multiplied with every h, until r grows (FP64, 12 x 12 x 8, p = 2, lmax 400: from 1e-16 to
+    // 1e-8 of ||b|| in 60 cycles).  The update measures it, and the next one takes it out.
     case EPI_GRAM1: {
       const int l = st->l;
       const double naz2 = sums[l], nw2 = naz2 - sums[l + 2];   // [l + 2]: sum of the squared coefficients
@@ -94,7 +97,7 @@ static __device__ void epilogue(const EpiArgs& e, const double* sums) {
       else if (l > 0 && nw2 < kPythagoras * naz2) f |= F_REORTH;
       else {
         st->gamma = 1.0 / sqrt(nw2);
-        st->alpha = st->gamma * sums[l + 1];
+        st->alpha = st->gamma * (sums[l + 1] - (l > 0 ? sums[l - 1] * st->left : 0.0));
       }
       if (!isfinite(naz2) && st->level == 0) st->status = KCMG_NONFINITE;
       st->flags = f;
@@ -112,12 +115,13 @@ static __device__ void epilogue(const EpiArgs& e, const double* sums) {
         st->flags |= F_DISCARD;
       } else {
         st->gamma = 1.0 / sqrt(nw2);
-        st->alpha = st->gamma * sums[l + 1];
+        st->alpha = st->gamma * (sums[l + 1] - sums[l - 1] * st->left);   // l > 0 here
       }
     } break;
     case EPI_FINISH: {
       if (!(st->flags & F_DISCARD)) {
         st->l++;
+        st->left = sums[1];
         st->breakdowns = 0;
       } else if (st->level == 0) {
         if (++st->breakdowns >= 2 && st->status == KCMG_OK) st->status = KCMG_BREAKDOWN;
@@ -136,6 +140,7 @@ static __device__ void epilogue(const EpiArgs& e, const double* sums) {
     case EPI_RESTART: {
       st->rnorm = sqrt(sums[0]);
       st->l = 0;
+      st->left = 0.0;
       st->restart_req = 0;
       st->nrestart++;
       if (!isfinite(st->rnorm) && st->status == KCMG_OK) st->status = KCMG_NONFINITE;

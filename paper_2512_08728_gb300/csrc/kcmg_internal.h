@@ -43,6 +43,7 @@ struct LevelState {
   double rnorm, rnorm0, eps, rtol, atol;
   double naz2;      // ||A z||^2 of the RM call in flight
   double gamma, alpha;
+  double left;      // w_{l-1} . r: what the last step has left of its column in r
   double brk;       // breakdown threshold relative to ||A z||
 };
 
@@ -57,7 +58,7 @@ enum EpiKind : int {
   EPI_MG_BEGIN,     // sum = ||r0||^2: start of an MG call on the level
   EPI_GRAM1,        // sums = W^T w, ||w||^2, w . r
   EPI_GRAM2,        // sums = W^T w', ||w'||^2, w' . r (reorthogonalisation pass)
-  EPI_FINISH,       // sum = ||r||^2 after the x, r update
+  EPI_FINISH,       // sums = ||r||^2 and w_l . r after the r update
   EPI_RESTART,      // sum = ||b - A x||^2: restart of the level
   EPI_NORM          // sum = ||y||^2 stored into *out (component calls, refinement)
 };

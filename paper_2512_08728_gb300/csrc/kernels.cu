@@ -428,8 +428,8 @@ k_gram_apply(const T* __restrict__ W, int N, const T* __restrict__ w, T* __restr
   }
 }
 
-// The step of Alg. 1: w_l = gamma (w_src - W c) as column l of W, r -= alpha w_l; ||r||^2 ->
-// EPI_FINISH.  gamma and alpha are known from the Gram pass, so the column is normalised and applied
+// The step of Alg. 1: w_l = gamma (w_src - W c) as column l of W, r -= alpha w_l + left w_{l-1} (what
+// the last step has left of its column); ||r||^2 and w_l . r -> EPI_FINISH.  gamma and alpha are known from the Gram pass, so the column is normalised and applied
 // as it is formed.  Without reorthogonalisation w_src = w, c = h; with it w_src = w' = w - W h,
 // c = h2.  The correction itself is stored as it comes, with its column of R (h, or h + h2):
 // A Z = W R with R_ll = 1 / gamma_l, so x follows from R y = alpha when it is needed (k_solve_y,
@@ -441,8 +441,8 @@ k_gram_apply(const T* __restrict__ W, int N, const T* __restrict__ w, T* __restr
 // from it, normalises and applies it (own_norm): one block's bandwidth, which is rare enough not to
 // matter, in place of two more launches in every minimisation.
 template <typename T>
-__device__ __noinline__ void own_norm(T* Wl, int N, T* r, const RmCoef& co, LevelState* st, double* r2, double* sh) {
-  __shared__ double sc[2];
+__device__ __noinline__ void own_norm(T* Wl, int N, T* r, const RmCoef& co, LevelState* st, double* sums, double* sh) {
+  __shared__ double sc[3];
   double v[2] = {0.0, 0.0};
   for (int j = threadIdx.x; j < N; j += blockDim.x) {   // written by other blocks: through L2
     const double a = __ldcg(Wl + j);
@@ -461,20 +461,28 @@ __device__ __noinline__ void own_norm(T* Wl, int N, T* r, const RmCoef& co, Leve
       st->alpha = sc[1] = v[1] / nw;
       co.gm[st->l] = sc[0];
       co.al[st->l] = sc[1];
+      if (st->l > 0) co.al[st->l - 1] += st->left;
     }
+    sc[2] = st->left;
   }
   __syncthreads();
   if (sc[0] == 0.0) return;   // discarded: r and its norm stay
-  const T gam = (T)sc[0], al = (T)sc[1];
-  double s[1] = {0.0};
+  const T gam = (T)sc[0], al = (T)sc[1], lf = (T)sc[2];
+  const T* Wp = Wl - (st->l > 0 ? N : 0);
+  v[0] = v[1] = 0.0;
   for (int j = threadIdx.x; j < N; j += blockDim.x) {
-    const T a = __ldcg(Wl + j) * gam, rv = fma(-al, a, __ldcg(r + j));
+    const T wp = lf != T(0) ? Wp[j] : T(0);
+    const T a = __ldcg(Wl + j) * gam, rv = fma(-al, a, fma(-lf, wp, __ldcg(r + j)));
     Wl[j] = a;
     r[j] = rv;
-    s[0] = fma((double)rv, (double)rv, s[0]);
+    v[0] = fma((double)rv, (double)rv, v[0]);
+    v[1] = fma((double)a, (double)rv, v[1]);
   }
-  bsum_n<1>(s, sh);
-  if (threadIdx.x == 0) *r2 = s[0];
+  bsum_n<2>(v, sh);
+  if (threadIdx.x == 0) {
+    sums[0] = v[0];
+    sums[1] = v[1];
+  }
 }
 
 template <typename T, bool PAIR>
@@ -487,7 +495,7 @@ k_gram_update(T* W, T* Z, int N, const T* __restrict__ w, const T* __restrict__ 
   __shared__ double sh[32 * 8];   // bsum_n<NC> needs 32 * NC
   const int l = st->l;
   const bool re = (st->flags & F_REORTH) != 0, keep = !(st->flags & F_DISCARD), own = (st->flags & F_OWN_NORM) != 0;
-  const T gam = own ? T(1) : (T)st->gamma, al = own ? T(0) : (T)st->alpha;
+  const T gam = own ? T(1) : (T)st->gamma, al = own ? T(0) : (T)st->alpha, lf = (T)st->left;
   if (keep)
     for (int i = threadIdx.x; i < l; i += blockDim.x) {
       cs[i] = re ? e.h2[i] : e.h[i];
@@ -496,12 +504,13 @@ k_gram_update(T* W, T* Z, int N, const T* __restrict__ w, const T* __restrict__ 
   if (keep && blockIdx.x == 0 && threadIdx.x == 0) {
     co.gm[l] = st->gamma;
     co.al[l] = st->alpha;
+    if (!own && l > 0) co.al[l - 1] += st->left;
   }
   __syncthreads();
   const T* ws = re ? wre : w;
   T* Wl = W + (size_t)l * N;
   T* Zl = Z + (size_t)l * N;
-  double r2 = 0.0;   // FP64 products and sums also of FP32 vectors: two FMAs a pair beside l
+  double r2 = 0.0, wr = 0.0;   // FP64 products and sums also of FP32 vectors: four FMAs a pair beside 2 l
   if (PAIR) {
     const int units = N / 2;
     for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < units; u += gridDim.x * blockDim.x) {
@@ -509,9 +518,10 @@ k_gram_update(T* W, T* Z, int N, const T* __restrict__ w, const T* __restrict__ 
       if (keep) {
         T2 a = __ldg(reinterpret_cast<const T2*>(ws) + u);
         reinterpret_cast<T2*>(Zl)[u] = __ldg(reinterpret_cast<const T2*>(z) + u);
+        T2 wi = {T(0), T(0)};
 #pragma unroll 4
         for (int i = 0; i < l; ++i) {
-          const T2 wi = __ldg(reinterpret_cast<const T2*>(W + (size_t)i * N) + u);
+          wi = __ldg(reinterpret_cast<const T2*>(W + (size_t)i * N) + u);
           const T cw = (T)(-cs[i]);
           a.x = fma(cw, wi.x, a.x);
           a.y = fma(cw, wi.y, a.y);
@@ -520,10 +530,12 @@ k_gram_update(T* W, T* Z, int N, const T* __restrict__ w, const T* __restrict__ 
         a.y *= gam;
         reinterpret_cast<T2*>(Wl)[u] = a;
         if (!own) {
-          rv.x = fma(-al, a.x, rv.x);
-          rv.y = fma(-al, a.y, rv.y);
+          rv.x = fma(-al, a.x, fma(-lf, wi.x, rv.x));
+          rv.y = fma(-al, a.y, fma(-lf, wi.y, rv.y));
           reinterpret_cast<T2*>(r)[u] = rv;
         }
+        wr = fma((double)a.x, (double)rv.x, wr);
+        wr = fma((double)a.y, (double)rv.y, wr);
       }
       r2 = fma((double)rv.x, (double)rv.x, r2);
       r2 = fma((double)rv.y, (double)rv.y, r2);
@@ -534,24 +546,32 @@ k_gram_update(T* W, T* Z, int N, const T* __restrict__ w, const T* __restrict__ 
       if (keep) {
         T a = ws[j];
         Zl[j] = z[j];
+        T wi = T(0);
 #pragma unroll 4
-        for (int i = 0; i < l; ++i) a = fma((T)(-cs[i]), __ldg(W + (size_t)i * N + j), a);
+        for (int i = 0; i < l; ++i) {
+          wi = __ldg(W + (size_t)i * N + j);
+          a = fma((T)(-cs[i]), wi, a);
+        }
         a *= gam;
         Wl[j] = a;
         if (!own) {
-          rv = fma(-al, a, rv);
+          rv = fma(-al, a, fma(-lf, wi, rv));
           r[j] = rv;
         }
+        wr = fma((double)a, (double)rv, wr);
       }
       r2 = fma((double)rv, (double)rv, r2);
     }
   }
-  double v[1] = {r2};
-  bsum_n<1>(v, sh);
-  if (threadIdx.x == 0) partial[blockIdx.x] = v[0];
+  double v[2] = {r2, wr};
+  bsum_n<2>(v, sh);
+  if (threadIdx.x == 0) {
+    partial[2 * blockIdx.x] = v[0];
+    partial[2 * blockIdx.x + 1] = v[1];
+  }
   if (last_block(&st->ticket)) {
-    __shared__ double sums[1];
-    reduce_few(partial, gridDim.x, 1, sums, sh);
+    __shared__ double sums[2];
+    reduce_few(partial, gridDim.x, 2, sums, sh);
     if (own && keep) own_norm<T>(Wl, N, r, co, st, sums, sh);
     if (threadIdx.x == 0) {
       epilogue(e, sums);

@@ -1,0 +1,37 @@
+"""Alg. 1 never raises the residual, also where the tolerance is out of reach and the basis goes on
+growing over corrections that depend on it: the solve ends at its iteration cap, not in a breakdown.
+
+A step takes out of r what it has along the new column and rounds it: 2^-53 of ||r|| for each of two
+updates of every entry, which near the rounding level of ||b||, kept over 400 columns, is up to
+sqrt(400) x 2^-52 = 4e-15 of ||b||; FP32 sweeps change the corrections, not this."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import paper_2512_08728_gb300 as pkg
+from workloads import make_problem
+
+pytestmark = pytest.mark.gpu
+FLOOR = 4e-15
+
+CASES = [(3, 2, (12, 12, 8), 3, 0), (3, 1, (24, 20, 20), 3, 1), (3, 2, (16, 10, 10), 2, 1), (2, 2, (32, 16), 3, 0)]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    pkg.build()
+
+
+@pytest.mark.parametrize("d,p,n,lv,seed", CASES)
+@pytest.mark.parametrize("precision", ["fp64", "mixed", "mixed_bf16"])
+def test_residual_past_the_attainable_accuracy(d, p, n, lv, seed, precision):
+    pr = make_problem(d, p, n, lv, nu_kind="jump", seed=seed)
+    s = pkg.KCycleSolver(pr, precision=precision, lmax=400, coarse_persistent=False)
+    x, info = s.solve(pr.b, rtol=1e-30, maxiter=130)
+    s.close()
+    h = info["hist"] / info["hist"][0]
+    assert info["status"] == 1 and info["iters"] == 130 and info["restarts"] == 0
+    assert np.all(h[1:] <= h[:-1] + FLOOR)
