@@ -59,6 +59,7 @@ struct MState {
   int act[kMaxRhs], l[kMaxRhs], flags[kMaxRhs], claim[kMaxRhs], brk[kMaxRhs], restart[kMaxRhs];
   double rtol, atol, brk_tol, pad2;
   double rnorm[kMaxRhs], rnorm0[kMaxRhs], eps[kMaxRhs], naz2[kMaxRhs], gam[kMaxRhs], alp[kMaxRhs];
+  double left[kMaxRhs];      // w_{l-1} . r: what the last step has left of its column in r
 };
 
 // Control steps; up to eight run one after another at the end of a reduction (packed, 4 bits each)
@@ -69,7 +70,7 @@ enum CtlKind : unsigned {
   CTL_TEST,     // loop test (level-local criteria); restart / claim flags, to the host as well
   CTL_GRAM1,    // sums = W^T w (columns < l), ||w||^2 (column lcap), w . r (column lcap + 1)
   CTL_GRAM2,    // sums = W^T w' and so on (reorthogonalisation pass)
-  CTL_FINISH,   // sums = ||r||^2 after the update
+  CTL_FINISH,   // sums = ||r||^2 and w_l . r after the update
   CTL_RESTART,  // sums = ||b - A x||^2 for the restarting right-hand sides
   CTL_CONFIRM,  // level 0: sums = true ||b - A x||^2 of the claiming right-hand sides
   CTL_ITEND     // end of an iteration
@@ -155,6 +156,7 @@ __device__ void mctl_step(const CtlArgs& c, unsigned kind) {
         st->act[r] = n0 > st->eps[r] && isfinite(n0);
         if (!isfinite(n0)) st->status = KCMG_NONFINITE;
         st->l[r] = 0;
+        st->left[r] = 0.0;
         st->flags[r] = 0;
         st->brk[r] = 0;
         st->claim[r] = 0;
@@ -168,6 +170,7 @@ __device__ void mctl_step(const CtlArgs& c, unsigned kind) {
         st->eps[r] = st->rtol * n0;
         st->act[r] = parent->act[r] && n0 > 0.0;
         st->l[r] = 0;
+        st->left[r] = 0.0;
         st->flags[r] = 0;
         st->restart[r] = 0;
         break;
@@ -187,7 +190,8 @@ __device__ void mctl_step(const CtlArgs& c, unsigned kind) {
         break;
       }
       // the norm of w_hat = w - W h by Pythagoras (kPythagoras; else a second pass is requested),
-      // alpha = w_hat . r = w . r (r is orthogonal to W)
+      // alpha = w_hat . r = w . r - h . (W^T r), where r is orthogonal to W but for what the last
+      // step has left of its column (epilogue.cuh, EPI_GRAM1)
       case CTL_GRAM1: {
         const int l = st->l[r];
         double hh = 0.0;
@@ -206,7 +210,8 @@ __device__ void mctl_step(const CtlArgs& c, unsigned kind) {
         st->gam[r] = st->alp[r] = 0.0;
         if (!discard && !reorth) {
           st->gam[r] = 1.0 / sqrt(nw2);
-          st->alp[r] = st->gam[r] * __ldcg(sums + (size_t)(lcap + 1) * 32 + r);
+          const double back = l > 0 ? __ldcg(sums + (size_t)(l - 1) * 32 + r) * st->left[r] : 0.0;
+          st->alp[r] = st->gam[r] * (__ldcg(sums + (size_t)(lcap + 1) * 32 + r) - back);
         }
         f_reorth = reorth;
         break;
@@ -232,8 +237,9 @@ __device__ void mctl_step(const CtlArgs& c, unsigned kind) {
           } else if (!(nw2 > st->brk_tol * st->brk_tol * st->naz2[r])) {
             st->flags[r] |= MF_DISCARD;
           } else {
+            const double back = __ldcg(sums + (size_t)(l - 1) * 32 + r) * st->left[r];   // l > 0 here
             st->gam[r] = 1.0 / sqrt(nw2);
-            st->alp[r] = st->gam[r] * __ldcg(sums + (size_t)(lcap + 1) * 32 + r);
+            st->alp[r] = st->gam[r] * (__ldcg(sums + (size_t)(lcap + 1) * 32 + r) - back);
           }
         }
         f_reorth = (st->flags[r] & MF_REORTH) != 0;
@@ -244,6 +250,7 @@ __device__ void mctl_step(const CtlArgs& c, unsigned kind) {
         if (!discard) {
           st->l[r] += 1;
           st->rnorm[r] = sqrt(__ldcg(sums + r));
+          st->left[r] = __ldcg(sums + 32 + r);
           st->brk[r] = 0;
         } else if (st->act[r]) {
           if (++st->brk[r] >= 2 && st->level == 0) {   // two consecutive discards
@@ -261,6 +268,7 @@ __device__ void mctl_step(const CtlArgs& c, unsigned kind) {
         if (st->restart[r]) {
           st->rnorm[r] = sqrt(__ldcg(sums + r));
           st->l[r] = 0;
+          st->left[r] = 0.0;
           st->restart[r] = 0;
         }
         break;
@@ -270,6 +278,7 @@ __device__ void mctl_step(const CtlArgs& c, unsigned kind) {
           const double rn = sqrt(__ldcg(sums + r));
           st->rnorm[r] = rn;
           st->l[r] = 0;
+          st->left[r] = 0.0;
           st->act[r] = rn > st->eps[r];
           st->claim[r] = 0;
         }
@@ -342,7 +351,7 @@ __device__ void mctl_run(const CtlArgs& c) {
 
 // The columns whose norm is taken from themselves (MF_OWN_NORM; k_mupdate has formed them and left x
 // and r): gamma, alpha, x and r as k_mupdate does for the others, by one block, which is rare enough
-// not to matter.  sums: the ||r||^2 of these right-hand sides.
+// not to matter.  sums: ||r||^2 and w_l . r of these right-hand sides.
 __device__ __noinline__ void own_columns(MState* st, MColumns col, double* sums) {
   __shared__ double red[2][kGramWarps][32], sc[2][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5, R = st->R, N = col.N;
@@ -380,24 +389,32 @@ __device__ __noinline__ void own_columns(MState* st, MColumns col, double* sums)
     }
   }
   __syncthreads();
-  const double g = sc[0][lane], al = sc[1][lane];
-  double r2 = 0.0;
+  const double g = sc[0][lane], al = sc[1][lane], lf = lane < R ? st->left[lane] : 0.0;
+  const size_t back = lf != 0.0 ? (size_t)N * R : 0;   // the column before (l > 0 where lf is not zero)
+  nn = wr = 0.0;
   if (g != 0.0)
     for (int j = warp; j < N; j += nw) {
       const size_t o = (size_t)j * R;
-      const double wv = __ldcg(Wl + o) * g, zv = __ldcg(Zl + o) * g, r_ = fma(-al, wv, __ldcg(rv + o));
+      const double wp = back ? (Wl - back)[o] : 0.0, zp = back ? (Zl - back)[o] : 0.0;
+      const double wv = __ldcg(Wl + o) * g, zv = __ldcg(Zl + o) * g, r_ = fma(-al, wv, fma(-lf, wp, __ldcg(rv + o)));
       Wl[o] = wv;
       Zl[o] = zv;
-      x[o] = fma(al, zv, __ldcg(x + o));
+      x[o] = fma(al, zv, fma(lf, zp, __ldcg(x + o)));
       rv[o] = r_;
-      r2 = fma(r_, r_, r2);
+      nn = fma(r_, r_, nn);
+      wr = fma(wv, r_, wr);
     }
-  red[0][warp][lane] = r2;
+  red[0][warp][lane] = nn;
+  red[1][warp][lane] = wr;
   __syncthreads();
   if (warp == 0 && g != 0.0) {
-    r2 = 0.0;
-    for (int w = 0; w < nw; ++w) r2 += red[0][w][lane];
-    sums[lane] = r2;
+    nn = wr = 0.0;
+    for (int w = 0; w < nw; ++w) {
+      nn += red[0][w][lane];
+      wr += red[1][w][lane];
+    }
+    sums[lane] = nn;
+    sums[32 + lane] = wr;
   }
   __threadfence_block();
   __syncthreads();
@@ -435,15 +452,17 @@ __device__ __forceinline__ void mfinish_reduction(const double* part, int pstrid
   if (!c.steps) return;
   if (!mlast_block(&c.st->ticket)) return;
   const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5, n = L + pstride - lcap, nblk = gridDim.x;
-  if (n == 1 && nw > 1) {   // one column: the warps take shares of the blocks
+  if ((n == 1 || FINISH) && nw > n) {   // one or two columns: the warps take shares of the blocks
     __shared__ double seg[32][32];
-    const int per = (nblk + nw - 1) / nw;
-    seg[warp][threadIdx.x & 31] = mreduce_col(part, min(nblk, warp * per), min(nblk, (warp + 1) * per), pstride, lcap - L);
+    const int k = warp % n, share = warp / n, ns = nw / n, per = (nblk + ns - 1) / ns;
+    if (share < ns)
+      seg[warp][threadIdx.x & 31] =
+          mreduce_col(part, min(nblk, share * per), min(nblk, (share + 1) * per), pstride, lcap - L + k);
     __syncthreads();
-    if (warp == 0) {
+    if (warp < n) {
       double t = 0.0;
-      for (int w = 0; w < nw; ++w) t += seg[w][threadIdx.x];
-      c.sums[(size_t)(lcap - L) * 32 + threadIdx.x] = t;
+      for (int w = warp; w < ns * n; w += n) t += seg[w][threadIdx.x & 31];
+      c.sums[(size_t)(lcap - L + warp) * 32 + (threadIdx.x & 31)] = t;
     }
   } else {
     for (int k = warp; k < n; k += nw) {
@@ -1072,8 +1091,9 @@ __global__ void __launch_bounds__(256) k_mapply(const double* __restrict__ W, co
 }
 
 // The step of Alg. 1 per right-hand side: w_l = gamma (wsrc - W cw), z_l = gamma (z - Z cz) into
-// column l_r, x += alpha z_l, r -= alpha w_l (gamma, alpha from the Gram pass, or own_columns() does
-// that part; discarded corrections change nothing); part[blk][32] = ||r||^2.  UNROLL columns' loads in flight: eight on
+// column l_r, x += alpha z_l + left z_{l-1}, r -= alpha w_l + left w_{l-1} (gamma, alpha from the Gram pass, or own_columns() does
+// that part; discarded corrections change nothing); part[blk][2][32] = ||r||^2,
+// w_l . r.  UNROLL columns' loads in flight: eight on
 // small levels, where they are what takes the time, four where many warps hide it and the
 // registers cost occupancy (32^3 x 32: eight 60.1, four 57.2 ms a cycle).
 template <int UNROLL>
@@ -1083,14 +1103,14 @@ __global__ void __launch_bounds__(256) k_mupdate(double* __restrict__ W, double*
                                                  double* __restrict__ rv, const double* __restrict__ cw,
                                                  const double* __restrict__ cz, double* __restrict__ part,
                                                  CtlArgs ctl) {
-  __shared__ double red[kGramWarps * 32];
+  __shared__ double red[kGramWarps * 2 * 32];
   const MState* st = ctl.st;
   const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
-  double v[1] = {0.0};
+  double v[2] = {0.0, 0.0};
   if (lane < R) {
     const bool upd = !(st->flags[lane] & MF_DISCARD), own = (st->flags[lane] & MF_OWN_NORM) != 0;
     const int lr = st->l[lane];
-    const double g = own ? 1.0 : st->gam[lane], al = st->alp[lane];
+    const double g = own ? 1.0 : st->gam[lane], al = st->alp[lane], lf = st->left[lane];
     const double* wsrc = (st->flags[lane] & MF_REORTH) ? wre : w;
     double* Wl = W + (size_t)lr * N * R;
     double* Zl = Z + (size_t)lr * N * R;
@@ -1100,27 +1120,31 @@ __global__ void __launch_bounds__(256) k_mupdate(double* __restrict__ W, double*
       if (upd) {
         double av = wsrc[o], zv = __ldg(z + o);
         const double xo = x[o];
+        double wi = 0.0, zi = 0.0;
 #pragma unroll UNROLL
         for (int i = 0; i < lr; ++i) {
           const size_t oi = ((size_t)i * N + j) * R + lane;
-          av = fma(-cw[(size_t)i * 32 + lane], __ldg(W + oi), av);
-          zv = fma(-cz[(size_t)i * 32 + lane], __ldg(Z + oi), zv);
+          wi = __ldg(W + oi);
+          zi = __ldg(Z + oi);
+          av = fma(-cw[(size_t)i * 32 + lane], wi, av);
+          zv = fma(-cz[(size_t)i * 32 + lane], zi, zv);
         }
         av *= g;
         zv *= g;
         Wl[o] = av;
         Zl[o] = zv;
         if (!own) {
-          x[o] = fma(al, zv, xo);
-          r_ = fma(-al, av, r_);
+          x[o] = fma(al, zv, fma(lf, zi, xo));
+          r_ = fma(-al, av, fma(-lf, wi, r_));
           rv[o] = r_;
         }
+        v[1] = fma(av, r_, v[1]);
       }
       v[0] = fma(r_, r_, v[0]);
     }
   }
-  block_cols<1>(v, red, part, 1, 0, 1);
-  mfinish_reduction<true>(part, 1, 0, 0, ctl);
+  block_cols<2>(v, red, part, 2, 0, 2);
+  mfinish_reduction<true>(part, 2, 0, 0, ctl);
 }
 
 // part[blk][32] = sum of v^2 per right-hand side
@@ -1847,7 +1871,7 @@ void rm(MrhsEngine* E, int lev, const double* zcor = nullptr, unsigned tail = 0)
   MLev& L = E->lv[lev];
   const int R = E->R, g = gram_grid(L), gv = vec_grid(L), thr = kGramWarps * 32, ps = L.lcap + 2;
   const double* zz = zcor ? zcor : L.z;
-  const bool in = in_kernel(g, ps), in1 = in_kernel(gv, 1);
+  const bool in = in_kernel(g, ps), in1 = in_kernel(gv, 2);
   const CtlArgs none = ctl_args(E, lev, CTL_NONE);
   const CtlArgs g1 = ctl_args(E, lev, CTL_GRAM1), g2 = ctl_args(E, lev, CTL_GRAM2);
   const CtlArgs fin = ctl_args(E, lev, ctl_seq(CTL_FINISH) | (tail << 4));
@@ -1859,7 +1883,7 @@ void rm(MrhsEngine* E, int lev, const double* zcor = nullptr, unsigned tail = 0)
   if (!in) reduce(E, g, ps, L.lcap, 1, g2);
   auto update = gv < kGramBlocks ? k_mupdate<8> : k_mupdate<4>;
   update<<<gv, thr, 0, E->s>>>(L.W, L.Z, L.N, R, L.w, L.wre, zz, L.x, L.r, E->cw, E->cz, E->part, in1 ? fin : none);
-  if (!in1) reduce(E, gv, 1, 0, 0, fin);
+  if (!in1) reduce(E, gv, 2, 0, 0, fin);
   E->launches += 4;
 }
 

@@ -54,7 +54,7 @@ extern "C" int batched_second_pass(int N, int R, int l, double* W, double* Z, co
   if (!in_kernel) k_mreduce<<<ps, 256>>>(part.p, blocks, ps, lcap, 1, g2);
   auto update = in_kernel ? k_mupdate<8> : k_mupdate<4>;
   update<<<blocks, thr>>>(dW.p, dZ.p, N, R, dw.p, dw.p, dz.p, dx.p, dr.p, cw.p, cz.p, part.p, in_kernel ? fin : none);
-  if (!in_kernel) k_mreduce<<<1, 256>>>(part.p, blocks, 1, 0, 0, fin);
+  if (!in_kernel) k_mreduce<<<2, 256>>>(part.p, blocks, 2, 0, 0, fin);
   const bool ok = cudaDeviceSynchronize() == cudaSuccess;
   cudaMemcpy(&h, st, sizeof h, cudaMemcpyDeviceToHost);
   cudaFree(st);
