@@ -558,14 +558,14 @@ struct CoarseCycle {
     return pt;
   }
 
-  // this block's sums of column c < l: W_c . w, l: w . w, l + 1: w . r, l + 2: r . r over the own
-  // rows; LPC lanes of a warp share a column.  The columns' per-thread sums are in T (coefficients of
+  // this block's sums of column c < l: W_c . w, l: w . w, l + 1: w . r, l + 2: r . r, l + 3 (l > 0):
+  // W_{l-1} . r over the own rows; LPC lanes of a warp share a column.  The columns' per-thread sums are in T (coefficients of
   // the size of ||w||); those of norms and w . r are FP64 products and sums in every form.
   template <int LPC>
   __device__ void dots_lpc(const T* W, int N, int l, double* pt) {
     constexpr int CPW = 32 / LPC;
     const int warp = threadIdx.x >> 5, ln = threadIdx.x & 31, nw = blockDim.x >> 5;
-    const int sub = ln / LPC, lc = ln - sub * LPC, n = l + 3, nsum = summands();
+    const int sub = ln / LPC, lc = ln - sub * LPC, n = sums_of(l), nsum = summands();
     const T* w = ws();
     const T* rs = rs_();
     for (int c0 = warp * CPW; c0 < n; c0 += nw * CPW) {
@@ -573,11 +573,11 @@ struct CoarseCycle {
       T s0 = T(0), s1 = T(0);
       double d = 0.0;
       if (sizeof(T) == 4 && c >= l && c < n) {
-        const T* u = c == l + 2 ? rs : w;
+        const T* u = c == l + 3 ? W + (size_t)(l - 1) * N + row0 : c == l + 2 ? rs : w;
         const T* v = c == l ? w : rs;
         for (int j = lc; j < rows; j += LPC) d = fma((double)u[j], (double)v[j], d);
       } else if (c < n) {
-        const T* u = c < l ? W + (size_t)c * N + row0 : c == l + 2 ? rs : w;
+        const T* u = c < l || c == l + 3 ? W + (size_t)(c < l ? c : l - 1) * N + row0 : c == l + 2 ? rs : w;
         const T* v = c <= l ? w : rs;
         int j = lc;
         for (; j + LPC < rows; j += 2 * LPC) {
@@ -598,8 +598,9 @@ struct CoarseCycle {
   __device__ bool dots(const T* W, int N, int l) {
     double* pt = next_partial();
     dots_lpc<8>(W, N, l, pt);   // few lanes a column: fewer FP64 instructions in the lanes' sum
-    return reduce_cols(pt, l + 3);
+    return reduce_cols(pt, sums_of(l));
   }
+  __device__ static int sums_of(int l) { return l > 0 ? l + 4 : 3; }
 
   // v[row] - sum_c W[c][row] cf[c] -> f(own row, value), columns split over lpr threads a row
   template <typename F>
@@ -650,6 +651,15 @@ struct CoarseCycle {
     // w_hat = w - W W^T w: its norm by Pythagoras; another pass whenever that leaves too little
     // of it (kPythagoras; classical Gram-Schmidt, "twice is enough" but for a few columns of FP32 forms)
     double* Rc = R + (size_t)l * (l - 1) / 2;
+    // r is orthogonal to W but for what the last step has left of its column (epilogue.cuh, EPI_GRAM1):
+    // out of r now, by the warps that do not decide, and into that step's alpha
+    if (l > 0) {
+      const int q = (int)blockDim.x - 1 - (int)threadIdx.x;
+      const T left = (T)red_s[l + 3];
+      const T* Wp = W + (size_t)(l - 1) * N + row0;
+      for (int lr = q; lr < rows; lr += blockDim.x) rs[lr] = fma(-left, Wp[lr], rs[lr]);
+      if (q == 0 && own_coef()) al[l - 1] += red_s[l + 3];
+    }
     for (int pass = 0;; ++pass) {
       decide(l, pass);
       for (int i = threadIdx.x; i < l; i += blockDim.x) {
@@ -672,7 +682,7 @@ struct CoarseCycle {
       sc.r2 = rms->rr;
       return true;
     }
-    const T g = (T)rms->gam, al_t = (T)rms->alp;   // alpha = w_hat . r (r is orthogonal to W)
+    const T g = (T)rms->gam, al_t = (T)rms->alp;
     T* Wl = W + (size_t)l * N + row0;
     T* Zl = vec(C.Z) + (size_t)l * N + row0;
     project(W, N, l, w, [&](int lr, T v) {
@@ -706,10 +716,11 @@ struct CoarseCycle {
 #pragma unroll
       for (int o = 16; o; o >>= 1) hh += __shfl_xor_sync(0xffffffffu, hh, o);
     if (threadIdx.x != 0) return;
-    const double n2 = red_s[l], nw2 = n2 - hh;
+    const double n2 = red_s[l], nw2 = n2 - hh, left = pass == 0 && l > 0 ? red_s[l + 3] : 0.0;
     if (pass == 0) {
       rms->naz2 = n2;
-      rms->rr = red_s[l + 2];
+      const double rr = red_s[l + 2] - left * left;
+      rms->rr = rr < 0.0 ? 0.0 : rr;   // (a NaN stays one)
     }
     const double tiny = a.brk * a.brk * rms->naz2;
     // n2 is the sum over the vector as the passes have left it, so it tells what is rounding; every
@@ -720,7 +731,7 @@ struct CoarseCycle {
     else if (!(nw2 > tiny)) v = 2;
     rms->verdict = v;
     if (v == 0) {
-      const double gam = rsqrt(nw2), alp = gam * red_s[l + 1];
+      const double gam = rsqrt(nw2), alp = gam * (red_s[l + 1] - (l > 0 ? red_s[l - 1] * left : 0.0));
       rms->gam = gam;
       rms->alp = alp;
       rms->r2new = rms->rr - alp * alp;

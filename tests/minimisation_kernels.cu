@@ -88,7 +88,8 @@ int second_pass(int N, int l, T* W, const T* w, const T* z, double naz2, T* r, i
   return st.l == l + 1 ? 0 : 2;
 }
 
-// the persistent kernel's sums over a block that is alone on its level: W^T w, w . w, w . r, r . r
+// the persistent kernel's sums over a block that is alone on its level: W^T w, w . w, w . r, r . r, and
+// the last column's with r
 constexpr int kNP = 3;
 template <typename T>
 __global__ void k_dots(const __grid_constant__ CoarseArgs a, const T* W, int N, int l, const T* w, const T* r,
@@ -107,7 +108,7 @@ __global__ void k_dots(const __grid_constant__ CoarseArgs a, const T* W, int N, 
   }
   __syncthreads();
   cc.dots(W, N, l);
-  for (int i = threadIdx.x; i < l + 3; i += blockDim.x) out[i] = red_s[i];
+  for (int i = threadIdx.x; i < l + 4; i += blockDim.x) out[i] = l > 0 || i < 3 ? red_s[i] : 0.0;
 }
 
 // what the persistent kernel does after a Gram pass with these sums (l coefficients, the last of them h)
@@ -118,7 +119,7 @@ __global__ void k_decide(const __grid_constant__ CoarseArgs a, int l, int pass, 
   CoarseCycle<double, double, double, kNP, 2, false> cc{a, nullptr, red_s, nullptr, &rms, nullptr, nullptr, nullptr};
   for (int p = 0; p <= pass; p += max(1, pass)) {   // the first pass leaves ||A z||^2
     __syncthreads();
-    for (int i = threadIdx.x; i < l + 3; i += blockDim.x) red_s[i] = 0.0;
+    for (int i = threadIdx.x; i < l + 4; i += blockDim.x) red_s[i] = 0.0;
     __syncthreads();
     if (threadIdx.x == 0) {
       red_s[l] = p == 0 && pass > 0 ? naz2 : n2;
@@ -135,7 +136,7 @@ __global__ void k_decide(const __grid_constant__ CoarseArgs a, int l, int pass, 
 template <typename T>
 int dots(int N, int l, const T* W, const T* w, const T* r, double* out) {
   Dev<T> dW(W, (size_t)(l + 1) * N), dw(w, N), dr(r, N);
-  Dev<double> dout(nullptr, l + 3);
+  Dev<double> dout(nullptr, l + 4);
   CoarseArgs a{};
   a.nlev = 2;
   a.cols = l + 1;

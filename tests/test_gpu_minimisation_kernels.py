@@ -69,10 +69,10 @@ def test_norms_of_the_persistent_kernel_sum_in_fp64(lib, t, N, l):
     w, r = np.full(N, 2.0**-13, dtype=T), np.full(N, -(2.0**-13), dtype=T)
     w[:16], r[:16] = 1.0, 1.0
     W = np.random.default_rng(1).standard_normal((l + 1, N)).astype(T)
-    out = np.zeros(l + 3)
+    out = np.zeros(l + 4)
     assert getattr(lib, "dots_" + t)(N, l, _p(W), _p(w), _p(r), _p(out)) == 0
     tol = (N / 8 + 5) * 2.0**-53
-    for got, a, b in ((out[l], w, w), (out[l + 1], w, r), (out[l + 2], r, r)):
+    for got, a, b in ((out[l], w, w), (out[l + 1], w, r), (out[l + 2], r, r)) + (((out[l + 3], W[l - 1], r),) if l else ()):
         terms = a.astype(np.float64) * b.astype(np.float64)
         assert abs(got - math.fsum(terms)) <= tol * np.abs(terms).sum()
     # the columns' sums are in the vectors' type: N / 16 terms an accumulator

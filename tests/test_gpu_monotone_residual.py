@@ -27,9 +27,10 @@ def _built():
 
 @pytest.mark.parametrize("d,p,n,lv,seed", CASES)
 @pytest.mark.parametrize("precision", ["fp64", "mixed", "mixed_bf16"])
-def test_residual_past_the_attainable_accuracy(d, p, n, lv, seed, precision):
+@pytest.mark.parametrize("persistent", [False, True])
+def test_residual_past_the_attainable_accuracy(d, p, n, lv, seed, precision, persistent):
     pr = make_problem(d, p, n, lv, nu_kind="jump", seed=seed)
-    s = pkg.KCycleSolver(pr, precision=precision, lmax=400, coarse_persistent=False)
+    s = pkg.KCycleSolver(pr, precision=precision, lmax=400, coarse_persistent=persistent)
     x, info = s.solve(pr.b, rtol=1e-30, maxiter=130)
     s.close()
     h = info["hist"] / info["hist"][0]
@@ -39,12 +40,13 @@ def test_residual_past_the_attainable_accuracy(d, p, n, lv, seed, precision):
 
 @pytest.mark.parametrize("d,p,n,lv,seed", CASES)
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
-def test_batched_solve_past_the_attainable_accuracy(d, p, n, lv, seed, precision):
+@pytest.mark.parametrize("persistent", [False, True])
+def test_batched_solve_past_the_attainable_accuracy(d, p, n, lv, seed, precision, persistent):
     """Batched solves record no residuals: a breakdown shows, or a solution that got worse.  390 columns
     that depend on one another cost x up to 1e-8 of ||b|| in its true residual in exact-norm arithmetic,
     too; 1e-6 is asked for."""
     pr = make_problem(d, p, n, lv, nu_kind="jump", seed=seed, nrhs=3)
-    s = pkg.KCycleSolver(pr, precision=precision, lmax=400, coarse_persistent=False)
+    s = pkg.KCycleSolver(pr, precision=precision, lmax=400, coarse_persistent=persistent)
     x, info = s.solve(pr.b, rtol=1e-30, maxiter=130)
     s.close()
     assert info["status"] == 1 and info["rel_res"] <= 1e-6
