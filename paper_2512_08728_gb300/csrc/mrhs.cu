@@ -1095,9 +1095,11 @@ __global__ void __launch_bounds__(256) k_mapply(const double* __restrict__ W, co
 // that part; discarded corrections change nothing); part[blk][2][32] = ||r||^2,
 // w_l . r.  UNROLL columns' loads in flight: eight on
 // small levels, where they are what takes the time, four where many warps hide it and the
-// registers cost occupancy (32^3 x 32: eight 60.1, four 57.2 ms a cycle).
+// registers cost occupancy (32^3 x 32: eight 60.1, four 57.2 ms a cycle).  Five blocks' registers
+// there, where own_columns() alone would take four's (32^3 x 32, eight cycles of m = 12: 1,658 ->
+// 1,564 ms).
 template <int UNROLL>
-__global__ void __launch_bounds__(256) k_mupdate(double* __restrict__ W, double* __restrict__ Z, int N, int R,
+__global__ void __launch_bounds__(256, UNROLL == 4 ? 5 : 4) k_mupdate(double* __restrict__ W, double* __restrict__ Z, int N, int R,
                                                  const double* __restrict__ w, const double* __restrict__ wre,
                                                  const double* __restrict__ z, double* __restrict__ x,
                                                  double* __restrict__ rv, const double* __restrict__ cw,
