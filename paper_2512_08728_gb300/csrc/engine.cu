@@ -1707,17 +1707,27 @@ bool in_place_ok(const kcmg_ctx* ctx, const void* in, const void* out, size_t n)
   return true;
 }
 
+// first waits for what second has been given so far.  A null stream is the default one of the current
+// device, so that is the context's for the duration.
+void stream_waits(kcmg_ctx* ctx, cudaStream_t first, cudaStream_t second) {
+  int cur = 0;
+  CK(cudaGetDevice(&cur));
+  if (cur != ctx->dev) CK(cudaSetDevice(ctx->dev));
+  cudaError_t e = cudaEventRecord(ctx->ev, second);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(first, ctx->ev, 0);
+  if (cur != ctx->dev) CK(cudaSetDevice(cur));
+  CK(e);
+}
+
 template <typename F>
 kcmg_status guarded(kcmg_ctx* ctx, F&& f) {
   if (!ctx) return KCMG_INVALID_ARG;
   try {
     // also where the caller's stream is the default one (null): the library's own stream does not
     // wait for that by itself
-    CK(cudaEventRecord(ctx->ev, ctx->user));
-    CK(cudaStreamWaitEvent(ctx->s, ctx->ev, 0));
+    stream_waits(ctx, ctx->s, ctx->user);
     kcmg_status st = f();
-    CK(cudaEventRecord(ctx->ev, ctx->s));
-    CK(cudaStreamWaitEvent(ctx->user, ctx->ev, 0));
+    stream_waits(ctx, ctx->user, ctx->s);
     return st;
   } catch (Fail& e) {
     return e.st;
@@ -1787,10 +1797,7 @@ kcmg_status kcmg_solve_adjoint(kcmg_ctx* ctx, const double* g, double* lambda, i
     kcmg_status st = ensure_adjoint(ctx);
     if (st != KCMG_OK) return st;
     kcmg_ctx* a = ctx->adj;
-    if (a != ctx) {   // its stream waits for the caller's work, as this context's does
-      CK(cudaEventRecord(ctx->ev, ctx->s));
-      CK(cudaStreamWaitEvent(a->s, ctx->ev, 0));
-    }
+    if (a != ctx) stream_waits(ctx, a->s, ctx->s);   // for the caller's work, as this context's stream does
     kcmg_status s2 = nrhs > 1 ? solve_multi(a, g, lambda, nrhs, rtol, atol, maxiter, info)
                               : solve_impl(a, g, lambda, rtol, atol, maxiter, info);
     if (a == ctx) return s2;
