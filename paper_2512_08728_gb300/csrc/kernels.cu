@@ -485,8 +485,10 @@ __device__ __noinline__ void own_norm(T* Wl, int N, T* r, const RmCoef& co, Leve
   }
 }
 
+// Registers for six blocks an SM with FP32 vectors and four with FP64 (64^3, np = 10, l = 206: 0.92
+// -> 0.59 ms with FP32 vectors, which own_norm alone would give five; 0.98 ms with FP64).
 template <typename T, bool PAIR>
-__global__ void __launch_bounds__(kVecThreads)
+__global__ void __launch_bounds__(kVecThreads, sizeof(T) == 4 ? 6 : 4)
 k_gram_update(T* W, T* Z, int N, const T* __restrict__ w, const T* __restrict__ wre,
               const T* __restrict__ z, RmCoef co, T* __restrict__ r, double* partial, EpiArgs e) {
   using T2 = typename Pair<T>::type;
@@ -510,7 +512,10 @@ k_gram_update(T* W, T* Z, int N, const T* __restrict__ w, const T* __restrict__ 
   const T* ws = re ? wre : w;
   T* Wl = W + (size_t)l * N;
   T* Zl = Z + (size_t)l * N;
-  double r2 = 0.0, wr = 0.0;   // FP64 products and sums also of FP32 vectors: four FMAs a pair beside 2 l
+  // ||r||^2 with FP64 products and sums also of FP32 vectors (two FMAs a pair and the conversions, 2
+  // clocks of an SM beside the 3 of l = 200 columns); w_l . r, itself of the size of a rounding, in T
+  double r2 = 0.0;
+  T wr = T(0);
   if (PAIR) {
     const int units = N / 2;
     for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < units; u += gridDim.x * blockDim.x) {
@@ -534,8 +539,8 @@ k_gram_update(T* W, T* Z, int N, const T* __restrict__ w, const T* __restrict__ 
           rv.y = fma(-al, a.y, fma(-lf, wi.y, rv.y));
           reinterpret_cast<T2*>(r)[u] = rv;
         }
-        wr = fma((double)a.x, (double)rv.x, wr);
-        wr = fma((double)a.y, (double)rv.y, wr);
+        wr = fma(a.x, rv.x, wr);
+        wr = fma(a.y, rv.y, wr);
       }
       r2 = fma((double)rv.x, (double)rv.x, r2);
       r2 = fma((double)rv.y, (double)rv.y, r2);
@@ -558,12 +563,12 @@ k_gram_update(T* W, T* Z, int N, const T* __restrict__ w, const T* __restrict__ 
           rv = fma(-al, a, fma(-lf, wi, rv));
           r[j] = rv;
         }
-        wr = fma((double)a, (double)rv, wr);
+        wr = fma(a, rv, wr);
       }
       r2 = fma((double)rv, (double)rv, r2);
     }
   }
-  double v[2] = {r2, wr};
+  double v[2] = {r2, (double)wr};
   bsum_n<2>(v, sh);
   if (threadIdx.x == 0) {
     partial[2 * blockIdx.x] = v[0];
@@ -1099,7 +1104,7 @@ void launch_coarse_gemv(const double* Ainv, int n, const T* b, T* x, cudaStream_
 }
 
 // dynamic shared memory: the final sums (lcap + 3 doubles) or the coefficients
-// (lcap or 2 lcap doubles); lcap <= kLcapMax keeps it within the default 48 KB
+// (lcap doubles); lcap <= kLcapMax keeps it within the default 48 KB
 template <typename T>
 void launch_gram_dots(const T* W, int N, const T* w, const T* r, int lcap, int nblk, double* partial,
                       const EpiArgs& e, int conditional, cudaStream_t s) {
