@@ -87,17 +87,18 @@ FP64_PEAK_NOTE = ("FP64 FMA peak from unit counts and clock: 152 SMs x 2 FMA/clk
                   "2.07 GHz = %.3f TFLOP/s, i.e. %.0f GB/s of 8-byte operands at one FMA each"
                   % (FP64_TFLOPS, FP64_TFLOPS * 1e3 / 2 * 8))
 
-# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of the kernels the bench
-# reports, from one ncu capture each, as bytes per unit of work (k_gram_update: per
-# (basis column + 2.5) x DOF, the unit its algorithmic bytes (2 l + 5) N 8 count), keyed by
-# kernel; valid only while the kernel's sources hash to the recorded value (otherwise the
-# line reports null).
+# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of the Gram kernels, from one ncu
+# capture each of a level-0 launch on 48^3 p=2 with 199 basis vectors, as bytes per vector entry
+# that the algorithm reads or writes (k_gram_dots: l columns, w and r; k_gram_update: the same and
+# z, and three vectors written), keyed by kernel; valid only while the kernels' sources hash to
+# the recorded value (otherwise the line reports null).
+TRAFFIC_VECTORS = {"k_gram_dots": 2, "k_gram_update": 6}   # beside the l columns
+_GRAM_SOURCES = ["kernels.cu", "epilogue.cuh", "kcmg_internal.h", "reduce.cuh"]
+_GRAM_NOTE = ("ncu capture (dram__bytes_read.sum + dram__bytes_write.sum) of one level-0 launch on 48^3 "
+              "p=2 with 199 basis vectors: %.3f GB per launch, scaled to this launch by (l + %d) N")
 TRAFFIC = {
-    "k_gram_update": (3567589888.0 / ((2 * 199 + 5) * 1105920), "41bfa758cbb3ac94",
-                      ["kernels.cu", "kcmg_internal.h", "reduce.cuh"],
-                      "ncu capture (dram__bytes_read.sum + dram__bytes_write.sum) of one level-0 "
-                      "launch on 48^3 p=2 with 199 basis vectors: 3.568 GB per launch, scaled to "
-                      "this launch by (2 l + 5) N"),
+    "k_gram_dots": (0.0, "", _GRAM_SOURCES, _GRAM_NOTE % (0.0, 2)),
+    "k_gram_update": (0.0, "", _GRAM_SOURCES, _GRAM_NOTE % (0.0, 6)),
 }
 
 
@@ -113,10 +114,10 @@ def _traffic(kernel):
     t = TRAFFIC.get(kernel)
     if not t:
         return None, None
-    per_launch, sha, files, note = t
+    per_unit, sha, files, note = t
     if _sources_sha(files) != sha:
         return None, "kernel changed since the capture (" + note + ")"
-    return per_launch, note
+    return per_unit, note
 
 
 class ClockSampler:
@@ -611,8 +612,8 @@ def main():
     # Alg. 1's Gram kernels on level 0 (one launch of each per level-0 RM), timed at the
     # basis length halfway through a restart period; level-1 launches are not counted
     n_rm0 = cycles * rms0
-    for kname, key, what in (("k_gram_update", "gram_update", "Alg. 1 new column: w - W h, z - Z h (FP64), level 0"),
-                             ("k_gram_dots", "gram_dots", "Alg. 1 first Gram pass: W^T w, ||w||^2 (FP64), level 0")):
+    for kname, key, what in (("k_gram_update", "gram_update", "Alg. 1 new column: w - W h and r (FP64), level 0"),
+                             ("k_gram_dots", "gram_dots", "Alg. 1 first Gram pass: W^T w, ||w||^2, w . r (FP64), level 0")):
         t, fl = rep[key + "_ms"], rep[key + "_flop"]
         tf = fl / (t * 1e-3) / 1e12 if t > 0 else 0.0
         kernels.append({"name": kname, "what": what, "bound": "alu", "achieved": tf, "peak": FP64_TFLOPS,
@@ -624,8 +625,8 @@ def main():
     # the dominant kernel: the largest share of the solve among the kernels timed here
     dom = max(kernels, key=lambda k: k["share_of_step"] or 0.0)
     traffic, traffic_note = _traffic(dom["name"])
-    if traffic is not None and dom["name"] == "k_gram_update":   # bytes per unit -> per launch
-        traffic = traffic * (2 * rep["gram_l"] + 5) * pr.ndof
+    if traffic is not None:   # bytes per vector entry -> per launch
+        traffic *= (rep["gram_l"] + TRAFFIC_VECTORS[dom["name"]]) * pr.ndof
 
     # end to end through the C interface with pinned host buffers: every step copies b
     # and x0 to the device and x back inside the timed region

@@ -193,9 +193,10 @@ kcmg_status kcmg_setup(kcmg_ctx **out, const kcmg_params *p, void *cuda_stream);
    ||b_j - A x_j|| <= max(rtol ||b_j - A x0_j||, atol), confirmed by a compensated FP64
    true residual.  The batched form is host-driven (use_graph is ignored).  Its level-0
    basis holds lmax vectors per column (default 60 when lmax = 0) plus one cycle's
-   corrections, shrunk to what the device can hold.  Small problems (with coarse_persistent) run
-   in one kernel, every column on its own group of blocks with its own operator applications,
-   loop and stopping test; the sweeps of the mixed forms are then FP32 FMAs.  Otherwise, in the
+   corrections, shrunk to what the device can hold.  Small problems (with coarse_persistent, and
+   whole bases that fit in that share of the free memory) run in one kernel, every column on its
+   own group of blocks with its own operator applications, loop and stopping test; the sweeps of
+   the mixed forms are then FP32 FMAs.  Otherwise, in the
    mixed forms, the block-Jacobi sweeps run on the tensor cores (TF32 products, FP32
    accumulation) or the CUDA cores, with launch shapes chosen by an autotuner at the first such
    solve (see kcmg_mrhs_tuning).  info: iters and level_iters count the shared loop (in the one

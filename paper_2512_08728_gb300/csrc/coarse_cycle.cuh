@@ -14,9 +14,10 @@
 //     sum, a block copies its neighbours' slabs of the iterate (the ranges shifted by the grid's
 //     strides) to shared memory: one L2 round trip a phase in place of one per use.
 //   - A row's products are split over several threads where a block has fewer rows than threads.
-//   - One reduction per residual minimisation: W^T w, ||w||^2, w.r and ||r||^2 together give the
-//     coefficients, the new column's norm (Pythagoras, guarded by the reorthogonalisation test)
-//     and alpha, so the column is normalised as it is formed and no second reduction is needed.
+//   - One reduction per residual minimisation: W^T w, ||w||^2, w.r, ||r||^2 and the last column's
+//     product with r together give the coefficients, the new column's norm (Pythagoras, guarded by
+//     the reorthogonalisation test) and alpha, so the column is normalised as it is formed and no
+//     second reduction is needed.
 //     The next smoother's first sweep needs own rows only: no barrier in between.
 //   - Corrections are stored as they come; x = sum_k y_k z_k with R y = alpha (R: the
 //     orthogonalisation coefficients) is formed when the level returns or restarts, so Alg. 1's
@@ -32,8 +33,7 @@
 // neighbour value through L2 and reduced three times a minimisation): levels 16^3 and 8^3 at
 // np = 10 beside the finest level's kernels 971 -> 553 us; 64 x 48 and two levels below at
 // np = 10, 2-D, 16.7 -> 8.2 ms; 16^3 and 8^3 alone, 16 visits, 5.0 -> 2.7 ms; 192 unknowns
-// 749 -> 257 us.  Whole solves to 1e-11, finest level on a kernel a step before: 16 x 16, np = 3,
-// 20.4 -> 13.5 ms; 8^3, np = 10, mixed, 28.3 -> 21.5 ms.
+// 749 -> 257 us.  Whole solves: whole_solve() (engine.cu).
 // Every control decision is taken by all blocks from the same reduced values (fixed reduction
 // order), so all blocks follow the same path.  The grid barrier spins with a bound: if it ever
 // times out it raises an error flag and every block leaves the kernel, so a fault becomes a
@@ -148,7 +148,8 @@ struct RmScal {
 
 // Vectors, basis W, Z, the Alg. 1 operator and the transfers are in TV (FP64, or FP32 in
 // the inner solve of the iterative-refinement forms); the smoother sweeps run in TS with
-// inverses stored as TI.  Reductions and Gram coefficients are FP64 in every form.
+// inverses stored as TI.  Reductions over lanes and blocks, norms and alpha are FP64 in every form;
+// a lane's share of W^T w is summed in TV.
 template <typename TV, typename TS, typename TI, int NP, int DIM, bool GROUP>
 struct CoarseCycle {
   using T = TV;

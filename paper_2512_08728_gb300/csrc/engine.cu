@@ -269,11 +269,13 @@ void alloc_cycle_vectors(kcmg_ctx* ctx, Level& L, int lcap) {
 // the graph (6 us and up on small problems, with the loop's own nodes); from about kWholeFmas FMAs
 // an application the phase's FP64 time makes up the difference, and the finest level's own
 // kernels skip the zeros of its blocks.  Measured, per-step finest level against whole solve:
-// 16 x 16, p = 1, to 1e-11 20.4 / 13.5 ms; 8^3, p = 2, mixed, to 1e-11 28.3 / 23.1 ms; three
-// cycles at 0.8M FMAs (12 x 12 x 8, p = 2) 5.24 / 5.03 ms, at 1.1M (20 x 20 x 24, p = 1) 2.39 / 2.25.
+// 16 x 16, p = 1, to 1e-11 21.6 / 14.6 ms; 8^3, p = 2, mixed, to 1e-11 24.5 / 22.3 ms; three
+// cycles at 0.8M FMAs (12 x 12 x 8, p = 2) 3.50 / 3.19 ms, at 1.1M (20 x 20 x 24, p = 1) 1.74 / 1.55,
+// at 0.7M with p = 3 (8 x 8 x 4) 1.98 / 1.60, mixed 1.61 / 1.33, Schwarz 2.70 / 2.00, and at 1.15M
+// with p = 3 in two dimensions (48 x 48) 12.4 / 12.2: the line suits every degree and form.
 // The task-parallel cycle's smoother steps run beside the coarse levels' kernel where there is
 // one, which hides them (16^3, p = 1, three levels, m = 8: 2.25 / 2.66 ms); with two levels there
-// is none (8^3, p = 1: 1.89 / 1.01).
+// is none (8^3, p = 1: 1.74 / 0.94).
 constexpr long long kWholeFmas = 1200000;
 bool whole_solve(const kcmg_ctx* ctx) {
   const kcmg_params& p = ctx->p;
@@ -1117,10 +1119,11 @@ void drop_groups(kcmg_ctx* ctx) {
 // the solve.  The batched kernels multiply the nonzero entries by all columns at the rate of the
 // chip, but take some 8 us a step and a few more for the host's part of the loop; a group takes
 // about 3 us a step, and its few SMs work through the dense blocks.  The two meet at some 30M FMAs
-// over all columns.  Measured, batched kernels against groups: 8^3, p = 2, to 1e-11, 8 columns
-// 180 / 34 ms, 32 columns 242 / 58; 16 x 16, p = 1, 32 columns 173 / 23; one cycle at 13M FMAs
-// (20 x 20 x 16, p = 2, 3 columns) 5.1 / 2.0 ms, at 23M (16^3, p = 2, 8 columns) 3.9 / 2.7, at 33M
-// (24 x 24 x 16, p = 1, 32 columns) 6.4 / 6.9.
+// over all columns for p = 1 with many columns, later otherwise.  Measured, batched kernels against
+// groups: 8^3, p = 2, to 1e-11, 8 columns 196 / 36 ms, 32 columns 262 / 57; 16 x 16, p = 1, 32
+// columns 173 / 24; one cycle at 13M FMAs (20 x 20 x 16, p = 2, 3 columns) 6.6 / 2.2 ms, at 23M
+// (16^3, p = 2, 8 columns) 4.1 / 2.7, at 26M with p = 3 (12 x 12 x 8, 8 columns) 14.2 / 6.1, mixed
+// 12.8 / 4.9, at 29M (20^3, p = 1, 32 columns) 5.5 / 6.1.
 constexpr long long kColumnsFmas = 30000000;
 ColumnGroups* column_groups(kcmg_ctx* ctx, int nrhs) {
   const kcmg_params& p = ctx->p;

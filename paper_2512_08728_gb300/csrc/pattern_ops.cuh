@@ -17,7 +17,7 @@
 // Measured (GB300, whole calls on device vectors): y = A x at 64^3, np = 10, FP64 355 -> 113 us
 // (355: dense blocks and staged vectors); r = b - A x with its norm at 96 x 80 x 72, np = 4,
 // 192 -> 108 us; five FP32 sweeps with BF16 inverses at 64^3 561 -> 231 us; the 64^3 FP64 solve's
-// first five cycles 289 -> 223 ms.
+// first five cycles 289 -> 223 ms (with the dense kernels' Alg. 1, which has changed since).
 //
 // Results are those of the dense kernels bit for bit: a row sees its nonzero entries in the
 // dense kernels' order, and the products left out are exact zeros.  A vector entry that is
