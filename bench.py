@@ -62,8 +62,8 @@ STRETCHED_ASYNC_M = 12
 # Level-0 cycles and level-1 iterations of the headline FP64 solve of this workload (seed 0,
 # LMAX = 400, m = 12), measured on GB300; the reference arm (a separate process)
 # extrapolates its bounded sample with them.
-GPU_LEVEL1_ITERS_FP64 = 1064
-GPU_CYCLES_FP64 = 54
+GPU_LEVEL1_ITERS_FP64 = 1044
+GPU_CYCLES_FP64 = 53
 
 
 def _peaks():
@@ -97,8 +97,8 @@ _GRAM_SOURCES = ["kernels.cu", "epilogue.cuh", "kcmg_internal.h", "reduce.cuh"]
 _GRAM_NOTE = ("ncu capture (dram__bytes_read.sum + dram__bytes_write.sum) of one level-0 launch on 48^3 "
               "p=2 with 199 basis vectors: %.3f GB per launch, scaled to this launch by (l + %d) N")
 TRAFFIC = {
-    "k_gram_dots": (0.0, "", _GRAM_SOURCES, _GRAM_NOTE % (0.0, 2)),
-    "k_gram_update": (0.0, "", _GRAM_SOURCES, _GRAM_NOTE % (0.0, 6)),
+    "k_gram_dots": (1787656944.0 / ((199 + 2) * 1105920), "feb6d0a095654d5c", _GRAM_SOURCES, _GRAM_NOTE % (1.788, 2)),
+    "k_gram_update": (1814737584.0 / ((199 + 6) * 1105920), "feb6d0a095654d5c", _GRAM_SOURCES, _GRAM_NOTE % (1.815, 6)),
 }
 
 
